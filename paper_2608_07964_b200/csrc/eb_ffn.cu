@@ -19,11 +19,19 @@
 // MMA issuer (leader CTA only) and TMEM owner, warps 2..9 = epilogue.  A stage is 48 KB per CTA (W0 | W1 |
 // up to 128 token rows of one 64-wide k-block, bf16, 128-byte swizzled K-major) for up to 1024 tensor-core
 // cycles; four stages.  TMA completions of both CTAs count on the leader's barrier; the tcgen05.commit
-// that frees a stage is delivered to both CTAs; no load is multicast.  The two accumulators fill TMEM
-// (2 x 256 fp32 columns), so the epilogue of a tile does not overlap the next tile's MMAs; eight epilogue
-// warps (two per TMEM lane quadrant, alternating 16-column chunks) keep that gap short and the producer
-// keeps prefetching through it.  The accumulator holds outputs in lanes and tokens in columns: an
-// epilogue warp transposes each 16-token chunk through 1 KB of shared memory and stores 16-byte vectors.
+// that frees a stage is delivered to both CTAs; no load is multicast.
+//
+// Epilogue against the next tile's MMAs.  The two accumulators of a tile of more than 128 columns fill TMEM
+// (2 x 256 fp32 columns).  What bounds such a tile is then how soon the accumulators come back: the eight
+// epilogue warps (two per lane quadrant, alternating 16-column chunks) read the whole first accumulator into
+// registers and hand it back, then the second one, and only then transpose and store; the MMA warp starts the
+// next tile with the first accumulator alone, over the k-blocks that the ring holds, and follows up with the
+// second.  Storing chunk by chunk before handing anything back kept the tensor pipe idle for 6100 cycles per
+// tile (of 36000 in gate/up, 29000 in down at H 2048, I 1408), this order for 1900: the expert pass of 49152
+// rows over 66 matrices went from 725 to 689 us.  Tiles of at most 128 columns take one half of TMEM in turn,
+// so their epilogue runs beside the next tile's MMAs (16-434 rows a group over 788 matrices: 2245 -> 2236 us).
+// The accumulator holds outputs in lanes and tokens in columns: an epilogue warp transposes each 16-token
+// chunk through 1 KB of shared memory and stores 16-byte vectors.
 //
 // Tiles: a device-built list (plan_kernel, fill_kernel).  Tiles of one group are weight-tile-major and
 // token-tile-minor, so pairs working side by side share the weight tile in L2 and every weight byte leaves
@@ -47,9 +55,12 @@ constexpr int kStageBytes = 2 * kWBytes + kTBytes;             // W0 | W1 | toke
 constexpr int kRingBytes = kStages * kStageBytes;
 constexpr int kEpiWarps = 8;
 constexpr int kThreads = 64 + 32 * kEpiWarps;
+constexpr int kEpiChunks = 256 / 16 / 2;                       // 16-column chunks of an epilogue warp (two warps per quadrant)
 constexpr size_t kSmemBytes = (size_t)kRingBytes + 1024 /*alignment slack*/ + 256 /*barriers*/ + kEpiWarps * 2048 /*transposes*/;
 static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
 constexpr int kTmemCols = 512;
+constexpr int kTmemHalf = 256;                                 // a narrow tile's two accumulators share one half of TMEM
+constexpr int kNarrowCols = kTmemHalf / 2;                     // ... which takes tiles of up to 128 columns
 constexpr int kTileRows = 256;                                 // token rows of a tile at most
 constexpr int kFeat1 = 256;                                    // outputs of a gate/up tile
 constexpr int kFeat2 = 512;                                    // outputs of a down tile
@@ -198,6 +209,57 @@ __device__ __forceinline__ int merged_cols(int n_slots) { return ((n_slots + 1) 
 // Columns of a tile from its list entry (y = rows, or minus the slot count of a merged tile).
 __device__ __forceinline__ int entry_cols(int y) { return y < 0 ? merged_cols(-y) : tile_cols(y); }
 
+// Which part of TMEM a tile's two accumulators take.  TMEM is two halves of 256 columns, each with a full and an
+// empty barrier.  A tile of more than 128 columns takes both (one accumulator in each); a narrower one takes the
+// half that is next in turn, so that its epilogue runs while the next tile's MMAs fill the other half.  The MMA
+// warp and the epilogue warps walk the same tiles and so reach the same placement and the same barrier phases.
+struct TmemTurn {
+  uint32_t used = 0;      // bits 0, 1: halves of the current tile; bit 2: the half whose turn is next
+  uint32_t phases = 3;    // bit h: phase parity of the current use of half h (the first use has parity 0)
+  __device__ __forceinline__ void take(int cols) {
+    const uint32_t next = used >> 2;
+    used = cols > kNarrowCols ? (3u | (next << 2)) : ((1u << next) | ((next ^ 1u) << 2));
+    phases ^= used & 3u;
+  }
+  __device__ __forceinline__ bool wide() const { return (used & 3u) == 3u; }
+  __device__ __forceinline__ int half() const { return (int)((used >> 1) & 1u); }   // of a narrow tile
+  __device__ __forceinline__ uint32_t parity(int h) const { return (phases >> h) & 1u; }
+  __device__ __forceinline__ uint32_t col0() const { return (used & 3u) == 2u ? kTmemHalf : 0; }
+  __device__ __forceinline__ uint32_t step() const { return (used & 3u) == 3u ? kTmemHalf : kNarrowCols; }
+};
+
+// An epilogue warp whose TMEM reads are complete (wait::ld) hands its part of an accumulator back to the MMA warp.
+__device__ __forceinline__ void release_tmem(uint32_t bar, int lane) {
+  tc_fence_before();
+  __syncwarp();
+  if (lane == 0) mbar_arrive_cluster(map_to_cta(bar, 0));
+}
+
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+__device__ __forceinline__ bf16 low_half(uint32_t v) { return __ushort_as_bfloat16((unsigned short)(v & 0xffffu)); }
+__device__ __forceinline__ bf16 high_half(uint32_t v) { return __ushort_as_bfloat16((unsigned short)(v >> 16)); }
+
+// Chunks at columns 0, 32, .. below n_cols of an accumulator, rounded to bf16, two tokens per word.  Two loads are in flight at a time.
+template <int N>
+__device__ __forceinline__ void drain_packed(uint32_t acc, int n_cols, uint32_t (&out)[N][8]) {
+#pragma unroll
+  for (int i = 0; i < N; i += 2) {
+    if (32 * i >= n_cols) break;
+    uint32_t a[2][16];
+    tmem_ld16(acc + 32 * i, a[0]);
+    tmem_ld16(acc + 32 * (i + 1), a[1]);   // within the accumulator's 128 or 256 columns; unused if beyond n_cols
+    tmem_ld_wait();
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      out[i][j] = pack_bf16(__uint_as_float(a[0][2 * j]), __uint_as_float(a[0][2 * j + 1]));
+      out[i + 1][j] = pack_bf16(__uint_as_float(a[1][2 * j]), __uint_as_float(a[1][2 * j + 1]));
+    }
+  }
+}
+
 // ---- the grouped GEMM kernel -----------------------------------------------------------------
 // PHASE 1: gate/up + SwiGLU (256 outputs per tile);  PHASE 2: down (512 outputs per tile).
 // A tile is an int4 of the list: x = first row, y = rows (1..256), z = weight matrix, w = output tile.
@@ -222,9 +284,10 @@ ffn_kernel(const __grid_constant__ CUtensorMap tmT128, const __grid_constant__ C
   auto t_addr = [&](int s) { return base + s * kStageBytes + 2 * kWBytes; };
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
   auto empty_bar = [&](int s) { return bar0 + 8u * (NS + s); };
-  const uint32_t tfull_bar = bar0 + 8u * (2 * NS), tempty_bar = bar0 + 8u * (2 * NS + 1);
-  volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(bars + 2 * NS + 2);
-  volatile int* s_abort = reinterpret_cast<volatile int*>(bars + 2 * NS + 3);
+  auto tfull_bar = [&](int h) { return bar0 + 8u * (2 * NS + h); };
+  auto tempty_bar = [&](int h) { return bar0 + 8u * (2 * NS + 2 + h); };
+  volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(bars + 2 * NS + 4);
+  volatile int* s_abort = reinterpret_cast<volatile int*>(bars + 2 * NS + 5);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();   // CTA 0 of a pair is the leader
@@ -233,8 +296,10 @@ ffn_kernel(const __grid_constant__ CUtensorMap tmT128, const __grid_constant__ C
       mbar_init(full_bar(s), 1);    // the leader's arrive + all bytes of the stage of both CTAs
       mbar_init(empty_bar(s), 1);   // one tcgen05.commit (delivered to both CTAs)
     }
-    mbar_init(tfull_bar, 1);                // one tcgen05.commit
-    mbar_init(tempty_bar, 2 * kEpiWarps);   // one arrival per epilogue warp of both CTAs (leader's barrier)
+    for (int h = 0; h < 2; ++h) {
+      mbar_init(tfull_bar(h), 1);                // one tcgen05.commit
+      mbar_init(tempty_bar(h), 2 * kEpiWarps);   // one arrival per epilogue warp of both CTAs (leader's barrier)
+    }
     *s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     prefetch_tmap(&tmT128);
@@ -326,23 +391,60 @@ ffn_kernel(const __grid_constant__ CUtensorMap tmT128, const __grid_constant__ C
     if (lane == 0 && rank == 0) {
       int stage = 0;
       uint32_t phase = 0;
-      int local = -1;
+      TmemTurn turn;
       for (int r = 0; r * n_pairs < n_work; ++r) {
         const int w = tile_of_round(r);
         if (w >= n_work) continue;
-        ++local;
         const int4 it = __ldg(work + w);
-        const uint32_t idesc = kIdescBase | ((uint32_t)(entry_cols(it.y) >> 3) << 17);
-        if (!mbar_wait(tempty_bar, (uint32_t)(local & 1) ^ 1u, s_abort, status)) goto done;
-        tc_fence_after();
-        for (int kb = 0; kb < num_kb; ++kb) {
+        const int cols = entry_cols(it.y);
+        const uint32_t idesc = kIdescBase | ((uint32_t)(cols >> 3) << 17);
+        turn.take(cols);
+        const uint32_t acc0 = tmem_base + turn.col0(), acc1 = acc0 + turn.step();
+        int kb = 0;
+        if (turn.wide()) {
+          // the epilogue hands the first accumulator back well before the second: the k-blocks that fit the ring
+          // are multiplied into the first one, then into the second, then both go on together
+          const int lead = num_kb < NS ? num_kb : NS;
+          if (!mbar_wait(tempty_bar(0), turn.parity(0) ^ 1u, s_abort, status)) goto done;
+          tc_fence_after();
+          int st = stage;
+          uint32_t ph = phase;
+          for (int i = 0; i < lead; ++i) {
+            if (!mbar_wait(full_bar(st), ph, s_abort, status)) goto done;
+            tc_fence_after();
+            const uint64_t d0 = smem_desc(w0_addr(st)), dt = smem_desc(t_addr(st));
+#pragma unroll
+            for (int k = 0; k < BK / 16; ++k) umma_pair_bf16(acc0, d0 + 2 * k, dt + 2 * k, idesc, (i | k) != 0 ? 1u : 0u);
+            if (++st == NS) {
+              st = 0;
+              ph ^= 1u;
+            }
+          }
+          if (!mbar_wait(tempty_bar(1), turn.parity(1) ^ 1u, s_abort, status)) goto done;
+          tc_fence_after();
+          for (; kb < lead; ++kb) {
+            const uint64_t d1 = smem_desc(w1_addr(stage)), dt = smem_desc(t_addr(stage));
+#pragma unroll
+            for (int k = 0; k < BK / 16; ++k) umma_pair_bf16(acc1, d1 + 2 * k, dt + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
+            umma_pair_commit(empty_bar(stage));
+            if (++stage == NS) {
+              stage = 0;
+              phase ^= 1u;
+            }
+          }
+        } else {
+          const int h = turn.half();
+          if (!mbar_wait(tempty_bar(h), turn.parity(h) ^ 1u, s_abort, status)) goto done;
+          tc_fence_after();
+        }
+        for (; kb < num_kb; ++kb) {
           if (!mbar_wait(full_bar(stage), phase, s_abort, status)) goto done;
           tc_fence_after();
           const uint64_t d0 = smem_desc(w0_addr(stage)), d1 = smem_desc(w1_addr(stage)), dt = smem_desc(t_addr(stage));
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k) {
-            umma_pair_bf16(tmem_base, d0 + 2 * k, dt + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
-            umma_pair_bf16(tmem_base + 256, d1 + 2 * k, dt + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
+            umma_pair_bf16(acc0, d0 + 2 * k, dt + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
+            umma_pair_bf16(acc1, d1 + 2 * k, dt + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
           }
           umma_pair_commit(empty_bar(stage));   // the stage is reusable in both CTAs once these MMAs have read it
           if (++stage == NS) {
@@ -350,7 +452,13 @@ ffn_kernel(const __grid_constant__ CUtensorMap tmT128, const __grid_constant__ C
             phase ^= 1u;
           }
         }
-        umma_pair_commit(tfull_bar);   // both accumulators complete
+        // both accumulators complete
+        if (turn.wide()) {
+          umma_pair_commit(tfull_bar(0));
+          umma_pair_commit(tfull_bar(1));
+        } else {
+          umma_pair_commit(tfull_bar(turn.half()));
+        }
       }
     }
   } else {
@@ -359,26 +467,61 @@ ffn_kernel(const __grid_constant__ CUtensorMap tmT128, const __grid_constant__ C
     const int chunk0 = ((warp - 2) >> 2) * 16;   // the two warps of a quadrant take alternate 16-column chunks
     const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16);
     bf16* tile = reinterpret_cast<bf16*>(smem + kRingBytes + 256) + (warp - 2) * 1024;   // 2 KB per epilogue warp
-    int local = -1;
+    TmemTurn turn;
     for (int r = 0; r * n_pairs < n_work; ++r) {
       const int w = tile_of_round(r);
       if (w >= n_work) continue;
-      ++local;
       const int4 it = __ldg(work + w);
+      turn.take(entry_cols(it.y));
       const bool merged = it.y < 0;
       const int n_cols = merged ? -it.y * kSlotRows : it.y;   // columns that may hold rows to store
       // one lane waits, the outcome is made warp-uniform before any .aligned instruction
       int ok = 1;
-      if (lane == 0) ok = mbar_wait(tfull_bar, (uint32_t)(local & 1), s_abort, status) ? 1 : 0;
+      if (lane == 0) {
+        const int h = turn.wide() ? 0 : turn.half();
+        ok = mbar_wait(tfull_bar(h), turn.parity(h), s_abort, status) ? 1 : 0;
+        if (ok && turn.wide()) ok = mbar_wait(tfull_bar(1), turn.parity(1), s_abort, status) ? 1 : 0;
+      }
       ok = __shfl_sync(0xffffffffu, ok, 0);
       if (!ok) goto done;
       tc_fence_after();
+      const uint32_t acc0 = taddr + turn.col0(), acc1 = acc0 + turn.step();
       // this warp's 32 outputs start at fbase; a 16-token chunk is transposed through shared memory so that
       // global stores are 16-byte vectors: lane -> (token lane / 4 (+8), outputs 8 (lane % 4) .. +7)
       const int fbase = (PHASE == 1 ? it.w * kFeat1 : it.w * kFeat2) + (int)rank * 128 + q * 32;
       const int fcol = fbase + (lane & 3) * 8;
-#pragma unroll 1
-      for (int c0 = chunk0; c0 < n_cols; c0 += 32) {
+      // Both accumulators move to registers first, the first one as it is, the second one combined (gate/up) or
+      // rounded (down) on the way; each is handed back as soon as it is read, the stores come after.
+      uint32_t r0[kEpiChunks][PHASE == 1 ? 16 : 8];   // first accumulator; then outputs, two tokens per word, in [0..7]
+      uint32_t r1[PHASE == 1 ? 1 : kEpiChunks][8];
+      if constexpr (PHASE == 1) {
+#pragma unroll
+        for (int i = 0; i < kEpiChunks; ++i) {
+          if (chunk0 + 32 * i >= n_cols) break;
+          tmem_ld16(acc0 + chunk0 + 32 * i, r0[i]);
+        }
+        tmem_ld_wait();
+        if (turn.wide()) release_tmem(tempty_bar(0), lane);
+#pragma unroll
+        for (int i = 0; i < kEpiChunks; ++i) {
+          if (chunk0 + 32 * i >= n_cols) break;
+          uint32_t b[16];
+          tmem_ld16(acc1 + chunk0 + 32 * i, b);
+          tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            r0[i][j] = pack_bf16(silu_mul(r0[i][2 * j], b[2 * j]), silu_mul(r0[i][2 * j + 1], b[2 * j + 1]));
+        }
+      } else {
+        drain_packed(acc0 + chunk0, n_cols - chunk0, r0);
+        if (turn.wide()) release_tmem(tempty_bar(0), lane);
+        drain_packed(acc1 + chunk0, n_cols - chunk0, r1);
+      }
+      release_tmem(tempty_bar(turn.wide() ? 1 : turn.half()), lane);
+#pragma unroll
+      for (int i = 0; i < kEpiChunks; ++i) {
+        const int c0 = chunk0 + 32 * i;
+        if (c0 >= n_cols) break;
         // rows of this chunk: columns c0 .. c0 + 15 are rows row0 .. row0 + n_here - 1 (a merged tile: one slot)
         int row0 = it.x + c0, n_here = min(16, it.y - c0);
         if (merged) {
@@ -386,18 +529,13 @@ ffn_kernel(const __grid_constant__ CUtensorMap tmT128, const __grid_constant__ C
           row0 = sl.x;
           n_here = sl.y;
         }
-        uint32_t a[16], b[16];
-        tmem_ld16(taddr + c0, a);
-        tmem_ld16(taddr + 256 + c0, b);
-        tmem_ld_wait();
-        if (PHASE == 1) {
 #pragma unroll
-          for (int j = 0; j < 16; ++j) tile[j * 32 + lane] = __float2bfloat16_rn(silu_mul(a[j], b[j]));
-        } else {
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            tile[j * 32 + lane] = __float2bfloat16_rn(__uint_as_float(a[j]));
-            tile[512 + j * 32 + lane] = __float2bfloat16_rn(__uint_as_float(b[j]));
+        for (int j = 0; j < 8; ++j) {
+          tile[2 * j * 32 + lane] = low_half(r0[i][j]);
+          tile[(2 * j + 1) * 32 + lane] = high_half(r0[i][j]);
+          if (PHASE == 2) {
+            tile[512 + 2 * j * 32 + lane] = low_half(r1[i][j]);
+            tile[512 + (2 * j + 1) * 32 + lane] = high_half(r1[i][j]);
           }
         }
         __syncwarp();
@@ -413,10 +551,6 @@ ffn_kernel(const __grid_constant__ CUtensorMap tmT128, const __grid_constant__ C
         }
         __syncwarp();
       }
-      // all TMEM reads of this warp are complete (wait::ld above): hand the accumulators back
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(map_to_cta(tempty_bar, 0));
     }
   }
 

@@ -473,6 +473,14 @@ def test_group_sizes_around_the_tile_boundaries(H, I):
     assert sorted(np.diff(ref["group_off"]).tolist()) == sorted(sizes)
 
 
+@pytest.mark.parametrize("H,I", [(72, 2056), (2056, 72), (328, 2056)])
+def test_tile_sizes_mixed_over_many_tiles_per_pair(H, I):
+    """The same groups with enough output tiles that every CTA pair works through several of them, tiles of more than
+    128 columns (both halves of TMEM) and narrower ones (one half in turn) one after the other: with fewer k-blocks
+    than the ring has stages (72), and with more (328, 2056)."""
+    test_group_sizes_around_the_tile_boundaries(H, I)
+
+
 # ----------------------------------------------------------------------------------- failure reporting
 def test_bounded_wait_gives_up_and_reports_without_harming_the_context():
     B = _binding()
