@@ -87,8 +87,7 @@ static size_t carve(eb_ctx* c, char* base) {
   c->max_chunks = (g.max_tokens + 31) / 32 + EB_MAX_MB;
   int rows = ebi_rows_cap(c), gcap = ebi_groups_cap(c);
   c->max_tiles = rows / 256 + gcap;                    // a group of r rows has ceil(r / 256) tiles
-  c->max_work1 = c->max_tiles * ((g.I + 255) / 256);   // 256 outputs per gate/up tile
-  c->max_work2 = c->max_tiles * ((g.H + 511) / 512);   // 512 outputs per down tile
+  c->max_work = c->max_tiles * ((g.I + 255) / 256 + (g.H + 511) / 512);   // 256 outputs per gate/up tile, 512 per down tile
   c->chunk_hist = (int32_t*)take(sizeof(int32_t) * (size_t)c->max_chunks * g.E);
   c->chunk_base = (int32_t*)take(sizeof(int32_t) * (size_t)c->max_chunks * g.E);
   c->group_size = (int32_t*)take(sizeof(int32_t) * (size_t)gcap);
@@ -98,8 +97,8 @@ static size_t carve(eb_ctx* c, char* base) {
   c->order = (int32_t*)take(sizeof(int32_t) * (size_t)gcap);
   c->tile_pref = (int32_t*)take(sizeof(int32_t) * (size_t)(gcap + 1));
   c->work_count = (int32_t*)take(sizeof(int32_t) * 16);
-  c->work1 = (int4*)take(sizeof(int4) * (size_t)c->max_work1);
-  c->work2 = (int4*)take(sizeof(int4) * (size_t)c->max_work2);
+  c->work = take(32 * (size_t)c->max_work);
+  c->tile_ready = (int32_t*)take(sizeof(int32_t) * (size_t)c->max_tiles);
   c->slots = (int2*)take(sizeof(int2) * 16 * (size_t)c->max_tiles);
   c->act = (bf16*)take(sizeof(bf16) * (size_t)rows * g.I);
   return off;

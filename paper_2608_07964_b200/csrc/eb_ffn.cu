@@ -1,11 +1,12 @@
 // eb_expert_ffn_grouped: expert_i of Eq. 1 (bias-free SwiGLU MLP) for every (layer, expert) group
 // of a step in one grouped pass on the 5th-generation tensor cores.
 //
-// Two persistent launches over a device-built tile list (ragged groups, no padding rows in memory):
+// One persistent launch over a device-built tile list (ragged groups, no padding rows in memory), gate/up
+// tiles first, down tiles after them in the same order of groups:
 //   gate/up : act[r, i] = silu(sum_h xp[r,h] Wg[i,h]) * (sum_h xp[r,h] Wu[i,h])      (bf16 out)
 //   down    : yp[r, h]  = sum_i act[r,i] Wd[h,i]                                      (bf16 out)
 //
-// Both run ffn_kernel on CTA pairs (2-CTA clusters, one CTA per SM).  The WEIGHTS are the M operand of
+// ffn_kernel runs on CTA pairs (2-CTA clusters, one CTA per SM).  The WEIGHTS are the M operand of
 // tcgen05.mma cta_group::2 (M = 256 weight rows, 128 per CTA) and the TOKEN rows of the tile are the N
 // operand: N = the tile's rows rounded up to 16, at most 256.  Tensor-core work, shared-memory fill and
 // TMEM columns of a tile therefore follow the rows it really holds - a group of 45 rows costs a 48-column
@@ -38,11 +39,19 @@
 // HBM once per group.  The D replicas of a shared expert (one group per virtual device, all reading the
 // same matrix) are merged when all are small: their rows are packed into common tiles in slots of 16
 // rows, so the matrix is streamed once per step instead of D times.  Groups are listed widest tiles
-// first and the list is dealt out in rounds of alternating direction, which gives every pair nearly the
-// same total cost without a dynamic scheduler.
+// first; every pair takes the next tile of the list when it is nearly through with the one before (a dealer
+// thread per pair claims it and leaves it in both CTAs' mailboxes).  A down tile starts when the gate/up tiles
+// of its rows are counted complete; those were dealt earlier, to pairs that are running, so every wait ends.
+// With a launch per phase and tiles dealt out beforehand, pairs that were through waited for the last one twice
+// per step (20 us of 240 in gate/up, 13 of 130 in down at 133 matrices of 3 x 2048 x 1408) and the down launch
+// began with an empty ring: the expert pass took 372 us there, 116 at 126 matrices of 3 x 1000 x 712 and 109 at
+// 32 of the former, this way 361, 105 and 102.
 //
 // Every wait on an mbarrier is bounded: on expiry the kernel records EB_ERR_TIMEOUT in the
 // context status word, lets copies in flight land, frees its TMEM and returns.
+#include <cstddef>
+#include <type_traits>
+
 #include "eb_internal.cuh"
 
 namespace {
@@ -53,10 +62,10 @@ constexpr int kWBytes = 128 * BK * 2;                          // 128 weight row
 constexpr int kTBytes = 128 * BK * 2;                          // up to 128 token rows of one k-block
 constexpr int kStageBytes = 2 * kWBytes + kTBytes;             // W0 | W1 | token rows
 constexpr int kRingBytes = kStages * kStageBytes;
-constexpr int kEpiWarps = 8;
+constexpr int kEpiWarps = 8;                                   // two per TMEM lane quadrant
 constexpr int kThreads = 64 + 32 * kEpiWarps;
-constexpr int kEpiChunks = 256 / 16 / 2;                       // 16-column chunks of an epilogue warp (two warps per quadrant)
-constexpr size_t kSmemBytes = (size_t)kRingBytes + 1024 /*alignment slack*/ + 256 /*barriers*/ + kEpiWarps * 2048 /*transposes*/;
+constexpr int kChunkStep = 16 * (kEpiWarps / 4);               // columns between two chunks of an epilogue warp
+constexpr size_t kSmemBytes = (size_t)kRingBytes + 1024 /*alignment slack*/ + 256 /*barriers*/ + kEpiWarps * 1024 /*transposes*/;
 static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
 constexpr int kTmemCols = 512;
 constexpr int kTmemHalf = 256;                                 // a narrow tile's two accumulators share one half of TMEM
@@ -67,6 +76,10 @@ constexpr int kFeat2 = 512;                                    // outputs of a d
 constexpr int kSlotRows = 16;                                  // rows of one slot of a merged tile
 constexpr int kMergeSlots = kTileRows / kSlotRows;             // slots of a merged tile at most
 constexpr int kMergeMaxRows = 64;                              // replicas of a shared expert are merged when none has more rows
+constexpr int kItems = 2;                                      // mailbox slots of a CTA (tiles dealt ahead)
+constexpr int kParts = 4;                                      // tiles whose epilogues may be under way at once in a CTA: a tile is dealt
+                                                               // only when every warp has begun the one kItems before it, so at most kItems + 1
+constexpr int kAskAhead = 16;                                  // k-blocks before the end of a tile at which its successor is asked for
 constexpr long long kSpinLimitCycles = 4000000000LL;
 
 // ---- PTX wrappers ----------------------------------------------------------------------------
@@ -89,13 +102,24 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Bounded wait: false if the limit expired or another thread of the CTA already gave up.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* s_abort, int* status,
-                                          long long limit = kSpinLimitCycles) {
-  if (mbar_try(bar, parity)) return true;
+__device__ __forceinline__ bool mbar_try_cluster(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// Bounded waits: false if the limit expired or another thread of the CTA already gave up.
+template <typename Try>
+__device__ __forceinline__ bool bounded_wait(Try try_once, volatile int* s_abort, int* status, long long limit = kSpinLimitCycles) {
+  if (try_once()) return true;
   const long long t0 = clock64();
   for (uint32_t spin = 1;; ++spin) {
-    if (mbar_try(bar, parity)) return true;
+    if (try_once()) return true;
     if ((spin & 63u) == 0u) {
       if (*s_abort) return false;
       if (clock64() - t0 > limit) {
@@ -105,6 +129,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
       }
     }
   }
+}
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* s_abort, int* status,
+                                          long long limit = kSpinLimitCycles) {
+  return bounded_wait([&] { return mbar_try(bar, parity); }, s_abort, status, limit);
+}
+// the same for a barrier that the peer CTA's ordinary stores arrive with
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* s_abort, int* status) {
+  return bounded_wait([&] { return mbar_try_cluster(bar, parity); }, s_abort, status);
 }
 
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
@@ -125,9 +157,33 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// Says "done with it" to a barrier of the pair: nothing this thread wrote is handed over.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
+// The same with what this thread wrote before it.  Only the tile dealer uses it: a release at cluster scope waits for
+// the thread's earlier accesses, and in the producer, MMA and epilogue warps that cost 1 to 2 us per tile.
+__device__ __forceinline__ void mbar_arrive_release_cluster(uint32_t cluster_addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+__device__ __forceinline__ void st_cluster(uint32_t cluster_addr, const int4& v) {
+  asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+__device__ __forceinline__ int4 ld_shared(uint32_t addr) {
+  int4 v;
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ int ld_acquire(const int* p) {
+  int v;
+  asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void red_release(int* p) {
+  asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p) : "memory");
+}
+// orders ordinary memory accesses with those of the TMA unit
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
 // TMA loads whose completion is counted on a barrier that may live in the peer CTA (the data goes to the
 // issuing CTA only)
 __device__ __forceinline__ void tma_pair_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
@@ -179,6 +235,12 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr)
       : "memory");
+}
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
@@ -242,42 +304,143 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 __device__ __forceinline__ bf16 low_half(uint32_t v) { return __ushort_as_bfloat16((unsigned short)(v & 0xffffu)); }
 __device__ __forceinline__ bf16 high_half(uint32_t v) { return __ushort_as_bfloat16((unsigned short)(v >> 16)); }
 
-// Chunks at columns 0, 32, .. below n_cols of an accumulator, rounded to bf16, two tokens per word.  Two loads are in flight at a time.
+// Chunks at columns 0, kChunkStep, .. of an accumulator, rounded to bf16, two tokens per word.
 template <int N>
-__device__ __forceinline__ void drain_packed(uint32_t acc, int n_cols, uint32_t (&out)[N][8]) {
+__device__ __forceinline__ void drain_packed(uint32_t acc, uint32_t (&out)[N][8]) {
+  constexpr int P = N < 2 ? 1 : 2;   // loads in flight
 #pragma unroll
-  for (int i = 0; i < N; i += 2) {
-    if (32 * i >= n_cols) break;
-    uint32_t a[2][16];
-    tmem_ld16(acc + 32 * i, a[0]);
-    tmem_ld16(acc + 32 * (i + 1), a[1]);   // within the accumulator's 128 or 256 columns; unused if beyond n_cols
+  for (int i = 0; i < N; i += P) {
+    uint32_t a[P][16];
+#pragma unroll
+    for (int k = 0; k < P; ++k) tmem_ld16(acc + kChunkStep * (i + k), a[k]);
     tmem_ld_wait();
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      out[i][j] = pack_bf16(__uint_as_float(a[0][2 * j]), __uint_as_float(a[0][2 * j + 1]));
-      out[i + 1][j] = pack_bf16(__uint_as_float(a[1][2 * j]), __uint_as_float(a[1][2 * j + 1]));
-    }
+    for (int k = 0; k < P; ++k)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) out[i + k][j] = pack_bf16(__uint_as_float(a[k][2 * j]), __uint_as_float(a[k][2 * j + 1]));
   }
 }
 
 // ---- the grouped GEMM kernel -----------------------------------------------------------------
-// PHASE 1: gate/up + SwiGLU (256 outputs per tile);  PHASE 2: down (512 outputs per tile).
-// A tile is an int4 of the list: x = first row, y = rows (1..256), z = weight matrix, w = output tile.
-// y < 0 marks a merged tile of -y slots of 16 rows each, described by slots[x ..): (first row, rows).
-template <int PHASE>
+// One entry of the tile list.
+struct Tile {
+  int row;      // first row, or first slot of a merged tile
+  int rows;     // rows (1 .. 256); -n for a merged tile of n slots of 16 rows, slots[row ..): (first row, rows)
+  int w;        // weight matrix; negative: the list has ended
+  int out;      // output tile
+  int phase;    // 1: gate/up + SwiGLU (256 outputs per tile);  2: down (512 outputs per tile)
+  int done;     // the token tile this one belongs to: entry of `ready`
+  int need;     // phase 2: arrivals on that entry after which the rows of the intermediate are all written (0: they are)
+  int pad;
+};
+static_assert(sizeof(Tile) == 32, "two 16-byte words");
+
+// Token-row boxes of 128 / 64 / 32 / 16 / 8 rows over one activation tensor.
+struct TokenMaps {
+  CUtensorMap box[5];
+};
+struct FfnParams {
+  TokenMaps xp, act;                 // inputs of the two phases
+  CUtensorMap gate, up, down;        // with the above kMaps tensor maps in a row
+  const Tile* work;                  // the list: gate/up tiles, then down tiles
+  const int2* slots;
+  const int32_t* work_count;         // [0], [1]: tiles of the two phases
+  int32_t* next;                     // tiles dealt out beyond the first of every pair (second entry: of a launch of part 2)
+  int32_t* ready;                    // per token tile: arrivals, one per CTA for every finished gate/up tile
+  bf16 *act_out, *yp;
+  int H, I;
+  int max_work;                      // capacity of the list
+  int part;                          // 0: the whole list; 1, 2: the tiles of that phase only
+  int* status;
+};
+
+constexpr int kMaps = 13;
+static_assert(offsetof(FfnParams, down) == (kMaps - 1) * sizeof(CUtensorMap), "the maps are prefetched as an array");
+
+// Chunks of 16 token columns of a finished tile: registers -> transposed through shared memory -> rows.  NC chunks
+// of this warp are read, of which those below the tile's columns hold rows (every chunk read lies in the accumulator).
+// A chunk's rows: columns c0 .. c0 + 15 are rows row0 .. row0 + n_here - 1 (a merged tile: one slot).
+// Global stores are 16-byte vectors: lane -> (token lane / 4 (+8), outputs 8 (lane % 4) .. +7).
+template <int PHASE, int NC>
+__device__ __forceinline__ void epilogue_tile(const Tile& it, const TmemTurn& turn, uint32_t taddr, int chunk0, int lane, int fbase,
+                                              bf16* tile, const int2* __restrict__ slots, bf16* __restrict__ out, int n_out,
+                                              uint32_t tempty0, uint32_t tempty1) {
+  const bool merged = it.rows < 0;
+  const int n_cols = merged ? -it.rows * kSlotRows : it.rows;   // columns that may hold rows to store
+  const uint32_t acc0 = taddr + turn.col0() + chunk0, acc1 = acc0 + turn.step();
+  // chunk i of one accumulator, two tokens per word, to its rows; its outputs start at column f
+  auto store_chunk = [&](const uint32_t* v, int i, int f) {
+    const int c0 = chunk0 + kChunkStep * i;
+    if (c0 < n_cols) {
+      int row0 = it.row + c0, n_here = min(16, it.rows - c0);
+      if (merged) {
+        const int2 sl = __ldg(slots + it.row + (c0 >> 4));
+        row0 = sl.x;
+        n_here = sl.y;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        tile[2 * j * 32 + lane] = low_half(v[j]);
+        tile[(2 * j + 1) * 32 + lane] = high_half(v[j]);
+      }
+      __syncwarp();
+      const int fcol = f + (lane & 3) * 8;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int tok = (lane >> 2) + 8 * h;
+        if (tok < n_here && fcol < n_out)
+          *reinterpret_cast<uint4*>(out + (size_t)(row0 + tok) * n_out + fcol) =
+              *reinterpret_cast<const uint4*>(tile + tok * 32 + (lane & 3) * 8);
+      }
+      __syncwarp();
+    }
+  };
+  // The accumulators move to registers, rounded (down) or combined (gate/up), and are handed back as soon as they are
+  // read; the stores come after.
+  const uint32_t tempty_last = turn.wide() || turn.half() ? tempty1 : tempty0;
+  if constexpr (PHASE == 1) {
+    uint32_t r[NC][16];   // the gate accumulator; then outputs in [0..7]
+#pragma unroll
+    for (int i = 0; i < NC; ++i) tmem_ld16(acc0 + kChunkStep * i, r[i]);
+    tmem_ld_wait();
+    if (turn.wide()) release_tmem(tempty0, lane);
+#pragma unroll
+    for (int i = 0; i < 2 * NC; ++i) {   // eight columns at a time: no register is left for more
+      uint32_t b[8];
+      uint32_t* const g = r[i / 2] + (i % 2) * 8;
+      tmem_ld8(acc1 + kChunkStep * (i / 2) + (i % 2) * 8, b);
+      tmem_ld_wait();
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        r[i / 2][(i % 2) * 4 + j] = pack_bf16(silu_mul(g[2 * j], b[2 * j]), silu_mul(g[2 * j + 1], b[2 * j + 1]));
+    }
+    release_tmem(tempty_last, lane);
+#pragma unroll
+    for (int i = 0; i < NC; ++i) store_chunk(r[i], i, fbase);
+  } else {
+    uint32_t r0[NC][8], r1[NC][8];
+    drain_packed(acc0, r0);
+    if (turn.wide()) release_tmem(tempty0, lane);
+    // half of it is stored while the next tile's first MMAs run, which makes room for the second accumulator
+#pragma unroll
+    for (int i = 0; i < NC / 2; ++i) store_chunk(r0[i], i, fbase);
+    drain_packed(acc1, r1);
+    release_tmem(tempty_last, lane);
+#pragma unroll
+    for (int i = NC / 2; i < NC; ++i) store_chunk(r0[i], i, fbase);
+#pragma unroll
+    for (int i = 0; i < NC; ++i) store_chunk(r1[i], i, fbase + 256);
+  }
+}
+
 __global__ void __launch_bounds__(kThreads, 1)
-ffn_kernel(const __grid_constant__ CUtensorMap tmT128, const __grid_constant__ CUtensorMap tmT64,
-           const __grid_constant__ CUtensorMap tmT32, const __grid_constant__ CUtensorMap tmT16,
-           const __grid_constant__ CUtensorMap tmT8, const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtensorMap tmW1,
-           const int4* __restrict__ work, const int2* __restrict__ slots, const int32_t* __restrict__ work_count,
-           bf16* __restrict__ out, int ld_out, int n_out, int k_total, int* status) {
+ffn_kernel(const __grid_constant__ FfnParams p) {
   EB_GRID_DEP_SYNC();
   constexpr int NS = kStages;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (base - raw);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kRingBytes);
   const uint32_t bar0 = base + (uint32_t)kRingBytes;
   auto w0_addr = [&](int s) { return base + s * kStageBytes; };
   auto w1_addr = [&](int s) { return base + s * kStageBytes + kWBytes; };
@@ -286,11 +449,20 @@ ffn_kernel(const __grid_constant__ CUtensorMap tmT128, const __grid_constant__ C
   auto empty_bar = [&](int s) { return bar0 + 8u * (NS + s); };
   auto tfull_bar = [&](int h) { return bar0 + 8u * (2 * NS + h); };
   auto tempty_bar = [&](int h) { return bar0 + 8u * (2 * NS + 2 + h); };
-  volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(bars + 2 * NS + 4);
-  volatile int* s_abort = reinterpret_cast<volatile int*>(bars + 2 * NS + 5);
+  auto item_full = [&](int i) { return bar0 + 8u * (2 * NS + 4 + i); };
+  auto item_empty = [&](int i) { return bar0 + 8u * (2 * NS + 4 + kItems + i); };
+  const uint32_t want_bar = bar0 + 8u * (2 * NS + 4 + 2 * kItems);
+  constexpr int kBarBytes = 8 * (2 * NS + 4 + 2 * kItems + 1);
+  static_assert(kBarBytes + 8 + 4 * kParts + sizeof(Tile) <= 192 && kItems * sizeof(Tile) <= 64, "256 bytes of barriers and mailbox");
+  volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(smem + kRingBytes + kBarBytes);
+  volatile int* s_abort = reinterpret_cast<volatile int*>(smem + kRingBytes + kBarBytes + 4);
+  int4* const s_first = reinterpret_cast<int4*>(smem + kRingBytes + 192 - sizeof(Tile));
+  const uint32_t items = bar0 + 192;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();   // CTA 0 of a pair is the leader
+  int* const status = p.status;
+  const int n_pairs = (int)(gridDim.x >> 1), my_pair = (int)(blockIdx.x >> 1);
   if (threadIdx.x == 0) {
     for (int s = 0; s < NS; ++s) {
       mbar_init(full_bar(s), 1);    // the leader's arrive + all bytes of the stage of both CTAs
@@ -300,15 +472,25 @@ ffn_kernel(const __grid_constant__ CUtensorMap tmT128, const __grid_constant__ C
       mbar_init(tfull_bar(h), 1);                // one tcgen05.commit
       mbar_init(tempty_bar(h), 2 * kEpiWarps);   // one arrival per epilogue warp of both CTAs (leader's barrier)
     }
+    for (int i = 0; i < kItems; ++i) {
+      mbar_init(item_full(i), 1);                        // the dealer's arrive
+      mbar_init(item_empty(i), 3 + 2 * kEpiWarps);       // every reader of both CTAs (CTA 1's barrier)
+    }
+    mbar_init(want_bar, 1);                              // the leader's producer (CTA 1's barrier)
     *s_abort = 0;
+    for (int i = 0; i < kParts; ++i) reinterpret_cast<int*>(smem + kRingBytes + kBarBytes + 8)[i] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    prefetch_tmap(&tmT128);
-    prefetch_tmap(&tmT64);
-    prefetch_tmap(&tmT32);
-    prefetch_tmap(&tmT16);
-    prefetch_tmap(&tmT8);
-    prefetch_tmap(&tmW0);
-    prefetch_tmap(&tmW1);
+  }
+  if (warp == 2 && lane < kMaps) prefetch_tmap(&p.xp.box[0] + lane);
+  if (threadIdx.x == 96) {
+    // The first tile of pair q is tile q of the part, fetched once per CTA beside the set-up; the others come from
+    // the tile dealer.
+    const int part_first = p.part == 2 ? p.work_count[0] : 0;
+    const int4* e = reinterpret_cast<const int4*>(p.work + min(part_first + my_pair, p.max_work - 1));
+    int4 a = __ldg(e), b = __ldg(e + 1);
+    if (part_first + my_pair >= (p.part == 1 ? p.work_count[0] : p.work_count[0] + p.work_count[1])) a.z = -1;
+    s_first[0] = a;
+    s_first[1] = b;
   }
   if (warp == 1) {
     tmem_alloc_pair(smem_u32((const void*)s_tmem), kTmemCols);
@@ -319,66 +501,122 @@ ffn_kernel(const __grid_constant__ CUtensorMap tmT128, const __grid_constant__ C
   cluster_sync_all();   // the peer's barriers are initialised before anything arrives on them
   tc_fence_after();
   const uint32_t tmem_base = *s_tmem;
-  const int n_work = work_count[PHASE - 1];
-  const int num_kb = (k_total + BK - 1) / BK;
-  // The list is ordered by cost, widest tiles first.  It is dealt out in rounds of one tile per pair, the
-  // direction alternating from round to round, so every pair ends up with nearly the same total cost.
-  const int n_pairs = (int)(gridDim.x >> 1), my_pair = (int)(blockIdx.x >> 1);
-  auto tile_of_round = [&](int r) { return r * n_pairs + ((r & 1) ? n_pairs - 1 - my_pair : my_pair); };
+  const int num_kb1 = (p.H + BK - 1) / BK, num_kb2 = (p.I + BK - 1) / BK;
+
+  // Tile number `seq` of this pair (false: gave up); all but the first come through the mailbox, where the reader frees
+  // the slot.
+  auto take_item = [&](int seq, Tile* it) {
+    const int i = seq % kItems;
+    uint32_t at = bar0 + 192u - (uint32_t)sizeof(Tile);
+    if (seq > 0) {
+      if (!mbar_wait_cluster(item_full(i), (uint32_t)((seq - 1) / kItems) & 1u, s_abort, status)) return false;
+      at = items + i * (uint32_t)sizeof(Tile);
+    }
+    const int4 a = ld_shared(at), b = ld_shared(at + 16);
+    *it = Tile{a.x, a.y, a.z, a.w, b.x, b.y, b.z, 0};
+    return true;
+  };
+  auto free_item = [&](int seq) {
+    if (seq > 0) mbar_arrive_cluster(map_to_cta(item_empty(seq % kItems), 1));
+  };
 
   if (warp == 0) {
     // ---------------- TMA producer (each CTA loads its own halves) ----------------
     if (lane == 0) {
       int stage = 0;
       uint32_t phase = 0;
-      for (int r = 0; r * n_pairs < n_work; ++r) {
-        const int w = tile_of_round(r);
-        if (w >= n_work) continue;
-        const int4 it = __ldg(work + w);
-        const bool merged = it.y < 0;
-        const int half = entry_cols(it.y) >> 1;   // token rows this CTA loads: a multiple of 8 (of 16 in a merged tile)
-        const int tok0 = it.x + (int)rank * half;
-        // merged tile: this CTA's slots are slots[x + rank * half / 16 ..); a slot beyond the tile's count
+      for (int seq = 0;; ++seq) {
+        Tile it;
+        if (!take_item(seq, &it)) goto done;
+        if (it.w < 0) break;
+        free_item(seq);
+        const bool merged = it.rows < 0;
+        const int half = entry_cols(it.rows) >> 1;   // token rows this CTA loads: a multiple of 8 (of 16 in a merged tile)
+        const int tok0 = it.row + (int)rank * half;
+        // merged tile: this CTA's slots are slots[row + rank * half / 16 ..); a slot beyond the tile's count
         // repeats the first one (its columns are never stored), so the byte count of a stage stays uniform
         int slot_row[kMergeSlots / 2];
 #pragma unroll
         for (int i = 0; i < kMergeSlots / 2; ++i) {
           const int sl = (int)rank * (half / kSlotRows) + i;
-          slot_row[i] = (merged && i < half / kSlotRows) ? __ldg(slots + it.x + (sl < -it.y ? sl : 0)).x : 0;
+          slot_row[i] = (merged && i < half / kSlotRows) ? __ldg(p.slots + it.row + (sl < -it.rows ? sl : 0)).x : 0;
         }
-        const int wrow0 = (PHASE == 1 ? it.w * kFeat1 : it.w * kFeat2) + (int)rank * 128;
-        const int wrow1 = PHASE == 1 ? wrow0 : wrow0 + 256;
+        const bool down = it.phase == 2;
+        const CUtensorMap* tmW0 = down ? &p.down : &p.gate;
+        const CUtensorMap* tmW1 = down ? &p.down : &p.up;
+        const TokenMaps* tmT = down ? &p.act : &p.xp;
+        const int num_kb = down ? num_kb2 : num_kb1;
+        const int wrow0 = it.out * (down ? kFeat2 : kFeat1) + (int)rank * 128;
+        const int wrow1 = down ? wrow0 + 256 : wrow0;
         const uint32_t tx = 2u * (2u * kWBytes + (uint32_t)half * (BK * 2));
-        for (int kb = 0; kb < num_kb; ++kb) {
-          if (!mbar_wait(empty_bar(stage), phase ^ 1u, s_abort, status)) goto done;
-          // both CTAs' copies are counted on the leader's barrier; the leader announces the total
-          const uint32_t fb = map_to_cta(full_bar(stage), 0);
-          if (rank == 0) mbar_expect_tx(full_bar(stage), tx);
-          tma_pair_load_3d(w0_addr(stage), &tmW0, kb * BK, wrow0, it.z, fb);
-          tma_pair_load_3d(w1_addr(stage), &tmW1, kb * BK, wrow1, it.z, fb);
-          const uint32_t ta = t_addr(stage);
+        // both CTAs' copies are counted on the leader's barrier; the leader announces the total
+        auto load_weights = [&](int st, int kb) {
+          const uint32_t fb = map_to_cta(full_bar(st), 0);
+          if (rank == 0) mbar_expect_tx(full_bar(st), tx);
+          tma_pair_load_3d(w0_addr(st), tmW0, kb * BK, wrow0, it.w, fb);
+          tma_pair_load_3d(w1_addr(st), tmW1, kb * BK, wrow1, it.w, fb);
+        };
+        auto load_tokens = [&](int st, int kb) {
+          const uint32_t fb = map_to_cta(full_bar(st), 0), ta = t_addr(st);
           if (merged) {
 #pragma unroll
             for (int i = 0; i < kMergeSlots / 2; ++i)
-              if (i < half / kSlotRows) tma_pair_load_2d(ta + i * (kSlotRows * BK * 2), &tmT16, kb * BK, slot_row[i], fb);
+              if (i < half / kSlotRows) tma_pair_load_2d(ta + i * (kSlotRows * BK * 2), &tmT->box[3], kb * BK, slot_row[i], fb);
           } else if (half == 128) {
-            tma_pair_load_2d(ta, &tmT128, kb * BK, tok0, fb);
+            tma_pair_load_2d(ta, &tmT->box[0], kb * BK, tok0, fb);
           } else {
             int r2 = 0;   // rows placed so far; every box starts on a multiple of 8 rows (1 KB), which keeps the swizzle phase
             if (half & 64) {
-              tma_pair_load_2d(ta, &tmT64, kb * BK, tok0, fb);
+              tma_pair_load_2d(ta, &tmT->box[1], kb * BK, tok0, fb);
               r2 = 64;
             }
             if (half & 32) {
-              tma_pair_load_2d(ta + r2 * (BK * 2), &tmT32, kb * BK, tok0 + r2, fb);
+              tma_pair_load_2d(ta + r2 * (BK * 2), &tmT->box[2], kb * BK, tok0 + r2, fb);
               r2 += 32;
             }
             if (half & 16) {
-              tma_pair_load_2d(ta + r2 * (BK * 2), &tmT16, kb * BK, tok0 + r2, fb);
+              tma_pair_load_2d(ta + r2 * (BK * 2), &tmT->box[3], kb * BK, tok0 + r2, fb);
               r2 += 16;
             }
-            if (half & 8) tma_pair_load_2d(ta + r2 * (BK * 2), &tmT8, kb * BK, tok0 + r2, fb);
+            if (half & 8) tma_pair_load_2d(ta + r2 * (BK * 2), &tmT->box[4], kb * BK, tok0 + r2, fb);
           }
+        };
+        const int ask = num_kb > kAskAhead ? num_kb - kAskAhead : 0;
+        int kb = 0;
+        if (down) {
+          const int* flag = p.ready + it.done;
+          if (it.need > 0 && ld_acquire(flag) < it.need) {
+            // the rows are still being made: the weights of the stages at hand go ahead of them
+            const int lead = num_kb < NS ? num_kb : NS;
+            int st = stage;
+            uint32_t ph = phase;
+            for (int i = 0; i < lead; ++i) {
+              if (!mbar_wait(empty_bar(st), ph ^ 1u, s_abort, status)) goto done;
+              load_weights(st, i);
+              if (++st == NS) {
+                st = 0;
+                ph ^= 1u;
+              }
+            }
+            if (!bounded_wait([&] { return ld_acquire(flag) >= it.need; }, s_abort, status)) goto done;
+            fence_proxy_async();
+            if (rank == 0 && ask < lead) mbar_arrive_cluster(map_to_cta(want_bar, 1));
+            for (; kb < lead; ++kb) {
+              load_tokens(stage, kb);
+              if (++stage == NS) {
+                stage = 0;
+                phase ^= 1u;
+              }
+            }
+          } else {
+            fence_proxy_async();
+          }
+        }
+        for (; kb < num_kb; ++kb) {
+          if (rank == 0 && kb == ask) mbar_arrive_cluster(map_to_cta(want_bar, 1));
+          if (!mbar_wait(empty_bar(stage), phase ^ 1u, s_abort, status)) goto done;
+          load_weights(stage, kb);
+          load_tokens(stage, kb);
           if (++stage == NS) {
             stage = 0;
             phase ^= 1u;
@@ -387,16 +625,18 @@ ffn_kernel(const __grid_constant__ CUtensorMap tmT128, const __grid_constant__ C
       }
     }
   } else if (warp == 1) {
-    // ---------------- MMA issuer (leader CTA only) ----------------
     if (lane == 0 && rank == 0) {
+      // ---------------- MMA issuer (leader CTA only) ----------------
       int stage = 0;
       uint32_t phase = 0;
       TmemTurn turn;
-      for (int r = 0; r * n_pairs < n_work; ++r) {
-        const int w = tile_of_round(r);
-        if (w >= n_work) continue;
-        const int4 it = __ldg(work + w);
-        const int cols = entry_cols(it.y);
+      for (int seq = 0;; ++seq) {
+        Tile it;
+        if (!take_item(seq, &it)) goto done;
+        if (it.w < 0) break;
+        free_item(seq);
+        const int num_kb = it.phase == 2 ? num_kb2 : num_kb1;
+        const int cols = entry_cols(it.rows);
         const uint32_t idesc = kIdescBase | ((uint32_t)(cols >> 3) << 17);
         turn.take(cols);
         const uint32_t acc0 = tmem_base + turn.col0(), acc1 = acc0 + turn.step();
@@ -460,24 +700,59 @@ ffn_kernel(const __grid_constant__ CUtensorMap tmT128, const __grid_constant__ C
           umma_pair_commit(tfull_bar(turn.half()));
         }
       }
+    } else if (lane == 0) {
+      // ---------------- tile dealer (CTA 1's otherwise idle MMA warp) ----------------
+      // Every tile of a pair but its first is the next one not yet dealt, claimed well before the leader's producer
+      // is through with the tile before it.  Both CTAs' mailboxes get a copy.
+      const int part_first = p.part == 2 ? p.work_count[0] : 0;
+      const int part_end = p.part == 1 ? p.work_count[0] : p.work_count[0] + p.work_count[1];
+      for (int seq = 1; part_first + my_pair < part_end; ++seq) {
+        const int i = seq % kItems;
+        if (!mbar_wait_cluster(want_bar, (uint32_t)(seq - 1) & 1u, s_abort, status)) goto done;
+        if (seq > kItems && !mbar_wait_cluster(item_empty(i), (uint32_t)((seq - 1) / kItems - 1) & 1u, s_abort, status)) goto done;
+        const int idx = part_first + n_pairs + atomicAdd(p.next + (p.part == 2 ? 1 : 0), 1);
+        int4 a = make_int4(0, 0, -1, 0), b = make_int4(0, 0, 0, 0);
+        if (idx < part_end) {
+          const int4* e = reinterpret_cast<const int4*>(p.work + idx);
+          a = __ldg(e);
+          b = __ldg(e + 1);
+          // a down tile whose rows are complete already, the usual case, spares the producers the question
+          if (b.x == 2 && ld_acquire(p.ready + b.y) >= b.z) b.z = 0;
+        }
+        const uint32_t at = items + i * (uint32_t)sizeof(Tile);
+        for (uint32_t r = 0; r < 2; ++r) {
+          const uint32_t dst = map_to_cta(at, r);
+          st_cluster(dst, a);
+          st_cluster(dst + 16, b);
+          mbar_arrive_release_cluster(map_to_cta(item_full(i), r));
+        }
+        if (idx >= part_end) break;
+      }
     }
   } else {
     // ---------------- epilogue warps ----------------
     const int q = warp & 3;                      // TMEM lane quadrant this warp may read
-    const int chunk0 = ((warp - 2) >> 2) * 16;   // the two warps of a quadrant take alternate 16-column chunks
+    const int chunk0 = ((warp - 2) >> 2) * 16;   // the warps of a quadrant take 16-column chunks in turn
     const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16);
-    bf16* tile = reinterpret_cast<bf16*>(smem + kRingBytes + 256) + (warp - 2) * 1024;   // 2 KB per epilogue warp
+    bf16* tile = reinterpret_cast<bf16*>(smem + kRingBytes + 256) + (warp - 2) * 512;   // 1 KB per epilogue warp
+    int* parts = reinterpret_cast<int*>(smem + kRingBytes + kBarBytes + 8);
     TmemTurn turn;
-    for (int r = 0; r * n_pairs < n_work; ++r) {
-      const int w = tile_of_round(r);
-      if (w >= n_work) continue;
-      const int4 it = __ldg(work + w);
-      turn.take(entry_cols(it.y));
-      const bool merged = it.y < 0;
-      const int n_cols = merged ? -it.y * kSlotRows : it.y;   // columns that may hold rows to store
+    for (int seq = 0;; ++seq) {
       // one lane waits, the outcome is made warp-uniform before any .aligned instruction
+      Tile it = {};
       int ok = 1;
+      if (lane == 0) ok = take_item(seq, &it) ? 1 : 0;
+      ok = __shfl_sync(0xffffffffu, ok, 0);
+      if (!ok) goto done;
+      it.row = __shfl_sync(0xffffffffu, it.row, 0);
+      it.rows = __shfl_sync(0xffffffffu, it.rows, 0);
+      it.w = __shfl_sync(0xffffffffu, it.w, 0);
+      it.out = __shfl_sync(0xffffffffu, it.out, 0);
+      it.phase = __shfl_sync(0xffffffffu, it.phase, 0);
+      if (it.w < 0) break;
+      turn.take(entry_cols(it.rows));
       if (lane == 0) {
+        free_item(seq);
         const int h = turn.wide() ? 0 : turn.half();
         ok = mbar_wait(tfull_bar(h), turn.parity(h), s_abort, status) ? 1 : 0;
         if (ok && turn.wide()) ok = mbar_wait(tfull_bar(1), turn.parity(1), s_abort, status) ? 1 : 0;
@@ -485,71 +760,31 @@ ffn_kernel(const __grid_constant__ CUtensorMap tmT128, const __grid_constant__ C
       ok = __shfl_sync(0xffffffffu, ok, 0);
       if (!ok) goto done;
       tc_fence_after();
-      const uint32_t acc0 = taddr + turn.col0(), acc1 = acc0 + turn.step();
-      // this warp's 32 outputs start at fbase; a 16-token chunk is transposed through shared memory so that
-      // global stores are 16-byte vectors: lane -> (token lane / 4 (+8), outputs 8 (lane % 4) .. +7)
-      const int fbase = (PHASE == 1 ? it.w * kFeat1 : it.w * kFeat2) + (int)rank * 128 + q * 32;
-      const int fcol = fbase + (lane & 3) * 8;
-      // Both accumulators move to registers first, the first one as it is, the second one combined (gate/up) or
-      // rounded (down) on the way; each is handed back as soon as it is read, the stores come after.
-      uint32_t r0[kEpiChunks][PHASE == 1 ? 16 : 8];   // first accumulator; then outputs, two tokens per word, in [0..7]
-      uint32_t r1[PHASE == 1 ? 1 : kEpiChunks][8];
-      if constexpr (PHASE == 1) {
-#pragma unroll
-        for (int i = 0; i < kEpiChunks; ++i) {
-          if (chunk0 + 32 * i >= n_cols) break;
-          tmem_ld16(acc0 + chunk0 + 32 * i, r0[i]);
-        }
-        tmem_ld_wait();
-        if (turn.wide()) release_tmem(tempty_bar(0), lane);
-#pragma unroll
-        for (int i = 0; i < kEpiChunks; ++i) {
-          if (chunk0 + 32 * i >= n_cols) break;
-          uint32_t b[16];
-          tmem_ld16(acc1 + chunk0 + 32 * i, b);
-          tmem_ld_wait();
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            r0[i][j] = pack_bf16(silu_mul(r0[i][2 * j], b[2 * j]), silu_mul(r0[i][2 * j + 1], b[2 * j + 1]));
+      // this warp's 32 outputs start at fbase
+      const int fbase = it.out * (it.phase == 1 ? kFeat1 : kFeat2) + (int)rank * 128 + q * 32;
+      const int cols = it.rows < 0 ? -it.rows * kSlotRows : it.rows;
+      auto run = [&](auto phase, bf16* out, int n_out) {
+        constexpr int PH = decltype(phase)::value;
+        if (cols <= 64) epilogue_tile<PH, 2>(it, turn, taddr, chunk0, lane, fbase, tile, p.slots, out, n_out, tempty_bar(0), tempty_bar(1));
+        else if (cols <= 128) epilogue_tile<PH, 4>(it, turn, taddr, chunk0, lane, fbase, tile, p.slots, out, n_out, tempty_bar(0), tempty_bar(1));
+        else epilogue_tile<PH, 8>(it, turn, taddr, chunk0, lane, fbase, tile, p.slots, out, n_out, tempty_bar(0), tempty_bar(1));
+      };
+      if (it.phase == 1) {
+        run(std::integral_constant<int, 1>(), p.act_out, p.I);
+        // this warp's part of the intermediate is written; the CTA's last warp counts it on the token tile, whose down
+        // tiles wait for all parts.  The stores are ordered before the TMA reads of whoever sees the count.
+        __syncwarp();
+        if (lane == 0) {
+          __threadfence_block();
+          if (atomicAdd(&parts[seq % kParts], 1) == kEpiWarps - 1) {
+            parts[seq % kParts] = 0;
+            __threadfence();
+            fence_proxy_async();
+            red_release(p.ready + it.done);
+          }
         }
       } else {
-        drain_packed(acc0 + chunk0, n_cols - chunk0, r0);
-        if (turn.wide()) release_tmem(tempty_bar(0), lane);
-        drain_packed(acc1 + chunk0, n_cols - chunk0, r1);
-      }
-      release_tmem(tempty_bar(turn.wide() ? 1 : turn.half()), lane);
-#pragma unroll
-      for (int i = 0; i < kEpiChunks; ++i) {
-        const int c0 = chunk0 + 32 * i;
-        if (c0 >= n_cols) break;
-        // rows of this chunk: columns c0 .. c0 + 15 are rows row0 .. row0 + n_here - 1 (a merged tile: one slot)
-        int row0 = it.x + c0, n_here = min(16, it.y - c0);
-        if (merged) {
-          const int2 sl = __ldg(slots + it.x + (c0 >> 4));
-          row0 = sl.x;
-          n_here = sl.y;
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          tile[2 * j * 32 + lane] = low_half(r0[i][j]);
-          tile[(2 * j + 1) * 32 + lane] = high_half(r0[i][j]);
-          if (PHASE == 2) {
-            tile[512 + 2 * j * 32 + lane] = low_half(r1[i][j]);
-            tile[512 + (2 * j + 1) * 32 + lane] = high_half(r1[i][j]);
-          }
-        }
-        __syncwarp();
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int tok = (lane >> 2) + 8 * h;
-          if (tok < n_here) {
-            bf16* dst = out + (size_t)(row0 + tok) * ld_out + fcol;
-            const uint4* src = reinterpret_cast<const uint4*>(tile + tok * 32 + (lane & 3) * 8);
-            if (fcol < n_out) *reinterpret_cast<uint4*>(dst) = src[0];
-            if (PHASE == 2 && fcol + 256 < n_out) *reinterpret_cast<uint4*>(dst + 256) = src[64];   // second accumulator: +1 KB
-          }
-        }
-        __syncwarp();
+        run(std::integral_constant<int, 2>(), p.yp, p.H);
       }
     }
   }
@@ -787,18 +1022,19 @@ plan_kernel(ModelParams mp, const int32_t* __restrict__ group_off, const int32_t
     work_count[3] = g0;
     work_count[4] = ng;
     work_count[5] = n_listed;
+    work_count[6] = work_count[7] = 0;   // tiles dealt out by the expert kernel
     work_count[8] = nl;
     work_count[9] = device;
   }
 }
 
-// fill: one thread per tile of the two lists (gate/up, down); tiles of a group are ordered weight-tile
+// fill: one thread per tile of the list (gate/up tiles, then down tiles); tiles of a group are ordered weight-tile
 // major, token-tile minor.
 __global__ void __launch_bounds__(256)
 fill_kernel(ModelParams mp, const int32_t* __restrict__ group_off, const int32_t* __restrict__ group_w,
             const int32_t* __restrict__ pgroup, const int32_t* __restrict__ pslots, const int32_t* __restrict__ order,
-            const int32_t* __restrict__ tile_pref, const int32_t* __restrict__ work_count, int nt1, int nt2, int max1,
-            int max2, int4* __restrict__ work1, int4* __restrict__ work2, int2* __restrict__ slots) {
+            const int32_t* __restrict__ tile_pref, const int32_t* __restrict__ work_count, int nt1, int nt2, int max_work,
+            Tile* __restrict__ work, int32_t* __restrict__ ready, int2* __restrict__ slots) {
   EB_GRID_DEP_SYNC();
   extern __shared__ int s_pref[];   // tile_pref staged once per block: the binary search below then stays on chip
   const int n_listed = work_count[5];
@@ -820,7 +1056,7 @@ fill_kernel(ModelParams mp, const int32_t* __restrict__ group_off, const int32_t
     const int rem = local - s_pref[lo] * nt;
     const int n = rem / t_g, m = rem % t_g;
     const int pos = order[lo], g = pgroup[pos], n_slots = pslots[pos];
-    int4 it;
+    Tile it;
     if (n_slots >= 0) {
       // tile m of a merged class holds the next 16 slots of the class, replicas in device order
       const int base = kMergeSlots * (s_pref[lo] + m);
@@ -836,18 +1072,23 @@ fill_kernel(ModelParams mp, const int32_t* __restrict__ group_off, const int32_t
               slots[base + c - first] = make_int2(r0 + k * kSlotRows, min(kSlotRows, rows - k * kSlotRows));
         }
       }
-      it.x = base;
-      it.y = -n_here;
+      it.row = base;
+      it.rows = -n_here;
     } else {
       // t_g tiles of nearly equal size: the first (rows % t_g) tiles hold one row more
       const int rows = group_off[g + 1] - group_off[g];
       const int each = rows / t_g, more = rows % t_g;
-      it.x = group_off[g] + m * each + min(m, more);
-      it.y = each + (m < more ? 1 : 0);
+      it.row = group_off[g] + m * each + min(m, more);
+      it.rows = each + (m < more ? 1 : 0);
     }
-    it.z = group_w[g];
-    it.w = n;
-    if (local < (list ? max2 : max1)) (list ? work2 : work1)[local] = it;
+    it.w = group_w[g];
+    it.out = n;
+    it.phase = list + 1;
+    it.done = s_pref[lo] + m;
+    it.need = nt1 * 2;
+    it.pad = 0;
+    if (list == 0 && n == 0) ready[it.done] = 0;
+    if (idx < max_work) work[idx] = it;
   }
 }
 
@@ -883,9 +1124,7 @@ bool make_map(CUtensorMap* m, const void* ptr, uint64_t d0, uint64_t d1, uint64_
   return r == CUDA_SUCCESS;
 }
 
-template <int PHASE>
-cudaError_t launch_ffn(eb_ctx* c, cudaStream_t st, const CUtensorMap* tT, const CUtensorMap& tW0, const CUtensorMap& tW1,
-                       const int4* work, bf16* out, int ld_out, int n_out, int k_total) {
+cudaError_t launch_ffn(eb_ctx* c, cudaStream_t st, const FfnParams& p) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(c->pair_grid);
   cfg.blockDim = dim3(kThreads);
@@ -900,11 +1139,8 @@ cudaError_t launch_ffn(eb_ctx* c, cudaStream_t st, const CUtensorMap* tT, const 
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  const int2* slots = c->slots;
-  const int32_t* wc = c->work_count;
   ++g_ebi_launches;
-  return cudaLaunchKernelEx(&cfg, ffn_kernel<PHASE>, tT[0], tT[1], tT[2], tT[3], tT[4], tW0, tW1, work, slots, wc, out, ld_out, n_out,
-                            k_total, c->d_status);
+  return cudaLaunchKernelEx(&cfg, ffn_kernel, p);
 }
 
 }  // namespace
@@ -924,8 +1160,7 @@ eb_status ebi_ffn_bind(eb_ctx* c) {
       !make_map(&c->tm_down, c->w_down, g.I, g.H, nw, BK, 128))
     return ebi_fail(c, EB_ERR_CUDA, "cuTensorMapEncodeTiled failed for the weights");
   // per context: function attributes and cluster occupancy belong to the current device
-  cudaError_t e = cudaFuncSetAttribute(ffn_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(ffn_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+  cudaError_t e = cudaFuncSetAttribute(ffn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
   if (e != cudaSuccess) return ebi_check_cuda(c, e, "cudaFuncSetAttribute");
   // how many 2-CTA clusters of this kernel the device can hold at once (one CTA per SM)
   cudaLaunchConfig_t cfg = {};
@@ -940,7 +1175,7 @@ eb_status ebi_ffn_bind(eb_ctx* c) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int clusters = 0;
-  e = cudaOccupancyMaxActiveClusters(&clusters, ffn_kernel<1>, &cfg);
+  e = cudaOccupancyMaxActiveClusters(&clusters, ffn_kernel, &cfg);
   if (e != cudaSuccess || clusters < 1) {
     cudaGetLastError();
     return ebi_fail(c, EB_ERR_CUDA, "the device cannot hold a 2-CTA cluster of the expert kernel");
@@ -959,11 +1194,26 @@ eb_status ebi_ffn_run(eb_ctx* c, cudaStream_t st, const void* xp, const int32_t*
   const eb_config& g = c->cfg;
   const int rows = ebi_rows_cap(c);
   // token-row boxes of 128 / 64 / 32 / 16 / 8 rows x one k-block, over the permuted rows and over the intermediate
-  CUtensorMap tok_x[5], tok_a[5];
+  FfnParams p;
   const int box_rows[5] = {128, 64, 32, 16, 8};
   for (int i = 0; i < 5; ++i)
-    if (!make_map(&tok_x[i], xp, g.H, rows, 0, BK, box_rows[i]) || !make_map(&tok_a[i], c->act, g.I, rows, 0, BK, box_rows[i]))
+    if (!make_map(&p.xp.box[i], xp, g.H, rows, 0, BK, box_rows[i]) || !make_map(&p.act.box[i], c->act, g.I, rows, 0, BK, box_rows[i]))
       return ebi_fail(c, EB_ERR_CUDA, "cuTensorMapEncodeTiled failed for the activations");
+  Tile* const work = (Tile*)c->work;
+  p.gate = c->tm_gate;
+  p.up = c->tm_up;
+  p.down = c->tm_down;
+  p.work = work;
+  p.max_work = c->max_work;
+  p.slots = c->slots;
+  p.work_count = c->work_count;
+  p.next = c->work_count + 6;
+  p.ready = c->tile_ready;
+  p.act_out = c->act;
+  p.yp = (bf16*)yp;
+  p.H = g.H;
+  p.I = g.I;
+  p.status = c->d_status;
   const int nt1 = (g.I + kFeat1 - 1) / kFeat1, nt2 = (g.H + kFeat2 - 1) / kFeat2;
   {
     KernelTimer timer(c, EBK_FFN_PLAN, st);
@@ -975,16 +1225,23 @@ eb_status ebi_ffn_run(eb_ctx* c, cudaStream_t st, const void* xp, const int32_t*
     ebi_launch(fill_kernel, dim3(c->num_sms), dim3(256), sizeof(int) * (size_t)(ebi_groups_cap(c) + 1), st, c->mp, group_off, group_w,
                (const int32_t*)c->pgroup,
                (const int32_t*)c->pslots, (const int32_t*)c->order, (const int32_t*)c->tile_pref,
-               (const int32_t*)c->work_count, nt1, nt2, c->max_work1, c->max_work2, c->work1, c->work2, c->slots);
+               (const int32_t*)c->work_count, nt1, nt2, c->max_work, work, c->tile_ready, c->slots);
   }
   cudaError_t e;
-  {
-    KernelTimer timer(c, EBK_FFN_GATEUP, st);
-    e = launch_ffn<1>(c, st, tok_x, c->tm_gate, c->tm_up, c->work1, c->act, g.I, g.I, g.H);
-  }
-  if (e == cudaSuccess) {
-    KernelTimer timer(c, EBK_FFN_DOWN, st);
-    e = launch_ffn<2>(c, st, tok_a, c->tm_down, c->tm_down, c->work2, (bf16*)yp, g.H, g.H, g.I);
+  if (!c->timing) {
+    p.part = 0;
+    e = launch_ffn(c, st, p);
+  } else {   // the same tiles in two launches, so that each phase gets a time of its own
+    {
+      KernelTimer timer(c, EBK_FFN_GATEUP, st);
+      p.part = 1;
+      e = launch_ffn(c, st, p);
+    }
+    if (e == cudaSuccess) {
+      KernelTimer timer(c, EBK_FFN_DOWN, st);
+      p.part = 2;
+      e = launch_ffn(c, st, p);
+    }
   }
   if (e != cudaSuccess) return ebi_check_cuda(c, e, "expert_ffn launch");
   EB_LAUNCH_CHECK(c, "expert_ffn");

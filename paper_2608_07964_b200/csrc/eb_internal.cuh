@@ -82,12 +82,12 @@ struct eb_ctx {
   int4* prank = nullptr;           // [G_cap] (cost class, rank and tiles before it inside the class) when a plan has more than 1024 positions
   int32_t* order = nullptr;        // [G_cap] positions that own tiles, widest tiles first
   int32_t* tile_pref = nullptr;    // [G_cap + 1] tiles before each entry of `order`
-  int32_t* work_count = nullptr;   // [16]: tile counts of the two lists, group range, layers, device filter
-  int4* work1 = nullptr;           // gate/up tile list
-  int4* work2 = nullptr;           // down tile list
+  int32_t* work_count = nullptr;   // [16]: tile counts of the two phases, group range, dealt-out counters, layers, device filter
+  void* work = nullptr;            // [max_work] tile list: gate/up tiles, then down tiles (32 bytes each)
+  int32_t* tile_ready = nullptr;   // [max_tiles] per token tile: finished parts of its intermediate rows
   int2* slots = nullptr;           // [16 * max_tiles] (first row, rows) of the 16-row slots of merged tiles
   bf16* act = nullptr;             // [R_cap][I]
-  int32_t max_chunks = 0, max_tiles = 0, max_work1 = 0, max_work2 = 0;
+  int32_t max_chunks = 0, max_tiles = 0, max_work = 0;
 
   bool fused_attr_set = false;
   // eb_step_host_submit / eb_step_host_wait: copy streams and per-slot events, created on first use

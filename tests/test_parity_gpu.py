@@ -481,6 +481,27 @@ def test_tile_sizes_mixed_over_many_tiles_per_pair(H, I):
     test_group_sizes_around_the_tile_boundaries(H, I)
 
 
+@pytest.mark.parametrize("tokens,H,I", [([1], 64, 64), ([40, 300, 7], 264, 520), ([900, 900, 900], 512, 1288)])
+def test_one_launch_for_both_phases_equals_a_launch_each(tokens, H, I):
+    """With per-kernel timing on, the gate/up and the down tiles go out as two launches; otherwise as one, in which the
+    down tiles wait for the rows they need.  Fewer tiles than CTA pairs, a few per pair, many per pair: same bits."""
+    B = _binding()
+    wl = _small(L=2, E=12, K=3, S=1, D=4, N=len(tokens), T=max(tokens), H=H, I=I, mapping="mod")
+    case, store = Hn.make_case(wl, tokens, [j % 2 for j in range(len(tokens))]), Hn.WeightStore(wl)
+    step, _ = _full_step(case, store, len(tokens))
+    rows = step.meta()["rows"]
+    batch = B.Batch(case.tok_off, case.layers)
+    got = []
+    for timed in (True, False, False, True):
+        step.set_timing(timed)
+        step.yp.zero_()
+        step.eb_step(batch, len(tokens))
+        got.append(step.yp[:rows].clone())
+    step.set_timing(False)
+    assert step.device_status() == 0 and step.check_workspace_guards() == 0
+    assert all(torch.equal(got[0], g) for g in got[1:])
+
+
 # ----------------------------------------------------------------------------------- failure reporting
 def test_bounded_wait_gives_up_and_reports_without_harming_the_context():
     B = _binding()
