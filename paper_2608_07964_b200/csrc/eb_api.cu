@@ -90,6 +90,8 @@ static size_t carve(eb_ctx* c, char* base) {
   c->max_work = c->max_tiles * ((g.I + 255) / 256 + (g.H + 511) / 512);   // 256 outputs per gate/up tile, 512 per down tile
   c->chunk_hist = (int32_t*)take(sizeof(int32_t) * (size_t)c->max_chunks * g.E);
   c->chunk_base = (int32_t*)take(sizeof(int32_t) * (size_t)c->max_chunks * g.E);
+  c->chunk_seg = (int32_t*)take(sizeof(int32_t) * (size_t)(c->max_chunks / EB_SEG_CHUNKS + EB_MAX_MB) * g.E);
+  c->mb_base = (int32_t*)take(sizeof(int32_t) * (size_t)EB_MAX_MB * g.E);
   c->group_size = (int32_t*)take(sizeof(int32_t) * (size_t)gcap);
   c->pgroup = (int32_t*)take(sizeof(int32_t) * (size_t)gcap);
   c->pslots = (int32_t*)take(sizeof(int32_t) * (size_t)gcap);
@@ -251,11 +253,15 @@ extern "C" eb_status eb_step(eb_ctx* c, void* stream, const eb_batch* batch, uin
   if (!c) return EB_ERR_INVALID_ARG;
   eb_status s = check_buffers(c, b);
   if (s != EB_OK) return s;
-  if ((s = eb_route(c, stream, batch, route_mask, b->logits, b->topk_idx, b->topk_w, b->mb_load, b->mb_cnt)) != EB_OK) return s;
-  if ((s = eb_schedule(c, stream, batch, m, policy, b->mb_load, b->sched, nullptr)) != EB_OK) return s;
-  if ((s = eb_permute(c, stream, batch, b->sched, b->x, b->topk_idx, b->group_off, b->group_w, b->row_src, b->pos,
-                      b->xp, b->step_meta)) != EB_OK) return s;
-  if ((s = eb_expert_ffn_grouped(c, stream, b->xp, b->group_off, b->group_w, b->step_meta, b->yp)) != EB_OK) return s;
+  BatchParams bp;
+  if ((s = ebi_make_batch(c, batch, &bp)) != EB_OK) return s;
+  if (bp.n_mb < 32 && (route_mask >> bp.n_mb) != 0) return ebi_fail(c, EB_ERR_INVALID_ARG, "route_mask beyond n_mb");
+  if (m < 1) return ebi_fail(c, EB_ERR_INVALID_ARG, "m must be at least 1");
+  if ((int)policy < 0 || (int)policy > EB_POLICY_ALL) return ebi_fail(c, EB_ERR_INVALID_ARG, "unknown policy");
+  if (!c->ws) return ebi_fail(c, EB_ERR_WORKSPACE, "no workspace set");
+  cudaStream_t st = (cudaStream_t)stream;
+  if ((s = ebi_front_run(c, st, bp, batch->pool_mask, route_mask, m, policy, b)) != EB_OK) return s;
+  if ((s = ebi_ffn_run(c, st, b->xp, b->group_off, b->group_w, b->step_meta, b->yp, -1, true)) != EB_OK) return s;
   if (!ebi_aligned16(b->residual)) return ebi_fail(c, EB_ERR_INVALID_ARG, "residual not 16-byte aligned");
   return eb_combine_residual(c, stream, batch, b->sched, b->yp, b->pos, b->topk_w, b->residual, b->out);
 }

@@ -52,7 +52,7 @@
 #include <cstddef>
 #include <type_traits>
 
-#include "eb_internal.cuh"
+#include "eb_tiles.cuh"
 
 namespace {
 
@@ -70,12 +70,6 @@ static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
 constexpr int kTmemCols = 512;
 constexpr int kTmemHalf = 256;                                 // a narrow tile's two accumulators share one half of TMEM
 constexpr int kNarrowCols = kTmemHalf / 2;                     // ... which takes tiles of up to 128 columns
-constexpr int kTileRows = 256;                                 // token rows of a tile at most
-constexpr int kFeat1 = 256;                                    // outputs of a gate/up tile
-constexpr int kFeat2 = 512;                                    // outputs of a down tile
-constexpr int kSlotRows = 16;                                  // rows of one slot of a merged tile
-constexpr int kMergeSlots = kTileRows / kSlotRows;             // slots of a merged tile at most
-constexpr int kMergeMaxRows = 64;                              // replicas of a shared expert are merged when none has more rows
 constexpr int kItems = 2;                                      // mailbox slots of a CTA (tiles dealt ahead)
 constexpr int kParts = 4;                                      // tiles whose epilogues may be under way at once in a CTA: a tile is dealt
                                                                // only when every warp has begun the one kItems before it, so at most kItems + 1
@@ -260,17 +254,6 @@ __device__ __forceinline__ float silu_mul(uint32_t g_bits, uint32_t u_bits) {
   return fmaf(h, t, h) * u;
 }
 
-// Accumulator columns of a tile of `valid_rows` token rows: rounded up to 16 (each CTA of the pair supplies half
-// of them, whole 8-row groups of the swizzled layout).
-__device__ __forceinline__ int tile_cols(int valid_rows) {
-  const int n = (valid_rows + 15) & ~15;
-  return n > kTileRows ? kTileRows : n;
-}
-// Columns of a merged tile of n 16-row slots: an even number of slots, so that neither CTA's half cuts a slot.
-__device__ __forceinline__ int merged_cols(int n_slots) { return ((n_slots + 1) & ~1) * kSlotRows; }
-// Columns of a tile from its list entry (y = rows, or minus the slot count of a merged tile).
-__device__ __forceinline__ int entry_cols(int y) { return y < 0 ? merged_cols(-y) : tile_cols(y); }
-
 // Which part of TMEM a tile's two accumulators take.  TMEM is two halves of 256 columns, each with a full and an
 // empty barrier.  A tile of more than 128 columns takes both (one accumulator in each); a narrower one takes the
 // half that is next in turn, so that its epilogue runs while the next tile's MMAs fill the other half.  The MMA
@@ -322,19 +305,6 @@ __device__ __forceinline__ void drain_packed(uint32_t acc, uint32_t (&out)[N][8]
 }
 
 // ---- the grouped GEMM kernel -----------------------------------------------------------------
-// One entry of the tile list.
-struct Tile {
-  int row;      // first row, or first slot of a merged tile
-  int rows;     // rows (1 .. 256); -n for a merged tile of n slots of 16 rows, slots[row ..): (first row, rows)
-  int w;        // weight matrix; negative: the list has ended
-  int out;      // output tile
-  int phase;    // 1: gate/up + SwiGLU (256 outputs per tile);  2: down (512 outputs per tile)
-  int done;     // the token tile this one belongs to: entry of `ready`
-  int need;     // phase 2: arrivals on that entry after which the rows of the intermediate are all written (0: they are)
-  int pad;
-};
-static_assert(sizeof(Tile) == 32, "two 16-byte words");
-
 // Token-row boxes of 128 / 64 / 32 / 16 / 8 rows over one activation tensor.
 struct TokenMaps {
   CUtensorMap box[5];
@@ -821,275 +791,36 @@ __global__ void bounded_wait_probe_kernel(long long limit_cycles, int* status, i
   }
 }
 
-// ---- tile list construction ------------------------------------------------------------------
-// A group of `rows` rows is cut into ceil(rows / 256) tiles of nearly equal size, so no tile is a short
-// remainder that would still stream a whole weight tile.
-__device__ __forceinline__ int group_tiles(int rows) { return (rows + kTileRows - 1) / kTileRows; }
-// Columns (token rows rounded up to 16) of the largest tile of a group; its cost class is that count in steps of 32.
-__device__ __forceinline__ int group_cols(int rows) {
-  const int t = group_tiles(rows);
-  return t ? tile_cols((rows + t - 1) / t) : 0;
-}
-
-// Processing order of the groups.  The group table is device-major, so the D replicas of a shared
-// expert (one group per virtual device, all reading the same weight matrix) lie far apart in it.
-// Tiles are therefore listed in another order: first every routed group in table order, then the
-// shared groups sorted by (layer, shared expert, device), so the replicas of one matrix are worked on
-// side by side, share its tiles in L2 and the matrix leaves HBM once per step instead of D times.
-// With a device filter (per-device timing) the device's own range is listed in table order.
-__device__ __forceinline__ int group_at(const ModelParams& mp, const int* dev_off, int nl, int device, int g0, int i) {
-  if (device >= 0) return g0 + i;
-  const int routed = nl * mp.E;
-  if (i < routed) {
-    int d = 0;
-    while (d + 1 < mp.D && i >= nl * dev_off[d + 1]) ++d;
-    const int n_d = dev_off[d + 1] - dev_off[d];
-    const int rel = i - nl * dev_off[d];
-    return nl * (dev_off[d] + d * mp.S) + (rel / n_d) * (n_d + mp.S) + rel % n_d;
-  }
-  const int q = i - routed;
-  const int lr = q / (mp.S * mp.D), s = (q / mp.D) % mp.S, d = q % mp.D;
-  const int n_d = dev_off[d + 1] - dev_off[d];
-  return nl * (dev_off[d] + d * mp.S) + lr * (n_d + mp.S) + n_d + s;
-}
-
-// The D replicas of a shared expert, when all are small, are packed into common tiles: the rows of each
-// replica are cut into slots of 16 (one TMA box, one epilogue chunk), up to sixteen slots per tile, so the
-// weight tile is fetched once for all of them.  `i` is a position of the processing order; returns true if
-// it belongs to such a merged class and gives the class's first position and slot count.
-__device__ __forceinline__ bool merged_class(const ModelParams& mp, const int* dev_off, int nl, int device, int i,
-                                             const int32_t* __restrict__ group_off, int* head, int* n_slots) {
-  if (device >= 0 || mp.S == 0 || mp.D < 2 || i < nl * mp.E) return false;
-  const int q = i - nl * mp.E;
-  const int h = i - q % mp.D;   // position of the class's replica on device 0
-  int tot = 0, mx = 0;
-  for (int d = 0; d < mp.D; ++d) {
-    const int g = group_at(mp, dev_off, nl, device, 0, h + d);
-    const int rows = group_off[g + 1] - group_off[g];
-    tot += (rows + kSlotRows - 1) / kSlotRows;
-    mx = rows > mx ? rows : mx;
-  }
-  *head = h;
-  *n_slots = tot;
-  return mx <= kMergeMaxRows;
-}
-
-// Cost classes of the tiles: class c holds the positions whose tiles have 32 c + 1 .. 32 (c + 1) columns.
-constexpr int kClasses = kTileRows / 32;
-
-// Block-wide exclusive scan (1024 threads) of one value per thread that belongs to one of kClasses classes:
-// returns the sum of the values of the same class in the threads before this one, and adds every class's
-// block total to total[].  A value packs two counters (low / high 32 bits).  Ends with a barrier.
-__device__ __forceinline__ long long block_scan_by_class(int cls, long long v, long long (*s_warp)[kClasses],
-                                                         long long* total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  long long incl[kClasses];
-#pragma unroll
-  for (int c = 0; c < kClasses; ++c) incl[c] = c == cls ? v : 0;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-#pragma unroll
-    for (int c = 0; c < kClasses; ++c) {
-      const long long n = __shfl_up_sync(0xffffffffu, incl[c], o);
-      if (lane >= o) incl[c] += n;
-    }
-  }
-  if (lane == 31) {
-#pragma unroll
-    for (int c = 0; c < kClasses; ++c) s_warp[warp][c] = incl[c];
-  }
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int c = 0; c < kClasses; ++c) {
-      const long long wv = s_warp[lane][c];
-      long long wi = wv;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const long long n = __shfl_up_sync(0xffffffffu, wi, o);
-        if (lane >= o) wi += n;
-      }
-      s_warp[lane][c] = wi - wv;
-      if (lane == 31) s_warp[32][c] = wi;
-    }
-  }
-  __syncthreads();
-  long long excl = 0;
-#pragma unroll
-  for (int c = 0; c < kClasses; ++c) {
-    if (c == cls) excl = s_warp[warp][c] + incl[c] - v;
-    total[c] += s_warp[32][c];
-  }
-  __syncthreads();
-  return excl;
-}
-
-// plan: per position i of the processing order (requested group range), the group, its tile count and
-// cost class; then the positions that own tiles are listed by cost class (widest tiles first, processing
-// order inside a class) with the exclusive scan of their tile counts.  Widest-first order lets the
-// expert kernel deal its tiles out in rounds of near-equal cost.  One scan carries all classes at once.
+// ---- tile list construction: eb_tiles.cuh -----------------------------------------------------
 __global__ void __launch_bounds__(1024)
-plan_kernel(ModelParams mp, const int32_t* __restrict__ group_off, const int32_t* __restrict__ step_meta, int device,
-            int nt1, int nt2, int32_t* __restrict__ pgroup, int32_t* __restrict__ pslots, int4* __restrict__ prank,
-            int32_t* __restrict__ order, int32_t* __restrict__ tile_pref, int32_t* __restrict__ work_count) {
+plan_kernel(ModelParams mp, const int32_t* __restrict__ group_off, const int32_t* __restrict__ step_meta, int device, TilePlan out) {
   EB_GRID_DEP_SYNC();
-  __shared__ long long s_warp[33][kClasses];
+  __shared__ OrderShared sh;
   __shared__ int s_dev_off[EB_MAX_D + 1];
-  const int tid = threadIdx.x;
-  if (tid <= mp.D) s_dev_off[tid] = mp.dev_off[tid];
-  const int G = step_meta[1];
+  if (threadIdx.x <= mp.D) s_dev_off[threadIdx.x] = mp.dev_off[threadIdx.x];
   const int g0 = device < 0 ? 0 : step_meta[3 + device];
-  const int g1 = device < 0 ? G : step_meta[3 + device + 1];
-  const int ng = g1 - g0;
+  const int g1 = device < 0 ? step_meta[1] : step_meta[3 + device + 1];
   const int nl = step_meta[2];
   __syncthreads();
-  // pass 1: tiles and class of every position; its rank and tile prefix inside its class
-  long long total[kClasses];   // low 32 bits: positions of the class, high 32 bits: their tiles
-#pragma unroll
-  for (int c = 0; c < kClasses; ++c) total[c] = 0;
-  int my_cls = -1;             // of the position this thread handled in the last chunk (the only one, as a rule)
-  long long my_at = 0;
-  for (int b = 0; b < ng; b += 1024) {
-    const int i = b + tid;
-    int tiles = 0, cols = 0;
-    if (i < ng) {
-      const int g = group_at(mp, s_dev_off, nl, device, g0, i);
-      const int rows = group_off[g + 1] - group_off[g];
-      int head, n_slots;
-      pgroup[i] = g;
-      pslots[i] = -1;
-      if (merged_class(mp, s_dev_off, nl, device, i, group_off, &head, &n_slots)) {
-        pslots[i] = n_slots;
-        if (i == head && n_slots > 0) {   // the class's tiles sit at its first position
-          tiles = (n_slots + kMergeSlots - 1) / kMergeSlots;
-          cols = merged_cols(n_slots < kMergeSlots ? n_slots : kMergeSlots);
-        }
-      } else {
-        tiles = group_tiles(rows);
-        cols = group_cols(rows);
-      }
+  auto item = [&](int i) {
+    const int g = group_at(mp, s_dev_off, nl, device, g0, i);
+    int head, n_slots;
+    if (merged_class(mp, s_dev_off, nl, device, i, group_off, &head, &n_slots)) {
+      // the class's tiles sit at its first position
+      const int tiles = i == head ? (n_slots + kMergeSlots - 1) / kMergeSlots : 0;
+      return Position{g, n_slots, tiles, cost_class(tiles, merged_cols(min(n_slots, kMergeSlots)))};
     }
-    const int cls = tiles > 0 ? (cols + 31) / 32 - 1 : -1;
-    long long before[kClasses];
-#pragma unroll
-    for (int c = 0; c < kClasses; ++c) before[c] = total[c];
-    const long long excl = block_scan_by_class(cls, tiles > 0 ? (1LL | ((long long)tiles << 32)) : 0, s_warp, total);
-    my_cls = cls;
-    my_at = 0;
-#pragma unroll
-    for (int c = 0; c < kClasses; ++c)
-      if (c == cls) my_at = before[c] + excl;
-    // more than one chunk of positions: parked until the class bases are known (read back by the same thread)
-    if (ng > 1024 && i < ng) prank[i] = make_int4(cls, (int)(my_at & 0xffffffffLL), (int)(my_at >> 32), 0);
-  }
-  // class bases: widest class first
-  long long base[kClasses];
-  long long run = 0;
-#pragma unroll
-  for (int c = kClasses - 1; c >= 0; --c) {
-    base[c] = run;
-    run += total[c];
-  }
-  const int n_listed = (int)(run & 0xffffffffLL), nt = (int)(run >> 32);
-  // pass 2: place every position that owns tiles
-  for (int b = 0; b < ng; b += 1024) {
-    const int i = b + tid;
-    int cls = my_cls, rank = (int)(my_at & 0xffffffffLL), tpref = (int)(my_at >> 32);
-    if (ng > 1024) {
-      cls = -1;
-      if (i < ng) {
-        const int4 v = prank[i];
-        cls = v.x;
-        rank = v.y;
-        tpref = v.z;
-      }
-    }
-    if (cls >= 0) {
-      long long b2 = 0;
-#pragma unroll
-      for (int c = 0; c < kClasses; ++c)
-        if (c == cls) b2 = base[c];
-      const int at = (int)(b2 & 0xffffffffLL) + rank;
-      order[at] = i;
-      tile_pref[at] = (int)(b2 >> 32) + tpref;
-    }
-  }
-  if (tid == 0) {
-    tile_pref[n_listed] = nt;
-    work_count[0] = nt * nt1;
-    work_count[1] = nt * nt2;
-    work_count[2] = nt;
-    work_count[3] = g0;
-    work_count[4] = ng;
-    work_count[5] = n_listed;
-    work_count[6] = work_count[7] = 0;   // tiles dealt out by the expert kernel
-    work_count[8] = nl;
-    work_count[9] = device;
-  }
+    const int rows = group_off[g + 1] - group_off[g], tiles = group_tiles(rows);
+    return Position{g, -1, tiles, cost_class(tiles, group_cols(rows))};
+  };
+  order_tiles(g1 - g0, nl, device, g0, item, out, sh);
 }
 
-// fill: one thread per tile of the list (gate/up tiles, then down tiles); tiles of a group are ordered weight-tile
-// major, token-tile minor.
 __global__ void __launch_bounds__(256)
-fill_kernel(ModelParams mp, const int32_t* __restrict__ group_off, const int32_t* __restrict__ group_w,
-            const int32_t* __restrict__ pgroup, const int32_t* __restrict__ pslots, const int32_t* __restrict__ order,
-            const int32_t* __restrict__ tile_pref, const int32_t* __restrict__ work_count, int nt1, int nt2, int max_work,
-            Tile* __restrict__ work, int32_t* __restrict__ ready, int2* __restrict__ slots) {
+fill_kernel(ModelParams mp, const int32_t* __restrict__ group_off, const int32_t* __restrict__ group_w, TileList list) {
   EB_GRID_DEP_SYNC();
-  extern __shared__ int s_pref[];   // tile_pref staged once per block: the binary search below then stays on chip
-  const int n_listed = work_count[5];
-  const int cnt1 = work_count[0], total = cnt1 + work_count[1];
-  if ((int)(blockIdx.x * blockDim.x) >= total) return;
-  for (int i = threadIdx.x; i <= n_listed; i += blockDim.x) s_pref[i] = tile_pref[i];
-  __syncthreads();
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
-    const int list = idx >= cnt1 ? 1 : 0, local = idx - (list ? cnt1 : 0);
-    const int nt = list ? nt2 : nt1;
-    const int t_index = local / nt;
-    // largest entry with tile_pref <= t_index (every listed position owns at least one tile)
-    int lo = 0, hi = n_listed - 1;
-    while (lo < hi) {
-      int mid = (lo + hi + 1) >> 1;
-      if (s_pref[mid] <= t_index) lo = mid; else hi = mid - 1;
-    }
-    const int t_g = s_pref[lo + 1] - s_pref[lo];
-    const int rem = local - s_pref[lo] * nt;
-    const int n = rem / t_g, m = rem % t_g;
-    const int pos = order[lo], g = pgroup[pos], n_slots = pslots[pos];
-    Tile it;
-    if (n_slots >= 0) {
-      // tile m of a merged class holds the next 16 slots of the class, replicas in device order
-      const int base = kMergeSlots * (s_pref[lo] + m);
-      const int first = kMergeSlots * m, n_here = min(kMergeSlots, n_slots - first);
-      if (list == 0 && n == 0) {
-        int c = 0;   // slots before the current replica
-        for (int d = 0; d < mp.D; ++d) {
-          const int gd = pgroup[pos + d];
-          const int r0 = group_off[gd], rows = group_off[gd + 1] - r0;
-          const int nc = (rows + kSlotRows - 1) / kSlotRows;
-          for (int k = 0; k < nc; ++k, ++c)
-            if (c >= first && c < first + n_here)
-              slots[base + c - first] = make_int2(r0 + k * kSlotRows, min(kSlotRows, rows - k * kSlotRows));
-        }
-      }
-      it.row = base;
-      it.rows = -n_here;
-    } else {
-      // t_g tiles of nearly equal size: the first (rows % t_g) tiles hold one row more
-      const int rows = group_off[g + 1] - group_off[g];
-      const int each = rows / t_g, more = rows % t_g;
-      it.row = group_off[g] + m * each + min(m, more);
-      it.rows = each + (m < more ? 1 : 0);
-    }
-    it.w = group_w[g];
-    it.out = n;
-    it.phase = list + 1;
-    it.done = s_pref[lo] + m;
-    it.need = nt1 * 2;
-    it.pad = 0;
-    if (list == 0 && n == 0) ready[it.done] = 0;
-    if (idx < max_work) work[idx] = it;
-  }
+  extern __shared__ int s_pref[];
+  fill_tiles(mp, group_off, group_w, list, s_pref, blockIdx.x, gridDim.x);
 }
 
 // ---- host side ---------------------------------------------------------------------------------
@@ -1185,7 +916,7 @@ eb_status ebi_ffn_bind(eb_ctx* c) {
 }
 
 eb_status ebi_ffn_run(eb_ctx* c, cudaStream_t st, const void* xp, const int32_t* group_off, const int32_t* group_w,
-                      const int32_t* step_meta, void* yp, int32_t device) {
+                      const int32_t* step_meta, void* yp, int32_t device, bool planned) {
   if (!xp || !group_off || !group_w || !step_meta || !yp) return ebi_fail(c, EB_ERR_INVALID_ARG, "null pointer");
   if (eb_status ds = ebi_check_device(c)) return ds;
   if (!ebi_aligned16(xp) || !ebi_aligned16(yp)) return ebi_fail(c, EB_ERR_INVALID_ARG, "xp / yp must be 16-byte aligned");
@@ -1199,11 +930,10 @@ eb_status ebi_ffn_run(eb_ctx* c, cudaStream_t st, const void* xp, const int32_t*
   for (int i = 0; i < 5; ++i)
     if (!make_map(&p.xp.box[i], xp, g.H, rows, 0, BK, box_rows[i]) || !make_map(&p.act.box[i], c->act, g.I, rows, 0, BK, box_rows[i]))
       return ebi_fail(c, EB_ERR_CUDA, "cuTensorMapEncodeTiled failed for the activations");
-  Tile* const work = (Tile*)c->work;
   p.gate = c->tm_gate;
   p.up = c->tm_up;
   p.down = c->tm_down;
-  p.work = work;
+  p.work = (const Tile*)c->work;
   p.max_work = c->max_work;
   p.slots = c->slots;
   p.work_count = c->work_count;
@@ -1214,18 +944,14 @@ eb_status ebi_ffn_run(eb_ctx* c, cudaStream_t st, const void* xp, const int32_t*
   p.H = g.H;
   p.I = g.I;
   p.status = c->d_status;
-  const int nt1 = (g.I + kFeat1 - 1) / kFeat1, nt2 = (g.H + kFeat2 - 1) / kFeat2;
-  {
-    KernelTimer timer(c, EBK_FFN_PLAN, st);
-    ebi_launch(plan_kernel, dim3(1), dim3(1024), 0, st, c->mp, group_off, step_meta, (int)device, nt1, nt2, c->pgroup, c->pslots,
-               c->prank, c->order, c->tile_pref, c->work_count);
-  }
-  {
+  if (!planned) {
+    {
+      KernelTimer timer(c, EBK_FFN_PLAN, st);
+      ebi_launch(plan_kernel, dim3(1), dim3(1024), 0, st, c->mp, group_off, step_meta, (int)device, tile_plan_of(c));
+    }
     KernelTimer timer(c, EBK_FFN_FILL, st);
     ebi_launch(fill_kernel, dim3(c->num_sms), dim3(256), sizeof(int) * (size_t)(ebi_groups_cap(c) + 1), st, c->mp, group_off, group_w,
-               (const int32_t*)c->pgroup,
-               (const int32_t*)c->pslots, (const int32_t*)c->order, (const int32_t*)c->tile_pref,
-               (const int32_t*)c->work_count, nt1, nt2, c->max_work, work, c->tile_ready, c->slots);
+               tile_list_of(c));
   }
   cudaError_t e;
   if (!c->timing) {

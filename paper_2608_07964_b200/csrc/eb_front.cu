@@ -1,0 +1,481 @@
+// The front end of a whole step, eb_step: everything between the inputs and the expert pass in three launches.
+//
+//   front_kernel  : per chunk of <= 32 tokens: routing (a warp per token) and the chunk's assignments per expert
+//   tables_kernel : one block: loads, schedule, group table, tile plan
+//   scatter_kernel: per part of a chunk: ranks, positions, gather of the token rows; some blocks fill the tile list
+//
+// The stages called one by one (eb_route, eb_schedule, eb_permute, eb_expert_ffn_grouped) take eight to eleven
+// launches for the same tables.  What bounds these kernels is not work but the chain of hand-overs between them, each
+// a launch, a first trip to memory and a few block barriers (2-5 us), so the split here follows the dependences that
+// need the whole GPU to be through: the counts of all tokens, then the positions of all rows.  The counts travel as
+// chunk histograms, which also spares the routing its global atomics.
+#include "eb_dispatch.cuh"
+#include "eb_route.cuh"
+#include "eb_schedule.cuh"
+#include "eb_tiles.cuh"
+
+namespace {
+
+constexpr int kFrontThreads = 1024;   // a warp per token of the chunk
+
+// PL: logits per lane.  With two (E <= 64) the registers leave room for two blocks per SM.
+template <int PL>
+__global__ void __launch_bounds__(kFrontThreads, PL <= 2 ? 2 : 1)
+front_kernel(ModelParams mp, BatchParams bp, uint32_t pool_mask, uint32_t route_mask, const float* __restrict__ logits,
+             int32_t* __restrict__ topk_idx, float* __restrict__ topk_w, int32_t* __restrict__ chunk_hist) {
+  EB_GRID_DEP_SYNC();
+  __shared__ int s_hist[EB_MAX_E];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int c = blockIdx.x, j = mb_of_chunk(bp, c);
+  const bool routed = (route_mask >> j) & 1u;
+  if (!routed && !((pool_mask >> j) & 1u)) return;
+  for (int e = threadIdx.x; e < mp.E; e += kFrontThreads) s_hist[e] = 0;
+  __syncthreads();
+  const int t = bp.tok_off[j] + (c - bp.chunk_off[j]) * 32 + warp;
+  if (t < bp.tok_off[j + 1]) {
+    int e = -1;
+    if (routed) e = route_token<PL>(mp, t, lane, logits, topk_idx, topk_w);
+    else if (lane < mp.K) e = topk_idx[(size_t)t * mp.K + lane];   // deferred: routed when it reached its layer
+    // an index outside [0, E) (only in a table not written by the routing) is skipped here and reported by scatter_kernel
+    if (lane < mp.K && (unsigned)e < (unsigned)mp.E) atomicAdd(&s_hist[e], 1);
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < mp.E; e += kFrontThreads) chunk_hist[(size_t)c * mp.E + e] = s_hist[e];
+}
+
+// ---- tables ----------------------------------------------------------------------------------
+struct TablesArgs {
+  uint32_t pool_mask, route_mask;
+  int m, policy;
+  const int32_t* chunk_hist;
+  int32_t *chunk_base, *chunk_seg, *mb_base, *mb_load, *mb_cnt;
+  eb_sched_result* res;
+  int32_t *group_off, *group_w, *step_meta;
+  TilePlan plan;
+};
+
+// i / E for i < 2^16 (E <= 256): one multiplication by ceil(2^32 / E); larger i take the division
+__device__ __forceinline__ int div_by(int i, int E, unsigned magic) { return i < 65536 ? (int)__umulhi((unsigned)i, magic) : i / E; }
+
+// What bounds this kernel is its own chain of phases, a few hundred cycles each at best: every phase has a thread per
+// item of the widest kind ((micro-batch, expert) or (layer, expert)), takes what it needs from shared memory, and
+// decodes nothing by loops or divisions that a table or a multiplication gives.
+__global__ void __launch_bounds__(kSchedThreads)
+tables_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ BatchParams bp, const __grid_constant__ TablesArgs a) {
+  EB_GRID_DEP_SYNC();
+  extern __shared__ int4 s_dyn4[];
+  __shared__ int s_dev_off[EB_MAX_D + 1], s_dev_list[EB_MAX_E], s_e2d[EB_MAX_E], s_seg_off[EB_MAX_MB + 1];
+  __shared__ int s_home[EB_MAX_MB][EB_MAX_D + 1];   // first local token of every home device, per micro-batch
+  __shared__ int s_hrows[EB_MAX_MB][EB_MAX_D];      // rows of a shared expert's replica: (active layer, device)
+  __shared__ int s_hslots[EB_MAX_MB], s_hmax[EB_MAX_MB];   // slots of its merged class and its largest replica: per active layer
+  __shared__ int s_mbs[EB_MAX_MB];                  // chosen micro-batches of every active layer, as bits
+  __shared__ int s_warp[32];
+  __shared__ int s_carry;
+  __shared__ StepShape ss;
+  __shared__ OrderShared s_order;
+  SchedShared& sc = *reinterpret_cast<SchedShared*>(s_dyn4);
+  int* const s_cnt = reinterpret_cast<int*>(s_dyn4) + sizeof(SchedShared) / 4;   // [n_mb][E] assignments, then rows before
+  int* const s_goff = s_cnt + bp.n_mb * mp.E;                                    // [G + 1] group sizes, then offsets
+  const int g_cap = bp.n_mb * (mp.E + mp.D * mp.S);
+  int* const s_pgroup = s_goff + g_cap + 1;                                      // [G] group at every position
+  int* const s_ptiles = s_pgroup + g_cap;                                        // [G] its tiles and cost class
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int E = mp.E, S = mp.S, D = mp.D, n_mb = bp.n_mb;
+  const unsigned magic = (unsigned)(((1ULL << 32) + E - 1) / E);   // E = 1: wraps to 0, see div_e
+  auto div_e = [&](int i) { return E == 1 ? i : div_by(i, E, magic); };
+
+  // ---- small tables; loads of the micro-batches that keep their routing
+  if (tid <= D) s_dev_off[tid] = mp.dev_off[tid];
+  for (int e = tid; e < E; e += kSchedThreads) {
+    s_dev_list[e] = mp.dev_list[e];
+    s_e2d[e] = mp.e2d[e];
+  }
+  if (tid >= 512 && tid < 512 + EB_MAX_MB * EB_MAX_D) {
+    const int j = (tid - 512) / EB_MAX_D, d = tid % EB_MAX_D;
+    sc.load[j][d] = (j < n_mb && d < D && !((a.route_mask >> j) & 1u)) ? a.mb_load[j * D + d] : 0;
+  }
+  if (tid >= 256 && tid < 256 + EB_MAX_MB * 16) {
+    const int j = (tid - 256) / 16, d = tid % 16;
+    if (j < n_mb && d <= D) {
+      const int T = bp.tok_off[j + 1] - bp.tok_off[j];
+      s_home[j][d] = home_start(d, T, D);
+      if (d == 15 && D == 16) s_home[j][16] = T;
+    }
+  }
+  if (warp == 31) {
+    const int j = lane < n_mb ? lane : 0;
+    const int n = lane < n_mb ? (bp.chunk_off[j + 1] - bp.chunk_off[j] + EB_SEG_CHUNKS - 1) / EB_SEG_CHUNKS : 0;
+    int incl = n;
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    if (lane < EB_MAX_MB) s_seg_off[lane + 1] = incl;   // beyond n_mb: the total
+    if (lane == 0) s_seg_off[0] = s_carry = 0;
+  }
+  for (int i = tid; i < n_mb * E; i += kSchedThreads) s_cnt[i] = 0;
+  __syncthreads();
+
+  // ---- assignments of every (micro-batch, expert) from the chunk histograms; chunk_base = those before the chunk in its
+  // micro-batch.  One thread per segment of chunks and expert; a micro-batch of one segment (<= 1024 tokens) is done
+  // in one go, a longer one adds up its segments in between.
+  const int n_items = s_seg_off[EB_MAX_MB] * E;
+  const uint32_t counted = a.pool_mask | a.route_mask;
+  auto mb_of_seg = [&](int g) {   // the last micro-batch whose segments start at or before g
+    int j = 0;
+#pragma unroll
+    for (int step = 8; step > 0; step >>= 1)
+      if (s_seg_off[j + step] <= g) j += step;
+    return j;
+  };
+  bool any_long = false;
+  for (int i = tid; i < n_items; i += kSchedThreads) {
+    const int g = div_e(i), e = i - g * E, j = mb_of_seg(g);
+    if (!((counted >> j) & 1u)) continue;
+    const int c0 = bp.chunk_off[j] + (g - s_seg_off[j]) * EB_SEG_CHUNKS;
+    const int n = min((int)EB_SEG_CHUNKS, bp.chunk_off[j + 1] - c0);
+    const bool whole = s_seg_off[j + 1] - s_seg_off[j] == 1;
+    const int32_t* h = a.chunk_hist + (size_t)c0 * E + e;
+    int32_t* base = a.chunk_base + (size_t)c0 * E + e;
+    int run = 0;
+    for (int k0 = 0; k0 < n; k0 += 16) {
+      int v[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = k0 + k < n ? h[(size_t)(k0 + k) * E] : 0;
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        if (whole && k0 + k < n) base[(size_t)(k0 + k) * E] = run;
+        run += v[k];
+      }
+    }
+    if (whole) {
+      s_cnt[j * E + e] = run;
+    } else {
+      a.chunk_seg[i] = run;
+      any_long = true;
+    }
+  }
+  if (__syncthreads_or(any_long)) {
+    for (int i = tid; i < n_mb * E; i += kSchedThreads) {
+      const int j = div_e(i), e = i - j * E;
+      if (s_seg_off[j + 1] - s_seg_off[j] < 2 || !((counted >> j) & 1u)) continue;
+      int run = 0;
+      for (int g = s_seg_off[j]; g < s_seg_off[j + 1]; ++g) {
+        const int v = a.chunk_seg[(size_t)g * E + e];
+        a.chunk_seg[(size_t)g * E + e] = run;
+        run += v;
+      }
+      s_cnt[i] = run;
+    }
+    __syncthreads();
+    for (int i = tid; i < n_items; i += kSchedThreads) {
+      const int g = div_e(i), e = i - g * E, j = mb_of_seg(g);
+      if (s_seg_off[j + 1] - s_seg_off[j] < 2 || !((counted >> j) & 1u)) continue;
+      const int c0 = bp.chunk_off[j] + (g - s_seg_off[j]) * EB_SEG_CHUNKS;
+      const int n = min((int)EB_SEG_CHUNKS, bp.chunk_off[j + 1] - c0);
+      int run = a.chunk_seg[i];
+      for (int k = 0; k < n; ++k) {
+        const int v = a.chunk_hist[(size_t)(c0 + k) * E + e];
+        a.chunk_base[(size_t)(c0 + k) * E + e] = run;
+        run += v;
+      }
+    }
+    __syncthreads();
+  }
+
+  // ---- loads of the micro-batches routed now: four threads per (micro-batch, device)
+  for (int i = tid; i < n_mb * E; i += kSchedThreads)
+    if ((a.route_mask >> div_e(i)) & 1u) a.mb_cnt[i] = s_cnt[i];
+  {
+    const int j = tid >> 6, d = (tid >> 2) & 15;
+    int v = 0;
+    if (j < n_mb && d < D)
+      for (int i = s_dev_off[d] + (tid & 3); i < s_dev_off[d + 1]; i += 4) v += s_cnt[j * E + s_dev_list[i]];
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    if ((tid & 3) == 0 && j < n_mb && d < D && ((a.route_mask >> j) & 1u)) {
+      sc.load[j][d] = v;
+      a.mb_load[j * D + d] = v;
+    }
+  }
+  __syncthreads();
+
+  // ---- schedule
+  schedule_block(sc, D, a.pool_mask, a.m, a.policy, 0, 1);
+  const uint32_t run = sc.run;
+  if (warp == 1) write_schedule(sc, D, a.pool_mask, a.res);
+  if (warp == 2 && lane < EB_MAX_MB) s_mbs[lane] = 0;
+  step_shape_block(bp, run, &ss);
+  const int nl = ss.nl, G = nl * (E + D * S);
+  if (tid < EB_MAX_MB && ss.rank_of_mb[tid] >= 0) atomicOr(&s_mbs[ss.rank_of_mb[tid]], 1 << tid);
+  __syncthreads();
+
+  // ---- routed groups: sizes, weight matrices, tiles; s_cnt turns into the rows of a group before the micro-batch
+  for (int i = tid; i < nl * E; i += kSchedThreads) {
+    const int lr = div_e(i), k = i - lr * E;   // k: expert in (device, expert) order
+    const int e = s_dev_list[k], d = s_e2d[e], off = s_dev_off[d], n_d = s_dev_off[d + 1] - off;
+    int tot = 0;
+    for (unsigned mbs = s_mbs[lr]; mbs; mbs &= mbs - 1) {
+      int* at = s_cnt + (__ffs(mbs) - 1) * E + e;
+      const int v = *at;
+      *at = tot;
+      tot += v;
+    }
+    const int g = nl * (off + d * S) + lr * (n_d + S) + (k - off);
+    s_goff[g] = tot;
+    a.group_w[g] = ss.act_layer[lr] * (E + S) + e;
+    const int pos = nl * off + lr * n_d + (k - off), tiles = group_tiles(tot);
+    s_pgroup[pos] = g;
+    s_ptiles[pos] = tiles << 4 | (cost_class(tiles, group_cols(tot)) & 15);
+  }
+  // ---- shared experts: rows = chosen tokens at the layer whose home device is d
+  if (S > 0) {
+    if (tid < EB_MAX_MB * EB_MAX_D) {   // whole warps; a layer's devices are sixteen neighbouring lanes
+      const int lr = tid >> 4, d = tid & 15;
+      int rows = 0;
+      if (lr < nl && d < D)
+        for (unsigned mbs = s_mbs[lr]; mbs; mbs &= mbs - 1) {
+          const int j = __ffs(mbs) - 1;
+          rows += s_home[j][d + 1] - s_home[j][d];
+        }
+      s_hrows[lr][d] = rows;
+      int slots = (rows + kSlotRows - 1) / kSlotRows, mx = rows;
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) {
+        slots += __shfl_xor_sync(0xffffffffu, slots, o);
+        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      }
+      if (d == 0) {
+        s_hslots[lr] = slots;
+        s_hmax[lr] = mx;
+      }
+    }
+    __syncthreads();
+    for (int i = tid; i < nl * S * D; i += kSchedThreads) {   // position order: layer, shared expert, device
+      const int q = i / D, d = i - q * D, lr = q / S, s = q - lr * S;
+      const int off = s_dev_off[d], n_d = s_dev_off[d + 1] - off, rows = s_hrows[lr][d];
+      const int g = nl * (off + d * S) + lr * (n_d + S) + n_d + s;
+      s_goff[g] = rows;
+      a.group_w[g] = ss.act_layer[lr] * (E + S) + E + s;
+      const bool merged = D >= 2 && s_hmax[lr] <= kMergeMaxRows;
+      const int n_slots = s_hslots[lr];
+      const int tiles = !merged ? group_tiles(rows) : d == 0 ? (n_slots + kMergeSlots - 1) / kMergeSlots : 0;
+      const int cols = merged ? merged_cols(min(n_slots, kMergeSlots)) : group_cols(rows);
+      s_pgroup[nl * E + i] = g;
+      s_ptiles[nl * E + i] = tiles << 4 | (cost_class(tiles, cols) & 15);
+    }
+  }
+  __syncthreads();
+
+  // ---- exclusive scan over groups, step_meta
+  for (int base = 0; base < G; base += kSchedThreads) {
+    const int g = base + tid;
+    const int v = g < G ? s_goff[g] : 0;
+    int incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int n = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += n;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    // every warp adds up the warps before it
+    int before = lane < warp ? s_warp[lane] : 0;
+    before = __reduce_add_sync(0xffffffffu, before) + s_carry;
+    const int excl = before + incl - v;
+    if (g < G) {
+      s_goff[g] = excl;
+      a.group_off[g] = excl;
+    }
+    __syncthreads();
+    if (tid == kSchedThreads - 1) s_carry = excl + v;
+    __syncthreads();
+  }
+  if (tid == 0) {
+    s_goff[G] = s_carry;
+    a.group_off[G] = s_carry;
+    a.step_meta[0] = s_carry;
+    a.step_meta[1] = G;
+    a.step_meta[2] = nl;
+  }
+  if (tid >= 32 && tid < 32 + EB_META_LEN - 3) {
+    const int i = tid - 32;   // entries 3 .. EB_META_LEN-1
+    a.step_meta[3 + i] = i < D ? nl * (s_dev_off[i] + i * S) : i == D ? G : 0;
+  }
+
+  // ---- first row of every chosen (micro-batch, expert)
+  for (int i = tid; i < n_mb * E; i += kSchedThreads) {
+    const int j = div_e(i), e = i - j * E, lr = ss.rank_of_mb[j];
+    if (lr < 0) continue;
+    const int d = s_e2d[e];
+    a.mb_base[i] = s_cnt[i] + s_goff[group_id(s_dev_off, S, nl, d, lr, mp.e_local[e])];
+  }
+
+  // ---- order of the tiles of the expert pass
+  auto item = [&](int i) {
+    const int t = s_ptiles[i], lr = i < nl * E ? 0 : (i - nl * E) / (S * D);
+    const bool merged = i >= nl * E && D >= 2 && s_hmax[lr] <= kMergeMaxRows;
+    return Position{s_pgroup[i], merged ? s_hslots[lr] : -1, t >> 4, t >> 4 ? t & 15 : -1};
+  };
+  order_tiles(G, nl, -1, 0, item, a.plan, s_order);
+}
+
+// ---- scatter ---------------------------------------------------------------------------------
+constexpr int kScatterThreads = 256;
+
+struct ScatterArgs {
+  const eb_sched_result* res;
+  const int32_t *topk_idx, *chunk_base, *mb_base, *group_off, *group_w;
+  int32_t *pos, *row_src, *step_meta;
+  const uint4* x;
+  uint4* xp;
+  TileList list;
+  int fill_blocks;
+};
+
+// Blocks below fill_blocks write the tile list.  Each of the others places TB tokens of a chunk: one warp ranks the
+// chunk's assignments up to them (a few warp matches) while the others fetch the token rows, then every row goes out
+// to its K + S places.  TB is small while there are few tokens (a block each keeps the chip busy) and 8 when there are
+// many (the ranking is shared by more rows).
+template <int TB>
+__global__ void __launch_bounds__(kScatterThreads)
+scatter_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ BatchParams bp, const __grid_constant__ ScatterArgs a) {
+  EB_GRID_DEP_SYNC();
+  extern __shared__ int s_dyn[];
+  if ((int)blockIdx.x < a.fill_blocks) {
+    fill_tiles(mp, a.group_off, a.group_w, a.list, s_dyn, blockIdx.x, a.fill_blocks);
+    return;
+  }
+  __shared__ StepShape ss;
+  __shared__ int s_dev_off[EB_MAX_D + 1];
+  __shared__ int s_next[EB_MAX_E];
+  __shared__ int s_pos[TB][EB_MAX_K + EB_MAX_S];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int E = mp.E, K = mp.K, S = mp.S, KS = K + S, vec = mp.H / 8;
+  const int part = (int)blockIdx.x - a.fill_blocks, c = part / (32 / TB);
+  const int j = mb_of_chunk(bp, c);
+  const int c0 = bp.tok_off[j] + (c - bp.chunk_off[j]) * 32;      // first token of the chunk
+  const int t0 = c0 + part % (32 / TB) * TB;                      // and of this part
+  const int nt = min(TB, bp.tok_off[j + 1] - t0);
+  if (nt <= 0) return;
+  const uint32_t run = a.res->run_mask;
+  if (!((run >> j) & 1u)) {
+    for (int i = tid; i < nt * KS; i += kScatterThreads) a.pos[(size_t)t0 * KS + i] = -1;
+    return;
+  }
+  // the first columns of the rows are on their way while the positions are worked out
+  uint4 v[TB];
+#pragma unroll
+  for (int k = 0; k < TB; ++k)
+    if (k < nt && tid < vec) v[k] = __ldg(a.x + (size_t)(t0 + k) * vec + tid);
+  if (tid <= mp.D) s_dev_off[tid] = mp.dev_off[tid];
+  for (int e = tid; e < E; e += kScatterThreads) s_next[e] = a.mb_base[j * E + e] + a.chunk_base[(size_t)c * E + e];
+  step_shape_block(bp, run, &ss);   // ends with a barrier
+  if (tid < 32) {
+    const int lr = ss.rank_of_mb[j];
+    // routed slots in assignment order from the start of the chunk; the rows of the tokens before this part only count
+    const int first = (t0 - c0) * K, last = first + nt * K;
+    for (int a0 = 0; a0 < last; a0 += 32) {
+      const int i = a0 + lane;
+      bool valid = i < last;
+      int e = valid ? a.topk_idx[(size_t)c0 * K + i] : -1 - lane;   // distinct dummies never match
+      if (valid && (unsigned)e >= (unsigned)E) {
+        // an index outside [0, E) is never used: the slot gets no row and the step's meta data counts it
+        if (i >= first) {
+          a.pos[(size_t)(c0 + i / K) * KS + i % K] = -1;
+          s_pos[(i - first) / K][i % K] = -1;
+          atomicAdd(&a.step_meta[EB_META_LEN - 1], 1);
+        }
+        valid = false;
+        e = -1 - lane;
+      }
+      const unsigned peers = __match_any_sync(0xffffffffu, e);
+      const int before = __popc(peers & ((1u << lane) - 1u));
+      if (valid && i >= first) {
+        const int p = s_next[e] + before, t = c0 + i / K;
+        a.pos[(size_t)t * KS + i % K] = p;
+        a.row_src[p] = t;
+        s_pos[(i - first) / K][i % K] = p;
+      }
+      __syncwarp();
+      if (valid && before == 0) s_next[e] += __popc(peers);
+      __syncwarp();
+    }
+    // shared slots: closed-form rows
+    if (S > 0 && lane < nt) {
+      const int T = bp.tok_off[j + 1] - bp.tok_off[j], tl = t0 + lane - bp.tok_off[j];
+      const int d = home_device(tl, T, mp.D);
+      int before = 0;
+      for (int j2 = 0; j2 < j; ++j2)
+        if (ss.rank_of_mb[j2] == lr) {
+          const int T2 = bp.tok_off[j2 + 1] - bp.tok_off[j2];
+          before += home_start(d + 1, T2, mp.D) - home_start(d, T2, mp.D);
+        }
+      const int n_d = s_dev_off[d + 1] - s_dev_off[d];
+      const int g = group_id(s_dev_off, S, ss.nl, d, lr, n_d), at = before + (tl - home_start(d, T, mp.D));
+      for (int s = 0; s < S; ++s) {
+        const int p = a.group_off[g + s] + at;
+        a.pos[(size_t)(t0 + lane) * KS + K + s] = p;
+        a.row_src[p] = t0 + lane;
+        s_pos[lane][K + s] = p;
+      }
+    }
+  }
+  __syncthreads();
+  for (int col = tid; col < vec; col += kScatterThreads) {
+    if (col != tid) {
+#pragma unroll
+      for (int k = 0; k < TB; ++k)
+        if (k < nt) v[k] = __ldg(a.x + (size_t)(t0 + k) * vec + col);
+    }
+#pragma unroll
+    for (int k = 0; k < TB; ++k)
+      if (k < nt)
+        for (int s = 0; s < KS; ++s) {
+          const int p = s_pos[k][s];
+          if (p >= 0) a.xp[(size_t)p * vec + col] = v[k];
+        }
+  }
+}
+
+size_t tables_smem(const eb_ctx* c, int n_mb, int groups) {
+  return sizeof(SchedShared) + sizeof(int) * ((size_t)n_mb * c->cfg.E + 3 * (size_t)groups + 1);
+}
+
+}  // namespace
+
+eb_status ebi_front_run(eb_ctx* c, cudaStream_t st, const BatchParams& bp, uint32_t pool_mask, uint32_t route_mask, int32_t m,
+                        eb_policy policy, const eb_step_buffers* b) {
+  const eb_config& g = c->cfg;
+  if (!c->tables_attr_set) {   // per context: function attributes belong to the current device
+    EB_CUDA(c, cudaFuncSetAttribute(tables_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)tables_smem(c, EB_MAX_MB, ebi_groups_cap(c))));
+    c->tables_attr_set = true;
+  }
+  if (bp.n_chunks > 0) {
+    KernelTimer timer(c, EBK_ROUTE, st);
+    ebi_launch(g.E <= 64 ? front_kernel<2> : front_kernel<kMaxPerLane>, dim3(bp.n_chunks), dim3(kFrontThreads), 0, st, c->mp, bp, pool_mask, route_mask,
+               (const float*)b->logits, b->topk_idx, b->topk_w, c->chunk_hist);
+  }
+  {
+    KernelTimer timer(c, EBK_SCHEDULE, st);
+    const TablesArgs a{pool_mask, route_mask, (int)m, (int)policy, c->chunk_hist, c->chunk_base, c->chunk_seg, c->mb_base, b->mb_load,
+                       b->mb_cnt, b->sched, b->group_off, b->group_w, b->step_meta, tile_plan_of(c)};
+    ebi_launch(tables_kernel, dim3(1), dim3(kSchedThreads), tables_smem(c, bp.n_mb, bp.n_mb * (g.E + g.D * g.S)), st, c->mp, bp, a);
+  }
+  {
+    KernelTimer timer(c, EBK_PERMUTE_GATHER, st);
+    const ScatterArgs a{b->sched, b->topk_idx, c->chunk_base, c->mb_base, b->group_off, b->group_w, b->pos, b->row_src, b->step_meta,
+                        (const uint4*)b->x, (uint4*)b->xp, tile_list_of(c), c->num_sms / 2};
+    const size_t smem = sizeof(int) * (size_t)(ebi_groups_cap(c) + 1);
+    auto launch = [&](auto kernel, int tb) {
+      ebi_launch(kernel, dim3(a.fill_blocks + bp.n_chunks * (32 / tb)), dim3(kScatterThreads), smem, st, c->mp, bp, a);
+    };
+    if (bp.n_tok <= 2 * c->num_sms) launch(scatter_kernel<1>, 1);
+    else if (bp.n_tok <= 16 * c->num_sms) launch(scatter_kernel<4>, 4);
+    else launch(scatter_kernel<8>, 8);
+  }
+  EB_LAUNCH_CHECK(c, "step front end");
+  return EB_OK;
+}

@@ -16,6 +16,9 @@ typedef __nv_bfloat16 bf16;
 
 enum { EB_MAX_GUARDS = 24 };
 
+// Chunks whose histograms one thread of a whole step's table kernel adds up.
+enum { EB_SEG_CHUNKS = 32 };
+
 // Kernel ids for the optional per-kernel event timing.
 enum EbKernel {
   EBK_ROUTE = 0,
@@ -76,6 +79,8 @@ struct eb_ctx {
   size_t guard_off[EB_MAX_GUARDS] = {};
   int32_t* chunk_hist = nullptr;   // [max_chunks][E]
   int32_t* chunk_base = nullptr;   // [max_chunks][E]
+  int32_t* chunk_seg = nullptr;    // [max_segs][E] assignments of every segment of chunks (whole steps)
+  int32_t* mb_base = nullptr;      // [EB_MAX_MB][E] first row of every micro-batch in its groups (whole steps)
   int32_t* group_size = nullptr;   // [G_cap]
   int32_t* pgroup = nullptr;       // [G_cap] group at each position of the processing order
   int32_t* pslots = nullptr;       // [G_cap] 16-row slots of the merged shared-expert class of the position, -1 otherwise
@@ -89,7 +94,7 @@ struct eb_ctx {
   bf16* act = nullptr;             // [R_cap][I]
   int32_t max_chunks = 0, max_tiles = 0, max_work = 0;
 
-  bool fused_attr_set = false;
+  bool fused_attr_set = false, tables_attr_set = false;
   // eb_step_host_submit / eb_step_host_wait: copy streams and per-slot events, created on first use
   cudaStream_t s_in = nullptr, s_out = nullptr;
   cudaEvent_t ev_in[EB_HOST_SLOTS] = {}, ev_step[EB_HOST_SLOTS] = {}, ev_out[EB_HOST_SLOTS] = {};
@@ -167,6 +172,9 @@ static inline bool ebi_aligned16(const void* p) { return (reinterpret_cast<uintp
 
 // Entry points of the per-step stages (defined in their own translation units).
 eb_status ebi_ffn_run(eb_ctx* c, cudaStream_t st, const void* xp, const int32_t* group_off,
-                      const int32_t* group_w, const int32_t* step_meta, void* yp, int32_t device);
+                      const int32_t* group_w, const int32_t* step_meta, void* yp, int32_t device, bool planned = false);
+// Routing, schedule, dispatch tables, gather and tile list of a whole step (eb_front.cu).
+eb_status ebi_front_run(eb_ctx* c, cudaStream_t st, const BatchParams& bp, uint32_t pool_mask, uint32_t route_mask, int32_t m,
+                        eb_policy policy, const eb_step_buffers* b);
 eb_status ebi_ffn_bind(eb_ctx* c);
 eb_status ebi_selftest_wait(eb_ctx* c, cudaStream_t st, long long limit_cycles, int* d_gave_up);

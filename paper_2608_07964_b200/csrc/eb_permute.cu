@@ -12,73 +12,11 @@
 // No order-dependent atomics anywhere: rows inside a group are in (micro-batch, token) order.
 #include <cstring>
 
-#include "eb_internal.cuh"
+#include "eb_dispatch.cuh"
 
 namespace {
 
 constexpr int kWarps = 8;
-
-struct StepShape {
-  int nl;                       // active layers
-  int act_layer[EB_MAX_MB];     // ascending
-  int rank_of_mb[EB_MAX_MB];    // rank of the micro-batch's layer among active layers, -1 if not chosen
-};
-
-// first token (local index) of micro-batch of T tokens whose home device is >= d
-__device__ __forceinline__ int home_start(int d, int T, int D) {
-  if (T < (1 << 26)) return (int)(((unsigned)d * (unsigned)T + (unsigned)(D - 1)) / (unsigned)D);   // d <= 16: no overflow
-  return (int)(((long long)d * T + D - 1) / D);
-}
-// home device of local token tl of a micro-batch of T tokens: floor(tl * D / T)
-__device__ __forceinline__ int home_device(int tl, int T, int D) {
-  if (T < (1 << 26)) return (int)(((unsigned)tl * (unsigned)D) / (unsigned)T);
-  return (int)(((long long)tl * D) / T);
-}
-
-// Active layers of a step and every micro-batch's rank among them: threads 0..15 each place one
-// micro-batch, the result lands in shared memory.  Ends with a block barrier.
-__device__ __forceinline__ void step_shape_block(const BatchParams& bp, uint32_t run, StepShape* out) {
-  const int j = threadIdx.x;
-  if (j < 32) {   // warp 0; lanes 0..15 each own one micro-batch
-    const bool sel = j < bp.n_mb && ((run >> j) & 1u);
-    const int my_layer = j < bp.n_mb ? bp.layer[j] : -1;
-    // is j the first chosen micro-batch sitting at its layer?
-    bool first = sel;
-    for (int i = 0; i < EB_MAX_MB; ++i) {
-      const int li = __shfl_sync(0xffffffffu, my_layer, i);
-      const bool si = (run >> i) & 1u;
-      if (i < j && si && li == my_layer) first = false;
-    }
-    // distinct chosen layers below mine, and in total
-    int below = 0, total = 0;
-    for (int i = 0; i < EB_MAX_MB; ++i) {
-      const int li = __shfl_sync(0xffffffffu, my_layer, i);
-      const bool fi = __shfl_sync(0xffffffffu, (int)first, i) != 0;
-      if (fi) {
-        ++total;
-        if (li < my_layer) ++below;
-      }
-    }
-    if (j < EB_MAX_MB) {
-      out->rank_of_mb[j] = sel ? below : -1;
-      if (first) out->act_layer[below] = my_layer;
-      if (j == 0) out->nl = total;
-    }
-  }
-  __syncthreads();
-}
-
-// group id of (device d, active-layer rank lr, local slot) ; local slot < n_d + S
-__device__ __forceinline__ int group_id(const int* dev_off, int S, int nl, int d, int lr, int local) {
-  int n_d = dev_off[d + 1] - dev_off[d];
-  return nl * (dev_off[d] + d * S) + lr * (n_d + S) + local;
-}
-
-__device__ __forceinline__ int mb_of_chunk(const BatchParams& bp, int c) {
-  int j = 0;
-  while (j + 1 < bp.n_mb && c >= bp.chunk_off[j + 1]) ++j;
-  return j;
-}
 
 // ---- hist ----------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kWarps * 32)

@@ -656,6 +656,46 @@ def test_random_shapes_front_end_bit_exact():
         _full_step(case, Hn.WeightStore(wl), m, policy, pool_mask=pool, check_ffn=(trial % 6 == 0))
 
 
+
+@pytest.mark.parametrize("E,K,S,D,tokens,layers,pool,m,policy", [
+    (8, 2, 0, 3, [1, 33, 2100, 0, 1024, 1025], [0, 1, 1, 2, 2, 0], 0b111111, 4, O.POLICY_MAXUTIL),   # one, two, three segments
+    (1, 1, 1, 1, [5], [0], 0b1, 1, O.POLICY_ALL),
+    (70, 5, 2, 16, [40, 3, 64, 65], [2, 0, 1, 2], 0b1111, 2, O.POLICY_CUMUTIL),       # more than 64 experts, sixteen devices
+    (256, 16, 3, 5, [31, 32], [1, 1], 0b11, 1, O.POLICY_DIFFPEAK),
+    (60, 4, 4, 8, [20] * 16, [j % 3 for j in range(16)], 0xffff, 12, O.POLICY_MAXUTIL),   # pool of sixteen
+    (60, 4, 4, 8, [9 + j for j in range(16)], list(range(16)), 0xffff, 1, O.POLICY_MAXUTIL),   # more than 1024 groups
+    (9, 3, 1, 4, [10] * 11, [0] * 11, 0x7ff, 3, O.POLICY_MAXUTIL),
+    (9, 3, 1, 4, [10, 20, 0, 30], [0, 1, 2, 0], 0, 1, O.POLICY_MAXUTIL),              # nothing runs
+    (9, 3, 2, 4, [700] * 4, [0, 0, 1, 2], 0b1101, 2, O.POLICY_ALL),                   # pool smaller than the batch
+])
+def test_whole_step_front_end_bit_exact(E, K, S, D, tokens, layers, pool, m, policy):
+    """eb_step makes routing, schedule, group tables, positions and rows in three kernels of its own; bit for bit against
+    the oracle, then again with a route mask: the micro-batches outside it keep their routing although their logits
+    have changed, as in the five calls."""
+    B = _binding()
+    wl = _small(L=max(layers) + 1, E=E, K=K, S=S, D=D, N=len(tokens), T=max(tokens), H=72, I=64, mapping="mod")
+    case, store = Hn.make_case(wl, tokens, layers), Hn.WeightStore(wl)
+    step = B.from_workload(wl, max_tokens=max(case.T_tot, 1))
+    step.bind_weights(store.gate, store.up, store.down)
+    T, n = case.T_tot, len(tokens)
+    step.logits[:T].copy_(case.logits)
+    step.x[:T].copy_(case.x)
+    batch = B.Batch(case.tok_off, layers, pool)
+    step.eb_step(batch, m, policy)
+    ref = Hn.oracle_front(case, pool, m, policy)
+    Hn.check_front(step, case, ref, n)
+    assert step.check_permutation(batch) == 0 and step.check_workspace_guards() == 0 and step.device_status() == 0
+    keep = 0b0110 & ((1 << n) - 1)
+    fresh = Hn.make_case(wl, tokens, layers).logits.roll(1, dims=1)
+    step.logits[:T].copy_(fresh)
+    for j in range(n):
+        if not (keep >> j) & 1:
+            case.logits[case.tok_off[j]:case.tok_off[j + 1]] = fresh[case.tok_off[j]:case.tok_off[j + 1]]
+    step.eb_step(batch, m, policy, route_mask=((1 << n) - 1) & ~keep)
+    Hn.check_front(step, case, Hn.oracle_front(case, pool, m, policy), n)
+    assert step.check_permutation(batch) == 0 and step.check_workspace_guards() == 0 and step.device_status() == 0
+
+
 def test_other_policies_on_the_decode_and_fine_grained_shapes():
     for name in ("c2", "c3"):
         wl = synth.workload(name)
