@@ -32,7 +32,7 @@ struct Tile {
   int phase;    // 1: gate/up + SwiGLU (256 outputs per tile);  2: down (512 outputs per tile)
   int done;     // the token tile this one belongs to: entry of `ready`
   int need;     // phase 2: arrivals on that entry after which the rows of the intermediate are all written (0: they are)
-  int pad;
+  int once;     // no other tile reads its weights
 };
 static_assert(sizeof(Tile) == 32, "two 16-byte words");
 
@@ -275,7 +275,7 @@ __device__ __forceinline__ void fill_tiles(const ModelParams& mp, const int32_t*
     it.phase = list + 1;
     it.done = s_pref[lo] + m;
     it.need = nt1 * 2;
-    it.pad = 0;
+    it.once = t_g == 1;
     if (list == 0 && n == 0) l.ready[it.done] = 0;
     if (idx < l.max_work) l.work[idx] = it;
   }
