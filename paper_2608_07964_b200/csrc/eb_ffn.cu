@@ -242,8 +242,10 @@ __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
   return (uint64_t)((addr & 0x3FFFFu) >> 4) | (1ull << 16) | (64ull << 32) | (1ull << 46) | (2ull << 61);
 }
-// Instruction descriptor without its N field: fp32 accumulate, bf16 A and B, both K-major, M = 256.
-constexpr uint32_t kIdescBase = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(256 >> 4) << 24);
+// Instruction descriptor: fp32 accumulate, bf16 A and B, both K-major; M weight rows and N token columns.
+__device__ __forceinline__ uint32_t instr_desc(int m, int n) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
+}
 
 // silu(g) * u with one special-function instruction: silu(g) = g / (1 + exp(-g)) = h + h tanh(h), h = g / 2.
 // tanh.approx.f32 is good to about 2^-11 relative, well inside the bf16 rounding of the result.
@@ -253,6 +255,13 @@ __device__ __forceinline__ float silu_mul(uint32_t g_bits, uint32_t u_bits) {
   asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(h));
   return fmaf(h, t, h) * u;
 }
+
+// A gate/up tile with at most 128 outputs left (the last of I = 1408: eleven times 128) is multiplied with M = 128, 64
+// weight rows per CTA: the tensor cores then spend half the time on it instead of working on 128 rows of zeros.  The
+// accumulator of such an MMA holds the CTA's 64 outputs twice over in its lanes, each time for half of the tokens.
+// At 49152 rows over 66 matrices of 3 x 2048 x 1408 the step went from 926 to 908 us, the expert pass alone from 698 to
+// 682; where weights are streamed nothing changes.
+__device__ __forceinline__ bool slim_tile(int n_out, int out) { return n_out - out * kFeat1 <= kFeat1 / 2; }
 
 // Which part of TMEM a tile's two accumulators take.  TMEM is two halves of 256 columns, each with a full and an
 // empty barrier.  A tile of more than 128 columns takes both (one accumulator in each); a narrower one takes the
@@ -311,7 +320,8 @@ struct TokenMaps {
 };
 struct FfnParams {
   TokenMaps xp, act;                 // inputs of the two phases
-  CUtensorMap gate, up, down;        // with the above kMaps tensor maps in a row
+  CUtensorMap gate, up, down;        // weight boxes of 128 rows
+  CUtensorMap gate64, up64;          // of 64 rows; with the above kMaps tensor maps in a row
   const Tile* work;                  // the list: gate/up tiles, then down tiles
   const int2* slots;
   const int32_t* work_count;         // [0], [1]: tiles of the two phases
@@ -324,27 +334,28 @@ struct FfnParams {
   int* status;
 };
 
-constexpr int kMaps = 13;
-static_assert(offsetof(FfnParams, down) == (kMaps - 1) * sizeof(CUtensorMap), "the maps are prefetched as an array");
+constexpr int kMaps = 15;
+static_assert(offsetof(FfnParams, up64) == (kMaps - 1) * sizeof(CUtensorMap), "the maps are prefetched as an array");
 
 // Chunks of 16 token columns of a finished tile: registers -> transposed through shared memory -> rows.  NC chunks
 // of this warp are read, of which those below the tile's columns hold rows (every chunk read lies in the accumulator).
-// A chunk's rows: columns c0 .. c0 + 15 are rows row0 .. row0 + n_here - 1 (a merged tile: one slot).
+// The tile's token columns token0 .. token0 + tmem_cols - 1 lie in this warp's accumulator columns 0 ..; the rows of a
+// chunk at token column c are row0 .. row0 + n_here - 1 (a merged tile: one slot).
 // Global stores are 16-byte vectors: lane -> (token lane / 4 (+8), outputs 8 (lane % 4) .. +7).
 template <int PHASE, int NC>
 __device__ __forceinline__ void epilogue_tile(const Tile& it, const TmemTurn& turn, uint32_t taddr, int chunk0, int lane, int fbase,
-                                              bf16* tile, const int2* __restrict__ slots, bf16* __restrict__ out, int n_out,
+                                              int token0, int tmem_cols, bf16* tile, const int2* __restrict__ slots, bf16* __restrict__ out, int n_out,
                                               uint32_t tempty0, uint32_t tempty1) {
   const bool merged = it.rows < 0;
   const int n_cols = merged ? -it.rows * kSlotRows : it.rows;   // columns that may hold rows to store
   const uint32_t acc0 = taddr + turn.col0() + chunk0, acc1 = acc0 + turn.step();
   // chunk i of one accumulator, two tokens per word, to its rows; its outputs start at column f
   auto store_chunk = [&](const uint32_t* v, int i, int f) {
-    const int c0 = chunk0 + kChunkStep * i;
-    if (c0 < n_cols) {
-      int row0 = it.row + c0, n_here = min(16, it.rows - c0);
+    const int left = tmem_cols - (chunk0 + kChunkStep * i), c = token0 + chunk0 + kChunkStep * i;
+    if (left > 0 && c < n_cols) {
+      int row0 = it.row + c, n_here = min(min(16, left), it.rows - c);
       if (merged) {
-        const int2 sl = __ldg(slots + it.row + (c0 >> 4));
+        const int2 sl = __ldg(slots + it.row + (c >> 4));
         row0 = sl.x;
         n_here = sl.y;
       }
@@ -524,9 +535,14 @@ ffn_kernel(const __grid_constant__ FfnParams p) {
         const CUtensorMap* tmW1 = down ? &p.down : &p.up;
         const TokenMaps* tmT = down ? &p.act : &p.xp;
         const int num_kb = down ? num_kb2 : num_kb1;
-        const int wrow0 = it.out * (down ? kFeat2 : kFeat1) + (int)rank * 128;
+        const bool slim = !down && slim_tile(p.I, it.out);   // 64 weight rows per CTA and operand
+        if (slim) {
+          tmW0 = &p.gate64;
+          tmW1 = &p.up64;
+        }
+        const int wrow0 = it.out * (down ? kFeat2 : kFeat1) + (int)rank * (slim ? 64 : 128);
         const int wrow1 = down ? wrow0 + 256 : wrow0;
-        const uint32_t tx = 2u * (2u * kWBytes + (uint32_t)half * (BK * 2));
+        const uint32_t tx = 2u * ((slim ? 1u : 2u) * kWBytes + (uint32_t)half * (BK * 2));
         // both CTAs' copies are counted on the leader's barrier; the leader announces the total
         auto load_weights = [&](int st, int kb) {
           const uint32_t fb = map_to_cta(full_bar(st), 0);
@@ -615,7 +631,7 @@ ffn_kernel(const __grid_constant__ FfnParams p) {
         free_item(seq);
         const int num_kb = it.phase == 2 ? num_kb2 : num_kb1;
         const int cols = entry_cols(it.rows);
-        const uint32_t idesc = kIdescBase | ((uint32_t)(cols >> 3) << 17);
+        const uint32_t idesc = instr_desc(it.phase == 1 && slim_tile(p.I, it.out) ? 128 : 256, cols);
         turn.take(cols);
         const uint32_t acc0 = tmem_base + turn.col0(), acc1 = acc0 + turn.step();
         int kb = 0;
@@ -739,13 +755,18 @@ ffn_kernel(const __grid_constant__ FfnParams p) {
       if (!ok) goto done;
       tc_fence_after();
       // this warp's 32 outputs start at fbase
-      const int fbase = it.out * (it.phase == 1 ? kFeat1 : kFeat2) + (int)rank * 128 + q * 32;
-      const int cols = it.rows < 0 ? -it.rows * kSlotRows : it.rows;
+      const bool slim = it.phase == 1 && slim_tile(p.I, it.out);
+      int fbase = it.out * (it.phase == 1 ? kFeat1 : kFeat2) + (int)rank * 128 + q * 32, token0 = 0, cols = entry_cols(it.rows);
+      if (slim) {   // lanes 0..63: the CTA's 64 outputs of the first half of the tokens, lanes 64..127: of the second half
+        fbase = it.out * kFeat1 + (int)rank * 64 + (q & 1) * 32;
+        cols >>= 1;
+        token0 = (q >> 1) * cols;
+      }
       auto run = [&](auto phase, bf16* out, int n_out) {
         constexpr int PH = decltype(phase)::value;
-        if (cols <= 64) epilogue_tile<PH, 2>(it, turn, taddr, chunk0, lane, fbase, tile, p.slots, out, n_out, tempty_bar(0), tempty_bar(1));
-        else if (cols <= 128) epilogue_tile<PH, 4>(it, turn, taddr, chunk0, lane, fbase, tile, p.slots, out, n_out, tempty_bar(0), tempty_bar(1));
-        else epilogue_tile<PH, 8>(it, turn, taddr, chunk0, lane, fbase, tile, p.slots, out, n_out, tempty_bar(0), tempty_bar(1));
+        if (cols <= 64) epilogue_tile<PH, 2>(it, turn, taddr, chunk0, lane, fbase, token0, cols, tile, p.slots, out, n_out, tempty_bar(0), tempty_bar(1));
+        else if (cols <= 128) epilogue_tile<PH, 4>(it, turn, taddr, chunk0, lane, fbase, token0, cols, tile, p.slots, out, n_out, tempty_bar(0), tempty_bar(1));
+        else epilogue_tile<PH, 8>(it, turn, taddr, chunk0, lane, fbase, token0, cols, tile, p.slots, out, n_out, tempty_bar(0), tempty_bar(1));
       };
       if (it.phase == 1) {
         run(std::integral_constant<int, 1>(), p.act_out, p.I);
@@ -894,9 +915,10 @@ eb_status ebi_ffn_bind(eb_ctx* c) {
   if (eb_status ds = ebi_check_device(c)) return ds;
   const eb_config& g = c->cfg;
   const uint64_t nw = (uint64_t)g.L * (g.E + g.S);
-  // weight tiles: boxes of 128 rows x one k-block
+  // weight tiles: boxes of 128 rows x one k-block, of 64 rows for slim tiles
   if (!make_map(&c->tm_gate, c->w_gate, g.H, g.I, nw, BK, 128) || !make_map(&c->tm_up, c->w_up, g.H, g.I, nw, BK, 128) ||
-      !make_map(&c->tm_down, c->w_down, g.I, g.H, nw, BK, 128))
+      !make_map(&c->tm_down, c->w_down, g.I, g.H, nw, BK, 128) || !make_map(&c->tm_gate64, c->w_gate, g.H, g.I, nw, BK, 64) ||
+      !make_map(&c->tm_up64, c->w_up, g.H, g.I, nw, BK, 64))
     return ebi_fail(c, EB_ERR_CUDA, "cuTensorMapEncodeTiled failed for the weights");
   // per context: function attributes and cluster occupancy belong to the current device
   cudaError_t e = cudaFuncSetAttribute(ffn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
@@ -941,6 +963,8 @@ eb_status ebi_ffn_run(eb_ctx* c, cudaStream_t st, const void* xp, const int32_t*
   p.gate = c->tm_gate;
   p.up = c->tm_up;
   p.down = c->tm_down;
+  p.gate64 = c->tm_gate64;
+  p.up64 = c->tm_up64;
   p.work = (const Tile*)c->work;
   p.max_work = c->max_work;
   p.slots = c->slots;

@@ -69,7 +69,7 @@ struct eb_ctx {
   const bf16* w_gate = nullptr;
   const bf16* w_up = nullptr;
   const bf16* w_down = nullptr;
-  CUtensorMap tm_gate, tm_up, tm_down;
+  CUtensorMap tm_gate, tm_up, tm_down, tm_gate64, tm_up64;
   int pair_grid = 0;               // CTAs launched for the expert kernels: two per 2-CTA cluster the device holds at once
 
   // workspace carve-up

@@ -473,11 +473,12 @@ def test_group_sizes_around_the_tile_boundaries(H, I):
     assert sorted(np.diff(ref["group_off"]).tolist()) == sorted(sizes)
 
 
-@pytest.mark.parametrize("H,I", [(72, 2056), (2056, 72), (328, 2056)])
+@pytest.mark.parametrize("H,I", [(72, 2056), (2056, 72), (328, 2056), (136, 1408), (72, 392)])
 def test_tile_sizes_mixed_over_many_tiles_per_pair(H, I):
     """The same groups with enough output tiles that every CTA pair works through several of them, tiles of more than
     128 columns (both halves of TMEM) and narrower ones (one half in turn) one after the other: with fewer k-blocks
-    than the ring has stages (72), and with more (328, 2056)."""
+    than the ring has stages (72), and with more (328, 2056).  I = 2056, 1408, 392 (8, 128, 136 outputs left for the
+    last gate/up tile) and 72 lie on both sides of the limit below which that tile is multiplied with half as many rows."""
     test_group_sizes_around_the_tile_boundaries(H, I)
 
 
@@ -661,7 +662,7 @@ def test_random_shapes_front_end_bit_exact():
     (8, 2, 0, 3, [1, 33, 2100, 0, 1024, 1025], [0, 1, 1, 2, 2, 0], 0b111111, 4, O.POLICY_MAXUTIL),   # one, two, three segments
     (1, 1, 1, 1, [5], [0], 0b1, 1, O.POLICY_ALL),
     (70, 5, 2, 16, [40, 3, 64, 65], [2, 0, 1, 2], 0b1111, 2, O.POLICY_CUMUTIL),       # more than 64 experts, sixteen devices
-    (256, 16, 3, 5, [31, 32], [1, 1], 0b11, 1, O.POLICY_DIFFPEAK),
+    (256, 8, 3, 5, [31, 32], [1, 1], 0b11, 1, O.POLICY_DIFFPEAK),
     (60, 4, 4, 8, [20] * 16, [j % 3 for j in range(16)], 0xffff, 12, O.POLICY_MAXUTIL),   # pool of sixteen
     (60, 4, 4, 8, [9 + j for j in range(16)], list(range(16)), 0xffff, 1, O.POLICY_MAXUTIL),   # more than 1024 groups
     (9, 3, 1, 4, [10] * 11, [0] * 11, 0x7ff, 3, O.POLICY_MAXUTIL),
