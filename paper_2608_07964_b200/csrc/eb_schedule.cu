@@ -37,8 +37,9 @@ schedule_kernel(int D, int n_mb, uint32_t pool_mask, int m, int policy, const in
         if (better(o, b)) b = o;
       }
       b = warp_best(b);
+      const uint32_t mask = run_mask_of(s.member, __popc(pool_mask), b);
       if (tid == 0) {
-        s.run = run_mask_of(s.member, __popc(pool_mask), b);
+        s.run = mask;
         *block_counter = 0;   // ready for the next call
       }
     }

@@ -103,20 +103,34 @@ __device__ __forceinline__ Cand warp_best_narrow(const Cand& c0) {
 }
 
 
-// run set of a candidate
+// run set of a candidate; one warp
 __device__ __forceinline__ uint32_t run_mask_of(const int* member, int np, const Cand& b) {
-  uint32_t mask = 0;
-  for (int k = 0; k < np; ++k)
-    if ((b.sub >> k) & 1u) mask |= 1u << member[k];
-  return mask;
+  const int k = threadIdx.x & 31;
+  return __reduce_or_sync(0xffffffffu, k < np && ((b.sub >> k) & 1u) ? 1u << member[k] : 0u);
 }
+
+// The byte values, those with more bits set first, then ascending.
+struct ByCount {
+  alignas(4) unsigned char v[256];
+};
+constexpr ByCount make_by_count() {
+  ByCount t{};
+  int at = 0;
+  for (int n = 8; n >= 0; --n)
+    for (int u = 0; u < 256; ++u) {
+      int bits = 0;
+      for (int b = 0; b < 8; ++b) bits += (u >> b) & 1;
+      if (bits == n) t.v[at++] = (unsigned char)u;
+    }
+  return t;
+}
+static __device__ const ByCount kByCount = make_by_count();
 
 struct SchedShared {
   int4 lo[256 * kSchedRow / 4], hi[256 * kSchedRow / 4];   // summed loads of every subset of the two halves of the pool
   int load[EB_MAX_MB][EB_MAX_D];                           // zero beyond n_mb and D
   int nibble[4][16][EB_MAX_D];                             // summed loads of every subset of four pool positions
-  unsigned char by_count[256];                             // the byte values, those with more bits set first, then ascending
-  int n_with[9];                                           // byte values with at least k bits set
+  unsigned char by_count[256];                             // kByCount
   int member[EB_MAX_MB];                                   // micro-batch of every pool position
   Cand best[kSchedThreads / 32];
   uint32_t run;
@@ -170,7 +184,10 @@ __device__ __forceinline__ Cand maxutil_scan(const SchedShared& s, int D, int np
     for (int k = block; k < (1 << (np - 8)) / 32 + 1; k += n_blocks) {
       const int h = k * 32 + (warp ^ (k * 11 & 31)), n_h = __popc(h);
       if (h >= 1 << (np - 8)) continue;
-      const int need = max(0, m - n_h), n_lo = need > 8 ? 0 : s.n_with[need];
+      const int need = max(0, m - n_h);
+      if (need > 8) continue;
+      // byte values with at least `need` bits set: 256, 255, 247, 219, 163, 93, 37, 9, 1
+      const int n_lo = need == 0 ? 256 : (int)((0x0109255da3dbf7ffULL >> (8 * (need - 1))) & 255u);
       const int4* hi = s.hi + h * (kSchedRow / 4);
       for (int i = lane; i < n_lo; i += 32) {
         const int u = s.by_count[i];
@@ -217,33 +234,7 @@ __device__ __forceinline__ bool schedule_block(SchedShared& s, int D, uint32_t p
         if (quad * 4 + b < np && ((u >> b) & 1)) acc += s.load[s.member[quad * 4 + b]][d];
       s.nibble[quad][u][d] = acc;
     }
-    if (np > 10 && tid < 256) {   // place of byte value tid: values with more bits, then lower values with as many
-      const int n = __popc(tid);
-      int before = 0, choose = 1, left = 8, ones = n;
-      for (int k = 8; k > 0; --k) {   // choose = C(8, k), k from 8 down
-        if (k > n) before += choose;
-        choose = choose * k / (9 - k);
-      }
-      // combinatorial rank among the values of n bits: the bits from the highest down
-      for (int bit = 7; bit >= 0 && ones > 0; --bit) {
-        left = bit;
-        if ((tid >> bit) & 1) {
-          int c = 1;   // C(left, ones): values with this bit clear and as many ones below it
-          for (int k = 0; k < ones; ++k) c = c * (left - k) / (k + 1);
-          before += c;
-          --ones;
-        }
-      }
-      s.by_count[before] = (unsigned char)tid;
-      if (tid < 9) {
-        int c = 1, sum = 0;
-        for (int k = 8; k >= tid; --k) {
-          sum += c;
-          c = c * k / (9 - k);
-        }
-        s.n_with[tid] = sum;
-      }
-    }
+    if (np > 10 && tid < 64) reinterpret_cast<uint32_t*>(s.by_count)[tid] = reinterpret_cast<const uint32_t*>(kByCount.v)[tid];
     __syncthreads();
     for (int i = tid; i < (1 << nlo) * EB_MAX_D; i += kSchedThreads)
       lo[(i >> 4) * kSchedRow + (i & 15)] = s.nibble[0][(i >> 4) & 15][i & 15] + s.nibble[1][i >> 8][i & 15];
@@ -257,10 +248,10 @@ __device__ __forceinline__ bool schedule_block(SchedShared& s, int D, uint32_t p
     __syncthreads();
     if (tid < 32) {
       Cand b = any_wide ? warp_best(s.best[tid]) : warp_best_narrow(s.best[tid]);
-      __syncwarp();
+      const uint32_t mask = run_mask_of(s.member, np, b);
       if (tid == 0) {
         s.best[0] = b;
-        s.run = run_mask_of(s.member, np, b);
+        s.run = mask;
       }
     }
     __syncthreads();
