@@ -5,7 +5,8 @@
 // thread loads its vector from the K + S expert-output rows of the token (independent loads, all
 // in flight together), accumulates in fp32 in the
 // fixed order k = 0..K-1 then s = 0..S-1, and stores bf16 (round to nearest even).  Gather form
-// means no atomics and a result that does not depend on scheduling.
+// means no atomics and a result that does not depend on scheduling.  The expert-output rows are read once, so
+// they leave L2 first (streaming loads): 226 MB took 48 us instead of 54 between its neighbours.
 #include <utility>
 
 #include "eb_internal.cuh"
@@ -48,7 +49,7 @@ combine_kernel(int n_tok, int H, int K, int team, const uint4* __restrict__ yp, 
   for (int v = threadIdx.x % team; v < vec; v += team) {
     uint4 r[KS];
 #pragma unroll
-    for (int s = 0; s < KS; ++s) r[s] = p[s] >= 0 ? __ldg(yp + (size_t)p[s] * vec + v) : make_uint4(0, 0, 0, 0);   // no row: adds 0
+    for (int s = 0; s < KS; ++s) r[s] = p[s] >= 0 ? __ldcs(yp + (size_t)p[s] * vec + v) : make_uint4(0, 0, 0, 0);   // no row: adds 0
     uint4 res = make_uint4(0, 0, 0, 0);
     if (residual) res = residual[(size_t)t * vec + v];
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};

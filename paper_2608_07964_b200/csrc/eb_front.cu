@@ -350,7 +350,9 @@ scatter_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ B
   __shared__ StepShape ss;
   __shared__ int s_dev_off[EB_MAX_D + 1];
   __shared__ int s_next[EB_MAX_E];
+  __shared__ int s_topk[32 * EB_MAX_K];
   __shared__ int s_pos[TB][EB_MAX_K + EB_MAX_S];
+  static_assert(32 * EB_MAX_K <= kScatterThreads, "a thread per assignment of the chunk");
   const int tid = threadIdx.x, lane = tid & 31;
   const int E = mp.E, K = mp.K, S = mp.S, KS = K + S, vec = mp.H / 8;
   const int part = (int)blockIdx.x - a.fill_blocks, c = part / (32 / TB);
@@ -370,16 +372,18 @@ scatter_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ B
   for (int k = 0; k < TB; ++k)
     if (k < nt && tid < vec) v[k] = __ldg(a.x + (size_t)(t0 + k) * vec + tid);
   if (tid <= mp.D) s_dev_off[tid] = mp.dev_off[tid];
+  // assignments from the start of the chunk to the end of this part
+  const int first = (t0 - c0) * K, last = first + nt * K;
+  if (tid < last) s_topk[tid] = a.topk_idx[(size_t)c0 * K + tid];
   for (int e = tid; e < E; e += kScatterThreads) s_next[e] = a.mb_base[j * E + e] + a.chunk_base[(size_t)c * E + e];
   step_shape_block(bp, run, &ss);   // ends with a barrier
   if (tid < 32) {
     const int lr = ss.rank_of_mb[j];
     // routed slots in assignment order from the start of the chunk; the rows of the tokens before this part only count
-    const int first = (t0 - c0) * K, last = first + nt * K;
     for (int a0 = 0; a0 < last; a0 += 32) {
       const int i = a0 + lane;
       bool valid = i < last;
-      int e = valid ? a.topk_idx[(size_t)c0 * K + i] : -1 - lane;   // distinct dummies never match
+      int e = valid ? s_topk[i] : -1 - lane;   // distinct dummies never match
       if (valid && (unsigned)e >= (unsigned)E) {
         // an index outside [0, E) is never used: the slot gets no row and the step's meta data counts it
         if (i >= first) {
