@@ -318,8 +318,9 @@ class MoEStep:
         return _sched_dict(EbSchedResult.from_address(h_res.data_ptr()), self.D)
 
     # -- results and status --------------------------------------------------------------------
-    def sched_result(self) -> Dict:
-        raw = self.sched.cpu().numpy().tobytes()
+    def sched_result(self, host_copy: Optional[torch.Tensor] = None) -> Dict:
+        """The last schedule; read from the device, or from a host copy of `self.sched` that is complete."""
+        raw = (self.sched.cpu() if host_copy is None else host_copy).numpy().tobytes()
         return _sched_dict(EbSchedResult.from_buffer_copy(raw), self.D)
 
     def meta(self) -> Dict:

@@ -19,6 +19,25 @@ import torch
 from . import binding as B
 
 
+def _logit_rows(step: "B.MoEStep", tok_off: List[int]) -> List[torch.Tensor]:
+    return [step.logits[tok_off[j]:tok_off[j + 1]] for j in range(len(tok_off) - 1)]
+
+
+def _copy_logits(rows: List[torch.Tensor], logits_of: Callable[[int, int], torch.Tensor], layer: List[int], mask: int) -> None:
+    """Logits of the micro-batches in `mask` at their current layers, into their rows.  A copy per micro-batch is a
+    launch each (16 of them took half of a scheduling step's time on the host); plain device tensors of the rows' form
+    go together in one."""
+    js = [j for j in range(len(rows)) if (mask >> j) & 1]
+    src = [logits_of(j, layer[j]) for j in js]
+    dst = [rows[j] for j in js]
+    if len(js) > 1 and all(s.device == d.device and s.dtype == d.dtype and s.shape == d.shape and s.is_contiguous()
+                           and s.numel() > 0 and not s.requires_grad for s, d in zip(src, dst)):
+        torch._foreach_copy_(dst, src)
+    else:
+        for d, s in zip(dst, src):
+            d.copy_(s)
+
+
 def run_load_trace(step: "B.MoEStep", tok_off: List[int], L: int, m: int, policy: int,
                    logits_of: Callable[[int, int], torch.Tensor]) -> List[Dict]:
     """Runs Algorithm 1 with route + schedule only.  Returns one record per step:
@@ -28,16 +47,23 @@ def run_load_trace(step: "B.MoEStep", tok_off: List[int], L: int, m: int, policy
     pool = (1 << N) - 1 if L > 0 else 0
     route_mask = pool
     steps: List[Dict] = []
+    rows = _logit_rows(step, tok_off)
+    # the schedule and the loads come back in pinned memory behind one synchronisation
+    h_load = torch.empty((N, step.D), dtype=torch.int32).pin_memory()
+    h_sched = torch.empty_like(step.sched, device="cpu").pin_memory()
+    stream = torch.cuda.current_stream(step.dev)
     while pool:
-        for j in range(N):
-            if (route_mask >> j) & 1:
-                step.logits[tok_off[j]:tok_off[j + 1]].copy_(logits_of(j, layer[j]))
+        _copy_logits(rows, logits_of, layer, route_mask)
         batch = B.Batch(tok_off, [min(l, L - 1) for l in layer], pool)
         if route_mask:
             step.eb_route(batch, route_mask)
-        res = step.eb_schedule(batch, m, policy, to_host=True)
+        step.eb_schedule(batch, m, policy)
+        h_load.copy_(step.mb_load[:N], non_blocking=True)
+        h_sched.copy_(step.sched, non_blocking=True)
+        stream.synchronize()
+        res = step.sched_result(h_sched)
         run = res["run_mask"]
-        loads = step.mb_load[:N].cpu().tolist()
+        loads = h_load.tolist()
         steps.append(dict(pool=pool, run_mask=run, layers={j: layer[j] for j in range(N) if (run >> j) & 1},
                           joint_load=res["joint_load"], util_num=res["util_num"], util_den=res["util_den"],
                           member_loads={j: loads[j] for j in range(N) if (run >> j) & 1}))
@@ -95,12 +121,11 @@ def run_full(step: "B.MoEStep", tok_off: List[int], L: int, m: int, policy: int,
     route_mask = pool
     step.x[:T].copy_(x0)
     steps: List[Dict] = []
+    rows = _logit_rows(step, tok_off)
     t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     t0.record()
     while pool:
-        for j in range(N):
-            if (route_mask >> j) & 1:
-                step.logits[tok_off[j]:tok_off[j + 1]].copy_(logits_of(j, layer[j]))
+        _copy_logits(rows, logits_of, layer, route_mask)
         lay = [min(l, L - 1) for l in layer]
         if graphs is not None:
             graphs.run(lay, pool, route_mask, m, policy)
