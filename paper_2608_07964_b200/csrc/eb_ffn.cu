@@ -325,11 +325,10 @@ struct FfnParams {
   const Tile* work;                  // the list: gate/up tiles, then down tiles
   const int2* slots;
   const int32_t* work_count;         // [0], [1]: tiles of the two phases
-  int32_t* next;                     // tiles dealt out beyond the first of every pair (second entry: of a launch of part 2)
+  int32_t* next;                     // tiles dealt out (second entry: of a launch of part 2)
   int32_t* ready;                    // per token tile: arrivals, one per CTA for every finished gate/up tile
   bf16 *act_out, *yp;
   int H, I;
-  int max_work;                      // capacity of the list
   int part;                          // 0: the whole list; 1, 2: the tiles of that phase only
   int* status;
 };
@@ -434,16 +433,14 @@ ffn_kernel(const __grid_constant__ FfnParams p) {
   auto item_empty = [&](int i) { return bar0 + 8u * (2 * NS + 4 + kItems + i); };
   const uint32_t want_bar = bar0 + 8u * (2 * NS + 4 + 2 * kItems);
   constexpr int kBarBytes = 8 * (2 * NS + 4 + 2 * kItems + 1);
-  static_assert(kBarBytes + 8 + 4 * kParts + sizeof(Tile) <= 192 && kItems * sizeof(Tile) <= 64, "256 bytes of barriers and mailbox");
+  static_assert(kBarBytes + 8 + 4 * kParts <= 192 && kItems * sizeof(Tile) <= 64, "256 bytes of barriers and mailbox");
   volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(smem + kRingBytes + kBarBytes);
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + kRingBytes + kBarBytes + 4);
-  int4* const s_first = reinterpret_cast<int4*>(smem + kRingBytes + 192 - sizeof(Tile));
   const uint32_t items = bar0 + 192;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();   // CTA 0 of a pair is the leader
   int* const status = p.status;
-  const int n_pairs = (int)(gridDim.x >> 1), my_pair = (int)(blockIdx.x >> 1);
   if (threadIdx.x == 0) {
     for (int s = 0; s < NS; ++s) {
       mbar_init(full_bar(s), 1);    // the leader's arrive + all bytes of the stage of both CTAs
@@ -463,15 +460,19 @@ ffn_kernel(const __grid_constant__ FfnParams p) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 2 && lane < kMaps) prefetch_tmap(&p.xp.box[0] + lane);
-  if (threadIdx.x == 96) {
-    // The first tile of pair q is tile q of the part, fetched once per CTA beside the set-up; the others come from
-    // the tile dealer.
-    const int part_first = p.part == 2 ? p.work_count[0] : 0;
-    const int4* e = reinterpret_cast<const int4*>(p.work + min(part_first + my_pair, p.max_work - 1));
-    int4 a = __ldg(e), b = __ldg(e + 1);
-    if (part_first + my_pair >= (p.part == 1 ? p.work_count[0] : p.work_count[0] + p.work_count[1])) a.z = -1;
-    s_first[0] = a;
-    s_first[1] = b;
+  // The pair's first tile, claimed like all others: were it fixed beforehand, a pair that cannot run yet (another
+  // kernel of this kind holds its SMs) would keep it, and both kernels could wait for such tiles.  One thread of CTA 1
+  // claims it, so that the trip to memory passes beside the set-up.
+  int4 first_a = make_int4(0, 0, -1, 0), first_b = make_int4(0, 0, 0, 0);
+  const bool claims_first = rank == 1 && threadIdx.x == 96;
+  if (claims_first) {
+    const int cnt1 = p.work_count[0], cnt2 = p.work_count[1];
+    const int idx = (p.part == 2 ? cnt1 : 0) + atomicAdd(p.next + (p.part == 2 ? 1 : 0), 1);
+    if (idx < (p.part == 1 ? cnt1 : cnt1 + cnt2)) {
+      const int4* e = reinterpret_cast<const int4*>(p.work + idx);
+      first_a = __ldg(e);
+      first_b = __ldg(e + 1);
+    }
   }
   if (warp == 1) {
     tmem_alloc_pair(smem_u32((const void*)s_tmem), kTmemCols);
@@ -484,22 +485,25 @@ ffn_kernel(const __grid_constant__ FfnParams p) {
   const uint32_t tmem_base = *s_tmem;
   const int num_kb1 = (p.H + BK - 1) / BK, num_kb2 = (p.I + BK - 1) / BK;
 
-  // Tile number `seq` of this pair (false: gave up); all but the first come through the mailbox, where the reader frees
-  // the slot.
+  // leaves a tile in slot i of both CTAs' mailboxes
+  auto deal = [&](int i, const int4& a, const int4& b) {
+    for (uint32_t r = 0; r < 2; ++r) {
+      const uint32_t dst = map_to_cta(items + i * (uint32_t)sizeof(Tile), r);
+      st_cluster(dst, a);
+      st_cluster(dst + 16, b);
+      mbar_arrive_release_cluster(map_to_cta(item_full(i), r));
+    }
+  };
+  if (claims_first) deal(0, first_a, first_b);
+  // Tile number `seq` of this pair, from the mailbox (false: gave up); the reader then frees the slot.
   auto take_item = [&](int seq, Tile* it) {
     const int i = seq % kItems;
-    uint32_t at = bar0 + 192u - (uint32_t)sizeof(Tile);
-    if (seq > 0) {
-      if (!mbar_wait_cluster(item_full(i), (uint32_t)((seq - 1) / kItems) & 1u, s_abort, status)) return false;
-      at = items + i * (uint32_t)sizeof(Tile);
-    }
-    const int4 a = ld_shared(at), b = ld_shared(at + 16);
+    if (!mbar_wait_cluster(item_full(i), (uint32_t)(seq / kItems) & 1u, s_abort, status)) return false;
+    const int4 a = ld_shared(items + i * (uint32_t)sizeof(Tile)), b = ld_shared(items + i * (uint32_t)sizeof(Tile) + 16);
     *it = Tile{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
     return true;
   };
-  auto free_item = [&](int seq) {
-    if (seq > 0) mbar_arrive_cluster(map_to_cta(item_empty(seq % kItems), 1));
-  };
+  auto free_item = [&](int seq) { mbar_arrive_cluster(map_to_cta(item_empty(seq % kItems), 1)); };
 
   if (warp == 0) {
     // ---------------- TMA producer (each CTA loads its own halves) ----------------
@@ -696,15 +700,17 @@ ffn_kernel(const __grid_constant__ FfnParams p) {
       }
     } else if (lane == 0) {
       // ---------------- tile dealer (CTA 1's otherwise idle MMA warp) ----------------
-      // Every tile of a pair but its first is the next one not yet dealt, claimed well before the leader's producer
-      // is through with the tile before it.  Both CTAs' mailboxes get a copy.
+      // Every further tile of a pair is the next one not yet dealt, claimed well before the leader's producer is
+      // through with the tile before it.
       const int part_first = p.part == 2 ? p.work_count[0] : 0;
       const int part_end = p.part == 1 ? p.work_count[0] : p.work_count[0] + p.work_count[1];
-      for (int seq = 1; part_first + my_pair < part_end; ++seq) {
+      Tile it;
+      if (!take_item(0, &it)) goto done;
+      for (int seq = 1; it.w >= 0; ++seq) {
         const int i = seq % kItems;
         if (!mbar_wait_cluster(want_bar, (uint32_t)(seq - 1) & 1u, s_abort, status)) goto done;
-        if (seq > kItems && !mbar_wait_cluster(item_empty(i), (uint32_t)((seq - 1) / kItems - 1) & 1u, s_abort, status)) goto done;
-        const int idx = part_first + n_pairs + atomicAdd(p.next + (p.part == 2 ? 1 : 0), 1);
+        if (seq >= kItems && !mbar_wait_cluster(item_empty(i), (uint32_t)(seq / kItems - 1) & 1u, s_abort, status)) goto done;
+        const int idx = part_first + atomicAdd(p.next + (p.part == 2 ? 1 : 0), 1);
         int4 a = make_int4(0, 0, -1, 0), b = make_int4(0, 0, 0, 0);
         if (idx < part_end) {
           const int4* e = reinterpret_cast<const int4*>(p.work + idx);
@@ -713,13 +719,7 @@ ffn_kernel(const __grid_constant__ FfnParams p) {
           // a down tile whose rows are complete already, the usual case, spares the producers the question
           if (b.x == 2 && ld_acquire(p.ready + b.y) >= b.z) b.z = 0;
         }
-        const uint32_t at = items + i * (uint32_t)sizeof(Tile);
-        for (uint32_t r = 0; r < 2; ++r) {
-          const uint32_t dst = map_to_cta(at, r);
-          st_cluster(dst, a);
-          st_cluster(dst + 16, b);
-          mbar_arrive_release_cluster(map_to_cta(item_full(i), r));
-        }
+        deal(i, a, b);
         if (idx >= part_end) break;
       }
     }
@@ -966,7 +966,6 @@ eb_status ebi_ffn_run(eb_ctx* c, cudaStream_t st, const void* xp, const int32_t*
   p.gate64 = c->tm_gate64;
   p.up64 = c->tm_up64;
   p.work = (const Tile*)c->work;
-  p.max_work = c->max_work;
   p.slots = c->slots;
   p.work_count = c->work_count;
   p.next = c->work_count + 6;
