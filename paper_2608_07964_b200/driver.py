@@ -24,18 +24,11 @@ def _logit_rows(step: "B.MoEStep", tok_off: List[int]) -> List[torch.Tensor]:
 
 
 def _copy_logits(rows: List[torch.Tensor], logits_of: Callable[[int, int], torch.Tensor], layer: List[int], mask: int) -> None:
-    """Logits of the micro-batches in `mask` at their current layers, into their rows.  A copy per micro-batch is a
-    launch each (16 of them took half of a scheduling step's time on the host); plain device tensors of the rows' form
-    go together in one."""
-    js = [j for j in range(len(rows)) if (mask >> j) & 1]
-    src = [logits_of(j, layer[j]) for j in js]
-    dst = [rows[j] for j in js]
-    if len(js) > 1 and all(s.device == d.device and s.dtype == d.dtype and s.shape == d.shape and s.is_contiguous()
-                           and s.numel() > 0 and not s.requires_grad for s, d in zip(src, dst)):
-        torch._foreach_copy_(dst, src)
-    else:
-        for d, s in zip(dst, src):
-            d.copy_(s)
+    """Logits of the micro-batches in `mask` at their current layers, into their rows.  Each result is taken over before
+    the next one is asked for: `logits_of` may fill and return one and the same buffer every time."""
+    for j, row in enumerate(rows):
+        if (mask >> j) & 1:
+            row.copy_(logits_of(j, layer[j]))
 
 
 def run_load_trace(step: "B.MoEStep", tok_off: List[int], L: int, m: int, policy: int,

@@ -126,6 +126,26 @@ def test_full_chain_matches_oracle_chain(name):
     assert step.device_status() == 0
 
 
+@pytest.mark.parametrize("device", ["cuda", "pinned"])
+def test_logits_of_may_reuse_one_buffer(device):
+    """A logits function that fills and returns the same buffer every time (a gate GEMM with out=, a staging buffer):
+    what it returned is taken over before it is asked again, in both loops."""
+    from paper_2608_07964_b200 import binding as B, driver
+    wl = synth.Workload(name="reuse", L=3, E=6, K=2, S=1, H=72, I=64, D=3, mapping="mod", N=4, T=24, zipf_s=1.0)
+    bias = synth.zipf_bias(wl)
+    store = Hn.WeightStore(wl)
+    step = B.from_workload(wl)
+    step.bind_weights(store.gate, store.up, store.down)
+    x0 = torch.cat([synth.hidden_for(wl, j, 0, "cuda") for j in range(wl.N)], 0)
+    fresh = lambda j, l: synth.logits_for(wl, j, l, "cuda", bias)
+    buf = torch.empty((wl.T, wl.E), device="cuda") if device == "cuda" else torch.empty((wl.T, wl.E)).pin_memory()
+    reused = lambda j, l: buf.copy_(fresh(j, l))
+    args = (step, wl.tok_off, wl.L, wl.m, O.POLICY_MAXUTIL)
+    assert driver.run_load_trace(*args, reused) == driver.run_load_trace(*args, fresh)
+    want, got = driver.run_full(*args, fresh, x0), driver.run_full(*args, reused, x0)
+    assert torch.equal(got["x"], want["x"]) and got["steps"] == want["steps"]
+
+
 def test_combine_with_residual_alone():
     """eb_combine_residual fed with the oracle's expert outputs (rounded to bf16) against the oracle's aggregation
     with the residual, including the in-place form (residual and out the same buffer)."""
