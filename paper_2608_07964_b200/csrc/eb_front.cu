@@ -443,18 +443,21 @@ scatter_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ B
   }
 }
 
-size_t tables_smem(const eb_ctx* c, int n_mb, int groups) {
-  return sizeof(SchedShared) + sizeof(int) * ((size_t)n_mb * c->cfg.E + 3 * (size_t)groups + 1);
+constexpr size_t tables_smem(int n_mb, int E, int groups) {
+  return sizeof(SchedShared) + sizeof(int) * ((size_t)n_mb * E + 3 * (size_t)groups + 1);
 }
+// The most any shape takes.  The limit belongs to the kernel on its device: a context that set its own need would lower it for
+// the contexts of larger shapes.
+constexpr size_t kTablesSmemMax = tables_smem(EB_MAX_MB, EB_MAX_E, EB_MAX_MB * (EB_MAX_E + EB_MAX_D * EB_MAX_S));
+static_assert(kTablesSmemMax + 16384 <= 232448, "shared memory of one block, the static part within 16 KB");
 
 }  // namespace
 
 eb_status ebi_front_run(eb_ctx* c, cudaStream_t st, const BatchParams& bp, uint32_t pool_mask, uint32_t route_mask, int32_t m,
                         eb_policy policy, const eb_step_buffers* b) {
   const eb_config& g = c->cfg;
-  if (!c->tables_attr_set) {   // per context: function attributes belong to the current device
-    EB_CUDA(c, cudaFuncSetAttribute(tables_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)tables_smem(c, EB_MAX_MB, ebi_groups_cap(c))));
+  if (!c->tables_attr_set) {   // per context: a context is on one device
+    EB_CUDA(c, cudaFuncSetAttribute(tables_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTablesSmemMax));
     c->tables_attr_set = true;
   }
   if (bp.n_chunks > 0) {
@@ -466,7 +469,7 @@ eb_status ebi_front_run(eb_ctx* c, cudaStream_t st, const BatchParams& bp, uint3
     KernelTimer timer(c, EBK_SCHEDULE, st);
     const TablesArgs a{pool_mask, route_mask, (int)m, (int)policy, c->chunk_hist, c->chunk_base, c->chunk_seg, c->mb_base, b->mb_load,
                        b->mb_cnt, b->sched, b->group_off, b->group_w, b->step_meta, tile_plan_of(c)};
-    ebi_launch(tables_kernel, dim3(1), dim3(kSchedThreads), tables_smem(c, bp.n_mb, bp.n_mb * (g.E + g.D * g.S)), st, c->mp, bp, a);
+    ebi_launch(tables_kernel, dim3(1), dim3(kSchedThreads), tables_smem(bp.n_mb, g.E, bp.n_mb * (g.E + g.D * g.S)), st, c->mp, bp, a);
   }
   {
     KernelTimer timer(c, EBK_PERMUTE_GATHER, st);

@@ -1,0 +1,69 @@
+"""What the library's host code asks of the CUDA runtime, on the CPU: the sources are built against a stand-in runtime
+(fake_cudart.cpp) that keeps shared-memory limits, can refuse a launch and writes down which kernels were launched."""
+import ctypes as C
+import glob
+import os
+import subprocess
+
+import pytest
+
+from paper_2608_07964_b200 import binding as B, build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+EB_ERR_CUDA = 4
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("host") / "libeb_host.so")
+    # the device code is of no interest here: kept as PTX, which spares the assembler's time
+    cmd = [build._nvcc(), "-gencode", "arch=compute_100a,code=compute_100a", "-O0", "-std=c++17", "--shared", "-cudart", "none", "-t", "8",
+           "-Xcompiler", "-fPIC", "-Xlinker", "-Bsymbolic", "-I", os.path.join(build.ROOT, "include"),
+           "-I", os.path.join(build.PKG, "csrc"), "-o", so, os.path.join(HERE, "fake_cudart.cpp")] + build.SOURCES
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    l = B.load_library(so)
+    l.fake_name.restype = C.c_char_p
+    return l
+
+
+class Context:
+    """A context whose buffers are addresses that nothing ever reads."""
+
+    def __init__(self, lib, E, K, S, D, max_tokens, H=64, I=64, L=4):
+        self.lib, self.D = lib, D
+        self.ctx = C.c_void_p()
+        e2d = (C.c_int32 * E)(*[e % D for e in range(E)])
+        cfg = B.EbConfig(L, E, K, S, H, I, D, 1, max_tokens, e2d)
+        assert lib.eb_create(C.byref(cfg), C.byref(self.ctx)) == 0
+        assert lib.eb_set_workspace(self.ctx, 1 << 20, lib.eb_workspace_bytes(self.ctx)) == 0
+        assert lib.eb_bind_weights(self.ctx, 1 << 30, 1 << 30, 1 << 30) == 0
+        self.p = 1 << 30
+        self.bufs = B.EbStepBuffers(*([self.p] * 15), None)
+
+    def batch(self, n_mb, tokens):
+        return B.Batch([j * tokens for j in range(n_mb + 1)], [j % 4 for j in range(n_mb)])
+
+    def step(self, n_mb, tokens, m=1, policy=B.POLICY_MAXUTIL):
+        b = self.batch(n_mb, tokens)
+        return self.lib.eb_step(self.ctx, None, C.byref(b.c), b.pool_mask, m, policy, C.byref(self.bufs))
+
+    def names(self):
+        return [self.lib.fake_name(i).decode() for i in range(self.lib.fake_launched())]
+
+
+SHAPES = [dict(E=256, K=8, S=8, D=16), dict(E=64, K=6, S=2, D=8), dict(E=60, K=4, S=4, D=8), dict(E=8, K=2, S=0, D=4)]
+
+
+def test_a_context_keeps_its_shared_memory_whatever_others_do(lib):
+    """The shared-memory limit belongs to the kernel, not to the context that sets it: contexts of other shapes, smaller
+    and larger ones, may make their first step at any time between the steps of one."""
+    lib.fake_reset(-1)
+    ctxs = [Context(lib, max_tokens=16 * 96, **s) for s in SHAPES]
+    for order in ((0, 1, 2, 3), (3, 2, 1, 0), (1, 3, 0, 2)):
+        for i in order:
+            assert ctxs[i].step(16, 96) == 0 and ctxs[i].step(4, 3) == 0, SHAPES[i]
+    late = Context(lib, max_tokens=64, E=2, K=1, S=0, D=1)
+    assert late.step(4, 3) == 0
+    for c, s in zip(ctxs, SHAPES):
+        assert c.step(16, 96) == 0, s

@@ -411,6 +411,30 @@ def test_two_contexts_on_two_streams_do_not_disturb_each_other():
         assert steps[i].device_status() == 0
 
 
+def test_steps_of_a_large_context_between_first_steps_of_smaller_ones():
+    """The contexts of one process share the kernels and what is set on them: the large one (16 micro-batches, shared
+    experts) gives the same bits before and after smaller ones made their first steps."""
+    B = _binding()
+    wl = _small(L=4, E=64, K=6, S=2, D=8, N=16, T=9, H=72, I=64, mapping="mod")
+    case, store = Hn.make_case(wl, [9] * 16, [j % 4 for j in range(16)]), Hn.WeightStore(wl)
+    step, ref = _full_step(case, store, 12)
+    batch = B.Batch(case.tok_off, case.layers)
+    want = step.out[:case.T_tot].clone()
+    for E, D in ((8, 4), (2, 1)):
+        small = _small(L=2, E=E, K=1, S=0, D=D, N=4, T=5, H=64, I=64, mapping="mod")
+        small_case = Hn.make_case(small, [5] * 4, [0, 0, 1, 1])
+        other = B.from_workload(small, max_tokens=20)
+        other_store = Hn.WeightStore(small)
+        other.bind_weights(other_store.gate, other_store.up, other_store.down)
+        other.logits[:20].copy_(small_case.logits)
+        other.x[:20].copy_(small_case.x)
+        other.eb_step(B.Batch(small_case.tok_off, small_case.layers), 3)
+        step.pos.fill_(-9)
+        step.eb_step(batch, 12)
+        Hn.check_front(step, case, ref, 16)
+        assert torch.equal(step.out[:case.T_tot], want) and step.device_status() == 0
+
+
 def test_deferred_micro_batch_keeps_its_routing():
     B = _binding()
     wl = synth.workload("c1")
