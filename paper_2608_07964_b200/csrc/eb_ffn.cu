@@ -978,29 +978,25 @@ eb_status ebi_ffn_run(eb_ctx* c, cudaStream_t st, const void* xp, const int32_t*
   if (!planned) {
     {
       KernelTimer timer(c, EBK_FFN_PLAN, st);
-      ebi_launch(plan_kernel, dim3(1), dim3(1024), 0, st, c->mp, group_off, step_meta, (int)device, tile_plan_of(c));
+      EB_LAUNCH(c, "expert_ffn", ebi_launch(plan_kernel, dim3(1), dim3(1024), 0, st, c->mp, group_off, step_meta, (int)device, tile_plan_of(c)));
     }
     KernelTimer timer(c, EBK_FFN_FILL, st);
-    ebi_launch(fill_kernel, dim3(c->num_sms), dim3(256), sizeof(int) * (size_t)(ebi_groups_cap(c) + 1), st, c->mp, group_off, group_w,
-               tile_list_of(c));
+    EB_LAUNCH(c, "expert_ffn", ebi_launch(fill_kernel, dim3(c->num_sms), dim3(256), sizeof(int) * (size_t)(ebi_groups_cap(c) + 1), st, c->mp,
+                                          group_off, group_w, tile_list_of(c)));
   }
-  cudaError_t e;
   if (!c->timing) {
     p.part = 0;
-    e = launch_ffn(c, st, p);
+    EB_LAUNCH(c, "expert_ffn", launch_ffn(c, st, p));
   } else {   // the same tiles in two launches, so that each phase gets a time of its own
     {
       KernelTimer timer(c, EBK_FFN_GATEUP, st);
       p.part = 1;
-      e = launch_ffn(c, st, p);
+      EB_LAUNCH(c, "expert_ffn", launch_ffn(c, st, p));
     }
-    if (e == cudaSuccess) {
-      KernelTimer timer(c, EBK_FFN_DOWN, st);
-      p.part = 2;
-      e = launch_ffn(c, st, p);
-    }
+    KernelTimer timer(c, EBK_FFN_DOWN, st);
+    p.part = 2;
+    EB_LAUNCH(c, "expert_ffn", launch_ffn(c, st, p));
   }
-  if (e != cudaSuccess) return ebi_check_cuda(c, e, "expert_ffn launch");
   EB_LAUNCH_CHECK(c, "expert_ffn");
   return EB_OK;
 }

@@ -462,14 +462,15 @@ eb_status ebi_front_run(eb_ctx* c, cudaStream_t st, const BatchParams& bp, uint3
   }
   if (bp.n_chunks > 0) {
     KernelTimer timer(c, EBK_ROUTE, st);
-    ebi_launch(g.E <= 64 ? front_kernel<2> : front_kernel<kMaxPerLane>, dim3(bp.n_chunks), dim3(kFrontThreads), 0, st, c->mp, bp, pool_mask, route_mask,
-               (const float*)b->logits, b->topk_idx, b->topk_w, c->chunk_hist);
+    EB_LAUNCH(c, "front", ebi_launch(g.E <= 64 ? front_kernel<2> : front_kernel<kMaxPerLane>, dim3(bp.n_chunks), dim3(kFrontThreads), 0, st, c->mp, bp,
+                                     pool_mask, route_mask, (const float*)b->logits, b->topk_idx, b->topk_w, c->chunk_hist));
   }
   {
     KernelTimer timer(c, EBK_SCHEDULE, st);
     const TablesArgs a{pool_mask, route_mask, (int)m, (int)policy, c->chunk_hist, c->chunk_base, c->chunk_seg, c->mb_base, b->mb_load,
                        b->mb_cnt, b->sched, b->group_off, b->group_w, b->step_meta, tile_plan_of(c)};
-    ebi_launch(tables_kernel, dim3(1), dim3(kSchedThreads), tables_smem(bp.n_mb, g.E, bp.n_mb * (g.E + g.D * g.S)), st, c->mp, bp, a);
+    EB_LAUNCH(c, "tables", ebi_launch(tables_kernel, dim3(1), dim3(kSchedThreads), tables_smem(bp.n_mb, g.E, bp.n_mb * (g.E + g.D * g.S)), st,
+                                      c->mp, bp, a));
   }
   {
     KernelTimer timer(c, EBK_PERMUTE_GATHER, st);
@@ -477,11 +478,10 @@ eb_status ebi_front_run(eb_ctx* c, cudaStream_t st, const BatchParams& bp, uint3
                         (const uint4*)b->x, (uint4*)b->xp, tile_list_of(c), c->num_sms / 2};
     const size_t smem = sizeof(int) * (size_t)(ebi_groups_cap(c) + 1);
     auto launch = [&](auto kernel, int tb) {
-      ebi_launch(kernel, dim3(a.fill_blocks + bp.n_chunks * (32 / tb)), dim3(kScatterThreads), smem, st, c->mp, bp, a);
+      return ebi_launch(kernel, dim3(a.fill_blocks + bp.n_chunks * (32 / tb)), dim3(kScatterThreads), smem, st, c->mp, bp, a);
     };
-    if (bp.n_tok <= 2 * c->num_sms) launch(scatter_kernel<1>, 1);
-    else if (bp.n_tok <= 16 * c->num_sms) launch(scatter_kernel<4>, 4);
-    else launch(scatter_kernel<8>, 8);
+    EB_LAUNCH(c, "scatter", bp.n_tok <= 2 * c->num_sms ? launch(scatter_kernel<1>, 1) : bp.n_tok <= 16 * c->num_sms ? launch(scatter_kernel<4>, 4)
+                                                                                                              : launch(scatter_kernel<8>, 8));
   }
   EB_LAUNCH_CHECK(c, "step front end");
   return EB_OK;

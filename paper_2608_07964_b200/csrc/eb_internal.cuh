@@ -136,6 +136,16 @@ struct KernelTimer {
     if (_e != cudaSuccess) return ebi_check_cuda((ctx), _e, #expr);     \
   } while (0)
 
+// A launch.  The kernels of a call work from what those before them wrote, so one that is refused ends the call.
+#define EB_LAUNCH(ctx, what, expr)                                      \
+  do {                                                                  \
+    cudaError_t _e = (expr);                                            \
+    if (_e != cudaSuccess) {                                            \
+      cudaGetLastError();                                               \
+      return ebi_check_cuda((ctx), _e, what);                           \
+    }                                                                   \
+  } while (0)
+
 #define EB_LAUNCH_CHECK(ctx, what)                                      \
   do {                                                                  \
     cudaError_t _e = cudaGetLastError();                                \

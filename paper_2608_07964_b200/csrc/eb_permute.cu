@@ -486,34 +486,35 @@ extern "C" eb_status eb_permute(eb_ctx* c, void* stream, const eb_batch* batch, 
       c->fused_attr_set = true;
     }
     KernelTimer timer(c, EBK_PERMUTE_FUSED, st);
-    ebi_launch(permute_fused_kernel, dim3(1), dim3(kFusedThreads), sizeof(int) * ((size_t)bp.n_chunks * c->cfg.E + gcap + 1 + (size_t)bp.n_tok * c->cfg.K),
-               st, c->mp, bp, d_res, topk_idx, group_off, group_w, pos, row_src, step_meta);
+    EB_LAUNCH(c, "permute", ebi_launch(permute_fused_kernel, dim3(1), dim3(kFusedThreads),
+                                       sizeof(int) * ((size_t)bp.n_chunks * c->cfg.E + gcap + 1 + (size_t)bp.n_tok * c->cfg.K), st, c->mp, bp,
+                                       d_res, topk_idx, group_off, group_w, pos, row_src, step_meta));
   } else {
     if (bp.n_chunks > 0) {
       KernelTimer timer(c, EBK_PERMUTE_HIST, st);
-      ebi_launch(hist_kernel, dim3(chunk_blocks), dim3(kWarps * 32), 0, st, c->mp, bp, d_res, topk_idx, c->chunk_hist);
+      EB_LAUNCH(c, "permute", ebi_launch(hist_kernel, dim3(chunk_blocks), dim3(kWarps * 32), 0, st, c->mp, bp, d_res, topk_idx, c->chunk_hist));
     }
     {
       KernelTimer timer(c, EBK_PERMUTE_SIZES, st);
-      ebi_launch(sizes_kernel, dim3((gcap + kWarps - 1) / kWarps), dim3(kWarps * 32), 0, st, c->mp, bp, d_res,
-                 (const int32_t*)c->chunk_hist, c->chunk_base, c->group_size);
+      EB_LAUNCH(c, "permute", ebi_launch(sizes_kernel, dim3((gcap + kWarps - 1) / kWarps), dim3(kWarps * 32), 0, st, c->mp, bp, d_res,
+                                         (const int32_t*)c->chunk_hist, c->chunk_base, c->group_size));
     }
     {
       KernelTimer timer(c, EBK_PERMUTE_SCAN, st);
-      ebi_launch(scan_kernel, dim3(1), dim3(1024), 0, st, c->mp, bp, d_res, (const int32_t*)c->group_size, group_off, group_w,
-                 step_meta);
+      EB_LAUNCH(c, "permute", ebi_launch(scan_kernel, dim3(1), dim3(1024), 0, st, c->mp, bp, d_res, (const int32_t*)c->group_size, group_off,
+                                         group_w, step_meta));
     }
     if (bp.n_chunks > 0) {
       KernelTimer timer(c, EBK_PERMUTE_RANK, st);
-      ebi_launch(rank_kernel, dim3(chunk_blocks), dim3(kWarps * 32), 0, st, c->mp, bp, d_res, topk_idx,
-                 (const int32_t*)c->chunk_base, (const int32_t*)group_off, pos, row_src, step_meta);
+      EB_LAUNCH(c, "permute", ebi_launch(rank_kernel, dim3(chunk_blocks), dim3(kWarps * 32), 0, st, c->mp, bp, d_res, topk_idx,
+                                         (const int32_t*)c->chunk_base, (const int32_t*)group_off, pos, row_src, step_meta));
     }
   }
   if (bp.n_tok > 0) {
     KernelTimer timer(c, EBK_PERMUTE_GATHER, st);
     const int team = team_for(c->cfg.H / 8), tpb = kGatherThreads / team;
-    ebi_launch(gather_kernel, dim3((bp.n_tok + tpb - 1) / tpb), dim3(kGatherThreads), 0, st, bp.n_tok, c->cfg.H,
-               c->cfg.K + c->cfg.S, team, (const uint4*)x, (const int32_t*)pos, (uint4*)xp);
+    EB_LAUNCH(c, "permute", ebi_launch(gather_kernel, dim3((bp.n_tok + tpb - 1) / tpb), dim3(kGatherThreads), 0, st, bp.n_tok, c->cfg.H,
+                                       c->cfg.K + c->cfg.S, team, (const uint4*)x, (const int32_t*)pos, (uint4*)xp));
   }
   EB_LAUNCH_CHECK(c, "permute");
   return EB_OK;
@@ -608,8 +609,8 @@ extern "C" eb_status eb_check_permutation(eb_ctx* c, void* stream, const eb_batc
   cudaStream_t st = (cudaStream_t)stream;
   int32_t* d_err = c->group_size;   // scratch word; the next eb_permute rewrites it
   EB_CUDA(c, cudaMemsetAsync(d_err, 0, sizeof(int32_t), st));
-  ebi_launch(check_kernel, dim3(2 * c->num_sms), dim3(256), 0, st, c->mp, bp, ebi_rows_cap(c), ebi_groups_cap(c), d_res,
-             topk_idx, group_off, group_w, row_src, pos, step_meta, d_err);
+  EB_LAUNCH(c, "check_permutation", ebi_launch(check_kernel, dim3(2 * c->num_sms), dim3(256), 0, st, c->mp, bp, ebi_rows_cap(c), ebi_groups_cap(c), d_res,
+                                               topk_idx, group_off, group_w, row_src, pos, step_meta, d_err));
   EB_LAUNCH_CHECK(c, "check_permutation");
   EB_CUDA(c, cudaMemcpyAsync(out_errors, d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   EB_CUDA(c, cudaStreamSynchronize(st));
@@ -740,23 +741,27 @@ extern "C" eb_status eb_permute_noalloc(const eb_config* cfg, void* stream, cons
 
   cudaStream_t st = (cudaStream_t)stream;
   // the array keeps the previous call's contents: tables rewritten, counters start from zero every call
+  cudaError_t ce = cudaSuccess;
+  auto refused = [&] { return (ce = cudaGetLastError()) != cudaSuccess; };   // the last launch was; nothing is launched behind it
+  auto fail = [&] { return noalloc_fail(err, err_cap, EB_ERR_CUDA, cudaGetErrorString(ce)); };
   noalloc_setup_kernel<<<64, 256, 0, st>>>(tables, d_tab, d_hist, kNaHistWords, d_gsize, kNaGroupWords);
-  cudaError_t ce = cudaGetLastError();
-  if (ce != cudaSuccess) return noalloc_fail(err, err_cap, EB_ERR_CUDA, cudaGetErrorString(ce));
+  if (refused()) return fail();
 
   const int gcap = EB_MAX_MB * (g.E + g.D * g.S);
   const int chunk_blocks = (bp.n_chunks + kWarps - 1) / kWarps;
   if (bp.n_chunks > 0) hist_kernel<<<chunk_blocks, kWarps * 32, 0, st>>>(mp, bp, d_res, topk_idx, d_hist);
+  if (refused()) return fail();
   sizes_kernel<<<(gcap + kWarps - 1) / kWarps, kWarps * 32, 0, st>>>(mp, bp, d_res, d_hist, d_cbase, d_gsize);
+  if (refused()) return fail();
   scan_kernel<<<1, 1024, 0, st>>>(mp, bp, d_res, d_gsize, group_off, group_w, step_meta);
+  if (refused()) return fail();
   if (bp.n_chunks > 0)
     rank_kernel<<<chunk_blocks, kWarps * 32, 0, st>>>(mp, bp, d_res, topk_idx, d_cbase, group_off, pos, row_src, step_meta);
+  if (refused()) return fail();
   if (bp.n_tok > 0) {
     const int team = team_for(g.H / 8), tpb = kGatherThreads / team;
     gather_kernel<<<(bp.n_tok + tpb - 1) / tpb, kGatherThreads, 0, st>>>(bp.n_tok, g.H, g.K + g.S, team, (const uint4*)x,
                                                                          pos, (uint4*)xp);
   }
-  ce = cudaGetLastError();
-  if (ce != cudaSuccess) return noalloc_fail(err, err_cap, EB_ERR_CUDA, cudaGetErrorString(ce));
-  return EB_OK;
+  return refused() ? fail() : EB_OK;
 }

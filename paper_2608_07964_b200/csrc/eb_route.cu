@@ -58,11 +58,11 @@ extern "C" eb_status eb_route(eb_ctx* c, void* stream, const eb_batch* batch, ui
   cudaStream_t st = (cudaStream_t)stream;
   KernelTimer timer(c, EBK_ROUTE, st);
   int n = bp.n_mb * (c->cfg.E + c->cfg.D);
-  ebi_launch(route_clear_kernel, dim3((n + 255) / 256), dim3(256), 0, st, c->mp, bp, route_mask, mb_load, mb_cnt);
+  EB_LAUNCH(c, "route", ebi_launch(route_clear_kernel, dim3((n + 255) / 256), dim3(256), 0, st, c->mp, bp, route_mask, mb_load, mb_cnt));
   if (bp.n_tok > 0) {
     int blocks = (bp.n_tok + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    ebi_launch(c->cfg.E <= 64 ? route_kernel<2> : route_kernel<kMaxPerLane>, dim3(blocks), dim3(kWarpsPerBlock * 32), 0, st, c->mp, bp, route_mask, logits, topk_idx, topk_w,
-               mb_load, mb_cnt);
+    EB_LAUNCH(c, "route", ebi_launch(c->cfg.E <= 64 ? route_kernel<2> : route_kernel<kMaxPerLane>, dim3(blocks), dim3(kWarpsPerBlock * 32), 0, st,
+                                     c->mp, bp, route_mask, logits, topk_idx, topk_w, mb_load, mb_cnt));
   }
   EB_LAUNCH_CHECK(c, "route");
   return EB_OK;

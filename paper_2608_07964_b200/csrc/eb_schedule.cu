@@ -66,8 +66,9 @@ extern "C" eb_status eb_schedule(eb_ctx* c, void* stream, const eb_batch* batch,
     for (int j = 0; j < bp.n_mb; ++j) np += (batch->pool_mask >> j) & 1u;
     const int blocks = policy == EB_POLICY_MAXUTIL && np > m && np > 13 ? 1 << (np - 13) : 1;
     KernelTimer timer(c, EBK_SCHEDULE, st);
-    ebi_launch(schedule_kernel, dim3(blocks), dim3(kSchedThreads), 0, st, c->cfg.D, bp.n_mb, batch->pool_mask, (int)m,
-               (int)policy, mb_load, d_res, (Cand*)c->d_sched_scratch, (unsigned*)(c->d_sched_scratch + kMaxBlocks * sizeof(Cand)));
+    EB_LAUNCH(c, "schedule", ebi_launch(schedule_kernel, dim3(blocks), dim3(kSchedThreads), 0, st, c->cfg.D, bp.n_mb, batch->pool_mask, (int)m,
+                                        (int)policy, mb_load, d_res, (Cand*)c->d_sched_scratch,
+                                        (unsigned*)(c->d_sched_scratch + kMaxBlocks * sizeof(Cand))));
   }
   EB_LAUNCH_CHECK(c, "schedule");
   if (h_res) {

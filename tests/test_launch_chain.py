@@ -67,3 +67,47 @@ def test_a_context_keeps_its_shared_memory_whatever_others_do(lib):
     assert late.step(4, 3) == 0
     for c, s in zip(ctxs, SHAPES):
         assert c.step(16, 96) == 0, s
+
+
+def _calls(c, n_mb, tokens):
+    """Every call that enqueues kernels, by name."""
+    l, b, p = c.lib, c.batch(n_mb, tokens), c.p
+    ref = C.byref(b.c)
+    bad, gave_up = C.c_int32(), C.c_int32()
+    e2d = (C.c_int32 * 8)(*[e % 4 for e in range(8)])
+    cfg = B.EbConfig(4, 8, 2, 1, 64, 64, 4, 1, 4096, e2d)
+    err = C.create_string_buffer(256)
+    return dict(
+        route=lambda: l.eb_route(c.ctx, None, ref, b.pool_mask, p, p, p, p, p),
+        schedule=lambda: l.eb_schedule(c.ctx, None, ref, 1, 0, p, p, None),
+        permute=lambda: l.eb_permute(c.ctx, None, ref, p, p, p, p, p, p, p, p, p),
+        permute_noalloc=lambda: l.eb_permute_noalloc(C.byref(cfg), None, ref, p, p, p, p, p, p, p, p, p, err, 256),
+        expert_ffn=lambda: l.eb_expert_ffn_grouped(c.ctx, None, p, p, p, p, p),
+        expert_ffn_device=lambda: l.eb_expert_ffn_device(c.ctx, None, p, p, p, p, p, 1),
+        combine=lambda: l.eb_combine(c.ctx, None, ref, p, p, p, p, p),
+        step=lambda: c.step(n_mb, tokens),
+        step_host=lambda: l.eb_step_host(c.ctx, None, ref, b.pool_mask, 1, 0, C.byref(c.bufs), p, p, p, None),
+        check_permutation=lambda: l.eb_check_permutation(c.ctx, None, ref, p, p, p, p, p, p, p, C.byref(bad)),
+        check_guards=lambda: l.eb_check_workspace_guards(c.ctx, None, C.byref(bad)),
+        selftest=lambda: l.eb_selftest_bounded_wait(c.ctx, None, 1000, C.byref(gave_up)))
+
+
+@pytest.mark.parametrize("timing", [0, 1])
+@pytest.mark.parametrize("n_mb,tokens", [(3, 5), (8, 400)])   # the fused permute kernel, and the four it stands for
+def test_nothing_is_launched_behind_a_refused_kernel(lib, n_mb, tokens, timing):
+    """Each kernel of a call works from what the one before it wrote: when the runtime refuses one, the call says so and
+    launches no further kernel, and the next call starts clean."""
+    lib.fake_reset(-1)
+    c = Context(lib, E=8, K=2, S=1, D=4, max_tokens=4096)
+    assert lib.eb_set_timing(c.ctx, timing) == 0
+    for name, call in _calls(c, n_mb, tokens).items():
+        lib.fake_reset(-1)
+        assert call() == 0, name
+        chain = c.names()
+        assert chain, name
+        for i in range(len(chain)):
+            lib.fake_reset(i)
+            assert call() == EB_ERR_CUDA, (name, chain[i])
+            assert c.names() == chain[:i], (name, chain[i])
+            lib.fake_reset(-1)
+            assert call() == 0 and c.names() == chain, (name, chain[i], "afterwards")
