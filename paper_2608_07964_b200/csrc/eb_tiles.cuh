@@ -32,7 +32,7 @@ struct Tile {
   int phase;    // 1: gate/up + SwiGLU (256 outputs per tile);  2: down (512 outputs per tile)
   int done;     // the token tile this one belongs to: entry of `ready`
   int need;     // phase 2: arrivals on that entry after which the rows of the intermediate are all written (0: they are)
-  int once;     // no other tile reads its weights
+  int once;     // no other token tile of the launch reads its matrix
 };
 static_assert(sizeof(Tile) == 32, "two 16-byte words");
 
@@ -227,7 +227,7 @@ __device__ __forceinline__ void fill_tiles(const ModelParams& mp, const int32_t*
   const int nt1 = l.nt1, nt2 = l.nt2;
   int2* __restrict__ slots = l.slots;
   const int n_listed = l.work_count[5];
-  const int cnt1 = l.work_count[0], total = cnt1 + l.work_count[1];
+  const int cnt1 = l.work_count[0], total = cnt1 + l.work_count[1], nl = l.work_count[8], device = l.work_count[9];
   if (block * (int)blockDim.x >= total) return;
   for (int i = threadIdx.x; i <= n_listed; i += blockDim.x) s_pref[i] = tile_pref[i];
   __syncthreads();
@@ -275,7 +275,10 @@ __device__ __forceinline__ void fill_tiles(const ModelParams& mp, const int32_t*
     it.phase = list + 1;
     it.done = s_pref[lo] + m;
     it.need = nt1 * 2;
-    it.once = t_g == 1;
+    // the replicas of a shared expert that are not merged are tiles of their own over one matrix (with a device filter the
+    // list holds one replica only)
+    const bool replica = n_slots < 0 && device < 0 && mp.D > 1 && pos >= nl * mp.E;
+    it.once = t_g == 1 && !replica;
     if (list == 0 && n == 0) l.ready[it.done] = 0;
     if (idx < l.max_work) l.work[idx] = it;
   }

@@ -109,3 +109,29 @@ def check_front(step, case: Case, ref: Dict, n_mb: int):
     # first group of every virtual device
     firsts = [next((g for g, (d, _, _) in enumerate(ref["groups"]) if d >= dd), G) for dd in range(wl.D)] + [G]
     assert meta["dev_group_off"] == firsts
+
+
+def workspace_regions(step) -> Dict[str, torch.Tensor]:
+    """The workspace's regions by name, as bytes.  The guard area behind each one has to be where this layout puts it."""
+    E, gcap, rows = step.E, step.groups_cap, step.rows_cap
+    chunks = (step.max_tokens + 31) // 32 + 16
+    tiles = rows // 256 + gcap
+    work = tiles * (-(-step.I // 256) + -(-step.H // 512))
+    sizes = dict(chunk_hist=4 * chunks * E, chunk_base=4 * chunks * E, chunk_seg=4 * (chunks // 32 + 16) * E, mb_base=4 * 16 * E,
+                 group_size=4 * gcap, pgroup=4 * gcap, pslots=4 * gcap, prank=16 * gcap, order=4 * gcap, tile_pref=4 * (gcap + 1),
+                 work_count=64, work=32 * work, tile_ready=4 * tiles, slots=8 * 16 * tiles, act=2 * rows * step.I)
+    out, off = {}, 0
+    for name, n in sizes.items():
+        out[name] = step.workspace[off:off + n]
+        off = (off + n + 255) // 256 * 256
+        assert bool((step.workspace[off:off + 256] == 0xA5).all()), f"no guard behind {name}: the layout has changed"
+        off += 256
+    assert off == step.workspace.numel()
+    return out
+
+
+def tile_list(step) -> np.ndarray:
+    """The tiles of the last expert pass [n, 8]: row, rows, matrix, output tile, phase, token tile, need, once."""
+    r = workspace_regions(step)
+    counts = r["work_count"].view(torch.int32).cpu().numpy()
+    return r["work"].view(torch.int32).cpu().numpy().reshape(-1, 8)[:counts[0] + counts[1]]

@@ -527,6 +527,44 @@ def test_one_launch_for_both_phases_equals_a_launch_each(tokens, H, I):
     assert all(torch.equal(got[0], g) for g in got[1:])
 
 
+@pytest.mark.parametrize("S,D,tokens,layers", [
+    (2, 4, [70, 70, 70, 70], [0, 0, 0, 0]),        # 70 rows per replica of a shared expert: a tile each over one matrix
+    (1, 8, [256, 256, 30], [0, 0, 1]),             # 64 rows (packed into common tiles) and fewer
+    (1, 8, [264, 256, 30], [0, 0, 1]),             # 65 rows
+    (1, 2, [600, 3], [0, 1]),                      # 300 rows: two tiles per replica
+    (3, 1, [90, 300], [0, 1]),                     # one device: one tile, and two, without replicas
+    (0, 3, [300, 40], [0, 0]),
+])
+def test_weights_are_marked_once_where_one_tile_reads_them(S, D, tokens, layers):
+    """The mark by which weights leave L2 first: on a tile exactly when no other token tile of the launch reads its matrix,
+    in the lists of a whole step, of the expert pass alone, and of one device's groups."""
+    B = _binding()
+    wl = _small(L=2, E=6, K=2, S=S, D=D, N=len(tokens), T=max(tokens), H=72, I=264, mapping="mod", zipf_s=1.5)
+    case, store = Hn.make_case(wl, tokens, layers), Hn.WeightStore(wl)
+    step = B.from_workload(wl, max_tokens=case.T_tot)
+    step.bind_weights(store.gate, store.up, store.down)
+    step.logits[:case.T_tot].copy_(case.logits)
+    step.x[:case.T_tot].copy_(case.x)
+
+    def check():
+        tiles = Hn.tile_list(step)
+        readers = {}
+        for t in tiles:
+            readers.setdefault(int(t[2]), set()).add(int(t[5]))
+        assert [int(t[7]) for t in tiles] == [int(len(readers[int(t[2])]) == 1) for t in tiles]
+        return sum(len(v) > 1 for v in readers.values())
+
+    step.eb_step(B.Batch(case.tok_off, case.layers), len(tokens))
+    shared = check()
+    assert shared > 0 or max(tokens) < 70
+    step.eb_expert_ffn_grouped()
+    assert check() == shared
+    for d in range(D):
+        step.eb_expert_ffn_grouped(device=d)
+        check()
+    assert step.device_status() == 0
+
+
 # ----------------------------------------------------------------------------------- failure reporting
 def test_bounded_wait_gives_up_and_reports_without_harming_the_context():
     B = _binding()
