@@ -214,9 +214,9 @@ eb_status eb_combine_residual(eb_ctx* ctx, void* stream, const eb_batch* batch, 
 /* ---- whole step --------------------------------------------------------------------------- */
 
 /* What the five calls compute, back to back on `stream` with device-resident inputs (buf->logits, buf->x): the same
- * outputs, with everything before the expert pass in three launches; the
- * aggregation adds buf->residual when it is not NULL (Algorithm 1's step for a model that carries its
- * hidden states in buf->x: residual = out = x updates them in place). */
+ * outputs, with everything before the expert pass in three launches (four for many tokens); the aggregation adds
+ * buf->residual when it is not NULL (Algorithm 1's step for a model that carries its hidden states in buf->x:
+ * residual = out = x updates them in place). */
 eb_status eb_step(eb_ctx* ctx, void* stream, const eb_batch* batch, uint32_t route_mask, int32_t m,
                   eb_policy policy, const eb_step_buffers* buf);
 
@@ -311,7 +311,7 @@ eb_status eb_selftest_bounded_wait(eb_ctx* ctx, void* stream, int64_t limit_cycl
  * stream.  eb_kernel_ms synchronises and writes the duration in ms of the most recent launch of
  * each kernel (negative if it has not run since timing was enabled); `ms` is host [eb_num_kernels()].
  * In a whole step (eb_step) "route" is routing with the chunk histograms, "schedule" the block that makes loads,
- * schedule, group table and tile plan, "permute_gather" ranks, gather and tile list.  The expert pass runs as one
+ * schedule, group table and tile plan (for many tokens with the sums of the histograms before it), "permute_gather" ranks, gather and tile list.  The expert pass runs as one
  * launch when timing is off, as one per phase when it is on. */
 int32_t eb_num_kernels(void);
 const char* eb_kernel_name(int32_t i);

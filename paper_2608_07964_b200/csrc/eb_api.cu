@@ -91,6 +91,7 @@ static size_t carve(eb_ctx* c, char* base) {
   c->chunk_hist = (int32_t*)take(sizeof(int32_t) * (size_t)c->max_chunks * g.E);
   c->chunk_base = (int32_t*)take(sizeof(int32_t) * (size_t)c->max_chunks * g.E);
   c->chunk_seg = (int32_t*)take(sizeof(int32_t) * (size_t)(c->max_chunks / EB_SEG_CHUNKS + EB_MAX_MB) * g.E);
+  c->seg_base = (int32_t*)take(sizeof(int32_t) * (size_t)(c->max_chunks / EB_SEG_CHUNKS + EB_MAX_MB) * g.E);
   c->mb_base = (int32_t*)take(sizeof(int32_t) * (size_t)EB_MAX_MB * g.E);
   c->group_size = (int32_t*)take(sizeof(int32_t) * (size_t)gcap);
   c->pgroup = (int32_t*)take(sizeof(int32_t) * (size_t)gcap);

@@ -1,6 +1,8 @@
-// The front end of a whole step, eb_step: everything between the inputs and the expert pass in three launches.
+// The front end of a whole step, eb_step: everything between the inputs and the expert pass in three launches (four for
+// many tokens).
 //
 //   front_kernel  : per chunk of <= 32 tokens: routing (a warp per token) and the chunk's assignments per expert
+//   sums_kernel   : many tokens only: sums of the chunk histograms per 32 chunks, which one block would take too long over
 //   tables_kernel : one block: loads, schedule, group table, tile plan
 //   scatter_kernel: per part of a chunk: ranks, positions, gather of the token rows; some blocks fill the tile list
 //
@@ -9,6 +11,8 @@
 // a launch, a first trip to memory and a few block barriers (2-5 us), so the split here follows the dependences that
 // need the whole GPU to be through: the counts of all tokens, then the positions of all rows.  The counts travel as
 // chunk histograms, which also spares the routing its global atomics.
+#include <algorithm>
+
 #include "eb_dispatch.cuh"
 #include "eb_route.cuh"
 #include "eb_schedule.cuh"
@@ -43,12 +47,50 @@ front_kernel(ModelParams mp, BatchParams bp, uint32_t pool_mask, uint32_t route_
   for (int e = threadIdx.x; e < mp.E; e += kFrontThreads) chunk_hist[(size_t)c * mp.E + e] = s_hist[e];
 }
 
+// Running sum of n values that lie `stride` apart, left before each in `base`; returns the total.  Sixteen loads at a time.
+__device__ __forceinline__ int sum_chunks(const int32_t* __restrict__ h, int32_t* __restrict__ base, int n, int stride) {
+  int run = 0;
+  for (int k0 = 0; k0 < n; k0 += 16) {
+    int v[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = k0 + k < n ? h[(size_t)(k0 + k) * stride] : 0;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      if (k0 + k < n) base[(size_t)(k0 + k) * stride] = run;
+      run += v[k];
+    }
+  }
+  return run;
+}
+
+// ---- sums ------------------------------------------------------------------------------------
+// Segments of at most EB_SEG_CHUNKS chunks of one micro-batch.
+struct Segments {
+  int off[EB_MAX_MB + 1];   // first segment of every micro-batch; beyond n_mb: the total
+};
+
+// A thread per (segment, expert): chunk_base = assignments before the chunk in its segment, chunk_seg = of the segment.
+// Only for steps whose histograms are too much for the one block of tables_kernel to add up (see kSumsWords).
+__global__ void __launch_bounds__(256)
+sums_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ BatchParams bp, const __grid_constant__ Segments seg, uint32_t counted,
+            const int32_t* __restrict__ chunk_hist, int32_t* __restrict__ chunk_base, int32_t* __restrict__ chunk_seg) {
+  EB_GRID_DEP_SYNC();
+  const int i = blockIdx.x * 256 + threadIdx.x, g = i / mp.E, e = i - g * mp.E;
+  if (g >= seg.off[EB_MAX_MB]) return;
+  int j = 0;
+  while (seg.off[j + 1] <= g) ++j;
+  if (!((counted >> j) & 1u)) return;
+  const int c0 = bp.chunk_off[j] + (g - seg.off[j]) * EB_SEG_CHUNKS;
+  chunk_seg[i] = sum_chunks(chunk_hist + (size_t)c0 * mp.E + e, chunk_base + (size_t)c0 * mp.E + e, min((int)EB_SEG_CHUNKS, bp.chunk_off[j + 1] - c0), mp.E);
+}
+
 // ---- tables ----------------------------------------------------------------------------------
 struct TablesArgs {
   uint32_t pool_mask, route_mask;
   int m, policy;
-  const int32_t* chunk_hist;
-  int32_t *chunk_base, *chunk_seg, *mb_base, *mb_load, *mb_cnt;
+  const int32_t *chunk_hist, *chunk_seg;   // chunk_seg: null without sums_kernel
+  int32_t *chunk_base, *seg_base, *mb_base, *mb_load, *mb_cnt;
+  Segments seg;
   eb_sched_result* res;
   int32_t *group_off, *group_w, *step_meta;
   TilePlan plan;
@@ -64,7 +106,7 @@ __global__ void __launch_bounds__(kSchedThreads)
 tables_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ BatchParams bp, const __grid_constant__ TablesArgs a) {
   EB_GRID_DEP_SYNC();
   extern __shared__ int4 s_dyn4[];
-  __shared__ int s_dev_off[EB_MAX_D + 1], s_dev_list[EB_MAX_E], s_e2d[EB_MAX_E], s_seg_off[EB_MAX_MB + 1];
+  __shared__ int s_dev_off[EB_MAX_D + 1], s_dev_list[EB_MAX_E], s_e2d[EB_MAX_E];
   __shared__ int s_home[EB_MAX_MB][EB_MAX_D + 1];   // first local token of every home device, per micro-batch
   __shared__ int s_hrows[EB_MAX_MB][EB_MAX_D];      // rows of a shared expert's replica: (active layer, device)
   __shared__ int s_hslots[EB_MAX_MB], s_hmax[EB_MAX_MB];   // slots of its merged class and its largest replica: per active layer
@@ -102,87 +144,27 @@ tables_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ Ba
       if (d == 15 && D == 16) s_home[j][16] = T;
     }
   }
-  if (warp == 31) {
-    const int j = lane < n_mb ? lane : 0;
-    const int n = lane < n_mb ? (bp.chunk_off[j + 1] - bp.chunk_off[j] + EB_SEG_CHUNKS - 1) / EB_SEG_CHUNKS : 0;
-    int incl = n;
-#pragma unroll
-    for (int o = 1; o < 16; o <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += v;
-    }
-    if (lane < EB_MAX_MB) s_seg_off[lane + 1] = incl;   // beyond n_mb: the total
-    if (lane == 0) s_seg_off[0] = s_carry = 0;
-  }
-  for (int i = tid; i < n_mb * E; i += kSchedThreads) s_cnt[i] = 0;
+  if (tid == kSchedThreads - 1) s_carry = 0;
   __syncthreads();
 
-  // ---- assignments of every (micro-batch, expert) from the chunk histograms; chunk_base = those before the chunk in its
-  // micro-batch.  One thread per segment of chunks and expert; a micro-batch of one segment (<= 1024 tokens) is done
-  // in one go, a longer one adds up its segments in between.
-  const int n_items = s_seg_off[EB_MAX_MB] * E;
+  // ---- assignments of every (micro-batch, expert): from the segments' sums, or from the chunk histograms, which also gives
+  // chunk_base = those before the chunk in its micro-batch
   const uint32_t counted = a.pool_mask | a.route_mask;
-  auto mb_of_seg = [&](int g) {   // the last micro-batch whose segments start at or before g
-    int j = 0;
-#pragma unroll
-    for (int step = 8; step > 0; step >>= 1)
-      if (s_seg_off[j + step] <= g) j += step;
-    return j;
-  };
-  bool any_long = false;
-  for (int i = tid; i < n_items; i += kSchedThreads) {
-    const int g = div_e(i), e = i - g * E, j = mb_of_seg(g);
-    if (!((counted >> j) & 1u)) continue;
-    const int c0 = bp.chunk_off[j] + (g - s_seg_off[j]) * EB_SEG_CHUNKS;
-    const int n = min((int)EB_SEG_CHUNKS, bp.chunk_off[j + 1] - c0);
-    const bool whole = s_seg_off[j + 1] - s_seg_off[j] == 1;
-    const int32_t* h = a.chunk_hist + (size_t)c0 * E + e;
-    int32_t* base = a.chunk_base + (size_t)c0 * E + e;
-    int run = 0;
-    for (int k0 = 0; k0 < n; k0 += 16) {
-      int v[16];
-#pragma unroll
-      for (int k = 0; k < 16; ++k) v[k] = k0 + k < n ? h[(size_t)(k0 + k) * E] : 0;
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        if (whole && k0 + k < n) base[(size_t)(k0 + k) * E] = run;
-        run += v[k];
+  for (int i = tid; i < n_mb * E; i += kSchedThreads) {
+    const int j = div_e(i), e = i - j * E;
+    int n = 0;
+    if ((counted >> j) & 1u) {
+      if (a.chunk_seg) {
+        const size_t at = (size_t)a.seg.off[j] * E + e;
+        n = sum_chunks(a.chunk_seg + at, a.seg_base + at, a.seg.off[j + 1] - a.seg.off[j], E);
+      } else {
+        const size_t at = (size_t)bp.chunk_off[j] * E + e;
+        n = sum_chunks(a.chunk_hist + at, a.chunk_base + at, bp.chunk_off[j + 1] - bp.chunk_off[j], E);
       }
     }
-    if (whole) {
-      s_cnt[j * E + e] = run;
-    } else {
-      a.chunk_seg[i] = run;
-      any_long = true;
-    }
+    s_cnt[i] = n;
   }
-  if (__syncthreads_or(any_long)) {
-    for (int i = tid; i < n_mb * E; i += kSchedThreads) {
-      const int j = div_e(i), e = i - j * E;
-      if (s_seg_off[j + 1] - s_seg_off[j] < 2 || !((counted >> j) & 1u)) continue;
-      int run = 0;
-      for (int g = s_seg_off[j]; g < s_seg_off[j + 1]; ++g) {
-        const int v = a.chunk_seg[(size_t)g * E + e];
-        a.chunk_seg[(size_t)g * E + e] = run;
-        run += v;
-      }
-      s_cnt[i] = run;
-    }
-    __syncthreads();
-    for (int i = tid; i < n_items; i += kSchedThreads) {
-      const int g = div_e(i), e = i - g * E, j = mb_of_seg(g);
-      if (s_seg_off[j + 1] - s_seg_off[j] < 2 || !((counted >> j) & 1u)) continue;
-      const int c0 = bp.chunk_off[j] + (g - s_seg_off[j]) * EB_SEG_CHUNKS;
-      const int n = min((int)EB_SEG_CHUNKS, bp.chunk_off[j + 1] - c0);
-      int run = a.chunk_seg[i];
-      for (int k = 0; k < n; ++k) {
-        const int v = a.chunk_hist[(size_t)(c0 + k) * E + e];
-        a.chunk_base[(size_t)(c0 + k) * E + e] = run;
-        run += v;
-      }
-    }
-    __syncthreads();
-  }
+  __syncthreads();
 
   // ---- loads of the micro-batches routed now: four threads per (micro-batch, device)
   for (int i = tid; i < n_mb * E; i += kSchedThreads)
@@ -326,7 +308,8 @@ constexpr int kScatterThreads = 256;
 
 struct ScatterArgs {
   const eb_sched_result* res;
-  const int32_t *topk_idx, *chunk_base, *mb_base, *group_off, *group_w;
+  const int32_t *topk_idx, *chunk_base, *seg_base, *mb_base, *group_off, *group_w;   // seg_base: null without sums_kernel
+  Segments seg;
   int32_t *pos, *row_src, *step_meta;
   const uint4* x;
   uint4* xp;
@@ -375,7 +358,8 @@ scatter_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ B
   // assignments from the start of the chunk to the end of this part
   const int first = (t0 - c0) * K, last = first + nt * K;
   if (tid < last) s_topk[tid] = a.topk_idx[(size_t)c0 * K + tid];
-  for (int e = tid; e < E; e += kScatterThreads) s_next[e] = a.mb_base[j * E + e] + a.chunk_base[(size_t)c * E + e];
+  const int32_t* seg_base = a.seg_base ? a.seg_base + (size_t)(a.seg.off[j] + (c - bp.chunk_off[j]) / EB_SEG_CHUNKS) * E : nullptr;
+  for (int e = tid; e < E; e += kScatterThreads) s_next[e] = a.mb_base[j * E + e] + a.chunk_base[(size_t)c * E + e] + (seg_base ? seg_base[e] : 0);
   step_shape_block(bp, run, &ss);   // ends with a barrier
   if (tid < 32) {
     const int lr = ss.rank_of_mb[j];
@@ -443,6 +427,15 @@ scatter_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ B
   }
 }
 
+// tables_kernel adds the chunk histograms up itself below this many words (chunks times experts) and up to this many chunks
+// of one micro-batch: one block reads and writes them at the rate of one SM, and a thread per (micro-batch, expert) goes through
+// a micro-batch's chunks in turn.  A launch of sums_kernel costs 2-3 us.  Steps without / with it (us, H = I = 64): 64 experts,
+// 16 x 1024 tokens (32768 words) 128.1 / 131.2, 16 x 2048 225.2 / 223.9, 16 x 4096 400 / 389; 256 experts, 16 x 512 (65536)
+// 117.0 / 118.3, 16 x 1024 190 / 183, 16 x 4096 616 / 559; 8 experts, 1 x 2048 (64 chunks) 42.4 / 42.0, 1 x 4096 50.3 / 46.0,
+// 1 x 65536 346 / 193.
+constexpr int kSumsWords = 65536;
+constexpr int kSumsChunks = 64;
+
 constexpr size_t tables_smem(int n_mb, int E, int groups) {
   return sizeof(SchedShared) + sizeof(int) * ((size_t)n_mb * E + 3 * (size_t)groups + 1);
 }
@@ -465,16 +458,25 @@ eb_status ebi_front_run(eb_ctx* c, cudaStream_t st, const BatchParams& bp, uint3
     EB_LAUNCH(c, "front", ebi_launch(g.E <= 64 ? front_kernel<2> : front_kernel<kMaxPerLane>, dim3(bp.n_chunks), dim3(kFrontThreads), 0, st, c->mp, bp,
                                      pool_mask, route_mask, (const float*)b->logits, b->topk_idx, b->topk_w, c->chunk_hist));
   }
+  Segments seg;
+  seg.off[0] = 0;
+  for (int j = 0; j < EB_MAX_MB; ++j) seg.off[j + 1] = seg.off[j] + (bp.chunk_off[j + 1] - bp.chunk_off[j] + EB_SEG_CHUNKS - 1) / EB_SEG_CHUNKS;
+  int longest = 0;
+  for (int j = 0; j < bp.n_mb; ++j) longest = std::max(longest, bp.chunk_off[j + 1] - bp.chunk_off[j]);
+  const bool sums = bp.n_chunks * g.E >= kSumsWords || longest > kSumsChunks;
   {
     KernelTimer timer(c, EBK_SCHEDULE, st);
-    const TablesArgs a{pool_mask, route_mask, (int)m, (int)policy, c->chunk_hist, c->chunk_base, c->chunk_seg, c->mb_base, b->mb_load,
-                       b->mb_cnt, b->sched, b->group_off, b->group_w, b->step_meta, tile_plan_of(c)};
+    if (sums)
+      EB_LAUNCH(c, "sums", ebi_launch(sums_kernel, dim3((seg.off[EB_MAX_MB] * g.E + 255) / 256), dim3(256), 0, st, c->mp, bp, seg, pool_mask | route_mask,
+                                      (const int32_t*)c->chunk_hist, c->chunk_base, c->chunk_seg));
+    const TablesArgs a{pool_mask, route_mask, (int)m, (int)policy, c->chunk_hist, sums ? c->chunk_seg : nullptr, c->chunk_base, c->seg_base,
+                       c->mb_base, b->mb_load, b->mb_cnt, seg, b->sched, b->group_off, b->group_w, b->step_meta, tile_plan_of(c)};
     EB_LAUNCH(c, "tables", ebi_launch(tables_kernel, dim3(1), dim3(kSchedThreads), tables_smem(bp.n_mb, g.E, bp.n_mb * (g.E + g.D * g.S)), st,
                                       c->mp, bp, a));
   }
   {
     KernelTimer timer(c, EBK_PERMUTE_GATHER, st);
-    const ScatterArgs a{b->sched, b->topk_idx, c->chunk_base, c->mb_base, b->group_off, b->group_w, b->pos, b->row_src, b->step_meta,
+    const ScatterArgs a{b->sched, b->topk_idx, c->chunk_base, sums ? c->seg_base : nullptr, c->mb_base, b->group_off, b->group_w, seg, b->pos, b->row_src, b->step_meta,
                         (const uint4*)b->x, (uint4*)b->xp, tile_list_of(c), c->num_sms / 2};
     const size_t smem = sizeof(int) * (size_t)(ebi_groups_cap(c) + 1);
     auto launch = [&](auto kernel, int tb) {

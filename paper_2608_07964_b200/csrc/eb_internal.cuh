@@ -16,7 +16,7 @@ typedef __nv_bfloat16 bf16;
 
 enum { EB_MAX_GUARDS = 24 };
 
-// Chunks whose histograms one thread of a whole step's table kernel adds up.
+// Chunks whose histograms one thread adds up in a whole step of many tokens.
 enum { EB_SEG_CHUNKS = 32 };
 
 // Kernel ids for the optional per-kernel event timing.
@@ -79,7 +79,8 @@ struct eb_ctx {
   size_t guard_off[EB_MAX_GUARDS] = {};
   int32_t* chunk_hist = nullptr;   // [max_chunks][E]
   int32_t* chunk_base = nullptr;   // [max_chunks][E]
-  int32_t* chunk_seg = nullptr;    // [max_segs][E] assignments of every segment of chunks (whole steps)
+  int32_t* chunk_seg = nullptr;    // [max_segs][E] assignments of every segment of chunks (whole steps of many tokens)
+  int32_t* seg_base = nullptr;     // [max_segs][E] those before the segment in its micro-batch
   int32_t* mb_base = nullptr;      // [EB_MAX_MB][E] first row of every micro-batch in its groups (whole steps)
   int32_t* group_size = nullptr;   // [G_cap]
   int32_t* pgroup = nullptr;       // [G_cap] group at each position of the processing order

@@ -117,7 +117,7 @@ def workspace_regions(step) -> Dict[str, torch.Tensor]:
     chunks = (step.max_tokens + 31) // 32 + 16
     tiles = rows // 256 + gcap
     work = tiles * (-(-step.I // 256) + -(-step.H // 512))
-    sizes = dict(chunk_hist=4 * chunks * E, chunk_base=4 * chunks * E, chunk_seg=4 * (chunks // 32 + 16) * E, mb_base=4 * 16 * E,
+    sizes = dict(chunk_hist=4 * chunks * E, chunk_base=4 * chunks * E, chunk_seg=4 * (chunks // 32 + 16) * E, seg_base=4 * (chunks // 32 + 16) * E, mb_base=4 * 16 * E,
                  group_size=4 * gcap, pgroup=4 * gcap, pslots=4 * gcap, prank=16 * gcap, order=4 * gcap, tile_pref=4 * (gcap + 1),
                  work_count=64, work=32 * work, tile_ready=4 * tiles, slots=8 * 16 * tiles, act=2 * rows * step.I)
     out, off = {}, 0

@@ -93,7 +93,7 @@ def _calls(c, n_mb, tokens):
 
 
 @pytest.mark.parametrize("timing", [0, 1])
-@pytest.mark.parametrize("n_mb,tokens", [(3, 5), (8, 400)])   # the fused permute kernel, and the four it stands for
+@pytest.mark.parametrize("n_mb,tokens", [(3, 5), (8, 400), (1, 4096)])   # the fused permute kernel, the four it stands for, sums of histograms
 def test_nothing_is_launched_behind_a_refused_kernel(lib, n_mb, tokens, timing):
     """Each kernel of a call works from what the one before it wrote: when the runtime refuses one, the call says so and
     launches no further kernel, and the next call starts clean."""

@@ -727,6 +727,10 @@ def test_random_shapes_front_end_bit_exact():
     (256, 8, 3, 5, [31, 32], [1, 1], 0b11, 1, O.POLICY_DIFFPEAK),
     (60, 4, 4, 8, [20] * 16, [j % 3 for j in range(16)], 0xffff, 12, O.POLICY_MAXUTIL),   # pool of sixteen
     (60, 4, 4, 8, [9 + j for j in range(16)], list(range(16)), 0xffff, 1, O.POLICY_MAXUTIL),   # more than 1024 groups
+    (256, 8, 1, 16, [2080, 2048, 2049, 2050], [1, 0, 1, 1], 0b1111, 3, O.POLICY_MAXUTIL),   # more histograms than one block adds up
+    (256, 8, 1, 16, [2016, 2048, 2048, 2048], [1, 0, 1, 1], 0b1011, 2, O.POLICY_CUMUTIL),   # just fewer
+    (7, 2, 1, 3, [2048], [0], 0b1, 1, O.POLICY_ALL),                                  # 64 chunks of one micro-batch, and 65
+    (7, 2, 1, 3, [2049, 5], [0, 1], 0b11, 1, O.POLICY_DIFFPEAK),
     (9, 3, 1, 4, [10] * 11, [0] * 11, 0x7ff, 3, O.POLICY_MAXUTIL),
     (9, 3, 1, 4, [10, 20, 0, 30], [0, 1, 2, 0], 0, 1, O.POLICY_MAXUTIL),              # nothing runs
     (9, 3, 2, 4, [700] * 4, [0, 0, 1, 2], 0b1101, 2, O.POLICY_ALL),                   # pool smaller than the batch
