@@ -12,6 +12,7 @@
 // need the whole GPU to be through: the counts of all tokens, then the positions of all rows.  The counts travel as
 // chunk histograms, which also spares the routing its global atomics.
 #include <algorithm>
+#include <type_traits>
 
 #include "eb_dispatch.cuh"
 #include "eb_route.cuh"
@@ -305,6 +306,7 @@ tables_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ Ba
 
 // ---- scatter ---------------------------------------------------------------------------------
 constexpr int kScatterThreads = 256;
+constexpr int kScatterNarrow = 512;   // elements of a row up to which a block of many takes a whole chunk
 
 struct ScatterArgs {
   const eb_sched_result* res;
@@ -315,12 +317,18 @@ struct ScatterArgs {
   uint4* xp;
   TileList list;
   int fill_blocks;
+  int team;   // threads per token row
 };
 
-// Blocks below fill_blocks write the tile list.  Each of the others places TB tokens of a chunk: one warp ranks the
-// chunk's assignments up to them (a few warp matches) while the others fetch the token rows, then every row goes out
-// to its K + S places.  TB is small while there are few tokens (a block each keeps the chip busy) and 8 when there are
-// many (the ranking is shared by more rows).
+// Blocks below fill_blocks write the tile list.  Each of the others places TB tokens of a chunk: the chunk's assignments up to
+// them are ranked by warp matches while the token rows are on their way, then every row goes out to its K + S places, a team
+// of threads per row.  What bounds it is that chain of two trips to memory and three barriers per block, and the row traffic.
+// TB is small while there are few tokens (a block each keeps the chip busy) and 8 when there are many (ranking and tables are
+// shared by more rows); one warp ranks.  Very many narrow rows take the whole chunk to a block: all warps rank, an assignment
+// per thread, and the teams move several rows at once.  16 x 4096 tokens of 64 elements to 8 places took 109 us with one row at a
+// time and TB = 8, 84 with teams and 29 with the whole chunk (44 for separate rank, gather and fill kernels), 16 x 2048 of 512
+// elements 64 with teams and 46.  Wide rows need the blocks: with 2048 elements, 16 x 512 tokens take 45 us at TB = 8 and 74 at
+// 32, with 1000 and 16 x 2048 both take 90.
 template <int TB>
 __global__ void __launch_bounds__(kScatterThreads)
 scatter_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ BatchParams bp, const __grid_constant__ ScatterArgs a) {
@@ -334,10 +342,13 @@ scatter_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ B
   __shared__ int s_dev_off[EB_MAX_D + 1];
   __shared__ int s_next[EB_MAX_E];
   __shared__ int s_topk[32 * EB_MAX_K];
+  constexpr bool kWide = TB == 32;
+  __shared__ int s_count[kWide ? kScatterThreads / 32 : 1][EB_MAX_E];   // assignments of every expert in each warp
   __shared__ int s_pos[TB][EB_MAX_K + EB_MAX_S];
   static_assert(32 * EB_MAX_K <= kScatterThreads, "a thread per assignment of the chunk");
-  const int tid = threadIdx.x, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int E = mp.E, K = mp.K, S = mp.S, KS = K + S, vec = mp.H / 8;
+  auto expert = [&](int e, int lane) { return (unsigned)e < (unsigned)E ? e : -1 - lane; };   // outside [0, E): equal to no other
   const int part = (int)blockIdx.x - a.fill_blocks, c = part / (32 / TB);
   const int j = mb_of_chunk(bp, c);
   const int c0 = bp.tok_off[j] + (c - bp.chunk_off[j]) * 32;      // first token of the chunk
@@ -349,82 +360,100 @@ scatter_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ B
     for (int i = tid; i < nt * KS; i += kScatterThreads) a.pos[(size_t)t0 * KS + i] = -1;
     return;
   }
+  // a team of threads per token row (one 16-byte column each); team 0 moves rows 0, teams, ..
+  const int teams = kScatterThreads / a.team, team = tid / a.team, col0 = tid % a.team;
   // the first columns of the rows are on their way while the positions are worked out
-  uint4 v[TB];
+  constexpr int P = TB < 8 ? TB : 8;   // rows in flight per thread
+  uint4 v[P];
 #pragma unroll
-  for (int k = 0; k < TB; ++k)
-    if (k < nt && tid < vec) v[k] = __ldg(a.x + (size_t)(t0 + k) * vec + tid);
+  for (int k = 0; k < P; ++k)
+    if (team + k * teams < nt && col0 < vec) v[k] = __ldg(a.x + (size_t)(t0 + team + k * teams) * vec + col0);
   if (tid <= mp.D) s_dev_off[tid] = mp.dev_off[tid];
   // assignments from the start of the chunk to the end of this part
   const int first = (t0 - c0) * K, last = first + nt * K;
   if (tid < last) s_topk[tid] = a.topk_idx[(size_t)c0 * K + tid];
+  if constexpr (kWide)
+    for (int i = tid; i < E; i += kScatterThreads)
+      for (int w = 0; w * 32 < last; ++w) s_count[w][i] = 0;
   const int32_t* seg_base = a.seg_base ? a.seg_base + (size_t)(a.seg.off[j] + (c - bp.chunk_off[j]) / EB_SEG_CHUNKS) * E : nullptr;
-  for (int e = tid; e < E; e += kScatterThreads) s_next[e] = a.mb_base[j * E + e] + a.chunk_base[(size_t)c * E + e] + (seg_base ? seg_base[e] : 0);
+  for (int i = tid; i < E; i += kScatterThreads) s_next[i] = a.mb_base[j * E + i] + a.chunk_base[(size_t)c * E + i] + (seg_base ? seg_base[i] : 0);
   step_shape_block(bp, run, &ss);   // ends with a barrier
-  if (tid < 32) {
-    const int lr = ss.rank_of_mb[j];
+  // an index outside [0, E) is never used: the slot gets no row and the step's meta data counts it
+  auto place = [&](int i, int p) {   // assignment i of the chunk, of this part
+    const int t = c0 + i / K, k = i % K;
+    a.pos[(size_t)t * KS + k] = p;
+    s_pos[t - t0][k] = p;
+    if (p >= 0) a.row_src[p] = t;
+    else atomicAdd(&a.step_meta[EB_META_LEN - 1], 1);
+  };
+  const int ranker = kWide ? kScatterThreads / 32 - 1 : 0;   // the warp that also places the shared slots
+  if constexpr (kWide) {
+    // routed slots, a thread per assignment: the equal ones before it in its warp by a warp match, those of the warps before
+    // it from the counts that each warp leaves
+    const int e = tid < last ? expert(s_topk[tid], lane) : -1 - lane;
+    const unsigned peers = __match_any_sync(0xffffffffu, e);
+    const int before = __popc(peers & ((1u << lane) - 1u));
+    if (e >= 0 && before == 0) s_count[warp][e] = __popc(peers);
+    __syncthreads();
+    if (tid < last) {
+      int p = -1;
+      if (e >= 0) {
+        p = s_next[e] + before;
+        for (int w = 0; w < warp; ++w) p += s_count[w][e];
+      }
+      place(tid, p);
+    }
+  } else if (warp == 0) {
     // routed slots in assignment order from the start of the chunk; the rows of the tokens before this part only count
     for (int a0 = 0; a0 < last; a0 += 32) {
-      const int i = a0 + lane;
-      bool valid = i < last;
-      int e = valid ? s_topk[i] : -1 - lane;   // distinct dummies never match
-      if (valid && (unsigned)e >= (unsigned)E) {
-        // an index outside [0, E) is never used: the slot gets no row and the step's meta data counts it
-        if (i >= first) {
-          a.pos[(size_t)(c0 + i / K) * KS + i % K] = -1;
-          s_pos[(i - first) / K][i % K] = -1;
-          atomicAdd(&a.step_meta[EB_META_LEN - 1], 1);
-        }
-        valid = false;
-        e = -1 - lane;
-      }
+      const int i = a0 + lane, e = i < last ? expert(s_topk[i], lane) : -1 - lane;
       const unsigned peers = __match_any_sync(0xffffffffu, e);
       const int before = __popc(peers & ((1u << lane) - 1u));
-      if (valid && i >= first) {
-        const int p = s_next[e] + before, t = c0 + i / K;
-        a.pos[(size_t)t * KS + i % K] = p;
-        a.row_src[p] = t;
-        s_pos[(i - first) / K][i % K] = p;
-      }
+      if (i >= first && i < last) place(i, e >= 0 ? s_next[e] + before : -1);
       __syncwarp();
-      if (valid && before == 0) s_next[e] += __popc(peers);
+      if (e >= 0 && before == 0) s_next[e] += __popc(peers);
       __syncwarp();
     }
-    // shared slots: closed-form rows
-    if (S > 0 && lane < nt) {
-      const int T = bp.tok_off[j + 1] - bp.tok_off[j], tl = t0 + lane - bp.tok_off[j];
-      const int d = home_device(tl, T, mp.D);
-      int before = 0;
-      for (int j2 = 0; j2 < j; ++j2)
-        if (ss.rank_of_mb[j2] == lr) {
-          const int T2 = bp.tok_off[j2 + 1] - bp.tok_off[j2];
-          before += home_start(d + 1, T2, mp.D) - home_start(d, T2, mp.D);
-        }
-      const int n_d = s_dev_off[d + 1] - s_dev_off[d];
-      const int g = group_id(s_dev_off, S, ss.nl, d, lr, n_d), at = before + (tl - home_start(d, T, mp.D));
-      for (int s = 0; s < S; ++s) {
-        const int p = a.group_off[g + s] + at;
-        a.pos[(size_t)(t0 + lane) * KS + K + s] = p;
-        a.row_src[p] = t0 + lane;
-        s_pos[lane][K + s] = p;
+  }
+  // shared slots: closed-form rows
+  if (S > 0 && warp == ranker && lane < nt) {
+    const int lr = ss.rank_of_mb[j], T = bp.tok_off[j + 1] - bp.tok_off[j], tl = t0 + lane - bp.tok_off[j];
+    const int d = home_device(tl, T, mp.D);
+    int before = 0;
+    for (int j2 = 0; j2 < j; ++j2)
+      if (ss.rank_of_mb[j2] == lr) {
+        const int T2 = bp.tok_off[j2 + 1] - bp.tok_off[j2];
+        before += home_start(d + 1, T2, mp.D) - home_start(d, T2, mp.D);
       }
+    const int n_d = s_dev_off[d + 1] - s_dev_off[d];
+    const int g = group_id(s_dev_off, S, ss.nl, d, lr, n_d), at = before + (tl - home_start(d, T, mp.D));
+    for (int s = 0; s < S; ++s) {
+      const int p = a.group_off[g + s] + at;
+      a.pos[(size_t)(t0 + lane) * KS + K + s] = p;
+      a.row_src[p] = t0 + lane;
+      s_pos[lane][K + s] = p;
     }
   }
   __syncthreads();
-  for (int col = tid; col < vec; col += kScatterThreads) {
-    if (col != tid) {
+  auto move_rows = [&](int row0, auto first) {
+    for (int col = col0; col < vec; col += a.team) {
+      if (!first || col != col0) {
 #pragma unroll
-      for (int k = 0; k < TB; ++k)
-        if (k < nt) v[k] = __ldg(a.x + (size_t)(t0 + k) * vec + col);
+        for (int k = 0; k < P; ++k)
+          if (row0 + k * teams < nt) v[k] = __ldg(a.x + (size_t)(t0 + row0 + k * teams) * vec + col);
+      }
+#pragma unroll
+      for (int k = 0; k < P; ++k)
+        if (row0 + k * teams < nt)
+          for (int s = 0; s < KS; ++s) {
+            const int p = s_pos[row0 + k * teams][s];
+            if (p >= 0) a.xp[(size_t)p * vec + col] = v[k];
+          }
     }
-#pragma unroll
-    for (int k = 0; k < TB; ++k)
-      if (k < nt)
-        for (int s = 0; s < KS; ++s) {
-          const int p = s_pos[k][s];
-          if (p >= 0) a.xp[(size_t)p * vec + col] = v[k];
-        }
-  }
+  };
+  move_rows(team, std::true_type());
+  if constexpr (TB > P)
+    for (int row0 = team + P * teams; row0 < nt; row0 += P * teams) move_rows(row0, std::false_type());
 }
 
 // tables_kernel adds the chunk histograms up itself below this many words (chunks times experts) and up to this many chunks
@@ -443,6 +472,13 @@ constexpr size_t tables_smem(int n_mb, int E, int groups) {
 // the contexts of larger shapes.
 constexpr size_t kTablesSmemMax = tables_smem(EB_MAX_MB, EB_MAX_E, EB_MAX_MB * (EB_MAX_E + EB_MAX_D * EB_MAX_S));
 static_assert(kTablesSmemMax + 16384 <= 232448, "shared memory of one block, the static part within 16 KB");
+
+// Threads that move a row of `vec` 16-byte columns: the power of two that covers them, 8 to the whole block.
+int row_team(int vec) {
+  int t = 8;
+  while (t < vec && t < kScatterThreads) t *= 2;
+  return t;
+}
 
 }  // namespace
 
@@ -477,13 +513,15 @@ eb_status ebi_front_run(eb_ctx* c, cudaStream_t st, const BatchParams& bp, uint3
   {
     KernelTimer timer(c, EBK_PERMUTE_GATHER, st);
     const ScatterArgs a{b->sched, b->topk_idx, c->chunk_base, sums ? c->seg_base : nullptr, c->mb_base, b->group_off, b->group_w, seg, b->pos, b->row_src, b->step_meta,
-                        (const uint4*)b->x, (uint4*)b->xp, tile_list_of(c), c->num_sms / 2};
+                        (const uint4*)b->x, (uint4*)b->xp, tile_list_of(c), c->num_sms / 2, row_team(g.H / 8)};
     const size_t smem = sizeof(int) * (size_t)(ebi_groups_cap(c) + 1);
     auto launch = [&](auto kernel, int tb) {
       return ebi_launch(kernel, dim3(a.fill_blocks + bp.n_chunks * (32 / tb)), dim3(kScatterThreads), smem, st, c->mp, bp, a);
     };
-    EB_LAUNCH(c, "scatter", bp.n_tok <= 2 * c->num_sms ? launch(scatter_kernel<1>, 1) : bp.n_tok <= 16 * c->num_sms ? launch(scatter_kernel<4>, 4)
-                                                                                                              : launch(scatter_kernel<8>, 8));
+    EB_LAUNCH(c, "scatter", bp.n_tok <= 2 * c->num_sms     ? launch(scatter_kernel<1>, 1)
+                            : bp.n_tok <= 16 * c->num_sms  ? launch(scatter_kernel<4>, 4)
+                            : g.H > kScatterNarrow || bp.n_tok <= 64 * c->num_sms ? launch(scatter_kernel<8>, 8)
+                                                                                  : launch(scatter_kernel<32>, 32));
   }
   EB_LAUNCH_CHECK(c, "step front end");
   return EB_OK;
