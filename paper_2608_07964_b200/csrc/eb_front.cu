@@ -12,7 +12,6 @@
 // need the whole GPU to be through: the counts of all tokens, then the positions of all rows.  The counts travel as
 // chunk histograms, which also spares the routing its global atomics.
 #include <algorithm>
-#include <type_traits>
 
 #include "eb_dispatch.cuh"
 #include "eb_route.cuh"
@@ -435,13 +434,14 @@ scatter_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ B
     }
   }
   __syncthreads();
-  auto move_rows = [&](int row0, auto first) {
+  auto move_rows = [&](int row0, bool loaded) {
     for (int col = col0; col < vec; col += a.team) {
-      if (!first || col != col0) {
+      if (!loaded) {
 #pragma unroll
         for (int k = 0; k < P; ++k)
           if (row0 + k * teams < nt) v[k] = __ldg(a.x + (size_t)(t0 + row0 + k * teams) * vec + col);
       }
+      loaded = false;
 #pragma unroll
       for (int k = 0; k < P; ++k)
         if (row0 + k * teams < nt)
@@ -451,9 +451,9 @@ scatter_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ B
           }
     }
   };
-  move_rows(team, std::true_type());
+  move_rows(team, true);
   if constexpr (TB > P)
-    for (int row0 = team + P * teams; row0 < nt; row0 += P * teams) move_rows(row0, std::false_type());
+    for (int row0 = team + P * teams; row0 < nt; row0 += P * teams) move_rows(row0, false);
 }
 
 // tables_kernel adds the chunk histograms up itself below this many words (chunks times experts) and up to this many chunks
