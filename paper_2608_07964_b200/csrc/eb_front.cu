@@ -47,8 +47,9 @@ front_kernel(ModelParams mp, BatchParams bp, uint32_t pool_mask, uint32_t route_
   for (int e = threadIdx.x; e < mp.E; e += kFrontThreads) chunk_hist[(size_t)c * mp.E + e] = s_hist[e];
 }
 
-// Running sum of n values that lie `stride` apart, left before each in `base`; returns the total.  Sixteen loads at a time.
-__device__ __forceinline__ int sum_chunks(const int32_t* __restrict__ h, int32_t* __restrict__ base, int n, int stride) {
+// Running sum of n values that lie `stride` apart, left before each in `base` if `keep`; returns the total.  Sixteen loads at
+// a time.
+__device__ __forceinline__ int sum_chunks(const int32_t* __restrict__ h, int32_t* __restrict__ base, int n, int stride, bool keep) {
   int run = 0;
   for (int k0 = 0; k0 < n; k0 += 16) {
     int v[16];
@@ -56,7 +57,7 @@ __device__ __forceinline__ int sum_chunks(const int32_t* __restrict__ h, int32_t
     for (int k = 0; k < 16; ++k) v[k] = k0 + k < n ? h[(size_t)(k0 + k) * stride] : 0;
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
-      if (k0 + k < n) base[(size_t)(k0 + k) * stride] = run;
+      if (keep && k0 + k < n) base[(size_t)(k0 + k) * stride] = run;
       run += v[k];
     }
   }
@@ -81,7 +82,7 @@ sums_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ Batc
   while (seg.off[j + 1] <= g) ++j;
   if (!((counted >> j) & 1u)) return;
   const int c0 = bp.chunk_off[j] + (g - seg.off[j]) * EB_SEG_CHUNKS;
-  chunk_seg[i] = sum_chunks(chunk_hist + (size_t)c0 * mp.E + e, chunk_base + (size_t)c0 * mp.E + e, min((int)EB_SEG_CHUNKS, bp.chunk_off[j + 1] - c0), mp.E);
+  chunk_seg[i] = sum_chunks(chunk_hist + (size_t)c0 * mp.E + e, chunk_base + (size_t)c0 * mp.E + e, min((int)EB_SEG_CHUNKS, bp.chunk_off[j + 1] - c0), mp.E, true);
 }
 
 // ---- tables ----------------------------------------------------------------------------------
@@ -94,12 +95,14 @@ struct TablesArgs {
   eb_sched_result* res;
   int32_t *group_off, *group_w, *step_meta;
   TilePlan plan;
+  SchedGrid sched;
 };
 
 // i / E for i < 2^16 (E <= 256): one multiplication by ceil(2^32 / E); larger i take the division
 __device__ __forceinline__ int div_by(int i, int E, unsigned magic) { return i < 65536 ? (int)__umulhi((unsigned)i, magic) : i / E; }
 
-// What bounds this kernel is its own chain of phases, a few hundred cycles each at best: every phase has a thread per
+// One block, or several that all work out the loads, share the subsets of a MaxUtil schedule among them and leave the rest to
+// the last one to arrive.  What bounds this kernel is its own chain of phases, a few hundred cycles each at best: every phase has a thread per
 // item of the widest kind ((micro-batch, expert) or (layer, expert)), takes what it needs from shared memory, and
 // decodes nothing by loops or divisions that a table or a multiplication gives.
 __global__ void __launch_bounds__(kSchedThreads)
@@ -123,6 +126,7 @@ tables_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ Ba
   int* const s_ptiles = s_pgroup + g_cap;                                        // [G] its tiles and cost class
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int E = mp.E, S = mp.S, D = mp.D, n_mb = bp.n_mb;
+  const bool first_block = blockIdx.x == 0;
   const unsigned magic = (unsigned)(((1ULL << 32) + E - 1) / E);   // E = 1: wraps to 0, see div_e
   auto div_e = [&](int i) { return E == 1 ? i : div_by(i, E, magic); };
 
@@ -156,10 +160,10 @@ tables_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ Ba
     if ((counted >> j) & 1u) {
       if (a.chunk_seg) {
         const size_t at = (size_t)a.seg.off[j] * E + e;
-        n = sum_chunks(a.chunk_seg + at, a.seg_base + at, a.seg.off[j + 1] - a.seg.off[j], E);
+        n = sum_chunks(a.chunk_seg + at, a.seg_base + at, a.seg.off[j + 1] - a.seg.off[j], E, first_block);
       } else {
         const size_t at = (size_t)bp.chunk_off[j] * E + e;
-        n = sum_chunks(a.chunk_hist + at, a.chunk_base + at, bp.chunk_off[j + 1] - bp.chunk_off[j], E);
+        n = sum_chunks(a.chunk_hist + at, a.chunk_base + at, bp.chunk_off[j + 1] - bp.chunk_off[j], E, first_block);
       }
     }
     s_cnt[i] = n;
@@ -168,7 +172,7 @@ tables_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ Ba
 
   // ---- loads of the micro-batches routed now: four threads per (micro-batch, device)
   for (int i = tid; i < n_mb * E; i += kSchedThreads)
-    if ((a.route_mask >> div_e(i)) & 1u) a.mb_cnt[i] = s_cnt[i];
+    if (first_block && ((a.route_mask >> div_e(i)) & 1u)) a.mb_cnt[i] = s_cnt[i];
   {
     const int j = tid >> 6, d = (tid >> 2) & 15;
     int v = 0;
@@ -178,13 +182,13 @@ tables_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ Ba
     v += __shfl_xor_sync(0xffffffffu, v, 2);
     if ((tid & 3) == 0 && j < n_mb && d < D && ((a.route_mask >> j) & 1u)) {
       sc.load[j][d] = v;
-      a.mb_load[j * D + d] = v;
+      if (first_block) a.mb_load[j * D + d] = v;
     }
   }
   __syncthreads();
 
-  // ---- schedule
-  schedule_block(sc, D, a.pool_mask, a.m, a.policy, 0, 1);
+  // ---- schedule; of several blocks the last one to arrive goes on
+  if (!schedule_grid(sc, D, a.pool_mask, a.m, a.policy, a.sched)) return;
   const uint32_t run = sc.run;
   if (warp == 1) write_schedule(sc, D, a.pool_mask, a.res);
   if (warp == 2 && lane < EB_MAX_MB) s_mbs[lane] = 0;
@@ -465,6 +469,12 @@ scatter_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ B
 constexpr int kSumsWords = 65536;
 constexpr int kSumsChunks = 64;
 
+// tables_kernel runs on several blocks when the others take at least this many subsets of a MaxUtil schedule off the first:
+// below, meeting in memory (1-3 us) costs more than it saves.  Steps on one / several blocks (us, 16 x 1 tokens, 64 experts):
+// pool of 16, m = 12 (2517 subsets) 41.5 / 41.6, m = 8 (39203) 57.0 / 43.6, m = 1 (65535) 67.5 / 44.4; pool of 14 (two blocks),
+// m = 8 (9908) 41.6 / 42.4, m = 6 (14913) 43.8 / 43.3.  256 experts, pool of 16, m = 1: 102.1 / 55.0.
+constexpr int kSchedSubsets = 5000;
+
 constexpr size_t tables_smem(int n_mb, int E, int groups) {
   return sizeof(SchedShared) + sizeof(int) * ((size_t)n_mb * E + 3 * (size_t)groups + 1);
 }
@@ -506,8 +516,11 @@ eb_status ebi_front_run(eb_ctx* c, cudaStream_t st, const BatchParams& bp, uint3
       EB_LAUNCH(c, "sums", ebi_launch(sums_kernel, dim3((seg.off[EB_MAX_MB] * g.E + 255) / 256), dim3(256), 0, st, c->mp, bp, seg, pool_mask | route_mask,
                                       (const int32_t*)c->chunk_hist, c->chunk_base, c->chunk_seg));
     const TablesArgs a{pool_mask, route_mask, (int)m, (int)policy, c->chunk_hist, sums ? c->chunk_seg : nullptr, c->chunk_base, c->seg_base,
-                       c->mb_base, b->mb_load, b->mb_cnt, seg, b->sched, b->group_off, b->group_w, b->step_meta, tile_plan_of(c)};
-    EB_LAUNCH(c, "tables", ebi_launch(tables_kernel, dim3(1), dim3(kSchedThreads), tables_smem(bp.n_mb, g.E, bp.n_mb * (g.E + g.D * g.S)), st,
+                       c->mb_base, b->mb_load, b->mb_cnt, seg, b->sched, b->group_off, b->group_w, b->step_meta, tile_plan_of(c),
+                       sched_grid_of(c)};
+    int blocks = sched_blocks(pool_mask, m, policy);
+    if ((int64_t)sched_subsets(pool_mask, m) * (blocks - 1) / blocks < kSchedSubsets) blocks = 1;
+    EB_LAUNCH(c, "tables", ebi_launch(tables_kernel, dim3(blocks), dim3(kSchedThreads), tables_smem(bp.n_mb, g.E, bp.n_mb * (g.E + g.D * g.S)), st,
                                       c->mp, bp, a));
   }
   {

@@ -134,6 +134,7 @@ struct SchedShared {
   int member[EB_MAX_MB];                                   // micro-batch of every pool position
   Cand best[kSchedThreads / 32];
   uint32_t run;
+  bool last;                                               // this block is the last one of the grid to arrive
   long long seq_w[EB_MAX_D];
 };
 
@@ -325,6 +326,61 @@ __device__ __forceinline__ bool schedule_block(SchedShared& s, int D, uint32_t p
   }
   __syncthreads();
   return true;
+}
+
+// schedule_block by all blocks of the grid: each leaves its best candidate in global memory and the block that arrives last
+// goes on with the choice among them.  False: this block is done.  The counter is ready for the next launch again.
+struct SchedGrid {
+  Cand* best;          // [gridDim.x]
+  unsigned* arrived;
+};
+__device__ __forceinline__ bool schedule_grid(SchedShared& s, int D, uint32_t pool_mask, int m, int policy, const SchedGrid& g) {
+  if (schedule_block(s, D, pool_mask, m, policy, blockIdx.x, gridDim.x)) return gridDim.x == 1 || blockIdx.x == 0;
+  const int tid = threadIdx.x;
+  if (tid == 0) {
+    g.best[blockIdx.x] = s.best[0];
+    __threadfence();
+    s.last = atomicAdd(g.arrived, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s.last) return false;
+  __threadfence();
+  if (tid < 32) {
+    Cand b;
+    b.n = -1; b.num = 0; b.peak = 1; b.sub = 0;
+    for (int i = tid; i < (int)gridDim.x; i += 32) {
+      const Cand o = g.best[i];
+      if (better(o, b)) b = o;
+    }
+    b = warp_best(b);
+    const uint32_t mask = run_mask_of(s.member, __popc(pool_mask), b);
+    if (tid == 0) {
+      s.run = mask;
+      *g.arrived = 0;
+    }
+  }
+  __syncthreads();
+  return true;
+}
+
+// Blocks for a schedule: MaxUtil over a pool of more than 13 takes one per 32 high halves of its subsets.
+constexpr int kMaxSchedBlocks = 1 << (EB_MAX_MB - 13);
+inline int sched_blocks(uint32_t pool_mask, int m, int policy) {
+  const int np = __builtin_popcount(pool_mask);
+  return policy == EB_POLICY_MAXUTIL && np > m && np > 13 ? 1 << (np - 13) : 1;
+}
+// Subsets that MaxUtil looks at: those of at least m members.
+inline int sched_subsets(uint32_t pool_mask, int m) {
+  const int np = __builtin_popcount(pool_mask);
+  int total = 0, c = 1;   // c: n out of np
+  for (int n = 0; n <= np; ++n) {
+    if (n >= m) total += c;
+    c = c * (np - n) / (n + 1);
+  }
+  return total;
+}
+inline SchedGrid sched_grid_of(const eb_ctx* c) {
+  return SchedGrid{(Cand*)c->d_sched_scratch, (unsigned*)(c->d_sched_scratch + kMaxSchedBlocks * sizeof(Cand))};
 }
 
 // The result record, by one warp, s.run final.

@@ -729,6 +729,9 @@ def test_random_shapes_front_end_bit_exact():
     (60, 4, 4, 8, [9 + j for j in range(16)], list(range(16)), 0xffff, 1, O.POLICY_MAXUTIL),   # more than 1024 groups
     (256, 8, 1, 16, [2080, 2048, 2049, 2050], [1, 0, 1, 1], 0b1111, 3, O.POLICY_MAXUTIL),   # more histograms than one block adds up
     (256, 8, 1, 16, [2016, 2048, 2048, 2048], [1, 0, 1, 1], 0b1011, 2, O.POLICY_CUMUTIL),   # just fewer
+    (60, 4, 4, 8, [7] * 16, [j % 5 for j in range(16)], 0xfeff, 5, O.POLICY_MAXUTIL),     # fifteen of sixteen, on four blocks
+    (9, 3, 0, 4, [5] * 16, [0] * 16, 0x7ff7, 6, O.POLICY_MAXUTIL),                    # fourteen, on two; many ties
+    (256, 8, 1, 16, [512] * 16, [j % 2 for j in range(16)], 0xffff, 4, O.POLICY_MAXUTIL), # eight blocks, histograms summed before
     (7, 2, 1, 3, [2048], [0], 0b1, 1, O.POLICY_ALL),                                  # 64 chunks of one micro-batch, and 65
     (7, 2, 1, 3, [2049, 5], [0, 1], 0b11, 1, O.POLICY_DIFFPEAK),
     (9, 3, 1, 4, [10] * 11, [0] * 11, 0x7ff, 3, O.POLICY_MAXUTIL),
@@ -736,7 +739,7 @@ def test_random_shapes_front_end_bit_exact():
     (9, 3, 2, 4, [700] * 4, [0, 0, 1, 2], 0b1101, 2, O.POLICY_ALL),                   # pool smaller than the batch
 ])
 def test_whole_step_front_end_bit_exact(E, K, S, D, tokens, layers, pool, m, policy):
-    """eb_step makes routing, schedule, group tables, positions and rows in three kernels of its own; bit for bit against
+    """eb_step makes routing, schedule, group tables, positions and rows in kernels of its own; bit for bit against
     the oracle, then again with a route mask: the micro-batches outside it keep their routing although their logits
     have changed, as in the five calls."""
     B = _binding()
