@@ -20,31 +20,17 @@
 
 namespace {
 
-constexpr int kFrontThreads = 1024;   // a warp per token of the chunk
-
-// PL: logits per lane.  With two (E <= 64) the registers leave room for two blocks per SM.
 template <int PL>
-__global__ void __launch_bounds__(kFrontThreads, PL <= 2 ? 2 : 1)
+__global__ void __launch_bounds__(kChunkThreads, PL <= 2 ? 2 : 1)
 front_kernel(ModelParams mp, BatchParams bp, uint32_t pool_mask, uint32_t route_mask, const float* __restrict__ logits,
              int32_t* __restrict__ topk_idx, float* __restrict__ topk_w, int32_t* __restrict__ chunk_hist) {
   EB_GRID_DEP_SYNC();
   __shared__ int s_hist[EB_MAX_E];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c = blockIdx.x, j = mb_of_chunk(bp, c);
   const bool routed = (route_mask >> j) & 1u;
   if (!routed && !((pool_mask >> j) & 1u)) return;
-  for (int e = threadIdx.x; e < mp.E; e += kFrontThreads) s_hist[e] = 0;
-  __syncthreads();
-  const int t = bp.tok_off[j] + (c - bp.chunk_off[j]) * 32 + warp;
-  if (t < bp.tok_off[j + 1]) {
-    int e = -1;
-    if (routed) e = route_token<PL>(mp, t, lane, logits, topk_idx, topk_w);
-    else if (lane < mp.K) e = topk_idx[(size_t)t * mp.K + lane];   // deferred: routed when it reached its layer
-    // an index outside [0, E) (only in a table not written by the routing) is skipped here and reported by scatter_kernel
-    if (lane < mp.K && (unsigned)e < (unsigned)mp.E) atomicAdd(&s_hist[e], 1);
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < mp.E; e += kFrontThreads) chunk_hist[(size_t)c * mp.E + e] = s_hist[e];
+  route_chunk<PL>(mp, bp, c, j, routed, logits, topk_idx, topk_w, s_hist);
+  for (int e = threadIdx.x; e < mp.E; e += kChunkThreads) chunk_hist[(size_t)c * mp.E + e] = s_hist[e];
 }
 
 // Running sum of n values that lie `stride` apart, left before each in `base` if `keep`; returns the total.  Sixteen loads at
@@ -501,7 +487,7 @@ eb_status ebi_front_run(eb_ctx* c, cudaStream_t st, const BatchParams& bp, uint3
   }
   if (bp.n_chunks > 0) {
     KernelTimer timer(c, EBK_ROUTE, st);
-    EB_LAUNCH(c, "front", ebi_launch(g.E <= 64 ? front_kernel<2> : front_kernel<kMaxPerLane>, dim3(bp.n_chunks), dim3(kFrontThreads), 0, st, c->mp, bp,
+    EB_LAUNCH(c, "front", ebi_launch(g.E <= 64 ? front_kernel<2> : front_kernel<kMaxPerLane>, dim3(bp.n_chunks), dim3(kChunkThreads), 0, st, c->mp, bp,
                                      pool_mask, route_mask, (const float*)b->logits, b->topk_idx, b->topk_w, c->chunk_hist));
   }
   Segments seg;

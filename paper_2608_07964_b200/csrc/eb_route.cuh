@@ -4,7 +4,7 @@
 // round is two warp reductions (redux) instead of ten shuffles.
 #pragma once
 
-#include "eb_internal.cuh"
+#include "eb_dispatch.cuh"
 
 namespace {
 
@@ -70,6 +70,27 @@ __device__ __forceinline__ int route_token(const ModelParams& mp, int t, int lan
     topk_w[(size_t)t * K + lane] = my_p / p_sum;
   }
   return my_e;
+}
+
+constexpr int kChunkThreads = 1024;   // a warp per token of a chunk.  With PL = 2 (E <= 64) the registers leave room for two blocks per SM
+
+// Chunk c of micro-batch j by one block: its tokens are routed (or keep their routing), s_hist [E] gets their assignments per
+// expert.  Ends with a block barrier.
+template <int PL>
+__device__ __forceinline__ void route_chunk(const ModelParams& mp, const BatchParams& bp, int c, int j, bool routed, const float* __restrict__ logits,
+                                            int32_t* __restrict__ topk_idx, float* __restrict__ topk_w, int* s_hist) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int e = threadIdx.x; e < mp.E; e += kChunkThreads) s_hist[e] = 0;
+  __syncthreads();
+  const int t = bp.tok_off[j] + (c - bp.chunk_off[j]) * 32 + warp;
+  if (t < bp.tok_off[j + 1]) {
+    int e = -1;
+    if (routed) e = route_token<PL>(mp, t, lane, logits, topk_idx, topk_w);
+    else if (lane < mp.K) e = topk_idx[(size_t)t * mp.K + lane];   // deferred: routed when it reached its layer
+    // an index outside [0, E) (only in a table not written by the routing) is skipped here and reported by the dispatch
+    if (lane < mp.K && (unsigned)e < (unsigned)mp.E) atomicAdd(&s_hist[e], 1);
+  }
+  __syncthreads();
 }
 
 }  // namespace
