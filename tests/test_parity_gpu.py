@@ -509,22 +509,25 @@ def test_tile_sizes_mixed_over_many_tiles_per_pair(H, I):
 @pytest.mark.parametrize("tokens,H,I", [([1], 64, 64), ([40, 300, 7], 264, 520), ([900, 900, 900], 512, 1288)])
 def test_one_launch_for_both_phases_equals_a_launch_each(tokens, H, I):
     """With per-kernel timing on, the gate/up and the down tiles go out as two launches; otherwise as one, in which the
-    down tiles wait for the rows they need.  Fewer tiles than CTA pairs, a few per pair, many per pair: same bits."""
+    down tiles wait for the rows they need.  Fewer tiles than CTA pairs, a few per pair, many per pair: the bits that were
+    compared with the oracle.  The intermediate is filled with NaN before every pass, so that a row read before it is
+    written shows up in the outputs."""
     B = _binding()
     wl = _small(L=2, E=12, K=3, S=1, D=4, N=len(tokens), T=max(tokens), H=H, I=I, mapping="mod")
     case, store = Hn.make_case(wl, tokens, [j % 2 for j in range(len(tokens))]), Hn.WeightStore(wl)
     step, _ = _full_step(case, store, len(tokens))
     rows = step.meta()["rows"]
     batch = B.Batch(case.tok_off, case.layers)
-    got = []
-    for timed in (True, False, False, True):
+    want = step.yp[:rows].clone()     # of _full_step: within the bar of the oracle's
+    act = Hn.workspace_regions(step)["act"]
+    for timed in (True, False, False, False, False, True, False):
         step.set_timing(timed)
-        step.yp.zero_()
+        step.yp.fill_(-7.0)
+        act.fill_(0xFF)
         step.eb_step(batch, len(tokens))
-        got.append(step.yp[:rows].clone())
+        assert torch.equal(step.yp[:rows], want), timed
     step.set_timing(False)
     assert step.device_status() == 0 and step.check_workspace_guards() == 0
-    assert all(torch.equal(got[0], g) for g in got[1:])
 
 
 @pytest.mark.parametrize("S,D,tokens,layers", [
@@ -732,6 +735,8 @@ def test_random_shapes_front_end_bit_exact():
     (60, 4, 4, 8, [7] * 16, [j % 5 for j in range(16)], 0xfeff, 5, O.POLICY_MAXUTIL),     # fifteen of sixteen, on four blocks
     (9, 3, 0, 4, [5] * 16, [0] * 16, 0x7ff7, 6, O.POLICY_MAXUTIL),                    # fourteen, on two; many ties
     (256, 8, 1, 16, [512] * 16, [j % 2 for j in range(16)], 0xffff, 4, O.POLICY_MAXUTIL), # eight blocks, histograms summed before
+    (6, 2, 2, 4, [70, 290, 3, 700], [1, 0, 2, 1], 0b1111, 4, O.POLICY_MAXUTIL),       # replicas of 1, 73 and 193 rows, merged or a tile each
+    (6, 2, 1, 2, [1100, 560, 40], [0, 1, 0], 0b111, 3, O.POLICY_MAXUTIL),             # replicas of 570 and 280 rows: several tiles each
     (7, 2, 1, 3, [2048], [0], 0b1, 1, O.POLICY_ALL),                                  # 64 chunks of one micro-batch, and 65
     (7, 2, 1, 3, [2049, 5], [0, 1], 0b11, 1, O.POLICY_DIFFPEAK),
     (9, 3, 1, 4, [10] * 11, [0] * 11, 0x7ff, 3, O.POLICY_MAXUTIL),
@@ -741,7 +746,7 @@ def test_random_shapes_front_end_bit_exact():
 def test_whole_step_front_end_bit_exact(E, K, S, D, tokens, layers, pool, m, policy):
     """eb_step makes routing, schedule, group tables, positions and rows in kernels of its own; bit for bit against
     the oracle, then again with a route mask: the micro-batches outside it keep their routing although their logits
-    have changed, as in the five calls."""
+    have changed, as in the five calls.  Its tile list is the one that the expert pass alone makes, and so are its outputs."""
     B = _binding()
     wl = _small(L=max(layers) + 1, E=E, K=K, S=S, D=D, N=len(tokens), T=max(tokens), H=72, I=64, mapping="mod")
     case, store = Hn.make_case(wl, tokens, layers), Hn.WeightStore(wl)
@@ -751,9 +756,15 @@ def test_whole_step_front_end_bit_exact(E, K, S, D, tokens, layers, pool, m, pol
     step.logits[:T].copy_(case.logits)
     step.x[:T].copy_(case.x)
     batch = B.Batch(case.tok_off, layers, pool)
+    step.yp.fill_(-7.0)
     step.eb_step(batch, m, policy)
     ref = Hn.oracle_front(case, pool, m, policy)
     Hn.check_front(step, case, ref, n)
+    R, tiles, yp = int(ref["group_off"][-1]), Hn.tile_list(step), step.yp.clone()
+    step.yp.fill_(-7.0)
+    step.eb_expert_ffn_grouped()
+    assert np.array_equal(Hn.tile_list(step), tiles) and torch.equal(step.yp, yp)
+    assert bool((yp[R:] == -7.0).all()) and bool((yp[:R] != -7.0).any(dim=1).all())
     assert step.check_permutation(batch) == 0 and step.check_workspace_guards() == 0 and step.device_status() == 0
     keep = 0b0110 & ((1 << n) - 1)
     fresh = Hn.make_case(wl, tokens, layers).logits.roll(1, dims=1)
