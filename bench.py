@@ -34,8 +34,9 @@ from paper_2608_07964_b200 import synth  # noqa: E402
 
 METRIC = "cross-layer MoE step tokens/s"
 UNIT = "tokens/s"
-# Kernels per step: route, schedule, permute (one fused kernel or four, plus the gather), expert pass 4 (plan, fill,
-# gate/up, down), combine 1.  bench counts them from the library's own launch counter.
+# Kernels per step: front (and sums for many tokens), tables, scatter, expert pass, combine.  bench counts them from the
+# library's own launch counter.  With per-kernel timing on the expert pass goes out as one launch per phase: the per-launch
+# figures are of those two launches of the same kernel, the step figures of the one.
 
 # DRAM traffic of the dominant kernel (ffn gate/up) from an ncu capture: (dram__bytes_read.sum +
 # dram__bytes_write.sum) over the algorithmic bytes of the captured launch.  The captures ran on cut-down cases
@@ -507,8 +508,9 @@ def run_ours(args, wl):
     if res["sustained"]:
         su = res["sustained"]
         flops = res["alg"]["gateup_flops"] + res["alg"]["down_flops"]
-        # share of the step the two expert launches take in the K-step run (their event times over the step time)
-        share = min(1.0, (res["kern_ms"].get("ffn_gateup", 0.0) + res["kern_ms"].get("ffn_down", 0.0)) / ms_step)
+        # share of the expert pass in the step: of the sum of all kernels' event times, those of its two launches
+        times = {k: v for k, v in res["kern_ms"].items() if v > 0}
+        share = (times["ffn_gateup"] + times["ffn_down"]) / sum(times.values())
         su["tokens_per_s"] = res["tokens_run"] / (su["ms_per_step"] / 1e3)
         # expert pass of the settled loop (same share of the step) against the sustained GEMM peak
         su["expert_pass_tflops"] = flops / (su["ms_per_step"] * share / 1e3) / 1e12

@@ -266,7 +266,7 @@ class MoEStep:
     # -- whole step ----------------------------------------------------------------------------
     def eb_step(self, batch: Batch, m: int, policy: int = POLICY_MAXUTIL, route_mask: Optional[int] = None,
                 in_place: bool = False):
-        """The five calls back to back.  With `in_place` the hidden states self.x take x + MoE(x) for the chosen
+        """What the five calls compute, in five or six launches.  With `in_place` the hidden states self.x take x + MoE(x) for the chosen
         micro-batches (the aggregation adds the residual and writes over x); otherwise the MoE output goes to self.out."""
         rm = ((1 << batch.n_mb) - 1) if route_mask is None else route_mask
         bufs = self.bufs_inplace if in_place else self.bufs

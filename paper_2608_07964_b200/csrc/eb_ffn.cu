@@ -17,7 +17,7 @@
 //            (256 outputs per tile);
 //   down   : W0, W1 = two consecutive 256-row blocks of W_down (512 outputs per tile).
 // Per CTA: warp 0 = TMA producer (its own 128 rows of W0 and W1 and its half of the token rows), warp 1 =
-// MMA issuer (leader CTA only) and TMEM owner, warps 2..9 = epilogue.  A stage is 48 KB per CTA (W0 | W1 |
+// MMA issuer (leader CTA only) and TMEM owner, warps 2..9 = epilogue, warp 10 = publisher of finished rows.  A stage is 48 KB per CTA (W0 | W1 |
 // up to 128 token rows of one 64-wide k-block, bf16, 128-byte swizzled K-major) for up to 1024 tensor-core
 // cycles; four stages.  TMA completions of both CTAs count on the leader's barrier; the tcgen05.commit
 // that frees a stage is delivered to both CTAs; no load is multicast.
@@ -34,7 +34,7 @@
 // The accumulator holds outputs in lanes and tokens in columns: an epilogue warp transposes each 16-token
 // chunk through 1 KB of shared memory and stores 16-byte vectors.
 //
-// Tiles: a device-built list (plan_kernel, fill_kernel).  Tiles of one group are weight-tile-major and
+// Tiles: a device-built list (eb_tiles.cuh).  Tiles of one group are weight-tile-major and
 // token-tile-minor, so pairs working side by side share the weight tile in L2 and every weight byte leaves
 // HBM once per group.  The D replicas of a shared expert (one group per virtual device, all reading the
 // same matrix) are merged when all are small: their rows are packed into common tiles in slots of 16
@@ -63,16 +63,17 @@ constexpr int kTBytes = 128 * BK * 2;                          // up to 128 toke
 constexpr int kStageBytes = 2 * kWBytes + kTBytes;             // W0 | W1 | token rows
 constexpr int kRingBytes = kStages * kStageBytes;
 constexpr int kEpiWarps = 8;                                   // two per TMEM lane quadrant
-constexpr int kThreads = 64 + 32 * kEpiWarps;
+constexpr int kThreads = 96 + 32 * kEpiWarps;
 constexpr int kChunkStep = 16 * (kEpiWarps / 4);               // columns between two chunks of an epilogue warp
-constexpr size_t kSmemBytes = (size_t)kRingBytes + 1024 /*alignment slack*/ + 256 /*barriers*/ + kEpiWarps * 1024 /*transposes*/;
+constexpr size_t kSmemBytes = (size_t)kRingBytes + 1024 /*alignment slack*/ + 512 /*barriers*/ + kEpiWarps * 1024 /*transposes*/;
 static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
 constexpr int kTmemCols = 512;
 constexpr int kTmemHalf = 256;                                 // a narrow tile's two accumulators share one half of TMEM
 constexpr int kNarrowCols = kTmemHalf / 2;                     // ... which takes tiles of up to 128 columns
 constexpr int kItems = 2;                                      // mailbox slots of a CTA (tiles dealt ahead)
 constexpr int kParts = 4;                                      // tiles whose epilogues may be under way at once in a CTA: a tile is dealt
-                                                               // only when every warp has begun the one kItems before it, so at most kItems + 1
+                                                               // only when every reader has taken the one kItems before it, so at most kItems + 1
+static_assert(kParts > kItems, "a barrier of the publisher is free again before it comes round");
 constexpr int kAskAhead = 16;                                  // k-blocks before the end of a tile at which its successor is asked for
 constexpr long long kSpinLimitCycles = 4000000000LL;
 
@@ -155,7 +156,11 @@ __device__ __forceinline__ void cluster_sync_all() {
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
-// The same with what this thread wrote before it.  Only the tile dealer uses it: a release at cluster scope waits for
+// Hands what the warp wrote to a thread of the same CTA.
+__device__ __forceinline__ void mbar_arrive_release(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// The same as mbar_arrive_cluster with what this thread wrote before it.  Only the tile dealer uses it: a release at cluster scope waits for
 // the thread's earlier accesses, and in the producer, MMA and epilogue warps that cost 1 to 2 us per tile.
 __device__ __forceinline__ void mbar_arrive_release_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
@@ -432,11 +437,12 @@ ffn_kernel(const __grid_constant__ FfnParams p) {
   auto item_full = [&](int i) { return bar0 + 8u * (2 * NS + 4 + i); };
   auto item_empty = [&](int i) { return bar0 + 8u * (2 * NS + 4 + kItems + i); };
   const uint32_t want_bar = bar0 + 8u * (2 * NS + 4 + 2 * kItems);
-  constexpr int kBarBytes = 8 * (2 * NS + 4 + 2 * kItems + 1);
-  static_assert(kBarBytes + 8 + 4 * kParts <= 192 && kItems * sizeof(Tile) <= 64, "256 bytes of barriers and mailbox");
+  auto part_bar = [&](int i) { return bar0 + 8u * (2 * NS + 4 + 2 * kItems + 1 + i); };
+  constexpr int kBarBytes = 8 * (2 * NS + 4 + 2 * kItems + 1 + kParts), kMailbox = 512 - kItems * (int)sizeof(Tile);
+  static_assert(kBarBytes + 8 <= kMailbox, "512 bytes of barriers and mailbox");
   volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(smem + kRingBytes + kBarBytes);
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + kRingBytes + kBarBytes + 4);
-  const uint32_t items = bar0 + 192;
+  const uint32_t items = bar0 + kMailbox;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();   // CTA 0 of a pair is the leader
@@ -452,11 +458,11 @@ ffn_kernel(const __grid_constant__ FfnParams p) {
     }
     for (int i = 0; i < kItems; ++i) {
       mbar_init(item_full(i), 1);                        // the dealer's arrive
-      mbar_init(item_empty(i), 3 + 2 * kEpiWarps);       // every reader of both CTAs (CTA 1's barrier)
+      mbar_init(item_empty(i), 5 + 2 * kEpiWarps);       // every reader of both CTAs (CTA 1's barrier)
     }
+    for (int i = 0; i < kParts; ++i) mbar_init(part_bar(i), kEpiWarps);   // one arrival per epilogue warp of the CTA
     mbar_init(want_bar, 1);                              // the leader's producer (CTA 1's barrier)
     *s_abort = 0;
-    for (int i = 0; i < kParts; ++i) reinterpret_cast<int*>(smem + kRingBytes + kBarBytes + 8)[i] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 2 && lane < kMaps) prefetch_tmap(&p.xp.box[0] + lane);
@@ -723,13 +729,33 @@ ffn_kernel(const __grid_constant__ FfnParams p) {
         if (idx >= part_end) break;
       }
     }
+  } else if (warp == 2 + kEpiWarps) {
+    if (lane == 0) {
+      // ---------------- publisher: counts the CTA's share of a finished gate/up tile on its token tile ----------------
+      // The down tiles of these rows wait for all shares.  The epilogue warps' stores are ordered before the TMA reads of
+      // whoever sees the count.  A thread of its own, since the fence waits for those stores: in the CTA's last epilogue warp it
+      // held up the next tile's epilogue, 98 instead of 89 us at 49152 rows over 132 matrices of 3 x 256 x 512.
+      uint32_t uses = 0;   // bit i: phase parity of the next use of part_bar(i)
+      for (int seq = 0;; ++seq) {
+        Tile it;
+        if (!take_item(seq, &it)) goto done;
+        if (it.w < 0) break;
+        free_item(seq);
+        if (it.phase != 1) continue;
+        const int i = seq % kParts;
+        if (!mbar_wait(part_bar(i), (uses >> i) & 1u, s_abort, status)) goto done;
+        uses ^= 1u << i;
+        __threadfence();
+        fence_proxy_async();
+        red_release(p.ready + it.done);
+      }
+    }
   } else {
     // ---------------- epilogue warps ----------------
     const int q = warp & 3;                      // TMEM lane quadrant this warp may read
     const int chunk0 = ((warp - 2) >> 2) * 16;   // the warps of a quadrant take 16-column chunks in turn
     const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16);
-    bf16* tile = reinterpret_cast<bf16*>(smem + kRingBytes + 256) + (warp - 2) * 512;   // 1 KB per epilogue warp
-    int* parts = reinterpret_cast<int*>(smem + kRingBytes + kBarBytes + 8);
+    bf16* tile = reinterpret_cast<bf16*>(smem + kRingBytes + 512) + (warp - 2) * 512;   // 1 KB per epilogue warp
     TmemTurn turn;
     for (int seq = 0;; ++seq) {
       // one lane waits, the outcome is made warp-uniform before any .aligned instruction
@@ -770,18 +796,9 @@ ffn_kernel(const __grid_constant__ FfnParams p) {
       };
       if (it.phase == 1) {
         run(std::integral_constant<int, 1>(), p.act_out, p.I);
-        // this warp's part of the intermediate is written; the CTA's last warp counts it on the token tile, whose down
-        // tiles wait for all parts.  The stores are ordered before the TMA reads of whoever sees the count.
+        // this warp's part of the intermediate is written: the publisher counts the CTA's share of the tile
         __syncwarp();
-        if (lane == 0) {
-          __threadfence_block();
-          if (atomicAdd(&parts[seq % kParts], 1) == kEpiWarps - 1) {
-            parts[seq % kParts] = 0;
-            __threadfence();
-            fence_proxy_async();
-            red_release(p.ready + it.done);
-          }
-        }
+        if (lane == 0) mbar_arrive_release(part_bar(seq % kParts));
       } else {
         run(std::integral_constant<int, 2>(), p.yp, p.H);
       }

@@ -4,8 +4,8 @@
 step routes the micro-batches that just advanced (eb_route with a route mask, so deferred ones
 keep their routing), schedules (eb_schedule, result copied to the host to advance the layer
 counters) and records the run set and the joint per-device load; the expert pass is skipped.
-`run_full` does the same but executes every step completely (eb_step: the five calls, the last one adding
-the residual h <- h + MLP(h) in place), optionally replaying each step from a CUDA graph.
+`run_full` does the same but executes every step completely (eb_step: what the five calls compute, the aggregation
+adding the residual h <- h + MLP(h) in place), optionally replaying each step from a CUDA graph.
 
 Logits of (micro-batch j, layer l) come from a caller-supplied function, so the loop itself holds
 no routing or scheduling arithmetic: those run in the CUDA kernels.
@@ -75,7 +75,7 @@ class StepGraphs:
     """CUDA graphs of whole steps, one per distinct (pool, layers, route mask, m, policy): a step's launches are
     fixed by those host-side values (which micro-batches run is read from device memory by the kernels), so a
     state that comes up again - the same schedule trajectory on the next batch - is replayed as one graph
-    launch instead of about a dozen kernel launches."""
+    launch instead of five or six kernel launches."""
 
     def __init__(self, step: "B.MoEStep", tok_off: List[int], capacity: int = 256):
         self.step, self.tok_off, self.capacity = step, list(tok_off), capacity
