@@ -6,7 +6,8 @@
 // in flight together), accumulates in fp32 in the
 // fixed order k = 0..K-1 then s = 0..S-1, and stores bf16 (round to nearest even).  Gather form
 // means no atomics and a result that does not depend on scheduling.  The expert-output rows are read once, so
-// they leave L2 first (streaming loads): 226 MB took 48 us instead of 54 between its neighbours.
+// they leave L2 first (streaming loads): a step that moves 226 MB here (6144 tokens of 2048 elements from 8 places) took
+// 268 us instead of 277, steps whose rows fit L2 the same.
 #include <utility>
 
 #include "eb_internal.cuh"

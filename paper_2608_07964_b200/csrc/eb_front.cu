@@ -495,7 +495,7 @@ eb_status ebi_front_run(eb_ctx* c, cudaStream_t st, const BatchParams& bp, uint3
   for (int j = 0; j < EB_MAX_MB; ++j) seg.off[j + 1] = seg.off[j] + (bp.chunk_off[j + 1] - bp.chunk_off[j] + EB_SEG_CHUNKS - 1) / EB_SEG_CHUNKS;
   int longest = 0;
   for (int j = 0; j < bp.n_mb; ++j) longest = std::max(longest, bp.chunk_off[j + 1] - bp.chunk_off[j]);
-  const bool sums = bp.n_chunks * g.E >= kSumsWords || longest > kSumsChunks;
+  const bool sums = (int64_t)bp.n_chunks * g.E >= kSumsWords || longest > kSumsChunks;
   {
     KernelTimer timer(c, EBK_SCHEDULE, st);
     if (sums)
