@@ -41,22 +41,14 @@ def run_load_trace(step: "B.MoEStep", tok_off: List[int], L: int, m: int, policy
     route_mask = pool
     steps: List[Dict] = []
     rows = _logit_rows(step, tok_off)
-    # the schedule and the loads come back in pinned memory behind one synchronisation
-    h_load = torch.empty((N, step.D), dtype=torch.int32).pin_memory()
-    h_sched = torch.empty_like(step.sched, device="cpu").pin_memory()
-    stream = torch.cuda.current_stream(step.dev)
     while pool:
         _copy_logits(rows, logits_of, layer, route_mask)
         batch = B.Batch(tok_off, [min(l, L - 1) for l in layer], pool)
         if route_mask:
             step.eb_route(batch, route_mask)
-        step.eb_schedule(batch, m, policy)
-        h_load.copy_(step.mb_load[:N], non_blocking=True)
-        h_sched.copy_(step.sched, non_blocking=True)
-        stream.synchronize()
-        res = step.sched_result(h_sched)
+        res = step.eb_schedule(batch, m, policy, to_host=True)
         run = res["run_mask"]
-        loads = h_load.tolist()
+        loads = step.mb_load[:N].cpu().tolist()
         steps.append(dict(pool=pool, run_mask=run, layers={j: layer[j] for j in range(N) if (run >> j) & 1},
                           joint_load=res["joint_load"], util_num=res["util_num"], util_den=res["util_den"],
                           member_loads={j: loads[j] for j in range(N) if (run >> j) & 1}))
