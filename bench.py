@@ -41,10 +41,10 @@ UNIT = "tokens/s"
 # DRAM traffic of the dominant kernel (ffn gate/up) from an ncu capture: (dram__bytes_read.sum +
 # dram__bytes_write.sum) over the algorithmic bytes of the captured launch.  The captures ran on cut-down cases
 # of the same shapes (a full-size capture would hold tens of GB); traffic grows in proportion to the weight
-# bytes streamed, so a full launch is that ratio times its own algorithmic bytes.
-NCU_TRAFFIC_RATIO = {"c4": 4.093019 / 3.909091, "c4small": 4.093019 / 3.909091,          # captured on c4small
-                     "c2": 1.495264 / 1.487012, "c2small": 1.495264 / 1.487012,          # captured on c2small
-                     "c3init": 1.170937 / 1.101005, "c3initsmall": 1.170937 / 1.101005}  # captured on c3initsmall
+# bytes streamed, so a full launch is that ratio times its own algorithmic bytes.  (profiles/expert_pass_traffic.md)
+NCU_TRAFFIC_RATIO = {"c4": 4.061304 / 3.909091, "c4small": 4.061304 / 3.909091,          # captured on c4small
+                     "c2": 1.486126 / 1.487012, "c2small": 1.486126 / 1.487012,          # captured on c2small
+                     "c3init": 1.121521 / 1.101005, "c3initsmall": 1.121521 / 1.101005}  # captured on c3initsmall
 
 
 def measured_peaks():
