@@ -72,12 +72,21 @@ sums_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ Batc
 }
 
 // ---- tables ----------------------------------------------------------------------------------
+// The distinct layers of a batch, ascending.
+struct StepLayers {
+  int n;
+  int layer[EB_MAX_MB];
+  int mbs[EB_MAX_MB];     // micro-batches at the layer, as bits
+  int of_mb[EB_MAX_MB];   // index of every micro-batch's layer
+};
+
 struct TablesArgs {
   uint32_t pool_mask, route_mask;
   int m, policy;
   const int32_t *chunk_hist, *chunk_seg;   // chunk_seg: null without sums_kernel
   int32_t *chunk_base, *seg_base, *mb_base, *mb_load, *mb_cnt;
   Segments seg;
+  StepLayers layers;
   eb_sched_result* res;
   int32_t *group_off, *group_w, *step_meta;
   TilePlan plan;
@@ -88,43 +97,42 @@ struct TablesArgs {
 __device__ __forceinline__ int div_by(int i, int E, unsigned magic) { return i < 65536 ? (int)__umulhi((unsigned)i, magic) : i / E; }
 
 // One block, or several that all work out the loads, share the subsets of a MaxUtil schedule among them and leave the rest to
-// the last one to arrive.  What bounds this kernel is its own chain of phases, a few hundred cycles each at best: every phase has a thread per
-// item of the widest kind ((micro-batch, expert) or (layer, expert)), takes what it needs from shared memory, and
-// decodes nothing by loops or divisions that a table or a multiplication gives.
+// the last one to arrive.  What bounds this kernel is its own chain of phases, a few hundred cycles each at best, a fifth of it
+// waiting for instructions: every phase has a thread per item of the widest kind ((micro-batch, expert) or (layer, expert)), takes
+// what it needs from shared memory, and decodes nothing by loops or divisions that a table or a multiplication gives; what does not
+// depend on this step's routing is laid out while the kernel before still runs, the scans over groups and the order of the
+// tiles share their barriers.
 __global__ void __launch_bounds__(kSchedThreads)
 tables_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ BatchParams bp, const __grid_constant__ TablesArgs a) {
-  EB_GRID_DEP_SYNC();
   extern __shared__ int4 s_dyn4[];
-  __shared__ int s_dev_off[EB_MAX_D + 1], s_dev_list[EB_MAX_E], s_e2d[EB_MAX_E];
+  __shared__ int4 s_expert[EB_MAX_E];               // in (device, expert) order: expert, first of its device, experts of the device, device
+  __shared__ int s_dev_off[EB_MAX_D + 1], s_e2d[EB_MAX_E];
   __shared__ int s_home[EB_MAX_MB][EB_MAX_D + 1];   // first local token of every home device, per micro-batch
-  __shared__ int s_hrows[EB_MAX_MB][EB_MAX_D];      // rows of a shared expert's replica: (active layer, device)
-  __shared__ int s_hslots[EB_MAX_MB], s_hmax[EB_MAX_MB];   // slots of its merged class and its largest replica: per active layer
-  __shared__ int s_mbs[EB_MAX_MB];                  // chosen micro-batches of every active layer, as bits
+  __shared__ int s_layer[EB_MAX_MB], s_layer_mbs[EB_MAX_MB], s_layer_of[EB_MAX_MB];   // a.layers
+  __shared__ int s_act[EB_MAX_MB];                  // active layers, ascending
+  __shared__ int s_mbs[EB_MAX_MB];                  // their chosen micro-batches, as bits
+  __shared__ int s_rank[EB_MAX_MB];                 // rank of every micro-batch's layer among them, -1 if not chosen
+  __shared__ int s_nl;
   __shared__ int s_warp[32];
-  __shared__ int s_carry;
-  __shared__ StepShape ss;
   __shared__ OrderShared s_order;
   SchedShared& sc = *reinterpret_cast<SchedShared*>(s_dyn4);
   int* const s_cnt = reinterpret_cast<int*>(s_dyn4) + sizeof(SchedShared) / 4;   // [n_mb][E] assignments, then rows before
   int* const s_goff = s_cnt + bp.n_mb * mp.E;                                    // [G + 1] group sizes, then offsets
   const int g_cap = bp.n_mb * (mp.E + mp.D * mp.S);
-  int* const s_pgroup = s_goff + g_cap + 1;                                      // [G] group at every position
-  int* const s_ptiles = s_pgroup + g_cap;                                        // [G] its tiles and cost class
+  int* const s_ptiles = s_goff + g_cap + 1;                                      // [G] tiles and cost class of every position
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int E = mp.E, S = mp.S, D = mp.D, n_mb = bp.n_mb;
   const bool first_block = blockIdx.x == 0;
   const unsigned magic = (unsigned)(((1ULL << 32) + E - 1) / E);   // E = 1: wraps to 0, see div_e
   auto div_e = [&](int i) { return E == 1 ? i : div_by(i, E, magic); };
 
-  // ---- small tables; loads of the micro-batches that keep their routing
+  // ---- what depends on the model and on the arguments alone, before the kernels before this one are through: the expert tables
+  // are written once, by eb_create
   if (tid <= D) s_dev_off[tid] = mp.dev_off[tid];
-  for (int e = tid; e < E; e += kSchedThreads) {
-    s_dev_list[e] = mp.dev_list[e];
-    s_e2d[e] = mp.e2d[e];
-  }
-  if (tid >= 512 && tid < 512 + EB_MAX_MB * EB_MAX_D) {
-    const int j = (tid - 512) / EB_MAX_D, d = tid % EB_MAX_D;
-    sc.load[j][d] = (j < n_mb && d < D && !((a.route_mask >> j) & 1u)) ? a.mb_load[j * D + d] : 0;
+  if (tid < E) {
+    const int e = mp.dev_list[tid], d = mp.e2d[e], off = mp.dev_off[d];
+    s_expert[tid] = make_int4(e, off, mp.dev_off[d + 1] - off, d);
+    s_e2d[e] = d;
   }
   if (tid >= 256 && tid < 256 + EB_MAX_MB * 16) {
     const int j = (tid - 256) / 16, d = tid % 16;
@@ -134,12 +142,27 @@ tables_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ Ba
       if (d == 15 && D == 16) s_home[j][16] = T;
     }
   }
-  if (tid == kSchedThreads - 1) s_carry = 0;
+  if (tid >= 512 && tid < 512 + EB_MAX_MB * EB_MAX_D) sc.load[(tid - 512) / EB_MAX_D][tid % EB_MAX_D] = 0;
+  if (tid >= 768 && tid < 768 + EB_MAX_MB) {
+    const int i = tid - 768;
+    s_layer[i] = a.layers.layer[i];
+    s_layer_mbs[i] = i < a.layers.n ? a.layers.mbs[i] : 0;
+    s_layer_of[i] = a.layers.of_mb[i];
+  }
+  for (int i = tid; i < kClasses * 33; i += kSchedThreads) (&s_order.warp[0][0])[i] = 0;
+  if (tid < kClasses) s_order.carry[tid] = 0;
+  schedule_members(sc, a.pool_mask);
   __syncthreads();
+  EB_GRID_DEP_SYNC();
 
   // ---- assignments of every (micro-batch, expert): from the segments' sums, or from the chunk histograms, which also gives
-  // chunk_base = those before the chunk in its micro-batch
+  // chunk_base = those before the chunk in its micro-batch; loads of the micro-batches routed now
   const uint32_t counted = a.pool_mask | a.route_mask;
+  int kept = 0;   // a load of a micro-batch that keeps its routing
+  if (tid >= kSchedThreads - EB_MAX_MB * EB_MAX_D) {
+    const int j = (tid - (kSchedThreads - EB_MAX_MB * EB_MAX_D)) / EB_MAX_D, d = tid % EB_MAX_D;
+    if (j < n_mb && d < D && !((a.route_mask >> j) & 1u)) sc.load[j][d] = kept = a.mb_load[j * D + d];
+  }
   for (int i = tid; i < n_mb * E; i += kSchedThreads) {
     const int j = div_e(i), e = i - j * E;
     int n = 0;
@@ -153,40 +176,42 @@ tables_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ Ba
       }
     }
     s_cnt[i] = n;
-  }
-  __syncthreads();
-
-  // ---- loads of the micro-batches routed now: four threads per (micro-batch, device)
-  for (int i = tid; i < n_mb * E; i += kSchedThreads)
-    if (first_block && ((a.route_mask >> div_e(i)) & 1u)) a.mb_cnt[i] = s_cnt[i];
-  {
-    const int j = tid >> 6, d = (tid >> 2) & 15;
-    int v = 0;
-    if (j < n_mb && d < D)
-      for (int i = s_dev_off[d] + (tid & 3); i < s_dev_off[d + 1]; i += 4) v += s_cnt[j * E + s_dev_list[i]];
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    v += __shfl_xor_sync(0xffffffffu, v, 2);
-    if ((tid & 3) == 0 && j < n_mb && d < D && ((a.route_mask >> j) & 1u)) {
-      sc.load[j][d] = v;
-      if (first_block) a.mb_load[j * D + d] = v;
+    if ((a.route_mask >> j) & 1u) {
+      if (first_block) a.mb_cnt[i] = n;
+      if (n) atomicAdd(&sc.load[j][s_e2d[e]], n);
     }
   }
-  __syncthreads();
+  // the loads of micro-batches routed now are at most their assignments
+  const bool any_wide = __syncthreads_or(wide_load(kept)) || (long long)bp.n_tok * mp.K > kNarrowLoad;
+  if (first_block && tid < EB_MAX_MB * EB_MAX_D) {
+    const int j = tid / EB_MAX_D, d = tid % EB_MAX_D;
+    if (j < n_mb && d < D && ((a.route_mask >> j) & 1u)) a.mb_load[j * D + d] = sc.load[j][d];
+  }
 
   // ---- schedule; of several blocks the last one to arrive goes on
-  if (!schedule_grid(sc, D, a.pool_mask, a.m, a.policy, a.sched)) return;
-  const uint32_t run = sc.run;
-  if (warp == 1) write_schedule(sc, D, a.pool_mask, a.res);
-  if (warp == 2 && lane < EB_MAX_MB) s_mbs[lane] = 0;
-  step_shape_block(bp, run, &ss);
-  const int nl = ss.nl, G = nl * (E + D * S);
-  if (tid < EB_MAX_MB && ss.rank_of_mb[tid] >= 0) atomicOr(&s_mbs[ss.rank_of_mb[tid]], 1 << tid);
+  uint32_t run;
+  if (!schedule_grid(sc, D, a.pool_mask, a.m, a.policy, any_wide, a.sched, &run)) return;
+  if (warp == 0) {
+    // active layers: those with chosen micro-batches
+    const int mbs = lane < EB_MAX_MB ? s_layer_mbs[lane] & (int)run : 0;
+    const unsigned active = __ballot_sync(0xffffffffu, mbs != 0);
+    if (mbs) {
+      const int lr = __popc(active & ((1u << lane) - 1u));
+      s_act[lr] = s_layer[lane];
+      s_mbs[lr] = mbs;
+    }
+    if (lane < EB_MAX_MB) s_rank[lane] = (run >> lane) & 1u ? __popc(active & ((1u << s_layer_of[lane]) - 1u)) : -1;
+    if (lane == 0) s_nl = __popc(active);
+  }
+  if (warp == 1) write_schedule(sc, D, a.pool_mask, run, a.res);
   __syncthreads();
+  const int nl = s_nl, G = nl * (E + D * S);
 
   // ---- routed groups: sizes, weight matrices, tiles; s_cnt turns into the rows of a group before the micro-batch
   for (int i = tid; i < nl * E; i += kSchedThreads) {
     const int lr = div_e(i), k = i - lr * E;   // k: expert in (device, expert) order
-    const int e = s_dev_list[k], d = s_e2d[e], off = s_dev_off[d], n_d = s_dev_off[d + 1] - off;
+    const int4 x = s_expert[k];
+    const int e = x.x, off = x.y, n_d = x.z, d = x.w;
     int tot = 0;
     for (unsigned mbs = s_mbs[lr]; mbs; mbs &= mbs - 1) {
       int* at = s_cnt + (__ffs(mbs) - 1) * E + e;
@@ -196,54 +221,51 @@ tables_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ Ba
     }
     const int g = nl * (off + d * S) + lr * (n_d + S) + (k - off);
     s_goff[g] = tot;
-    a.group_w[g] = ss.act_layer[lr] * (E + S) + e;
+    a.group_w[g] = s_act[lr] * (E + S) + e;
     const int pos = nl * off + lr * n_d + (k - off), tiles = group_tiles(tot);
-    s_pgroup[pos] = g;
     s_ptiles[pos] = tiles << 4 | (cost_class(tiles, group_cols(tot)) & 15);
+    a.plan.pgroup[pos] = g;
+    a.plan.pslots[pos] = -1;
   }
-  // ---- shared experts: rows = chosen tokens at the layer whose home device is d
-  if (S > 0) {
-    if (tid < EB_MAX_MB * EB_MAX_D) {   // whole warps; a layer's devices are sixteen neighbouring lanes
-      const int lr = tid >> 4, d = tid & 15;
-      int rows = 0;
-      if (lr < nl && d < D)
-        for (unsigned mbs = s_mbs[lr]; mbs; mbs &= mbs - 1) {
-          const int j = __ffs(mbs) - 1;
-          rows += s_home[j][d + 1] - s_home[j][d];
-        }
-      s_hrows[lr][d] = rows;
-      int slots = (rows + kSlotRows - 1) / kSlotRows, mx = rows;
+  // ---- shared experts: rows = chosen tokens at the layer whose home device is d; the devices of a (layer, shared expert), as
+  // positions neighbours, are sixteen neighbouring lanes
+  for (int i0 = 0; i0 < nl * S * EB_MAX_D; i0 += kSchedThreads) {
+    const int i = i0 + tid, q = i / EB_MAX_D, d = i % EB_MAX_D;
+    const bool there = q < nl * S && d < D;
+    const int lr = there ? q / S : 0, s = there ? q - lr * S : 0;
+    int rows = 0;
+    if (there)
+      for (unsigned mbs = s_mbs[lr]; mbs; mbs &= mbs - 1) {
+        const int j = __ffs(mbs) - 1;
+        rows += s_home[j][d + 1] - s_home[j][d];
+      }
+    int n_slots = (rows + kSlotRows - 1) / kSlotRows, most = rows;
 #pragma unroll
-      for (int o = 8; o > 0; o >>= 1) {
-        slots += __shfl_xor_sync(0xffffffffu, slots, o);
-        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      }
-      if (d == 0) {
-        s_hslots[lr] = slots;
-        s_hmax[lr] = mx;
-      }
+    for (int o = 8; o > 0; o >>= 1) {
+      n_slots += __shfl_xor_sync(0xffffffffu, n_slots, o);
+      most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
     }
-    __syncthreads();
-    for (int i = tid; i < nl * S * D; i += kSchedThreads) {   // position order: layer, shared expert, device
-      const int q = i / D, d = i - q * D, lr = q / S, s = q - lr * S;
-      const int off = s_dev_off[d], n_d = s_dev_off[d + 1] - off, rows = s_hrows[lr][d];
-      const int g = nl * (off + d * S) + lr * (n_d + S) + n_d + s;
-      s_goff[g] = rows;
-      a.group_w[g] = ss.act_layer[lr] * (E + S) + E + s;
-      const bool merged = D >= 2 && s_hmax[lr] <= kMergeMaxRows;
-      const int n_slots = s_hslots[lr];
-      const int tiles = !merged ? group_tiles(rows) : d == 0 ? (n_slots + kMergeSlots - 1) / kMergeSlots : 0;
-      const int cols = merged ? merged_cols(min(n_slots, kMergeSlots)) : group_cols(rows);
-      s_pgroup[nl * E + i] = g;
-      s_ptiles[nl * E + i] = tiles << 4 | (cost_class(tiles, cols) & 15);
-    }
+    if (!there) continue;
+    const int off = s_dev_off[d], n_d = s_dev_off[d + 1] - off;
+    const int g = nl * (off + d * S) + lr * (n_d + S) + n_d + s, pos = nl * E + q * D + d;
+    s_goff[g] = rows;
+    a.group_w[g] = s_act[lr] * (E + S) + E + s;
+    const bool merged = D >= 2 && most <= kMergeMaxRows;
+    const int tiles = !merged ? group_tiles(rows) : d == 0 ? (n_slots + kMergeSlots - 1) / kMergeSlots : 0;
+    const int cols = merged ? merged_cols(min(n_slots, kMergeSlots)) : group_cols(rows);
+    s_ptiles[pos] = tiles << 4 | (cost_class(tiles, cols) & 15);
+    a.plan.pgroup[pos] = g;
+    a.plan.pslots[pos] = merged ? n_slots : -1;
   }
   __syncthreads();
 
-  // ---- exclusive scan over groups, step_meta
-  for (int base = 0; base < G; base += kSchedThreads) {
-    const int g = base + tid;
-    const int v = g < G ? s_goff[g] : 0;
+  // ---- exclusive scan over groups and order of the tiles of the expert pass, a chunk of 1024 groups and positions at a time (one
+  // chunk as a rule)
+  int carry = 0, my_cls = -1;
+  long long my_at = 0;
+  for (int b = 0; b < G; b += kSchedThreads) {
+    const int i = b + tid;
+    const int v = i < G ? s_goff[i] : 0, t = i < G ? s_ptiles[i] : 0;
     int incl = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -251,23 +273,44 @@ tables_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ Ba
       if (lane >= o) incl += n;
     }
     if (lane == 31) s_warp[warp] = incl;
+    my_cls = t >> 4 ? t & 15 : -1;
+    my_at = order_mark(t >> 4, my_cls, s_order);
     __syncthreads();
     // every warp adds up the warps before it
-    int before = lane < warp ? s_warp[lane] : 0;
-    before = __reduce_add_sync(0xffffffffu, before) + s_carry;
-    const int excl = before + incl - v;
-    if (g < G) {
-      s_goff[g] = excl;
-      a.group_off[g] = excl;
+    const int sum = s_warp[lane];
+    const int excl = carry + (int)__reduce_add_sync(0xffffffffu, lane < warp ? sum : 0) + incl - v;
+    carry += __reduce_add_sync(0xffffffffu, sum);
+    if (i < G) {
+      s_goff[i] = excl;
+      a.group_off[i] = excl;
     }
+    order_scan(s_order);
     __syncthreads();
-    if (tid == kSchedThreads - 1) s_carry = excl + v;
-    __syncthreads();
+    if (my_cls >= 0) my_at += s_order.warp[my_cls][warp];
+    if (G > kSchedThreads) {
+      if (i < G) order_park(i, my_cls, my_at, a.plan);
+      __syncthreads();
+      for (int k = tid; k < kClasses * 33; k += kSchedThreads) (&s_order.warp[0][0])[k] = 0;
+      __syncthreads();
+    }
+  }
+  if (G > kSchedThreads) {
+    for (int i = tid; i < G; i += kSchedThreads) order_unpark(i, a.plan, s_order);
+  } else {
+    order_place(tid, my_cls, my_at, a.plan, s_order);
+  }
+
+  // ---- first row of every chosen (micro-batch, expert)
+  for (int i = tid; i < n_mb * E; i += kSchedThreads) {
+    const int j = div_e(i), k = i - j * E, lr = s_rank[j];
+    if (lr < 0) continue;
+    const int4 x = s_expert[k];
+    const int at = j * E + x.x;
+    a.mb_base[at] = s_cnt[at] + s_goff[nl * (x.y + x.w * S) + lr * (x.z + S) + (k - x.y)];
   }
   if (tid == 0) {
-    s_goff[G] = s_carry;
-    a.group_off[G] = s_carry;
-    a.step_meta[0] = s_carry;
+    a.group_off[G] = carry;
+    a.step_meta[0] = carry;
     a.step_meta[1] = G;
     a.step_meta[2] = nl;
   }
@@ -275,22 +318,7 @@ tables_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ Ba
     const int i = tid - 32;   // entries 3 .. EB_META_LEN-1
     a.step_meta[3 + i] = i < D ? nl * (s_dev_off[i] + i * S) : i == D ? G : 0;
   }
-
-  // ---- first row of every chosen (micro-batch, expert)
-  for (int i = tid; i < n_mb * E; i += kSchedThreads) {
-    const int j = div_e(i), e = i - j * E, lr = ss.rank_of_mb[j];
-    if (lr < 0) continue;
-    const int d = s_e2d[e];
-    a.mb_base[i] = s_cnt[i] + s_goff[group_id(s_dev_off, S, nl, d, lr, mp.e_local[e])];
-  }
-
-  // ---- order of the tiles of the expert pass
-  auto item = [&](int i) {
-    const int t = s_ptiles[i], lr = i < nl * E ? 0 : (i - nl * E) / (S * D);
-    const bool merged = i >= nl * E && D >= 2 && s_hmax[lr] <= kMergeMaxRows;
-    return Position{s_pgroup[i], merged ? s_hslots[lr] : -1, t >> 4, t >> 4 ? t & 15 : -1};
-  };
-  order_tiles(G, nl, -1, 0, item, a.plan, s_order);
+  if (tid == 64) order_finish(G, nl, -1, 0, a.plan, s_order);
 }
 
 // ---- scatter ---------------------------------------------------------------------------------
@@ -462,12 +490,33 @@ constexpr int kSumsChunks = 64;
 constexpr int kSchedSubsets = 5000;
 
 constexpr size_t tables_smem(int n_mb, int E, int groups) {
-  return sizeof(SchedShared) + sizeof(int) * ((size_t)n_mb * E + 3 * (size_t)groups + 1);
+  return sizeof(SchedShared) + sizeof(int) * ((size_t)n_mb * E + 2 * (size_t)groups + 1);
 }
 // The most any shape takes.  The limit belongs to the kernel on its device: a context that set its own need would lower it for
 // the contexts of larger shapes.
 constexpr size_t kTablesSmemMax = tables_smem(EB_MAX_MB, EB_MAX_E, EB_MAX_MB * (EB_MAX_E + EB_MAX_D * EB_MAX_S));
 static_assert(kTablesSmemMax + 16384 <= 232448, "shared memory of one block, the static part within 16 KB");
+
+StepLayers layers_of(const BatchParams& bp) {
+  StepLayers l = {};
+  for (int j = 0; j < bp.n_mb; ++j) {
+    int i = 0;
+    while (i < l.n && l.layer[i] < bp.layer[j]) ++i;
+    if (i == l.n || l.layer[i] != bp.layer[j]) {
+      for (int k = l.n++; k > i; --k) {
+        l.layer[k] = l.layer[k - 1];
+        l.mbs[k] = l.mbs[k - 1];
+      }
+      l.layer[i] = bp.layer[j];
+      l.mbs[i] = 0;
+    }
+    l.mbs[i] |= 1 << j;
+  }
+  for (int i = 0; i < l.n; ++i)
+    for (int j = 0; j < bp.n_mb; ++j)
+      if ((l.mbs[i] >> j) & 1) l.of_mb[j] = i;
+  return l;
+}
 
 // Threads that move a row of `vec` 16-byte columns: the power of two that covers them, 8 to the whole block.
 int row_team(int vec) {
@@ -502,7 +551,7 @@ eb_status ebi_front_run(eb_ctx* c, cudaStream_t st, const BatchParams& bp, uint3
       EB_LAUNCH(c, "sums", ebi_launch(sums_kernel, dim3((seg.off[EB_MAX_MB] * g.E + 255) / 256), dim3(256), 0, st, c->mp, bp, seg, pool_mask | route_mask,
                                       (const int32_t*)c->chunk_hist, c->chunk_base, c->chunk_seg));
     const TablesArgs a{pool_mask, route_mask, (int)m, (int)policy, c->chunk_hist, sums ? c->chunk_seg : nullptr, c->chunk_base, c->seg_base,
-                       c->mb_base, b->mb_load, b->mb_cnt, seg, b->sched, b->group_off, b->group_w, b->step_meta, tile_plan_of(c),
+                       c->mb_base, b->mb_load, b->mb_cnt, seg, layers_of(bp), b->sched, b->group_off, b->group_w, b->step_meta, tile_plan_of(c),
                        sched_grid_of(c)};
     int blocks = sched_blocks(pool_mask, m, policy);
     if ((int64_t)sched_subsets(pool_mask, m) * (blocks - 1) / blocks < kSchedSubsets) blocks = 1;

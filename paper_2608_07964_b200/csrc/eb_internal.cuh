@@ -153,9 +153,9 @@ struct KernelTimer {
     if (_e != cudaSuccess) return ebi_check_cuda((ctx), _e, what);      \
   } while (0)
 
-// Every kernel of the library begins with EB_GRID_DEP_SYNC(): it waits until the kernels before it in
-// the stream have finished (and their writes are visible), then lets the kernel after it start being
-// scheduled.  With launches made through ebi_launch (programmatic stream serialisation) the launch
+// Every kernel of the library begins with EB_GRID_DEP_SYNC() (tables_kernel after laying out shared memory from its arguments and
+// from tables that no kernel writes): it waits until the kernels before it in the stream have finished (and their writes are
+// visible), then lets the kernel after it start being scheduled.  With launches made through ebi_launch (programmatic stream serialisation) the launch
 // latency of each small kernel overlaps the previous kernel; with ordinary launches it is a no-op.
 #define EB_GRID_DEP_SYNC() asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory")
 

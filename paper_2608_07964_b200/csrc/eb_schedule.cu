@@ -10,13 +10,17 @@ schedule_kernel(int D, int n_mb, uint32_t pool_mask, int m, int policy, const in
   EB_GRID_DEP_SYNC();
   __shared__ SchedShared s;
   const int tid = threadIdx.x;
+  int load = 0;
   if (tid < EB_MAX_MB * EB_MAX_D) {
     const int j = tid / EB_MAX_D, d = tid % EB_MAX_D;
-    s.load[j][d] = (j < n_mb && d < D) ? mb_load[j * D + d] : 0;
+    if (j < n_mb && d < D) load = mb_load[j * D + d];
+    s.load[j][d] = load;
   }
-  __syncthreads();
-  if (!schedule_grid(s, D, pool_mask, m, policy, grid)) return;
-  if (tid < 32) write_schedule(s, D, pool_mask, res);
+  schedule_members(s, pool_mask);
+  const bool any_wide = __syncthreads_or(wide_load(load));
+  uint32_t run;
+  if (!schedule_grid(s, D, pool_mask, m, policy, any_wide, grid, &run)) return;
+  if (tid < 32) write_schedule(s, D, pool_mask, run, res);
 }
 
 }  // namespace

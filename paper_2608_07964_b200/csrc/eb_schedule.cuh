@@ -9,10 +9,14 @@
 // CumUtil / DiffPeak (Section 5.2) go through the pool in order, one warp with a device per lane; topping their result
 // up to m members scores the remaining pool members in parallel, one lane each.
 //
-// What bounds the enumeration is instruction issue: 2^16 subsets on one SM.  Subsets that are too small are not visited:
-// the low halves are kept in the order of their member counts, so that for every high half the sufficient ones come
-// first (12 of 16 members: 212 warp turns instead of 2048).  Sums are 32-bit where the loads allow it, and the tables'
-// rows are 20 words apart, which 16-byte reads of neighbouring rows go through without bank conflicts.
+// What bounds small pools is latency, of large ones instruction issue: 2^16 subsets on one SM.  So there are three ways through
+// the subsets of MaxUtil, none of which visits those that are too small:
+//  - up to 10 members: a subset per thread, summed member by member; no tables, no barrier before the result is known.
+//  - more members of which at most 4 stay out (m = ceil(0.75 n) up to n = 16: 2517 subsets): the total less the loads of
+//    those left out, which come from a constant table in the order of their count.
+//  - otherwise the halves: summed loads of every half-subset in shared memory.  The low halves are kept in the order of their
+//    member counts, so that for every high half the sufficient ones come first.  Sums are 32-bit where the loads allow
+//    it, and the tables' rows are 20 words apart, which 16-byte reads of neighbouring rows go through without bank conflicts.
 #pragma once
 
 #include "eb_internal.cuh"
@@ -78,30 +82,45 @@ __device__ __forceinline__ Cand warp_best(Cand c) {
   }
   return c;
 }
-// the same for candidates whose numbers fit 32 bits and whose n is the member count of sub (or negative: none)
+// The same for candidates whose numbers fit 32 bits and whose n is the member count of sub (or negative: none).  The quotients
+// in floating point, off by less than four units in the last place, leave one candidate standing as a rule; for numbers up to
+// 2048 they order like the rationals (which differ by 2^-22 of their value at least), equal ones are told apart by one more
+// reduction; the rest goes through a tree of exact comparisons.
 __device__ __forceinline__ Cand warp_best_narrow(const Cand& c0) {
   int num = (int)c0.num, peak = (int)c0.peak;
   unsigned sub = c0.n < 0 ? 0u : c0.sub;   // the empty subset is never a candidate
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const int num2 = __shfl_xor_sync(0xffffffffu, num, o), peak2 = __shfl_xor_sync(0xffffffffu, peak, o);
-    const unsigned sub2 = __shfl_xor_sync(0xffffffffu, sub, o);
-    const long long l = (long long)num2 * peak, r = (long long)num * peak2;
-    const int n = __popc(sub), n2 = __popc(sub2);
-    if (n2 != 0 && (n == 0 || l > r || (l == r && (n2 > n || (n2 == n && sub2 < sub))))) {
-      num = num2;
-      peak = peak2;
-      sub = sub2;
-    }
+  const unsigned key = sub ? __float_as_uint(__fdiv_rn((float)num, (float)peak)) : 0u;   // quotients of at least 1: never 0
+  const unsigned top = __reduce_max_sync(0xffffffffu, key);
+  unsigned left = __ballot_sync(0xffffffffu, sub != 0 && key + 8u >= top);
+  const bool small = __all_sync(0xffffffffu, max(num, peak) <= 2048);
+  if (__popc(left) > 1 && small) {
+    const unsigned order = sub && key == top ? ((unsigned)__popc(sub) << 16 | (0xffffu ^ sub)) : 0u;
+    const unsigned most = __reduce_max_sync(0xffffffffu, order);   // of one lane: subsets are distinct
+    left = __ballot_sync(0xffffffffu, order == most);
   }
+  if (__popc(left) > 1) {
+#pragma unroll 1
+    for (int o = 16; o > 0; o >>= 1) {
+      const int num2 = __shfl_xor_sync(0xffffffffu, num, o), peak2 = __shfl_xor_sync(0xffffffffu, peak, o);
+      const unsigned sub2 = __shfl_xor_sync(0xffffffffu, sub, o);
+      const long long l = (long long)num2 * peak, r = (long long)num * peak2;
+      const int n = __popc(sub), n2 = __popc(sub2);
+      if (n2 != 0 && (n == 0 || l > r || (l == r && (n2 > n || (n2 == n && sub2 < sub))))) {
+        num = num2;
+        peak = peak2;
+        sub = sub2;
+      }
+    }
+    left = 1u;
+  }
+  const int at = left ? __ffs(left) - 1 : 0;   // no candidate at all: sub is 0 in every lane
   Cand c;
-  c.num = num;
-  c.peak = peak;
-  c.n = sub ? __popc(sub) : -1;
-  c.sub = sub;
+  c.num = __shfl_sync(0xffffffffu, num, at);
+  c.peak = __shfl_sync(0xffffffffu, peak, at);
+  c.sub = __shfl_sync(0xffffffffu, sub, at);
+  c.n = c.sub ? __popc(c.sub) : -1;
   return c;
 }
-
 
 // run set of a candidate; one warp
 __device__ __forceinline__ uint32_t run_mask_of(const int* member, int np, const Cand& b) {
@@ -126,9 +145,32 @@ constexpr ByCount make_by_count() {
 }
 static __device__ const ByCount kByCount = make_by_count();
 
+// The 16-bit values with at most kFewOut bits set, by bit count, ascending inside a count: the subsets of k of the first np positions are
+// the first C(np, k) values of count k.
+constexpr int kFewOut = 4;
+struct FewOut {
+  unsigned short v[1 + 16 + 120 + 560 + 1820];
+};
+constexpr FewOut make_few_out() {
+  FewOut t{};
+  int at = 1;
+  for (int a = 0; a < 16; ++a) t.v[at++] = (unsigned short)(1 << a);
+  for (int b = 1; b < 16; ++b)
+    for (int a = 0; a < b; ++a) t.v[at++] = (unsigned short)(1 << b | 1 << a);
+  for (int c = 2; c < 16; ++c)
+    for (int b = 1; b < c; ++b)
+      for (int a = 0; a < b; ++a) t.v[at++] = (unsigned short)(1 << c | 1 << b | 1 << a);
+  for (int d = 3; d < 16; ++d)
+    for (int c = 2; c < d; ++c)
+      for (int b = 1; b < c; ++b)
+        for (int a = 0; a < b; ++a) t.v[at++] = (unsigned short)(1 << d | 1 << c | 1 << b | 1 << a);
+  return t;
+}
+static __device__ const FewOut kFew = make_few_out();
+
 struct SchedShared {
   int4 lo[256 * kSchedRow / 4], hi[256 * kSchedRow / 4];   // summed loads of every subset of the two halves of the pool
-  int load[EB_MAX_MB][EB_MAX_D];                           // zero beyond n_mb and D
+  alignas(16) int load[EB_MAX_MB][EB_MAX_D];               // zero beyond n_mb and D
   int nibble[4][16][EB_MAX_D];                             // summed loads of every subset of four pool positions
   unsigned char by_count[256];                             // kByCount
   int member[EB_MAX_MB];                                   // micro-batch of every pool position
@@ -138,21 +180,14 @@ struct SchedShared {
   long long seq_w[EB_MAX_D];
 };
 
-// Joint load of the low-half subset lo and a high-half one whose loads are in hi: compared with the best so far.
+// The best subset a thread has seen.
 template <typename W>
 struct BestSubset {
   W num = 0, peak = 1;
   int n = -1;
   unsigned sub = 0;
-  __device__ __forceinline__ void offer(const int4* lo, const int4* hi, int quads, int D, int n2, unsigned sub2) {
-    W num2 = 0, peak2 = 0;
-    for (int q = 0; q < quads; ++q) {   // entries beyond D are zero
-      const int4 a = lo[q], b = hi[q];
-      const W w0 = (W)a.x + b.x, w1 = (W)a.y + b.y, w2 = (W)a.z + b.z, w3 = (W)a.w + b.w;
-      num2 += (w0 + w1) + (w2 + w3);
-      const W p0 = w0 > w1 ? w0 : w1, p1 = w2 > w3 ? w2 : w3, p = p0 > p1 ? p0 : p1;
-      peak2 = p > peak2 ? p : peak2;
-    }
+  // sum and maximum of the joint load of a subset of n2 members
+  __device__ __forceinline__ void offer(W num2, W peak2, int D, int n2, unsigned sub2) {
     if (peak2 == 0) {
       num2 = D;
       peak2 = 1;
@@ -165,97 +200,171 @@ struct BestSubset {
       sub = sub2;
     }
   }
+  __device__ __forceinline__ Cand cand() const {
+    Cand c;
+    c.num = num;
+    c.peak = peak;
+    c.n = n;
+    c.sub = sub;
+    return c;
+  }
 };
-
-// Best subset (pool positions as bits) of at least m members among this block's share.
 template <typename W>
-__device__ __forceinline__ Cand maxutil_scan(const SchedShared& s, int D, int np, int nlo, int m, int block, int n_blocks) {
+__device__ __forceinline__ W max4(W a, W b, W c, W d) {
+  const W p = a > b ? a : b, q = c > d ? c : d;
+  return p > q ? p : q;
+}
+
+// Best subset (pool positions as bits) of at least m members, of those this thread looks at.
+// Up to 10 members.
+template <typename W>
+__device__ __forceinline__ Cand maxutil_small(const SchedShared& s, int D, int np, int m) {
+  const int tid = threadIdx.x, n = __popc(tid), quads = (D + 3) / 4;
+  BestSubset<W> best;
+  if (tid < (1 << np) && n >= m) {
+    W num = 0, peak = 0;
+    for (int q = 0; q < quads; ++q) {   // entries beyond D are zero
+      W w0 = 0, w1 = 0, w2 = 0, w3 = 0;
+      for (int k = 0; k < np; ++k) {
+        const int4 v = reinterpret_cast<const int4*>(s.load[s.member[k]])[q];
+        if ((tid >> k) & 1) {
+          w0 += v.x;
+          w1 += v.y;
+          w2 += v.z;
+          w3 += v.w;
+        }
+      }
+      num += (w0 + w1) + (w2 + w3);
+      const W p = max4(w0, w1, w2, w3);
+      peak = p > peak ? p : peak;
+    }
+    best.offer(num, peak, D, n, tid);
+  }
+  return best.cand();
+}
+// All but at most kFewOut of up to 16 members.
+template <typename W>
+__device__ __forceinline__ Cand maxutil_few_out(const SchedShared& s, int D, int np, int m) {
+  const int tid = threadIdx.x, lane = tid & 31, quads = (D + 3) / 4, out = np - m;
+  W mine = 0;   // total load of device `lane` mod 16
+  for (int k = 0; k < np; ++k) mine += s.load[s.member[k]][lane & 15];
+  const int n1 = np, n2 = n1 * (np - 1) / 2, n3 = n2 * (np - 2) / 3, n4 = n3 * (np - 3) / 4;
+  const int end0 = 1, end1 = end0 + (out >= 1 ? n1 : 0), end2 = end1 + (out >= 2 ? n2 : 0), end3 = end2 + (out >= 3 ? n3 : 0),
+            end4 = end3 + (out >= 4 ? n4 : 0);
+  BestSubset<W> best;
+  for (int c0 = 0; c0 < end4; c0 += kSchedThreads) {   // whole warps go on together: the totals travel by shuffles
+    const int c = c0 + tid;
+    if (c - lane >= end4) break;
+    const int at = c < end0 ? 0 : c < end1 ? c : c < end2 ? c - end1 + 17 : c < end3 ? c - end2 + 137 : c - end3 + 697;
+    const unsigned off = c < end4 ? kFew.v[at] : 0u;
+    W num = 0, peak = 0;
+    for (int q = 0; q < quads; ++q) {
+      W w0 = __shfl_sync(0xffffffffu, mine, 4 * q), w1 = __shfl_sync(0xffffffffu, mine, 4 * q + 1), w2 = __shfl_sync(0xffffffffu, mine, 4 * q + 2),
+        w3 = __shfl_sync(0xffffffffu, mine, 4 * q + 3);
+      for (unsigned left = off; left; left &= left - 1) {
+        const int4 v = reinterpret_cast<const int4*>(s.load[s.member[__ffs(left) - 1]])[q];
+        w0 -= v.x;
+        w1 -= v.y;
+        w2 -= v.z;
+        w3 -= v.w;
+      }
+      num += (w0 + w1) + (w2 + w3);
+      const W p = max4(w0, w1, w2, w3);
+      peak = p > peak ? p : peak;
+    }
+    if (c < end4) best.offer(num, peak, D, np - __popc(off), ((1u << np) - 1u) ^ off);
+  }
+  return best.cand();
+}
+// More than 10 members, this block's share.
+template <typename W>
+__device__ __forceinline__ Cand maxutil_halves(const SchedShared& s, int D, int np, int m, int block, int n_blocks) {
   const int quads = (D + 3) / 4, tid = threadIdx.x;
   static_assert(EB_MAX_D == 16 && EB_MAX_MB == 16, "the tables are indexed in nibbles");
   BestSubset<W> best;
-  if (np <= 10) {   // a subset per thread
-    const int n = __popc(tid);
-    if (tid < (1 << np) && n >= m)
-      best.offer(s.lo + (tid & ((1 << nlo) - 1)) * (kSchedRow / 4), s.hi + (tid >> nlo) * (kSchedRow / 4), quads, D, n, tid);
-  } else {
-    // A warp takes high halves in turn and, for each, the low halves that bring it to m members: they come first in
-    // the order by member count.  Which warp takes which high half changes from turn to turn, so that the shares of
-    // large high halves even out.
-    const int lane = tid & 31, warp = tid >> 5;
-    for (int k = block; k < (1 << (np - 8)) / 32 + 1; k += n_blocks) {
-      const int h = k * 32 + (warp ^ (k * 11 & 31)), n_h = __popc(h);
-      if (h >= 1 << (np - 8)) continue;
-      const int need = max(0, m - n_h);
-      if (need > 8) continue;
-      // byte values with at least `need` bits set: 256, 255, 247, 219, 163, 93, 37, 9, 1
-      const int n_lo = need == 0 ? 256 : (int)((0x0109255da3dbf7ffULL >> (8 * (need - 1))) & 255u);
-      const int4* hi = s.hi + h * (kSchedRow / 4);
-      for (int i = lane; i < n_lo; i += 32) {
-        const int u = s.by_count[i];
-        if (u | h) best.offer(s.lo + u * (kSchedRow / 4), hi, quads, D, n_h + __popc(u), (unsigned)(h << 8 | u));
+  // A warp takes high halves in turn and, for each, the low halves that bring it to m members: they come first in
+  // the order by member count.  Which warp takes which high half changes from turn to turn, so that the shares of
+  // large high halves even out.
+  const int lane = tid & 31, warp = tid >> 5;
+  for (int k = block; k < (1 << (np - 8)) / 32 + 1; k += n_blocks) {
+    const int h = k * 32 + (warp ^ (k * 11 & 31)), n_h = __popc(h);
+    if (h >= 1 << (np - 8)) continue;
+    const int need = max(0, m - n_h);
+    if (need > 8) continue;
+    // byte values with at least `need` bits set: 256, 255, 247, 219, 163, 93, 37, 9, 1
+    const int n_lo = need == 0 ? 256 : (int)((0x0109255da3dbf7ffULL >> (8 * (need - 1))) & 255u);
+    const int4* hi = s.hi + h * (kSchedRow / 4);
+    for (int i = lane; i < n_lo; i += 32) {
+      const int u = s.by_count[i];
+      if (!(u | h)) continue;
+      const int4* lo = s.lo + u * (kSchedRow / 4);
+      W num = 0, peak = 0;
+      for (int q = 0; q < quads; ++q) {   // entries beyond D are zero
+        const int4 a = lo[q], b = hi[q];
+        const W w0 = (W)a.x + b.x, w1 = (W)a.y + b.y, w2 = (W)a.z + b.z, w3 = (W)a.w + b.w;
+        num += (w0 + w1) + (w2 + w3);
+        const W p = max4(w0, w1, w2, w3);
+        peak = p > peak ? p : peak;
       }
+      best.offer(num, peak, D, n_h + __popc(u), (unsigned)(h << 8 | u));
     }
   }
-  Cand c;
-  c.num = best.num;
-  c.peak = best.peak;
-  c.n = best.n;
-  c.sub = best.sub;
-  return c;
+  return best.cand();
 }
 
+// Which micro-batches are in the pool; before the barrier behind the writes of s.load.
+__device__ __forceinline__ void schedule_members(SchedShared& s, uint32_t pool_mask) {
+  const int tid = threadIdx.x;
+  if (tid < EB_MAX_MB && ((pool_mask >> tid) & 1u)) s.member[__popc(pool_mask & ((1u << tid) - 1u))] = tid;
+}
+__device__ __forceinline__ bool wide_load(int v) { return v < 0 || v > kNarrowLoad; }
+
 // Chooses the run set from s.load.  All kSchedThreads threads of the block call it after a barrier behind the writes of
-// s.load; `block` of n_blocks.  On return (after a barrier): s.run, or with n_blocks > 1 under MaxUtil this block's
-// candidate in s.best[0].  True: s.run is final.
-__device__ __forceinline__ bool schedule_block(SchedShared& s, int D, uint32_t pool_mask, int m, int policy, int block, int n_blocks) {
+// s.load and schedule_members; `any_wide` (uniform) unless no load is a wide_load; `block` of n_blocks.  True: *run is the run set;
+// false, with n_blocks > 1 under MaxUtil over a large pool: *mine is this block's candidate.  In every thread.
+__device__ __forceinline__ bool schedule_block(SchedShared& s, int D, uint32_t pool_mask, int m, int policy, bool any_wide, int block, int n_blocks,
+                                               uint32_t* run, Cand* mine) {
   const int tid = threadIdx.x;
   const int np = __popc(pool_mask);
-  if (tid < EB_MAX_MB && ((pool_mask >> tid) & 1u)) s.member[__popc(pool_mask & ((1u << tid) - 1u))] = tid;
   if (np <= m || policy == EB_POLICY_ALL) {
-    if (tid == 0) s.run = pool_mask;
-    __syncthreads();
+    *run = pool_mask;
     return true;
   }
-  bool wide = false;
-  if (tid < EB_MAX_MB * EB_MAX_D) {
-    const int v = s.load[tid / EB_MAX_D][tid % EB_MAX_D];
-    wide = v < 0 || v > kNarrowLoad;
-  }
-  const bool any_wide = __syncthreads_or(wide);
   if (policy == EB_POLICY_MAXUTIL) {
-    const int nlo = np < 8 ? np : 8, nhi = np - nlo;
-    int* lo = reinterpret_cast<int*>(s.lo);
-    int* hi = reinterpret_cast<int*>(s.hi);
-    // sums over four members at a time (one entry per thread), then over eight
-    {
-      const int quad = tid >> 8, u = (tid >> 4) & 15, d = tid & 15;
-      int acc = 0;
+    Cand best;
+    if (np <= 10) {
+      best = any_wide ? maxutil_small<long long>(s, D, np, m) : maxutil_small<int>(s, D, np, m);
+    } else if (np - m <= kFewOut) {
+      best = any_wide ? maxutil_few_out<long long>(s, D, np, m) : maxutil_few_out<int>(s, D, np, m);
+    } else {
+      const int nlo = 8, nhi = np - nlo;
+      int* lo = reinterpret_cast<int*>(s.lo);
+      int* hi = reinterpret_cast<int*>(s.hi);
+      // sums over four members at a time (one entry per thread), then over eight
+      {
+        const int quad = tid >> 8, u = (tid >> 4) & 15, d = tid & 15;
+        int acc = 0;
 #pragma unroll
-      for (int b = 0; b < 4; ++b)
-        if (quad * 4 + b < np && ((u >> b) & 1)) acc += s.load[s.member[quad * 4 + b]][d];
-      s.nibble[quad][u][d] = acc;
+        for (int b = 0; b < 4; ++b)
+          if (quad * 4 + b < np && ((u >> b) & 1)) acc += s.load[s.member[quad * 4 + b]][d];
+        s.nibble[quad][u][d] = acc;
+      }
+      if (tid < 64) reinterpret_cast<uint32_t*>(s.by_count)[tid] = reinterpret_cast<const uint32_t*>(kByCount.v)[tid];
+      __syncthreads();
+      for (int i = tid; i < (1 << nlo) * EB_MAX_D; i += kSchedThreads)
+        lo[(i >> 4) * kSchedRow + (i & 15)] = s.nibble[0][(i >> 4) & 15][i & 15] + s.nibble[1][i >> 8][i & 15];
+      for (int i = tid; i < (1 << nhi) * EB_MAX_D; i += kSchedThreads)
+        hi[(i >> 4) * kSchedRow + (i & 15)] = s.nibble[2][(i >> 4) & 15][i & 15] + s.nibble[3][i >> 8][i & 15];
+      __syncthreads();
+      best = any_wide ? maxutil_halves<long long>(s, D, np, m, block, n_blocks) : maxutil_halves<int>(s, D, np, m, block, n_blocks);
     }
-    if (np > 10 && tid < 64) reinterpret_cast<uint32_t*>(s.by_count)[tid] = reinterpret_cast<const uint32_t*>(kByCount.v)[tid];
-    __syncthreads();
-    for (int i = tid; i < (1 << nlo) * EB_MAX_D; i += kSchedThreads)
-      lo[(i >> 4) * kSchedRow + (i & 15)] = s.nibble[0][(i >> 4) & 15][i & 15] + s.nibble[1][i >> 8][i & 15];
-    for (int i = tid; i < (1 << nhi) * EB_MAX_D; i += kSchedThreads)
-      hi[(i >> 4) * kSchedRow + (i & 15)] = s.nibble[2][(i >> 4) & 15][i & 15] + s.nibble[3][i >> 8][i & 15];
-    __syncthreads();
-    Cand best = any_wide ? maxutil_scan<long long>(s, D, np, nlo, m, block, n_blocks) : maxutil_scan<int>(s, D, np, nlo, m, block, n_blocks);
-    // warp then block reduction under the total order (any reduction order gives the same winner)
+    // warp then block reduction under the total order (any reduction order gives the same winner); every warp makes the second
     best = any_wide ? warp_best(best) : warp_best_narrow(best);
     if ((tid & 31) == 0) s.best[tid >> 5] = best;
     __syncthreads();
-    if (tid < 32) {
-      Cand b = any_wide ? warp_best(s.best[tid]) : warp_best_narrow(s.best[tid]);
-      const uint32_t mask = run_mask_of(s.member, np, b);
-      if (tid == 0) {
-        s.best[0] = b;
-        s.run = mask;
-      }
-    }
-    __syncthreads();
+    best = any_wide ? warp_best(s.best[tid & 31]) : warp_best_narrow(s.best[tid & 31]);
+    *run = run_mask_of(s.member, np, best);
+    *mine = best;
     return n_blocks == 1;
   }
   if (tid < 32) {
@@ -263,7 +372,7 @@ __device__ __forceinline__ bool schedule_block(SchedShared& s, int D, uint32_t p
     const int lane = tid;
     auto load_of = [&](int j) { return lane < EB_MAX_D ? (long long)s.load[j][lane] : 0LL; };
     long long w = load_of(s.member[0]);
-    uint32_t run = 1u << s.member[0];
+    uint32_t chosen = 1u << s.member[0];
     int n = 1;
     if (policy == EB_POLICY_CUMUTIL) {
       Cand cur = warp_util(w, D, any_wide);
@@ -274,7 +383,7 @@ __device__ __forceinline__ bool schedule_block(SchedShared& s, int D, uint32_t p
         if (nxt.num * cur.peak > cur.num * nxt.peak) {
           w = w2;
           cur = nxt;
-          run |= 1u << j;
+          chosen |= 1u << j;
           ++n;
         }
       }
@@ -289,7 +398,7 @@ __device__ __forceinline__ bool schedule_block(SchedShared& s, int D, uint32_t p
         if (peaks & bit) continue;
         peaks |= bit;
         w += load_of(s.member[k]);
-        run |= 1u << s.member[k];
+        chosen |= 1u << s.member[k];
         ++n;
       }
     }
@@ -300,7 +409,7 @@ __device__ __forceinline__ bool schedule_block(SchedShared& s, int D, uint32_t p
     while (n < m) {
       Cand cu;
       cu.n = -1; cu.num = 0; cu.peak = 1; cu.sub = 0;
-      if (lane < np && !((run >> s.member[lane]) & 1u)) {
+      if (lane < np && !((chosen >> s.member[lane]) & 1u)) {
         long long num = 0, peak = 0;
 #pragma unroll
         for (int d = 0; d < EB_MAX_D; ++d) {   // zero beyond D
@@ -319,12 +428,13 @@ __device__ __forceinline__ bool schedule_block(SchedShared& s, int D, uint32_t p
       __syncwarp();
       if (lane < EB_MAX_D) s.seq_w[lane] += s.load[bj][lane];
       __syncwarp();
-      run |= 1u << bj;
+      chosen |= 1u << bj;
       ++n;
     }
-    if (lane == 0) s.run = run;
+    if (lane == 0) s.run = chosen;
   }
   __syncthreads();
+  *run = s.run;
   return true;
 }
 
@@ -334,11 +444,13 @@ struct SchedGrid {
   Cand* best;          // [gridDim.x]
   unsigned* arrived;
 };
-__device__ __forceinline__ bool schedule_grid(SchedShared& s, int D, uint32_t pool_mask, int m, int policy, const SchedGrid& g) {
-  if (schedule_block(s, D, pool_mask, m, policy, blockIdx.x, gridDim.x)) return gridDim.x == 1 || blockIdx.x == 0;
+__device__ __forceinline__ bool schedule_grid(SchedShared& s, int D, uint32_t pool_mask, int m, int policy, bool any_wide, const SchedGrid& g,
+                                              uint32_t* run) {
+  Cand mine;
+  if (schedule_block(s, D, pool_mask, m, policy, any_wide, blockIdx.x, gridDim.x, run, &mine)) return blockIdx.x == 0;
   const int tid = threadIdx.x;
   if (tid == 0) {
-    g.best[blockIdx.x] = s.best[0];
+    g.best[blockIdx.x] = mine;
     __threadfence();
     s.last = atomicAdd(g.arrived, 1u) == gridDim.x - 1;
   }
@@ -360,14 +472,15 @@ __device__ __forceinline__ bool schedule_grid(SchedShared& s, int D, uint32_t po
     }
   }
   __syncthreads();
+  *run = s.run;
   return true;
 }
 
-// Blocks for a schedule: MaxUtil over a pool of more than 13 takes one per 32 high halves of its subsets.
+// Blocks for a schedule: MaxUtil over the halves of a pool of more than 13 takes one per 32 high halves of its subsets.
 constexpr int kMaxSchedBlocks = 1 << (EB_MAX_MB - 13);
 inline int sched_blocks(uint32_t pool_mask, int m, int policy) {
   const int np = __builtin_popcount(pool_mask);
-  return policy == EB_POLICY_MAXUTIL && np > m && np > 13 ? 1 << (np - 13) : 1;
+  return policy == EB_POLICY_MAXUTIL && np - m > kFewOut && np > 13 ? 1 << (np - 13) : 1;
 }
 // Subsets that MaxUtil looks at: those of at least m members.
 inline int sched_subsets(uint32_t pool_mask, int m) {
@@ -383,11 +496,10 @@ inline SchedGrid sched_grid_of(const eb_ctx* c) {
   return SchedGrid{(Cand*)c->d_sched_scratch, (unsigned*)(c->d_sched_scratch + kMaxSchedBlocks * sizeof(Cand))};
 }
 
-// The result record, by one warp, s.run final.
-__device__ __forceinline__ void write_schedule(const SchedShared& s, int D, uint32_t pool_mask, eb_sched_result* __restrict__ res) {
+// The result record, by one warp.
+__device__ __forceinline__ void write_schedule(const SchedShared& s, int D, uint32_t pool_mask, uint32_t run, eb_sched_result* __restrict__ res) {
   const int tid = threadIdx.x & 31;
   // lane d sums the chosen micro-batches' load on device d (zero beyond D); the warp adds and maximises
-  const uint32_t run = s.run;
   long long v = 0;
   if (tid < EB_MAX_D) {
 #pragma unroll

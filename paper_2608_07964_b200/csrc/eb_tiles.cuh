@@ -108,14 +108,88 @@ struct OrderShared {
   long long carry[kClasses];      // of the chunks of positions before
 };
 
-// Lists the positions 0 .. ng - 1 that own tiles by cost class, widest tiles first, processing order inside a class, with
-// the exclusive scan of their tile counts.  Widest-first order is what lets the expert kernel hand its tiles out to
-// nearly equal ends.  One block of 1024 threads; item(i) gives position i.  Ranks inside a warp come from a warp match
-// of the classes, the sums over warps from one warp per class: a block scan carrying all eight classes through every
-// shuffle took three times as long (10 us of a step's latency together with the decoding of positions).
+// The parts of order_tiles, which lists the positions that own tiles by cost class, widest tiles first, processing order inside
+// a class, with the exclusive scan of their tile counts.  Widest-first order is what lets the expert kernel hand its tiles out to
+// nearly equal ends.  Ranks inside a warp come from a warp match of the classes, the sums over warps from one warp per class: a
+// block scan carrying all eight classes through every shuffle took three times as long.
+//
+// order_mark: a position per thread (class -1: none); returns the positions and tiles of its class in the lanes before it and
+// leaves the warp's sums in sh.warp, which is clear.  Then a barrier, order_scan and another barrier.
+__device__ __forceinline__ long long order_mark(int tiles, int cls, OrderShared& sh) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned peers = __match_any_sync(0xffffffffu, cls), below = peers & ((1u << lane) - 1u);
+  int pref = __popc(below);   // tiles of the class before this lane
+  if (__any_sync(0xffffffffu, tiles > 1)) {
+    unsigned todo = __ballot_sync(0xffffffffu, cls >= 0);
+    while (todo) {
+      const int c = __shfl_sync(0xffffffffu, cls, __ffs(todo) - 1);
+      int incl = cls == c ? tiles : 0;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int n = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += n;
+      }
+      if (cls == c) pref = incl - tiles;
+      todo &= ~__ballot_sync(0xffffffffu, cls == c);
+    }
+  }
+  if (cls >= 0 && lane == 31 - __clz(peers))   // the class's last lane knows its sums
+    sh.warp[cls][warp] = (long long)__popc(peers) | ((long long)(pref + tiles) << 32);
+  return (long long)__popc(below) | ((long long)pref << 32);
+}
+// order_scan: sh.warp turns into those of the chunks and warps before, sh.carry takes the chunk up.
+__device__ __forceinline__ void order_scan(OrderShared& sh) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp >= kClasses) return;
+  const long long v = sh.warp[warp][lane];
+  long long incl = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long n = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += n;
+  }
+  const long long before = sh.carry[warp];
+  sh.warp[warp][lane] = before + incl - v;
+  __syncwarp();
+  if (lane == 31) sh.carry[warp] = before + incl;
+}
+// order_place: position i of class cls, `at` of its class before it; sh.carry is final.
+__device__ __forceinline__ void order_place(int i, int cls, long long at, const TilePlan& out, const OrderShared& sh) {
+  if (cls < 0) return;
+  for (int c = cls + 1; c < kClasses; ++c) at += sh.carry[c];   // the wider classes come first
+  out.order[(int)(at & 0xffffffffLL)] = i;
+  out.tile_pref[(int)(at & 0xffffffffLL)] = (int)(at >> 32);
+}
+// More than one chunk of positions: parked until the class bases are known (read back by the same thread).
+__device__ __forceinline__ void order_park(int i, int cls, long long at, const TilePlan& out) {
+  out.prank[i] = make_int4(cls, (int)(at & 0xffffffffLL), (int)(at >> 32), 0);
+}
+__device__ __forceinline__ void order_unpark(int i, const TilePlan& out, const OrderShared& sh) {
+  const int4 v = out.prank[i];
+  order_place(i, v.x, (long long)v.y | ((long long)v.z << 32), out, sh);
+}
+// The counts of the list; one thread.
+__device__ __forceinline__ void order_finish(int ng, int nl, int device, int g0, const TilePlan& out, const OrderShared& sh) {
+  long long all = 0;
+  for (int c = 0; c < kClasses; ++c) all += sh.carry[c];
+  const int n_listed = (int)(all & 0xffffffffLL), nt = (int)(all >> 32);
+  out.tile_pref[n_listed] = nt;
+  int32_t* const work_count = out.work_count;
+  work_count[0] = nt * out.nt1;
+  work_count[1] = nt * out.nt2;
+  work_count[2] = nt;
+  work_count[3] = g0;
+  work_count[4] = ng;
+  work_count[5] = n_listed;
+  work_count[6] = work_count[7] = 0;   // tiles dealt out by the expert kernel
+  work_count[8] = nl;
+  work_count[9] = device;
+}
+
+// Orders the positions 0 .. ng - 1.  One block of 1024 threads; item(i) gives position i.
 template <typename Item>
 __device__ __forceinline__ void order_tiles(int ng, int nl, int device, int g0, Item item, const TilePlan& out, OrderShared& sh) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = tid >> 5;
   int my_cls = -1;             // of the position this thread handled in the last chunk (the only one, as a rule)
   long long my_at = 0;
   if (tid < kClasses) sh.carry[tid] = 0;
@@ -129,82 +203,24 @@ __device__ __forceinline__ void order_tiles(int ng, int nl, int device, int g0, 
     }
     if (tid < kClasses * 33) (&sh.warp[0][0])[tid] = 0;
     __syncthreads();
-    const unsigned peers = __match_any_sync(0xffffffffu, p.cls), below = peers & ((1u << lane) - 1u);
-    int pref = __popc(below);   // tiles of the class before this lane
-    if (__any_sync(0xffffffffu, p.tiles > 1)) {
-      unsigned todo = __ballot_sync(0xffffffffu, p.cls >= 0);
-      while (todo) {
-        const int c = __shfl_sync(0xffffffffu, p.cls, __ffs(todo) - 1);
-        int incl = p.cls == c ? p.tiles : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int n = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += n;
-        }
-        if (p.cls == c) pref = incl - p.tiles;
-        todo &= ~__ballot_sync(0xffffffffu, p.cls == c);
-      }
-    }
-    if (p.cls >= 0 && lane == 31 - __clz(peers))   // the class's last lane knows its sums
-      sh.warp[p.cls][warp] = (long long)__popc(peers) | ((long long)(pref + p.tiles) << 32);
+    my_at = order_mark(p.tiles, p.cls, sh);
     __syncthreads();
-    if (warp < kClasses) {
-      const long long v = sh.warp[warp][lane];
-      long long incl = v;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const long long n = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += n;
-      }
-      const long long before = sh.carry[warp];
-      sh.warp[warp][lane] = before + incl - v;
-      __syncwarp();
-      if (lane == 31) sh.carry[warp] = before + incl;
-    }
+    order_scan(sh);
     __syncthreads();
     my_cls = p.cls;
-    if (my_cls >= 0) my_at = sh.warp[my_cls][warp] + ((long long)__popc(below) | ((long long)pref << 32));
-    // more than one chunk of positions: parked until the class bases are known (read back by the same thread)
+    if (my_cls >= 0) my_at += sh.warp[my_cls][warp];
     if (ng > 1024) {
-      if (i < ng) out.prank[i] = make_int4(my_cls, (int)(my_at & 0xffffffffLL), (int)(my_at >> 32), 0);
+      if (i < ng) order_park(i, my_cls, my_at, out);
       __syncthreads();   // the table is cleared for the next chunk
     }
   }
   __syncthreads();
-  for (int b = 0; b < ng; b += 1024) {
-    const int i = b + tid;
-    int cls = my_cls;
-    long long at = my_at;
-    if (ng > 1024) {
-      cls = -1;
-      if (i < ng) {
-        const int4 v = out.prank[i];
-        cls = v.x;
-        at = (long long)v.y | ((long long)v.z << 32);
-      }
-    }
-    if (cls >= 0) {
-      for (int c = cls + 1; c < kClasses; ++c) at += sh.carry[c];   // the wider classes come first
-      out.order[(int)(at & 0xffffffffLL)] = i;
-      out.tile_pref[(int)(at & 0xffffffffLL)] = (int)(at >> 32);
-    }
+  if (ng > 1024) {
+    for (int i = tid; i < ng; i += 1024) order_unpark(i, out, sh);
+  } else {
+    order_place(tid, my_cls, my_at, out, sh);
   }
-  if (tid == 0) {
-    long long all = 0;
-    for (int c = 0; c < kClasses; ++c) all += sh.carry[c];
-    const int n_listed = (int)(all & 0xffffffffLL), nt = (int)(all >> 32);
-    out.tile_pref[n_listed] = nt;
-    int32_t* const work_count = out.work_count;
-    work_count[0] = nt * out.nt1;
-    work_count[1] = nt * out.nt2;
-    work_count[2] = nt;
-    work_count[3] = g0;
-    work_count[4] = ng;
-    work_count[5] = n_listed;
-    work_count[6] = work_count[7] = 0;   // tiles dealt out by the expert kernel
-    work_count[8] = nl;
-    work_count[9] = device;
-  }
+  if (tid == 0) order_finish(ng, nl, device, g0, out, sh);
 }
 
 // fill: one thread per tile of the list (gate/up tiles, then down tiles); tiles of a group are ordered weight-tile
