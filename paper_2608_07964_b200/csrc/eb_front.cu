@@ -151,7 +151,7 @@ tables_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ Ba
   }
   for (int i = tid; i < kClasses * 33; i += kSchedThreads) (&s_order.warp[0][0])[i] = 0;
   if (tid < kClasses) s_order.carry[tid] = 0;
-  schedule_members(sc, a.pool_mask);
+  schedule_prepare(sc, a.pool_mask, a.m, a.policy);
   __syncthreads();
   EB_GRID_DEP_SYNC();
 

@@ -16,7 +16,7 @@ schedule_kernel(int D, int n_mb, uint32_t pool_mask, int m, int policy, const in
     if (j < n_mb && d < D) load = mb_load[j * D + d];
     s.load[j][d] = load;
   }
-  schedule_members(s, pool_mask);
+  schedule_prepare(s, pool_mask, m, policy);
   const bool any_wide = __syncthreads_or(wide_load(load));
   uint32_t run;
   if (!schedule_grid(s, D, pool_mask, m, policy, any_wide, grid, &run)) return;

@@ -13,7 +13,7 @@
 // the subsets of MaxUtil, none of which visits those that are too small:
 //  - up to 10 members: a subset per thread, summed member by member; no tables, no barrier before the result is known.
 //  - more members of which at most 4 stay out (m = ceil(0.75 n) up to n = 16: 2517 subsets): the total less the loads of
-//    those left out, which come from a constant table in the order of their count.
+//    two pairs left out, whose sums are tabulated.
 //  - otherwise the halves: summed loads of every half-subset in shared memory.  The low halves are kept in the order of their
 //    member counts, so that for every high half the sufficient ones come first.  Sums are 32-bit where the loads allow
 //    it, and the tables' rows are 20 words apart, which 16-byte reads of neighbouring rows go through without bank conflicts.
@@ -70,7 +70,7 @@ __device__ __forceinline__ Cand warp_util(long long w, int D, bool wide) {
 }
 
 // best candidate of the warp, in every lane
-__device__ __forceinline__ Cand warp_best(Cand c) {
+static __device__ __noinline__ Cand warp_best(Cand c) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     Cand oth;
@@ -85,8 +85,8 @@ __device__ __forceinline__ Cand warp_best(Cand c) {
 // The same for candidates whose numbers fit 32 bits and whose n is the member count of sub (or negative: none).  The quotients
 // in floating point, off by less than four units in the last place, leave one candidate standing as a rule; for numbers up to
 // 2048 they order like the rationals (which differ by 2^-22 of their value at least), equal ones are told apart by one more
-// reduction; the rest goes through a tree of exact comparisons.
-__device__ __forceinline__ Cand warp_best_narrow(const Cand& c0) {
+// reduction; the rest goes through a tree of exact comparisons.  Not inlined: it is called twice.
+static __device__ __noinline__ Cand warp_best_narrow(const Cand& c0) {
   int num = (int)c0.num, peak = (int)c0.peak;
   unsigned sub = c0.n < 0 ? 0u : c0.sub;   // the empty subset is never a candidate
   const unsigned key = sub ? __float_as_uint(__fdiv_rn((float)num, (float)peak)) : 0u;   // quotients of at least 1: never 0
@@ -145,32 +145,44 @@ constexpr ByCount make_by_count() {
 }
 static __device__ const ByCount kByCount = make_by_count();
 
-// The 16-bit values with at most kFewOut bits set, by bit count, ascending inside a count: the subsets of k of the first np positions are
-// the first C(np, k) values of count k.
+// What may be left out of a pool, when that is at most kFewOut members: "pairs", the sets of at most two positions by count and
+// ascending (the sets within the first np positions are the first of their count), and the sets of at most four as two pairs, the
+// lower positions in the low byte, by count and ascending in the same way.
 constexpr int kFewOut = 4;
+constexpr int kPairs = 1 + 16 + 120;
+constexpr int kFewSets = 1 + 16 + 120 + 560 + 1820;
 struct FewOut {
-  unsigned short v[1 + 16 + 120 + 560 + 1820];
+  alignas(16) unsigned short few[(kFewSets + 7) / 8 * 8];
+  alignas(16) unsigned short pair[(kPairs + 7) / 8 * 8];   // as bits
 };
+constexpr int single_index(int a) { return 1 + a; }
+constexpr int pair_index(int a, int b) { return 17 + b * (b - 1) / 2 + a; }   // a < b
 constexpr FewOut make_few_out() {
   FewOut t{};
   int at = 1;
-  for (int a = 0; a < 16; ++a) t.v[at++] = (unsigned short)(1 << a);
+  for (int a = 0; a < 16; ++a, ++at) {
+    t.few[at] = (unsigned short)single_index(a);
+    t.pair[single_index(a)] = (unsigned short)(1 << a);
+  }
   for (int b = 1; b < 16; ++b)
-    for (int a = 0; a < b; ++a) t.v[at++] = (unsigned short)(1 << b | 1 << a);
+    for (int a = 0; a < b; ++a, ++at) {
+      t.few[at] = (unsigned short)pair_index(a, b);
+      t.pair[pair_index(a, b)] = (unsigned short)(1 << b | 1 << a);
+    }
   for (int c = 2; c < 16; ++c)
     for (int b = 1; b < c; ++b)
-      for (int a = 0; a < b; ++a) t.v[at++] = (unsigned short)(1 << c | 1 << b | 1 << a);
+      for (int a = 0; a < b; ++a) t.few[at++] = (unsigned short)(pair_index(a, b) | single_index(c) << 8);
   for (int d = 3; d < 16; ++d)
     for (int c = 2; c < d; ++c)
       for (int b = 1; b < c; ++b)
-        for (int a = 0; a < b; ++a) t.v[at++] = (unsigned short)(1 << d | 1 << c | 1 << b | 1 << a);
+        for (int a = 0; a < b; ++a) t.few[at++] = (unsigned short)(pair_index(a, b) | pair_index(c, d) << 8);
   return t;
 }
 static __device__ const FewOut kFew = make_few_out();
 
 struct SchedShared {
-  int4 lo[256 * kSchedRow / 4], hi[256 * kSchedRow / 4];   // summed loads of every subset of the two halves of the pool
-  alignas(16) int load[EB_MAX_MB][EB_MAX_D];               // zero beyond n_mb and D
+  int4 lo[256 * kSchedRow / 4], hi[256 * kSchedRow / 4];   // summed loads of every subset of the two halves of the pool; or of pairs, and kFew
+  alignas(16) int load[EB_MAX_MB][kSchedRow];              // zero beyond n_mb and D
   int nibble[4][16][EB_MAX_D];                             // summed loads of every subset of four pool positions
   unsigned char by_count[256];                             // kByCount
   int member[EB_MAX_MB];                                   // micro-batch of every pool position
@@ -178,7 +190,10 @@ struct SchedShared {
   uint32_t run;
   bool last;                                               // this block is the last one of the grid to arrive
   long long seq_w[EB_MAX_D];
+  __device__ __forceinline__ FewOut& few() { return *reinterpret_cast<FewOut*>(hi); }
+  __device__ __forceinline__ const FewOut& few() const { return *reinterpret_cast<const FewOut*>(hi); }
 };
+static_assert(sizeof(FewOut) <= sizeof(SchedShared::hi), "the two ways through a large pool share the space");
 
 // The best subset a thread has seen.
 template <typename W>
@@ -242,36 +257,32 @@ __device__ __forceinline__ Cand maxutil_small(const SchedShared& s, int D, int n
   }
   return best.cand();
 }
-// All but at most kFewOut of up to 16 members.
+// All but at most kFewOut of up to 16 members; s.lo holds the loads of the pairs.
 template <typename W>
 __device__ __forceinline__ Cand maxutil_few_out(const SchedShared& s, int D, int np, int m) {
   const int tid = threadIdx.x, lane = tid & 31, quads = (D + 3) / 4, out = np - m;
+  const FewOut& few = s.few();
   W mine = 0;   // total load of device `lane` mod 16
   for (int k = 0; k < np; ++k) mine += s.load[s.member[k]][lane & 15];
   const int n1 = np, n2 = n1 * (np - 1) / 2, n3 = n2 * (np - 2) / 3, n4 = n3 * (np - 3) / 4;
   const int end0 = 1, end1 = end0 + (out >= 1 ? n1 : 0), end2 = end1 + (out >= 2 ? n2 : 0), end3 = end2 + (out >= 3 ? n3 : 0),
             end4 = end3 + (out >= 4 ? n4 : 0);
   BestSubset<W> best;
-  for (int c0 = 0; c0 < end4; c0 += kSchedThreads) {   // whole warps go on together: the totals travel by shuffles
-    const int c = c0 + tid;
-    if (c - lane >= end4) break;
+#pragma unroll 1
+  for (int c = tid; c - lane < end4; c += kSchedThreads) {   // whole warps go on together: the totals travel by shuffles
     const int at = c < end0 ? 0 : c < end1 ? c : c < end2 ? c - end1 + 17 : c < end3 ? c - end2 + 137 : c - end3 + 697;
-    const unsigned off = c < end4 ? kFew.v[at] : 0u;
+    const int set = c < end4 ? few.few[at] : 0, p = set & 255, r = set >> 8;
+    const int4 *x = s.lo + p * (kSchedRow / 4), *y = s.lo + r * (kSchedRow / 4);
     W num = 0, peak = 0;
-    for (int q = 0; q < quads; ++q) {
-      W w0 = __shfl_sync(0xffffffffu, mine, 4 * q), w1 = __shfl_sync(0xffffffffu, mine, 4 * q + 1), w2 = __shfl_sync(0xffffffffu, mine, 4 * q + 2),
-        w3 = __shfl_sync(0xffffffffu, mine, 4 * q + 3);
-      for (unsigned left = off; left; left &= left - 1) {
-        const int4 v = reinterpret_cast<const int4*>(s.load[s.member[__ffs(left) - 1]])[q];
-        w0 -= v.x;
-        w1 -= v.y;
-        w2 -= v.z;
-        w3 -= v.w;
-      }
+    for (int q = 0; q < quads; ++q) {   // entries beyond D are zero
+      const int4 a = x[q], b = y[q];
+      const W w0 = __shfl_sync(0xffffffffu, mine, 4 * q) - ((W)a.x + b.x), w1 = __shfl_sync(0xffffffffu, mine, 4 * q + 1) - ((W)a.y + b.y),
+              w2 = __shfl_sync(0xffffffffu, mine, 4 * q + 2) - ((W)a.z + b.z), w3 = __shfl_sync(0xffffffffu, mine, 4 * q + 3) - ((W)a.w + b.w);
       num += (w0 + w1) + (w2 + w3);
-      const W p = max4(w0, w1, w2, w3);
-      peak = p > peak ? p : peak;
+      const W p4 = max4(w0, w1, w2, w3);
+      peak = p4 > peak ? p4 : peak;
     }
+    const unsigned off = few.pair[p] | few.pair[r];
     if (c < end4) best.offer(num, peak, D, np - __popc(off), ((1u << np) - 1u) ^ off);
   }
   return best.cand();
@@ -312,29 +323,45 @@ __device__ __forceinline__ Cand maxutil_halves(const SchedShared& s, int D, int 
   return best.cand();
 }
 
-// Which micro-batches are in the pool; before the barrier behind the writes of s.load.
-__device__ __forceinline__ void schedule_members(SchedShared& s, uint32_t pool_mask) {
+// Whether a schedule goes the way of maxutil_few_out.
+__host__ __device__ __forceinline__ bool few_out(int np, int m, int policy) { return policy == EB_POLICY_MAXUTIL && np > 10 && np > m && np - m <= kFewOut; }
+// Which micro-batches are in the pool, and the tables that the schedule takes; before the barrier behind the writes of s.load.
+__device__ __forceinline__ void schedule_prepare(SchedShared& s, uint32_t pool_mask, int m, int policy) {
   const int tid = threadIdx.x;
   if (tid < EB_MAX_MB && ((pool_mask >> tid) & 1u)) s.member[__popc(pool_mask & ((1u << tid) - 1u))] = tid;
+  static_assert(sizeof(FewOut) / 16 <= kSchedThreads, "a thread per 16 bytes");
+  if (few_out(__popc(pool_mask), m, policy) && tid < (int)sizeof(FewOut) / 16)
+    reinterpret_cast<int4*>(&s.few())[tid] = reinterpret_cast<const int4*>(&kFew)[tid];
 }
 __device__ __forceinline__ bool wide_load(int v) { return v < 0 || v > kNarrowLoad; }
 
-// Chooses the run set from s.load.  All kSchedThreads threads of the block call it after a barrier behind the writes of
-// s.load and schedule_members; `any_wide` (uniform) unless no load is a wide_load; `block` of n_blocks.  True: *run is the run set;
-// false, with n_blocks > 1 under MaxUtil over a large pool: *mine is this block's candidate.  In every thread.
-__device__ __forceinline__ bool schedule_block(SchedShared& s, int D, uint32_t pool_mask, int m, int policy, bool any_wide, int block, int n_blocks,
-                                               uint32_t* run, Cand* mine) {
+// Chooses the run set from s.load and returns it.  All kSchedThreads threads of the block call it after a barrier behind the writes
+// of s.load and schedule_prepare; `any_wide` (uniform) unless no load is a wide_load; `block` of n_blocks.  With n_blocks > 1, which
+// is for MaxUtil over a large pool, s.best[0] is this block's candidate.  Ends with a barrier.
+__device__ __forceinline__ uint32_t schedule_block(SchedShared& s, int D, uint32_t pool_mask, int m, int policy, bool any_wide, int block, int n_blocks) {
   const int tid = threadIdx.x;
   const int np = __popc(pool_mask);
   if (np <= m || policy == EB_POLICY_ALL) {
-    *run = pool_mask;
-    return true;
+    __syncthreads();
+    return pool_mask;
   }
   if (policy == EB_POLICY_MAXUTIL) {
     Cand best;
     if (np <= 10) {
       best = any_wide ? maxutil_small<long long>(s, D, np, m) : maxutil_small<int>(s, D, np, m);
-    } else if (np - m <= kFewOut) {
+    } else if (few_out(np, m, policy)) {
+      int* pairs = reinterpret_cast<int*>(s.lo);
+      for (int i = tid; i < kPairs * EB_MAX_D; i += kSchedThreads) {
+        const int p = i / EB_MAX_D, d = i % EB_MAX_D;
+        const unsigned bits = s.few().pair[p];
+        int v = 0;
+        if (bits >> np == 0) {   // the other pairs are in no set that is looked at
+          if (bits) v = s.load[s.member[__ffs(bits) - 1]][d];
+          if (bits & (bits - 1)) v += s.load[s.member[31 - __clz(bits)]][d];
+        }
+        pairs[p * kSchedRow + d] = v;
+      }
+      __syncthreads();
       best = any_wide ? maxutil_few_out<long long>(s, D, np, m) : maxutil_few_out<int>(s, D, np, m);
     } else {
       const int nlo = 8, nhi = np - nlo;
@@ -358,14 +385,21 @@ __device__ __forceinline__ bool schedule_block(SchedShared& s, int D, uint32_t p
       __syncthreads();
       best = any_wide ? maxutil_halves<long long>(s, D, np, m, block, n_blocks) : maxutil_halves<int>(s, D, np, m, block, n_blocks);
     }
-    // warp then block reduction under the total order (any reduction order gives the same winner); every warp makes the second
+    // warp then block reduction under the total order (any reduction order gives the same winner), the second by one warp: all at
+    // once, each for itself, they were in each other's way (800 to 1700 cycles instead of 300)
     best = any_wide ? warp_best(best) : warp_best_narrow(best);
     if ((tid & 31) == 0) s.best[tid >> 5] = best;
     __syncthreads();
-    best = any_wide ? warp_best(s.best[tid & 31]) : warp_best_narrow(s.best[tid & 31]);
-    *run = run_mask_of(s.member, np, best);
-    *mine = best;
-    return n_blocks == 1;
+    if (tid < 32) {
+      best = any_wide ? warp_best(s.best[tid]) : warp_best_narrow(s.best[tid]);
+      const uint32_t mask = run_mask_of(s.member, np, best);
+      if (tid == 0) {
+        s.run = mask;
+        s.best[0] = best;
+      }
+    }
+    __syncthreads();
+    return s.run;
   }
   if (tid < 32) {
     // CumUtil / DiffPeak: ascending pool members, the first always taken; lane d holds the joint load of device d
@@ -434,8 +468,7 @@ __device__ __forceinline__ bool schedule_block(SchedShared& s, int D, uint32_t p
     if (lane == 0) s.run = chosen;
   }
   __syncthreads();
-  *run = s.run;
-  return true;
+  return s.run;
 }
 
 // schedule_block by all blocks of the grid: each leaves its best candidate in global memory and the block that arrives last
@@ -446,11 +479,11 @@ struct SchedGrid {
 };
 __device__ __forceinline__ bool schedule_grid(SchedShared& s, int D, uint32_t pool_mask, int m, int policy, bool any_wide, const SchedGrid& g,
                                               uint32_t* run) {
-  Cand mine;
-  if (schedule_block(s, D, pool_mask, m, policy, any_wide, blockIdx.x, gridDim.x, run, &mine)) return blockIdx.x == 0;
+  *run = schedule_block(s, D, pool_mask, m, policy, any_wide, blockIdx.x, gridDim.x);
+  if (gridDim.x == 1) return true;
   const int tid = threadIdx.x;
   if (tid == 0) {
-    g.best[blockIdx.x] = mine;
+    g.best[blockIdx.x] = s.best[0];
     __threadfence();
     s.last = atomicAdd(g.arrived, 1u) == gridDim.x - 1;
   }
@@ -480,7 +513,7 @@ __device__ __forceinline__ bool schedule_grid(SchedShared& s, int D, uint32_t po
 constexpr int kMaxSchedBlocks = 1 << (EB_MAX_MB - 13);
 inline int sched_blocks(uint32_t pool_mask, int m, int policy) {
   const int np = __builtin_popcount(pool_mask);
-  return policy == EB_POLICY_MAXUTIL && np - m > kFewOut && np > 13 ? 1 << (np - 13) : 1;
+  return policy == EB_POLICY_MAXUTIL && np > m && np > 13 && !few_out(np, m, policy) ? 1 << (np - 13) : 1;
 }
 // Subsets that MaxUtil looks at: those of at least m members.
 inline int sched_subsets(uint32_t pool_mask, int m) {
