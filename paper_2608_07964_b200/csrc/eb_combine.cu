@@ -31,10 +31,11 @@ template <int KS>
 __global__ void __launch_bounds__(kThreads)
 combine_kernel(int n_tok, int H, int K, int team, const uint4* __restrict__ yp, const int32_t* __restrict__ pos,
                const float* __restrict__ topk_w, const uint4* residual, uint4* out) {   // residual may be `out` itself
-  EB_GRID_DEP_SYNC();
   const int t = blockIdx.x * (kThreads / team) + threadIdx.x / team;   // team >= 32: a warp serves one token
-  if (t >= n_tok) return;
   const int lane = threadIdx.x & 31;
+  if (t < n_tok && lane < 3) touch_ahead(lane == 0 ? (const void*)(pos + (size_t)t * KS) : lane == 1 ? (const void*)(topk_w + (size_t)t * K) : (const void*)(out + (size_t)t * (H / 8)));
+  EB_GRID_DEP_SYNC();
+  if (t >= n_tok) return;
   // lane s fetches slot s once per warp; the values are broadcast with shuffles
   const int my_pos = lane < KS ? pos[(size_t)t * KS + lane] : -1;
   const float my_w = lane < K ? topk_w[(size_t)t * K + lane] : 1.0f;

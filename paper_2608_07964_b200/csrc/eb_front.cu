@@ -24,9 +24,15 @@ template <int PL>
 __global__ void __launch_bounds__(kChunkThreads, PL <= 2 ? 2 : 1)
 front_kernel(ModelParams mp, BatchParams bp, uint32_t pool_mask, uint32_t route_mask, const float* __restrict__ logits,
              int32_t* __restrict__ topk_idx, float* __restrict__ topk_w, int32_t* __restrict__ chunk_hist) {
-  EB_GRID_DEP_SYNC();
   __shared__ int s_hist[EB_MAX_E];
   const int c = blockIdx.x, j = mb_of_chunk(bp, c);
+  const int t = bp.tok_off[j] + (c - bp.chunk_off[j]) * 32 + (threadIdx.x >> 5), lane = threadIdx.x & 31;   // a warp per token
+  if (t < bp.tok_off[j + 1]) {
+    if (lane * 32 < mp.E) touch_ahead(logits + (size_t)t * mp.E + lane * 32);
+    if (lane == 8) touch_ahead(topk_idx + (size_t)t * mp.K);
+    if (lane == 9) touch_ahead(topk_w + (size_t)t * mp.K);
+  }
+  EB_GRID_DEP_SYNC();
   const bool routed = (route_mask >> j) & 1u;
   if (!routed && !((pool_mask >> j) & 1u)) return;
   route_chunk<PL>(mp, bp, c, j, routed, logits, topk_idx, topk_w, s_hist);
@@ -349,9 +355,9 @@ struct ScatterArgs {
 template <int TB>
 __global__ void __launch_bounds__(kScatterThreads)
 scatter_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ BatchParams bp, const __grid_constant__ ScatterArgs a) {
-  EB_GRID_DEP_SYNC();
   extern __shared__ int s_dyn[];
   if ((int)blockIdx.x < a.fill_blocks) {
+    EB_GRID_DEP_SYNC();
     fill_tiles(mp, a.group_off, a.group_w, a.list, s_dyn, blockIdx.x, a.fill_blocks);
     return;
   }
@@ -371,6 +377,14 @@ scatter_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ B
   const int c0 = bp.tok_off[j] + (c - bp.chunk_off[j]) * 32;      // first token of the chunk
   const int t0 = c0 + part % (32 / TB) * TB;                      // and of this part
   const int nt = min(TB, bp.tok_off[j + 1] - t0);
+  if (nt > 0) {
+    // a line of 128 bytes per thread
+    for (int i = tid * 8; i < nt * vec; i += kScatterThreads * 8) touch_ahead(a.x + (size_t)t0 * vec + i);
+    if (tid * 32 < E) touch_ahead(a.mb_base + j * E + tid * 32);
+    if (tid == 32) touch_ahead(a.topk_idx + (size_t)c0 * K);
+    if (tid == 64) touch_ahead(a.pos + (size_t)t0 * KS);
+  }
+  EB_GRID_DEP_SYNC();
   if (nt <= 0) return;
   const uint32_t run = a.res->run_mask;
   if (!((run >> j) & 1u)) {
