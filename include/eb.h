@@ -165,6 +165,22 @@ eb_status eb_route(eb_ctx* ctx, void* stream, const eb_batch* batch, uint32_t ro
 eb_status eb_schedule(eb_ctx* ctx, void* stream, const eb_batch* batch, int32_t m, eb_policy policy,
                       const int32_t* mb_load, eb_sched_result* d_res, eb_sched_result* h_res);
 
+/* The schedule in host memory as soon as it is made, without waiting for the rest of a step.  With a ticket other than 0,
+ * eb_schedule and eb_step on this context (and graphs captured from them, whenever they are replayed) also leave the result and the
+ * loads it was made from in a record in pinned host memory, which the context owns and allocates on the first such call, and mark it
+ * with the ticket last.  Setting a ticket clears the mark, so it must not be done while marked work is in flight that is yet to
+ * be waited for.  Ticket 0 (the state after eb_create): later calls do not write the record; the mark stays.
+ * eb_schedule_wait blocks until the mark is `ticket` and copies the record; should all work on `stream` be over without it, it
+ * copies d_res and mb_load from the device instead.  h_load: host, [n_mb, D], or NULL. */
+eb_status eb_watch_schedule(eb_ctx* ctx, uint32_t ticket);
+eb_status eb_schedule_wait(eb_ctx* ctx, void* stream, uint32_t ticket, int32_t n_mb, const eb_sched_result* d_res,
+                           const int32_t* mb_load, eb_sched_result* h_res, int32_t* h_load);
+
+/* Device-to-device copy on `stream`, for loops that hand the library many small pieces (logits of one micro-batch at a time).
+ * The two ranges are the same or
+ * do not overlap. */
+eb_status eb_copy(eb_ctx* ctx, void* stream, void* dst, const void* src, size_t bytes);
+
 /* Dispatch on one GPU (Section 2.2; stands in for the first all-to-all): histogram of the chosen micro-batches' assignments per
  * group, exclusive prefix sum, stable ranks, and a 16-byte-vector gather of the token rows into
  * group-contiguous order.  Reads the run mask from d_res on the device.

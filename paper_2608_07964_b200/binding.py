@@ -44,7 +44,7 @@ class EbStepBuffers(C.Structure):
                                           "residual")]
 
 
-SYMBOLS = ["eb_create", "eb_destroy", "eb_bind_weights", "eb_workspace_bytes", "eb_set_workspace",
+SYMBOLS = ["eb_copy", "eb_watch_schedule", "eb_schedule_wait", "eb_create", "eb_destroy", "eb_bind_weights", "eb_workspace_bytes", "eb_set_workspace",
            "eb_rows_capacity", "eb_groups_capacity", "eb_route", "eb_schedule", "eb_permute",
            "eb_expert_ffn_grouped", "eb_expert_ffn_device", "eb_combine", "eb_combine_residual", "eb_step", "eb_step_host",
            "eb_step_host_submit", "eb_step_host_wait",
@@ -79,6 +79,9 @@ def load_library(path: Optional[str] = None) -> C.CDLL:
     lib.eb_groups_capacity.argtypes = [vp]
     lib.eb_route.argtypes = [vp, vp, C.POINTER(EbBatch), u32, vp, vp, vp, vp, vp]
     lib.eb_schedule.argtypes = [vp, vp, C.POINTER(EbBatch), i32, i32, vp, vp, vp]
+    lib.eb_copy.argtypes = [vp, vp, vp, vp, C.c_size_t]
+    lib.eb_watch_schedule.argtypes = [vp, u32]
+    lib.eb_schedule_wait.argtypes = [vp, vp, u32, i32, vp, vp, vp, vp]
     lib.eb_permute.argtypes = [vp, vp, C.POINTER(EbBatch), vp, vp, vp, vp, vp, vp, vp, vp, vp]
     lib.eb_expert_ffn_grouped.argtypes = [vp, vp, vp, vp, vp, vp, vp]
     lib.eb_expert_ffn_device.argtypes = [vp, vp, vp, vp, vp, vp, vp, i32]
@@ -124,7 +127,8 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    # the handle of torch.cuda.current_stream() without the object around it: 0.2 us a call instead of 3.2
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 class Batch:
@@ -234,6 +238,34 @@ class MoEStep:
         self._check(self.lib.eb_schedule(self.ctx, _stream(), C.byref(batch.c), m, policy, ld.data_ptr(),
                                          self.sched.data_ptr(), C.addressof(h) if to_host else None))
         return _sched_dict(h, self.D) if to_host else None
+
+    def copy(self, dst: torch.Tensor, src: torch.Tensor):
+        """dst.copy_(src) on the current stream.  The plain case - one device, type and shape, both contiguous and apart - is a kernel
+        of the library (4.3 us of host time instead of 5.9)."""
+        if (type(src) is torch.Tensor and src.dtype is dst.dtype and src.layout is torch.strided and src.device == dst.device and src.shape == dst.shape
+                and dst.is_cuda and src.is_contiguous() and dst.is_contiguous() and not src.requires_grad and not src.is_neg()):
+            d, s, n = dst.data_ptr(), src.data_ptr(), dst.numel() * dst.element_size()
+            if d == s or abs(d - s) >= n:
+                self._check(self.lib.eb_copy(self.ctx, _stream(), d, s, n))
+                return
+        dst.copy_(src)
+
+    def watch_schedule(self, ticket: int):
+        """With a ticket other than 0 the schedules of this context are left in host memory too, see `schedule_wait`."""
+        self._check(self.lib.eb_watch_schedule(self.ctx, ticket))
+
+    def schedule_wait(self, ticket: int, n_mb: int) -> Dict:
+        """The schedule marked with `ticket` as soon as it is made, whatever the step has yet to do; with the load vectors it was
+        made from under "loads"."""
+        if not hasattr(self, "_wait_res"):
+            self._wait_res, self._wait_load = EbSchedResult(), (C.c_int32 * (EB_MAX_MB * self.D))()
+        h, ld = self._wait_res, self._wait_load
+        self._check(self.lib.eb_schedule_wait(self.ctx, _stream(), ticket, n_mb, self.sched.data_ptr(), self.mb_load.data_ptr(),
+                                              C.addressof(h), C.addressof(ld)))
+        res = _sched_dict(h, self.D)
+        v = ld[:n_mb * self.D]
+        res["loads"] = [v[j * self.D:(j + 1) * self.D] for j in range(n_mb)]
+        return res
 
     def eb_permute(self, batch: Batch, x: Optional[torch.Tensor] = None):
         xx = self.x if x is None else x

@@ -177,6 +177,7 @@ extern "C" eb_status eb_destroy(eb_ctx* c) {
   if (c->d_tables) cudaFree(c->d_tables);
   if (c->d_status) cudaFree(c->d_status);
   if (c->d_sched_scratch) cudaFree(c->d_sched_scratch);
+  if (c->watch_rec) cudaFreeHost(c->watch_rec);
   for (int i = 0; i < 2 * EBK_COUNT; ++i)
     if (c->ev[i]) cudaEventDestroy(c->ev[i]);
   for (int i = 0; i < EB_HOST_SLOTS; ++i) {
@@ -337,6 +338,32 @@ extern "C" eb_status eb_step_host_wait(eb_ctx* c, int32_t slot) {
   if (!c->slot_busy[slot]) return EB_OK;
   c->slot_busy[slot] = false;
   EB_CUDA(c, cudaEventSynchronize(c->ev_out[slot]));
+  return EB_OK;
+}
+
+namespace {
+// Bound by the launch: a cudaMemcpyAsync between two places of one device takes the host 4 us, this 2.
+template <typename V>
+__global__ void __launch_bounds__(256) copy_kernel(V* dst, const V* src, size_t n) {
+  EB_GRID_DEP_SYNC();
+  for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (size_t)gridDim.x * 256) dst[i] = src[i];
+}
+template <typename V>
+cudaError_t launch_copy(const eb_ctx* c, cudaStream_t st, void* dst, const void* src, size_t bytes) {
+  const size_t n = bytes / sizeof(V), blocks = std::min<size_t>((n + 255) / 256, 8 * (size_t)c->num_sms);
+  return ebi_launch(copy_kernel<V>, dim3((unsigned)blocks), dim3(256), 0, st, (V*)dst, (const V*)src, n);
+}
+}  // namespace
+
+extern "C" eb_status eb_copy(eb_ctx* c, void* stream, void* dst, const void* src, size_t bytes) {
+  if (!c) return EB_ERR_INVALID_ARG;
+  if (bytes && (!dst || !src)) return ebi_fail(c, EB_ERR_INVALID_ARG, "null pointer");
+  if (eb_status ds = ebi_check_device(c)) return ds;
+  const uintptr_t bits = (uintptr_t)dst | (uintptr_t)src | bytes;
+  if (bytes == 0) return EB_OK;
+  EB_LAUNCH(c, "copy", bits % 16 == 0  ? launch_copy<uint4>(c, (cudaStream_t)stream, dst, src, bytes)
+                       : bits % 4 == 0 ? launch_copy<uint32_t>(c, (cudaStream_t)stream, dst, src, bytes)
+                                       : launch_copy<unsigned char>(c, (cudaStream_t)stream, dst, src, bytes));
   return EB_OK;
 }
 

@@ -97,6 +97,7 @@ struct TablesArgs {
   int32_t *group_off, *group_w, *step_meta;
   TilePlan plan;
   SchedGrid sched;
+  ScheduleWatch watch;
 };
 
 // i / E for i < 2^16 (E <= 256): one multiplication by ceil(2^32 / E); larger i take the division
@@ -209,7 +210,7 @@ tables_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ Ba
     if (lane < EB_MAX_MB) s_rank[lane] = (run >> lane) & 1u ? __popc(active & ((1u << s_layer_of[lane]) - 1u)) : -1;
     if (lane == 0) s_nl = __popc(active);
   }
-  if (warp == 1) write_schedule(sc, D, a.pool_mask, run, a.res);
+  if (warp == 1) write_schedule(sc, D, a.pool_mask, run, a.res, a.watch);
   __syncthreads();
   const int nl = s_nl, G = nl * (E + D * S);
 
@@ -566,7 +567,7 @@ eb_status ebi_front_run(eb_ctx* c, cudaStream_t st, const BatchParams& bp, uint3
                                       (const int32_t*)c->chunk_hist, c->chunk_base, c->chunk_seg));
     const TablesArgs a{pool_mask, route_mask, (int)m, (int)policy, c->chunk_hist, sums ? c->chunk_seg : nullptr, c->chunk_base, c->seg_base,
                        c->mb_base, b->mb_load, b->mb_cnt, seg, layers_of(bp), b->sched, b->group_off, b->group_w, b->step_meta, tile_plan_of(c),
-                       sched_grid_of(c)};
+                       sched_grid_of(c), schedule_watch_of(c)};
     int blocks = sched_blocks(pool_mask, m, policy);
     if ((int64_t)sched_subsets(pool_mask, m) * (blocks - 1) / blocks < kSchedSubsets) blocks = 1;
     EB_LAUNCH(c, "tables", ebi_launch(tables_kernel, dim3(blocks), dim3(kSchedThreads), tables_smem(bp.n_mb, g.E, bp.n_mb * (g.E + g.D * g.S)), st,

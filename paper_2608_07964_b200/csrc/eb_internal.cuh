@@ -56,6 +56,18 @@ struct ModelParams {
   const int32_t* e_local;   // [E] index of the expert among its device's experts
 };
 
+// Record of a schedule in pinned host memory (eb_watch_schedule).
+struct ScheduleRecord {
+  eb_sched_result res;
+  int32_t load[EB_MAX_MB * EB_MAX_D];
+  uint32_t ticket;   // written last
+};
+// Where a kernel leaves it: null: nowhere.
+struct ScheduleWatch {
+  ScheduleRecord* rec;
+  uint32_t ticket;
+};
+
 struct eb_ctx {
   eb_config cfg;
   int device = 0;
@@ -64,6 +76,8 @@ struct eb_ctx {
   int32_t* d_tables = nullptr;  // e2d | dev_off | dev_list | e_local
   ModelParams mp;
   int32_t* d_status = nullptr;
+  ScheduleRecord* watch_rec = nullptr;   // pinned host memory, allocated on first use
+  uint32_t watch_ticket = 0;
   char* d_sched_scratch = nullptr;  // per-block candidates and arrival counter of the multi-block scheduler
 
   const bf16* w_gate = nullptr;
@@ -106,6 +120,8 @@ struct eb_ctx {
 
   std::string err;
 };
+
+inline ScheduleWatch schedule_watch_of(const eb_ctx* c) { return ScheduleWatch{c->watch_ticket ? c->watch_rec : nullptr, c->watch_ticket}; }
 
 int32_t ebi_rows_cap(const eb_ctx* c);
 int32_t ebi_groups_cap(const eb_ctx* c);

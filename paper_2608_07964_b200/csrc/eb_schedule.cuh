@@ -529,8 +529,9 @@ inline SchedGrid sched_grid_of(const eb_ctx* c) {
   return SchedGrid{(Cand*)c->d_sched_scratch, (unsigned*)(c->d_sched_scratch + kMaxSchedBlocks * sizeof(Cand))};
 }
 
-// The result record, by one warp.
-__device__ __forceinline__ void write_schedule(const SchedShared& s, int D, uint32_t pool_mask, uint32_t run, eb_sched_result* __restrict__ res) {
+// The result record, by one warp; and its copy in host memory, if that is watched.
+__device__ __forceinline__ void write_schedule(const SchedShared& s, int D, uint32_t pool_mask, uint32_t run, eb_sched_result* res,
+                                               const ScheduleWatch& watch) {
   const int tid = threadIdx.x & 31;
   // lane d sums the chosen micro-batches' load on device d (zero beyond D); the warp adds and maximises
   long long v = 0;
@@ -538,6 +539,7 @@ __device__ __forceinline__ void write_schedule(const SchedShared& s, int D, uint
 #pragma unroll
     for (int j = 0; j < EB_MAX_MB; ++j) v += ((run >> j) & 1u) ? s.load[j][tid] : 0;
     res->joint_load[tid] = (int32_t)v;
+    if (watch.rec) watch.rec->res.joint_load[tid] = (int32_t)v;
   }
   long long num = v, peak = v;
 #pragma unroll
@@ -547,12 +549,20 @@ __device__ __forceinline__ void write_schedule(const SchedShared& s, int D, uint
     peak = p2 > peak ? p2 : peak;
   }
   if (tid == 0) {
-    res->run_mask = run;
-    res->defer_mask = pool_mask & ~run;
-    res->n_run = __popc(run);
-    res->status = EB_OK;
-    res->util_num = num;
-    res->util_den = (long long)D * peak;
+    for (eb_sched_result* r = res; r; r = watch.rec && r == res ? &watch.rec->res : nullptr) {
+      r->run_mask = run;
+      r->defer_mask = pool_mask & ~run;
+      r->n_run = __popc(run);
+      r->status = EB_OK;
+      r->util_num = num;
+      r->util_den = (long long)D * peak;
+    }
+  }
+  if (watch.rec) {
+    for (int i = tid; i < EB_MAX_MB * D; i += 32) watch.rec->load[i] = s.load[i / D][i % D];
+    __threadfence_system();
+    __syncwarp();
+    if (tid == 0) asm volatile("st.release.sys.global.u32 [%0], %1;" ::"l"(&watch.rec->ticket), "r"(watch.ticket) : "memory");
   }
 }
 

@@ -2,7 +2,7 @@
 
 `run_load_trace` drives the scheduling loop of Algorithm 1 on the GPU in load-trace mode: each
 step routes the micro-batches that just advanced (eb_route with a route mask, so deferred ones
-keep their routing), schedules (eb_schedule, result copied to the host to advance the layer
+keep their routing), schedules (eb_schedule, the result left in host memory by the kernel to advance the layer
 counters) and records the run set and the joint per-device load; the expert pass is skipped.
 `run_full` does the same but executes every step completely (eb_step: what the five calls compute, the aggregation
 adding the residual h <- h + MLP(h) in place), optionally replaying each step from a CUDA graph.
@@ -12,6 +12,7 @@ no routing or scheduling arithmetic: those run in the CUDA kernels.
 """
 from __future__ import annotations
 
+import itertools
 from typing import Callable, Dict, List, Optional
 
 import torch
@@ -19,16 +20,20 @@ import torch
 from . import binding as B
 
 
+# marks of watched schedules: each names one launch, or one graph, of the process
+_tickets = itertools.count(1)
+
+
 def _logit_rows(step: "B.MoEStep", tok_off: List[int]) -> List[torch.Tensor]:
     return [step.logits[tok_off[j]:tok_off[j + 1]] for j in range(len(tok_off) - 1)]
 
 
-def _copy_logits(rows: List[torch.Tensor], logits_of: Callable[[int, int], torch.Tensor], layer: List[int], mask: int) -> None:
+def _copy_logits(step: "B.MoEStep", rows: List[torch.Tensor], logits_of: Callable[[int, int], torch.Tensor], layer: List[int], mask: int) -> None:
     """Logits of the micro-batches in `mask` at their current layers, into their rows.  Each result is taken over before
     the next one is asked for: `logits_of` may fill and return one and the same buffer every time."""
     for j, row in enumerate(rows):
         if (mask >> j) & 1:
-            row.copy_(logits_of(j, layer[j]))
+            step.copy(row, logits_of(j, layer[j]))
 
 
 def run_load_trace(step: "B.MoEStep", tok_off: List[int], L: int, m: int, policy: int,
@@ -41,25 +46,32 @@ def run_load_trace(step: "B.MoEStep", tok_off: List[int], L: int, m: int, policy
     route_mask = pool
     steps: List[Dict] = []
     rows = _logit_rows(step, tok_off)
-    while pool:
-        _copy_logits(rows, logits_of, layer, route_mask)
-        batch = B.Batch(tok_off, [min(l, L - 1) for l in layer], pool)
-        if route_mask:
-            step.eb_route(batch, route_mask)
-        res = step.eb_schedule(batch, m, policy, to_host=True)
-        run = res["run_mask"]
-        loads = step.mb_load[:N].cpu().tolist()
-        steps.append(dict(pool=pool, run_mask=run, layers={j: layer[j] for j in range(N) if (run >> j) & 1},
-                          joint_load=res["joint_load"], util_num=res["util_num"], util_den=res["util_den"],
-                          member_loads={j: loads[j] for j in range(N) if (run >> j) & 1}))
-        route_mask = 0
-        for j in range(N):
-            if (run >> j) & 1:
-                layer[j] += 1
-                if layer[j] >= L:
-                    pool &= ~(1 << j)
-                else:
-                    route_mask |= 1 << j
+    try:
+        while pool:
+            _copy_logits(step, rows, logits_of, layer, route_mask)
+            batch = B.Batch(tok_off, [min(l, L - 1) for l in layer], pool)
+            ticket = next(_tickets)
+            step.watch_schedule(ticket)
+            if route_mask:
+                step.eb_route(batch, route_mask)
+            step.eb_schedule(batch, m, policy)
+            # schedule and loads come by way of host memory, not by two copies with a wait each
+            res = step.schedule_wait(ticket, N)
+            run, loads = res["run_mask"], res["loads"]
+            steps.append(dict(pool=pool, run_mask=run, layers={j: layer[j] for j in range(N) if (run >> j) & 1},
+                              joint_load=res["joint_load"], util_num=res["util_num"], util_den=res["util_den"],
+                              member_loads={j: loads[j] for j in range(N) if (run >> j) & 1}))
+            route_mask = 0
+            for j in range(N):
+                if (run >> j) & 1:
+                    layer[j] += 1
+                    if layer[j] >= L:
+                        pool &= ~(1 << j)
+                    else:
+                        route_mask |= 1 << j
+    finally:
+        step.watch_schedule(0)
+    torch.cuda.current_stream().synchronize()
     return steps
 
 
@@ -74,21 +86,30 @@ class StepGraphs:
         self.graphs: Dict = {}
         self.hits = self.captures = 0
 
-    def run(self, layers: List[int], pool: int, route_mask: int, m: int, policy: int):
+    def run(self, layers: List[int], pool: int, route_mask: int, m: int, policy: int) -> int:
+        """Launches the step; returns the ticket that its schedule is marked with (MoEStep.schedule_wait)."""
         key = (pool, tuple(layers), route_mask, m, policy)
         g = self.graphs.get(key)
         if g is None:
             if len(self.graphs) >= self.capacity:
                 self.graphs.pop(next(iter(self.graphs)))
             batch = B.Batch(self.tok_off, layers, pool)
+            ticket = next(_tickets)
             graph = torch.cuda.CUDAGraph()
-            with torch.cuda.graph(graph):
-                self.step.eb_step(batch, m, policy, route_mask, in_place=True)
-            g = self.graphs[key] = (graph, batch)
+            self.step.watch_schedule(ticket)
+            try:
+                with torch.cuda.graph(graph):
+                    self.step.eb_step(batch, m, policy, route_mask, in_place=True)
+            finally:
+                self.step.watch_schedule(0)
+            g = self.graphs[key] = (graph, batch, ticket)
             self.captures += 1
         else:
             self.hits += 1
+            self.step.watch_schedule(g[2])   # clears the mark of the last replay
+            self.step.watch_schedule(0)
         g[0].replay()
+        return g[2]
 
 
 def run_full(step: "B.MoEStep", tok_off: List[int], L: int, m: int, policy: int,
@@ -109,20 +130,24 @@ def run_full(step: "B.MoEStep", tok_off: List[int], L: int, m: int, policy: int,
     rows = _logit_rows(step, tok_off)
     t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     t0.record()
+    stream = torch.cuda.current_stream()
     while pool:
-        _copy_logits(rows, logits_of, layer, route_mask)
+        _copy_logits(step, rows, logits_of, layer, route_mask)
         lay = [min(l, L - 1) for l in layer]
         if graphs is not None:
-            graphs.run(lay, pool, route_mask, m, policy)
+            ticket = graphs.run(lay, pool, route_mask, m, policy)
         else:
+            ticket = next(_tickets)
+            step.watch_schedule(ticket)
             step.eb_step(B.Batch(tok_off, lay, pool), m, policy, route_mask, in_place=True)
-        res = step.sched_result()          # the host needs the run set to advance the layer counters
+            step.watch_schedule(0)
+        # the host needs the run set to advance the layer counters, and has it while the expert pass runs; on_step and logits_of
+        # are called when the step is through, as they may look at its results from anywhere
+        res = step.schedule_wait(ticket, N)
         run = res["run_mask"]
         rec = dict(pool=pool, run_mask=run, layers={j: layer[j] for j in range(N) if (run >> j) & 1},
                    joint_load=res["joint_load"], util_num=res["util_num"], util_den=res["util_den"])
         steps.append(rec)
-        if on_step is not None:
-            on_step(len(steps) - 1, rec)
         route_mask = 0
         for j in range(N):
             if (run >> j) & 1:
@@ -131,6 +156,9 @@ def run_full(step: "B.MoEStep", tok_off: List[int], L: int, m: int, policy: int,
                     pool &= ~(1 << j)
                 else:
                     route_mask |= 1 << j
+        stream.synchronize()
+        if on_step is not None:
+            on_step(len(steps) - 1, rec)
     t1.record()
     torch.cuda.synchronize()
     return dict(x=step.x[:T].clone(), steps=steps, ms=t0.elapsed_time(t1), token_layers=T * L)

@@ -1,0 +1,74 @@
+"""Schedules left in host memory, and the copy of logits, against the calls they stand in for."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def _step(n_mb, tokens, E=12, K=3, D=5):
+    from paper_2608_07964_b200 import binding as B
+    step = B.MoEStep(3, E, K, 1, 64, 64, D, [e % D for e in range(E)], n_mb * tokens)
+    g = torch.Generator(device="cuda").manual_seed(7)
+    step.logits.normal_(generator=g)
+    step.x.normal_(generator=g)
+    w = [torch.empty(s, dtype=torch.bfloat16, device="cuda").normal_(0, 0.05, generator=g) for s in ((3, E + 1, 64, 64),) * 3]
+    step.bind_weights(*w)
+    return B, step
+
+
+@pytest.mark.parametrize("n_mb,m,policy", [(1, 1, 0), (4, 3, 0), (11, 8, 0), (16, 12, 0), (16, 1, 0), (9, 2, 1), (9, 2, 2), (5, 1, 3)])
+def test_a_watched_schedule_is_the_one_on_the_device(n_mb, m, policy):
+    B, step = _step(n_mb, 37)
+    batch = B.Batch([37 * j for j in range(n_mb + 1)], [j % 3 for j in range(n_mb)])
+    step.watch_schedule(5)
+    step.eb_step(batch, m, policy)
+    got = step.schedule_wait(5, n_mb)
+    loads = got.pop("loads")
+    assert got == step.sched_result() and loads == step.mb_load[:n_mb].cpu().tolist()
+    step.watch_schedule(6)
+    step.eb_route(batch)
+    step.eb_schedule(batch, m, policy)
+    again = step.schedule_wait(6, n_mb)
+    assert again.pop("loads") == loads and again == got
+    # nothing is watched: the wait falls back on the device's record once the stream is idle
+    step.watch_schedule(9)
+    step.watch_schedule(0)
+    step.eb_step(batch, m, policy)
+    last = step.schedule_wait(9, n_mb)
+    assert last.pop("loads") == loads and last == got
+
+
+def test_a_watched_graph_marks_every_replay():
+    B, step = _step(4, 16)
+    batch = B.Batch([0, 16, 32, 48, 64], [0, 1, 2, 0])
+    step.eb_step(batch, 3)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    step.watch_schedule(3)
+    with torch.cuda.graph(graph):
+        step.eb_step(batch, 3)
+    for seed in range(4):
+        step.logits.normal_(generator=torch.Generator(device="cuda").manual_seed(seed))
+        step.watch_schedule(3)
+        step.watch_schedule(0)
+        graph.replay()
+        got = step.schedule_wait(3, 4)
+        assert got.pop("loads") == step.mb_load[:4].cpu().tolist() and got == step.sched_result()
+
+
+@pytest.mark.parametrize("rows,cols,lead", [(1, 1, 0), (3, 5, 1), (77, 64, 4), (1000, 8, 2), (4097, 64, 0), (31, 12, 3)])
+def test_copy_equals_torch(rows, cols, lead):
+    B, step = _step(1, 1)
+    src = torch.randn(lead + rows * cols, device="cuda")[lead:].view(rows, cols)
+    for d in (0, 1):
+        buf = torch.zeros(d + rows * cols + 8, device="cuda")
+        step.copy(buf[d:d + rows * cols].view(rows, cols), src)
+        assert torch.equal(buf[d:d + rows * cols].view(rows, cols), src)
+        assert not buf[:d].any() and not buf[d + rows * cols:].any()
+    for other in (src.double(), src.cpu(), src.t().contiguous().t(), src[:1].expand(rows, cols)):   # the general way
+        dst = torch.zeros(rows, cols, device="cuda")
+        step.copy(dst, other)
+        assert torch.equal(dst, other.to(dst).contiguous())
+    one = torch.arange(rows * cols + 1, device="cuda", dtype=torch.float32)
+    step.copy(one[1:].view(rows, cols), one[1:].view(rows, cols))   # onto itself
+    assert torch.equal(one, torch.arange(rows * cols + 1, device="cuda", dtype=torch.float32))
