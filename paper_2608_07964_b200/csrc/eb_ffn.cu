@@ -190,8 +190,13 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
   asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ void red_release(int* p) {
-  asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p) : "memory");
+// Counts one up; what the thread has seen written goes before (release: a fence and a relaxed addition).  Between the two, what it has
+// seen is also put before later accesses of TMA units.  A step of 4 x 64 tokens, where every down tile waits for this, 33.5 -> 33.2 us
+// against a __threadfence and a red.release.
+__device__ __forceinline__ void red_publish(int* p) {
+  asm volatile("fence.acq_rel.gpu;" ::: "memory");
+  asm volatile("fence.proxy.async;" ::: "memory");
+  asm volatile("red.relaxed.gpu.global.add.s32 [%0], 1;" ::"l"(p) : "memory");
 }
 // orders ordinary memory accesses with those of the TMA unit
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
@@ -759,9 +764,7 @@ ffn_kernel(const __grid_constant__ FfnParams p) {
         const int i = seq % kParts;
         if (!mbar_wait(part_bar(i), (uses >> i) & 1u, s_abort, status)) goto done;
         uses ^= 1u << i;
-        __threadfence();
-        fence_proxy_async();
-        red_release(p.ready + it.done);
+        red_publish(p.ready + it.done);
       }
     }
   } else {

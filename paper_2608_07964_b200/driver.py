@@ -139,8 +139,10 @@ def run_full(step: "B.MoEStep", tok_off: List[int], L: int, m: int, policy: int,
         else:
             ticket = next(_tickets)
             step.watch_schedule(ticket)
-            step.eb_step(B.Batch(tok_off, lay, pool), m, policy, route_mask, in_place=True)
-            step.watch_schedule(0)
+            try:
+                step.eb_step(B.Batch(tok_off, lay, pool), m, policy, route_mask, in_place=True)
+            finally:
+                step.watch_schedule(0)
         # the host needs the run set to advance the layer counters, and has it while the expert pass runs; on_step and logits_of
         # are called when the step is through, as they may look at its results from anywhere
         res = step.schedule_wait(ticket, N)
