@@ -17,6 +17,8 @@
 //  - otherwise the halves: summed loads of every half-subset in shared memory.  The low halves are kept in the order of their
 //    member counts, so that for every high half the sufficient ones come first.  Sums are 32-bit where the loads allow
 //    it, and the tables' rows are 20 words apart, which 16-byte reads of neighbouring rows go through without bank conflicts.
+// In a step the schedule of 4 members took 6300 cycles by halves and takes 3300 the first way, that of 12 out of 16 18000 and 11000 the
+// second; 10 members is what a subset per thread of the block reaches, 4 left out what pairs and a byte per pair describe.
 #pragma once
 
 #include "eb_internal.cuh"
