@@ -170,8 +170,10 @@ eb_status eb_schedule(eb_ctx* ctx, void* stream, const eb_batch* batch, int32_t 
  * loads it was made from in a record in pinned host memory, which the context owns and allocates on the first such call, and mark it
  * with the ticket last.  Setting a ticket clears the mark, so it must not be done while marked work is in flight that is yet to
  * be waited for.  Ticket 0 (the state after eb_create): later calls do not write the record; the mark stays.
- * eb_schedule_wait blocks until the mark is `ticket` and copies the record; should all work on `stream` be over without it, it
- * copies d_res and mb_load from the device instead.  h_load: host, [n_mb, D], or NULL. */
+ * eb_schedule_wait blocks until the mark is `ticket` and copies the record.  What a call launched with the ticket is waited for on
+ * whatever stream that was.  Of graphs the library knows nothing: `stream` is the one that they are replayed on, and should all work on
+ * it be over without the mark (a graph captured while nothing was watched), d_res and mb_load are copied from the device
+ * instead.  h_load: host, [n_mb, D], or NULL. */
 eb_status eb_watch_schedule(eb_ctx* ctx, uint32_t ticket);
 eb_status eb_schedule_wait(eb_ctx* ctx, void* stream, uint32_t ticket, int32_t n_mb, const eb_sched_result* d_res,
                            const int32_t* mb_load, eb_sched_result* h_res, int32_t* h_load);

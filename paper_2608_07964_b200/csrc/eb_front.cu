@@ -572,6 +572,7 @@ eb_status ebi_front_run(eb_ctx* c, cudaStream_t st, const BatchParams& bp, uint3
     if ((int64_t)sched_subsets(pool_mask, m) * (blocks - 1) / blocks < kSchedSubsets) blocks = 1;
     EB_LAUNCH(c, "tables", ebi_launch(tables_kernel, dim3(blocks), dim3(kSchedThreads), tables_smem(bp.n_mb, g.E, bp.n_mb * (g.E + g.D * g.S)), st,
                                       c->mp, bp, a));
+    ebi_watch_launched(c, st);
   }
   {
     KernelTimer timer(c, EBK_PERMUTE_GATHER, st);

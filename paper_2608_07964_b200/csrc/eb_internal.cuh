@@ -78,6 +78,7 @@ struct eb_ctx {
   int32_t* d_status = nullptr;
   ScheduleRecord* watch_rec = nullptr;   // pinned host memory, allocated on first use
   uint32_t watch_ticket = 0;
+  uint32_t watch_sent = 0;               // ticket whose mark is sure to come: its kernels were launched, not captured
   char* d_sched_scratch = nullptr;  // per-block candidates and arrival counter of the multi-block scheduler
 
   const bf16* w_gate = nullptr;
@@ -121,6 +122,13 @@ struct eb_ctx {
   std::string err;
 };
 
+// After the launch of the kernel that leaves the record: its mark comes, on whatever stream that was.  A captured launch promises nothing.
+inline void ebi_watch_launched(eb_ctx* c, cudaStream_t st) {
+  if (!c->watch_ticket) return;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
+  else if (cap == cudaStreamCaptureStatusNone) c->watch_sent = c->watch_ticket;
+}
 inline ScheduleWatch schedule_watch_of(const eb_ctx* c) { return ScheduleWatch{c->watch_ticket ? c->watch_rec : nullptr, c->watch_ticket}; }
 
 int32_t ebi_rows_cap(const eb_ctx* c);

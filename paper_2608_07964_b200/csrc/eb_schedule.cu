@@ -41,6 +41,7 @@ extern "C" eb_status eb_schedule(eb_ctx* c, void* stream, const eb_batch* batch,
     KernelTimer timer(c, EBK_SCHEDULE, st);
     EB_LAUNCH(c, "schedule", ebi_launch(schedule_kernel, dim3(sched_blocks(batch->pool_mask, m, policy)), dim3(kSchedThreads), 0, st, c->cfg.D,
                                         bp.n_mb, batch->pool_mask, (int)m, (int)policy, mb_load, d_res, sched_grid_of(c), schedule_watch_of(c)));
+    ebi_watch_launched(c, st);
   }
   EB_LAUNCH_CHECK(c, "schedule");
   if (h_res) {
@@ -60,7 +61,10 @@ extern "C" eb_status eb_watch_schedule(eb_ctx* c, uint32_t ticket) {
     EB_CUDA(c, cudaHostAlloc(&p, sizeof(ScheduleRecord), cudaHostAllocMapped | cudaHostAllocPortable));
     c->watch_rec = (ScheduleRecord*)p;
   }
-  if (ticket) __atomic_store_n(&c->watch_rec->ticket, 0u, __ATOMIC_RELEASE);
+  if (ticket) {
+    __atomic_store_n(&c->watch_rec->ticket, 0u, __ATOMIC_RELEASE);
+    c->watch_sent = 0;
+  }
   c->watch_ticket = ticket;
   return EB_OK;
 }
@@ -84,7 +88,8 @@ extern "C" eb_status eb_schedule_wait(eb_ctx* c, void* stream, uint32_t ticket, 
     }
     EB_CUDA(c, e);
     if (marked()) break;
-    // everything enqueued is over: a graph captured while nothing was watched
+    if (c->watch_sent == ticket) continue;   // launched on another stream than this one: the mark comes
+    // everything enqueued here is over without a mark: a graph captured while nothing was watched
     EB_CUDA(c, cudaMemcpyAsync(h_res, d_res, sizeof(eb_sched_result), cudaMemcpyDeviceToHost, st));
     if (h_load) EB_CUDA(c, cudaMemcpyAsync(h_load, mb_load, load_bytes, cudaMemcpyDeviceToHost, st));
     EB_CUDA(c, cudaStreamSynchronize(st));

@@ -56,6 +56,36 @@ def test_a_watched_graph_marks_every_replay():
         assert got.pop("loads") == step.mb_load[:4].cpu().tolist() and got == step.sched_result()
 
 
+def test_a_schedule_is_waited_for_from_any_stream():
+    """The stream that asks is idle while the schedule is still behind other work on the one that makes it."""
+    B, step = _step(4, 16)
+    batch = B.Batch([0, 16, 32, 48, 64], [0, 1, 2, 0])
+    step.eb_step(batch, 3)
+    before = step.sched_result(), step.mb_load[:4].cpu().tolist()
+    busy = torch.randn(8192, 8192, device="cuda")
+    for alone in (False, True):   # a whole step, eb_schedule alone
+        step.logits.normal_(generator=torch.Generator(device="cuda").manual_seed(11 + alone))
+        launching, asking = torch.cuda.Stream(), torch.cuda.Stream()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(launching):
+            for _ in range(10):
+                busy @ busy
+            step.watch_schedule(21 + alone)
+            if alone:
+                step.eb_route(batch)
+                step.eb_schedule(batch, 3)
+            else:
+                step.eb_step(batch, 3)
+            step.watch_schedule(0)
+        with torch.cuda.stream(asking):
+            got = step.schedule_wait(21 + alone, 4)
+        loads = got.pop("loads")
+        torch.cuda.synchronize()
+        now = step.sched_result(), step.mb_load[:4].cpu().tolist()
+        assert (got, loads) == now and now[1] != before[1]
+        before = now
+
+
 @pytest.mark.parametrize("rows,cols,lead", [(1, 1, 0), (3, 5, 1), (77, 64, 4), (1000, 8, 2), (4097, 64, 0), (31, 12, 3)])
 def test_copy_equals_torch(rows, cols, lead):
     B, step = _step(1, 1)
