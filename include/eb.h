@@ -168,8 +168,10 @@ eb_status eb_schedule(eb_ctx* ctx, void* stream, const eb_batch* batch, int32_t 
 /* The schedule in host memory as soon as it is made, without waiting for the rest of a step.  With a ticket other than 0,
  * eb_schedule and eb_step on this context (and graphs captured from them, whenever they are replayed) also leave the result and the
  * loads it was made from in a record in pinned host memory, which the context owns and allocates on the first such call, and mark it
- * with the ticket last.  Setting a ticket clears the mark, so it must not be done while marked work is in flight that is yet to
- * be waited for.  Ticket 0 (the state after eb_create): later calls do not write the record; the mark stays.
+ * with the ticket last.  Setting a ticket clears the mark, and from then on it is the only one that can be waited for (others:
+ * EB_ERR_INVALID_ARG, as there is one record).  The same ticket may be set again, as for another replay of a graph, only when all
+ * work marked with it is over: a mark does not tell one replay from the next.  Ticket 0 (the state after eb_create): later calls
+ * do not write the record; the mark stays.
  * eb_schedule_wait blocks until the mark is `ticket` and copies the record.  What a call launched with the ticket is waited for on
  * whatever stream that was.  Of graphs the library knows nothing: `stream` is the one that they are replayed on, and should all work on
  * it be over without the mark (a graph captured while nothing was watched), d_res and mb_load are copied from the device

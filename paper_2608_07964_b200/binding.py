@@ -195,6 +195,7 @@ class MoEStep:
             self.logits, self.x, self.topk_idx, self.topk_w, self.mb_load, self.mb_cnt, self.sched, self.group_off,
             self.group_w, self.row_src, self.pos, self.xp, self.yp, self.step_meta, self.x)], self.x.data_ptr())
         self._weights = None
+        self._waited = 0          # ticket of the last schedule_wait
 
     # -- helpers -------------------------------------------------------------------------------
     def _check(self, code: int, ctx="self"):
@@ -256,12 +257,13 @@ class MoEStep:
 
     def schedule_wait(self, ticket: int, n_mb: int) -> Dict:
         """The schedule marked with `ticket` as soon as it is made, whatever the step has yet to do; with the load vectors it was
-        made from under "loads"."""
+        made from under "loads".  `ticket` is the last one that was set."""
         if not hasattr(self, "_wait_res"):
             self._wait_res, self._wait_load = EbSchedResult(), (C.c_int32 * (EB_MAX_MB * self.D))()
         h, ld = self._wait_res, self._wait_load
         self._check(self.lib.eb_schedule_wait(self.ctx, _stream(), ticket, n_mb, self.sched.data_ptr(), self.mb_load.data_ptr(),
                                               C.addressof(h), C.addressof(ld)))
+        self._waited = ticket
         res = _sched_dict(h, self.D)
         v = ld[:n_mb * self.D]
         res["loads"] = [v[j * self.D:(j + 1) * self.D] for j in range(n_mb)]

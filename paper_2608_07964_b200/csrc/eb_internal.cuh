@@ -78,6 +78,7 @@ struct eb_ctx {
   int32_t* d_status = nullptr;
   ScheduleRecord* watch_rec = nullptr;   // pinned host memory, allocated on first use
   uint32_t watch_ticket = 0;
+  uint32_t watch_newest = 0;             // last ticket set: the one that can be waited for
   uint32_t watch_sent = 0;               // ticket whose mark is sure to come: its kernels were launched, not captured
   char* d_sched_scratch = nullptr;  // per-block candidates and arrival counter of the multi-block scheduler
 

@@ -63,6 +63,7 @@ extern "C" eb_status eb_watch_schedule(eb_ctx* c, uint32_t ticket) {
   }
   if (ticket) {
     __atomic_store_n(&c->watch_rec->ticket, 0u, __ATOMIC_RELEASE);
+    c->watch_newest = ticket;
     c->watch_sent = 0;
   }
   c->watch_ticket = ticket;
@@ -75,6 +76,7 @@ extern "C" eb_status eb_schedule_wait(eb_ctx* c, void* stream, uint32_t ticket, 
   if (!ticket || !d_res || !mb_load || !h_res) return ebi_fail(c, EB_ERR_INVALID_ARG, "null pointer or ticket 0");
   if (n_mb < 0 || n_mb > EB_MAX_MB) return ebi_fail(c, EB_ERR_UNSUPPORTED, "n_mb out of range");
   if (!c->watch_rec) return ebi_fail(c, EB_ERR_INVALID_ARG, "no schedule is watched");
+  if (ticket != c->watch_newest) return ebi_fail(c, EB_ERR_INVALID_ARG, "not the last ticket that was set: its record may be written over");
   if (eb_status ds = ebi_check_device(c)) return ds;
   cudaStream_t st = (cudaStream_t)stream;
   const size_t load_bytes = sizeof(int32_t) * (size_t)n_mb * c->cfg.D;

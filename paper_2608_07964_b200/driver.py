@@ -85,9 +85,12 @@ class StepGraphs:
         self.step, self.tok_off, self.capacity = step, list(tok_off), capacity
         self.graphs: Dict = {}
         self.hits = self.captures = 0
+        self._last = 0            # ticket of the last step
 
     def run(self, layers: List[int], pool: int, route_mask: int, m: int, policy: int) -> int:
-        """Launches the step; returns the ticket that its schedule is marked with (MoEStep.schedule_wait)."""
+        """Launches the step; returns the ticket that its schedule is waited for with (MoEStep.schedule_wait), before the next step
+        is launched.  A step launched without waiting for the one before may find that one's replay of the same graph, and so the same
+        mark, still on its way: its ticket is then one that nothing marks, and the wait for it lasts until the step is over."""
         key = (pool, tuple(layers), route_mask, m, policy)
         g = self.graphs.get(key)
         if g is None:
@@ -106,10 +109,12 @@ class StepGraphs:
             self.captures += 1
         else:
             self.hits += 1
-            self.step.watch_schedule(g[2])   # clears the mark of the last replay
+            ticket = g[2] if self._last == self.step._waited else next(_tickets)
+            self.step.watch_schedule(ticket)   # clears the mark of the last replay
             self.step.watch_schedule(0)
+        self._last, self.step._waited = ticket, 0
         g[0].replay()
-        return g[2]
+        return ticket
 
 
 def run_full(step: "B.MoEStep", tok_off: List[int], L: int, m: int, policy: int,

@@ -86,6 +86,39 @@ def test_a_schedule_is_waited_for_from_any_stream():
         before = now
 
 
+@pytest.mark.parametrize("same", [True, False])
+def test_replays_in_a_row_give_the_last_ones_schedule(same):
+    """Steps replayed without waiting for the ones before, of one graph and of two."""
+    from paper_2608_07964_b200 import driver
+    B, step = _step(4, 16)
+    graphs = driver.StepGraphs(step, [0, 16, 32, 48, 64])
+    layers = [[0, 1, 2, 0], [0, 1, 2, 0] if same else [1, 1, 2, 0]]
+    for lay in layers:
+        ticket = graphs.run(lay, 15, 15, 3, 0)
+        step.schedule_wait(ticket, 4)
+    busy = torch.randn(8192, 8192, device="cuda")
+    for trial in range(4):
+        other = torch.randn(step.logits.shape, device="cuda", generator=torch.Generator(device="cuda").manual_seed(trial))
+        torch.cuda.synchronize()
+        for _ in range(4):
+            busy @ busy
+        first = graphs.run(layers[0], 15, 15, 3, 0)
+        step.logits.copy_(other)
+        for _ in range(4):
+            busy @ busy
+        last = graphs.run(layers[1], 15, 15, 3, 0)
+        got = step.schedule_wait(last, 4)
+        loads = got.pop("loads")
+        torch.cuda.synchronize()
+        assert got == step.sched_result() and loads == step.mb_load[:4].cpu().tolist(), trial
+        with pytest.raises(B.EbError):   # its record is gone
+            step.schedule_wait(first, 4)
+        again = graphs.run(layers[0], 15, 15, 3, 0)   # waited for: marked like any other
+        assert again == graphs.graphs[(15, tuple(layers[0]), 15, 3, 0)][2]
+        got = step.schedule_wait(again, 4)
+        assert got.pop("loads") == loads and got == step.sched_result()
+
+
 @pytest.mark.parametrize("rows,cols,lead", [(1, 1, 0), (3, 5, 1), (77, 64, 4), (1000, 8, 2), (4097, 64, 0), (31, 12, 3)])
 def test_copy_equals_torch(rows, cols, lead):
     B, step = _step(1, 1)
