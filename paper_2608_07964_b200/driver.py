@@ -24,16 +24,12 @@ from . import binding as B
 _tickets = itertools.count(1)
 
 
-def _logit_rows(step: "B.MoEStep", tok_off: List[int]) -> List[torch.Tensor]:
-    return [step.logits[tok_off[j]:tok_off[j + 1]] for j in range(len(tok_off) - 1)]
-
-
-def _copy_logits(step: "B.MoEStep", rows: List[torch.Tensor], logits_of: Callable[[int, int], torch.Tensor], layer: List[int], mask: int) -> None:
-    """Logits of the micro-batches in `mask` at their current layers, into their rows.  Each result is taken over before
+def _copy_logits(rows: List[Callable[[torch.Tensor], object]], logits_of: Callable[[int, int], torch.Tensor], layer: List[int], mask: int) -> None:
+    """Logits of the micro-batches in `mask` at their current layers, into their rows (a MoEStep.copier).  Each result is taken over before
     the next one is asked for: `logits_of` may fill and return one and the same buffer every time."""
-    for j, row in enumerate(rows):
+    for j, copy in enumerate(rows):
         if (mask >> j) & 1:
-            step.copy(row, logits_of(j, layer[j]))
+            copy(logits_of(j, layer[j]))
 
 
 def run_load_trace(step: "B.MoEStep", tok_off: List[int], L: int, m: int, policy: int,
@@ -45,10 +41,10 @@ def run_load_trace(step: "B.MoEStep", tok_off: List[int], L: int, m: int, policy
     pool = (1 << N) - 1 if L > 0 else 0
     route_mask = pool
     steps: List[Dict] = []
-    rows = _logit_rows(step, tok_off)
+    rows = step.copier(step.logits, tok_off)
     try:
         while pool:
-            _copy_logits(step, rows, logits_of, layer, route_mask)
+            _copy_logits(rows, logits_of, layer, route_mask)
             batch = B.Batch(tok_off, [min(l, L - 1) for l in layer], pool)
             ticket = next(_tickets)
             step.watch_schedule(ticket)
@@ -132,12 +128,12 @@ def run_full(step: "B.MoEStep", tok_off: List[int], L: int, m: int, policy: int,
     route_mask = pool
     step.x[:T].copy_(x0)
     steps: List[Dict] = []
-    rows = _logit_rows(step, tok_off)
+    rows = step.copier(step.logits, tok_off)
     t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     t0.record()
     stream = torch.cuda.current_stream()
     while pool:
-        _copy_logits(step, rows, logits_of, layer, route_mask)
+        _copy_logits(rows, logits_of, layer, route_mask)
         lay = [min(l, L - 1) for l in layer]
         if graphs is not None:
             ticket = graphs.run(lay, pool, route_mask, m, policy)

@@ -16,6 +16,10 @@ def _step(n_mb, tokens, E=12, K=3, D=5):
     return B, step
 
 
+def _copy(step, dst, src):
+    step.copier(dst)[0](src)
+
+
 @pytest.mark.parametrize("n_mb,m,policy", [(1, 1, 0), (4, 3, 0), (11, 8, 0), (16, 12, 0), (16, 1, 0), (9, 2, 1), (9, 2, 2), (5, 1, 3)])
 def test_a_watched_schedule_is_the_one_on_the_device(n_mb, m, policy):
     B, step = _step(n_mb, 37)
@@ -125,13 +129,78 @@ def test_copy_equals_torch(rows, cols, lead):
     src = torch.randn(lead + rows * cols, device="cuda")[lead:].view(rows, cols)
     for d in (0, 1):
         buf = torch.zeros(d + rows * cols + 8, device="cuda")
-        step.copy(buf[d:d + rows * cols].view(rows, cols), src)
+        _copy(step, buf[d:d + rows * cols].view(rows, cols), src)
         assert torch.equal(buf[d:d + rows * cols].view(rows, cols), src)
         assert not buf[:d].any() and not buf[d + rows * cols:].any()
     for other in (src.double(), src.cpu(), src.t().contiguous().t(), src[:1].expand(rows, cols)):   # the general way
         dst = torch.zeros(rows, cols, device="cuda")
-        step.copy(dst, other)
+        _copy(step, dst, other)
         assert torch.equal(dst, other.to(dst).contiguous())
     one = torch.arange(rows * cols + 1, device="cuda", dtype=torch.float32)
-    step.copy(one[1:].view(rows, cols), one[1:].view(rows, cols))   # onto itself
+    _copy(step, one[1:].view(rows, cols), one[1:].view(rows, cols))   # onto itself
     assert torch.equal(one, torch.arange(rows * cols + 1, device="cuda", dtype=torch.float32))
+
+
+def test_copy_does_what_autograd_and_views_ask_of_copy_():
+    """Where copy_ refuses, counts a version, resolves a view or carries a tangent, so does the copy."""
+    import torch.autograd.forward_ad as fwAD
+    B, step = _step(1, 1)
+    src = torch.randn(5, 7, device="cuda")
+    leaf = torch.zeros(5, 7, device="cuda", requires_grad=True)
+    with pytest.raises(RuntimeError, match="leaf"):
+        _copy(step, leaf, src)
+    assert not leaf.any()
+    base = torch.zeros(9, 7, device="cuda", requires_grad=True)
+    saved = torch.zeros(9, 7, device="cuda")
+    out = (base * saved).sum()
+    _copy(step, saved[2:7], src)   # what the backward pass would read is no longer what it was
+    with pytest.raises(RuntimeError, match="modified by an inplace operation"):
+        out.backward()
+    with torch.inference_mode():
+        frozen = torch.zeros(5, 7, device="cuda")
+    with pytest.raises(RuntimeError, match="[Ii]nference"):
+        _copy(step, frozen, src)
+    z = torch.randn(5, 7, device="cuda", dtype=torch.complex64)
+    for dst, other in ((torch.ones(5, 7, device="cuda"), torch._efficientzerotensor((5, 7), device="cuda")),
+                       (torch.zeros_like(z), z.conj()), (torch.zeros_like(z).conj(), z), (torch.zeros(5, 7, device="cuda"), torch._neg_view(src)),
+                       (torch._neg_view(torch.zeros(5, 7, device="cuda")), src)):
+        _copy(step, dst, other)
+        assert torch.equal(dst.resolve_conj().resolve_neg(), (other * 1).resolve_conj().resolve_neg())
+    with fwAD.dual_level():
+        dst = torch.zeros(5, 7, device="cuda")
+        _copy(step, dst, fwAD.make_dual(src, torch.full_like(src, 2)))
+        assert torch.equal(fwAD.unpack_dual(dst).tangent, torch.full_like(src, 2))
+
+    def doubled(x):
+        dst = torch.zeros_like(x)
+        _copy(step, dst, x)
+        return 2 * dst
+    assert torch.equal(torch.func.vmap(doubled)(src), 2 * src)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.uint8, torch.int64])
+@pytest.mark.parametrize("count,lead", [(1, 0), (1, 1), (7, 3), (255, 1), (4097, 2), (300001, 5)])
+def test_copies_of_types_that_are_no_multiple_of_four_bytes(dtype, count, lead):
+    B, step = _step(1, 1)
+    src = torch.randint(0, 100, (lead + count,), device="cuda").to(dtype)[lead:]
+    for d in (0, 1, 2):
+        buf = torch.zeros(d + count + 8, device="cuda", dtype=dtype)
+        _copy(step, buf[d:d + count], src)
+        assert torch.equal(buf[d:d + count], src) and not buf[:d].any() and not buf[d + count:].any()
+
+
+def test_a_copier_fills_the_rows_it_was_made_for():
+    B, step = _step(4, 16)
+    step.logits.zero_()
+    fill = step.copier(step.logits, [0, 5, 5, 33, 64])
+    want = torch.zeros_like(step.logits)
+    for i, (a, b) in enumerate(((0, 5), (5, 5), (5, 33), (33, 64))):
+        src = torch.full((b - a, step.E), float(i + 1), device="cuda")
+        fill[i](src)
+        want[a:b] = src
+        assert torch.equal(step.logits, want)
+    with pytest.raises(RuntimeError):   # as copy_ does: neither the shape nor broadcast to it
+        fill[0](torch.zeros(4, step.E, device="cuda"))
+    fill[3](torch.arange(step.E, device="cuda", dtype=torch.float64))
+    want[33:] = torch.arange(step.E, device="cuda")
+    assert torch.equal(step.logits, want)
