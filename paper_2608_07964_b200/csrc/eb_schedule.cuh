@@ -1,8 +1,6 @@
 // Schedule(S, m) of Algorithm 1 for one thread block: the policies and the result record.
 //
-// MaxUtil (Section 4.2) enumerates every subset of the pool with at least m members.  The pool
-// is split into a low and a high half; the summed load vector of each half-subset is tabulated
-// in shared memory (2 x 256 x D entries at most), so a subset costs D additions and a maximum.
+// MaxUtil (Section 4.2) enumerates every subset of the pool with at least m members.
 // Utilisation (Eq. 3 for one step) is sum(W) / (D * max(W)); D is common to all candidates, so
 // candidates are compared exactly by cross-multiplying sum and max in 64-bit integers.
 // Total order: higher utilisation, then more members, then the numerically smaller mask.
@@ -11,14 +9,20 @@
 //
 // What bounds small pools is latency, of large ones instruction issue: 2^16 subsets on one SM.  So there are three ways through
 // the subsets of MaxUtil, none of which visits those that are too small:
-//  - up to 10 members: a subset per thread, summed member by member; no tables, no barrier before the result is known.
-//  - more members of which at most 4 stay out (m = ceil(0.75 n) up to n = 16: 2517 subsets): the total less the loads of
+//  - up to 10 members: a subset per thread; no tables, no barrier before the result is known.  The members from the sixth on are
+//    the same for a whole warp, whose lanes add them up once, a device each; the other five are added member by member.
+//  - more members of which few may stay out (m = ceil(0.75 n) from 12 up to n = 16: 2517 subsets): the total less the loads of
 //    two pairs left out, whose sums are tabulated.
-//  - otherwise the halves: summed loads of every half-subset in shared memory.  The low halves are kept in the order of their
+//  - otherwise the halves: the pool is split in two, and the summed load vector of each half-subset is tabulated in shared memory
+//    (2 x 256 x D entries at most), so a subset costs D additions and a maximum.  The low halves are kept in the order of their
 //    member counts, so that for every high half the sufficient ones come first.  Sums are 32-bit where the loads allow
 //    it, and the tables' rows are 20 words apart, which 16-byte reads of neighbouring rows go through without bank conflicts.
 // In a step the schedule of 4 members took 6300 cycles by halves and takes 3300 the first way, that of 12 out of 16 18000 and 11000 the
-// second; 10 members is what a subset per thread of the block reaches, 4 left out what pairs and a byte per pair describe.
+// second; 10 members is what a subset per thread of the block reaches, 4 left out what pairs and a byte per pair describe.  eb_schedule
+// in a chain of its own (us, by halves / every member by itself / now): 8 members, m = 6, 16 devices 3.64 / 5.20 / 3.33, 8 devices
+// 3.65 / 3.99 / 3.15; 10 members, m = 8, 16 devices 3.93 / 5.96 / 4.15 (halves take 0.5 to 1.5 more inside a step).  The pairs have
+// tables of their own to lay out, which 11 members of which 1 or 2 stay out and 12 of which 1 does are too few subsets for: 3.81 / 4.06
+// for 11 and 1 by halves / by pairs, 4.00 / 4.06 for 11 and 2, 3.88 / 4.00 for 12 and 1, but 4.10 / 3.99 for 12 and 2.
 #pragma once
 
 #include "eb_internal.cuh"
@@ -236,14 +240,24 @@ __device__ __forceinline__ W max4(W a, W b, W c, W d) {
 // Up to 10 members.
 template <typename W>
 __device__ __forceinline__ Cand maxutil_small(const SchedShared& s, int D, int np, int m) {
-  const int tid = threadIdx.x, n = __popc(tid), quads = (D + 3) / 4;
+  const int tid = threadIdx.x, lane = tid & 31, n = __popc(tid), quads = (D + 3) / 4;
   BestSubset<W> best;
-  if (tid < (1 << np) && n >= m) {
+  if (tid - lane < 1 << np && __popc(tid - lane) + 5 >= m) {   // else the whole warp's are too small
+    W mine = 0;   // members from the sixth on are those of the whole warp: their load on device `lane` mod 16
+#pragma unroll 1
+    for (int k = 5; k < np; ++k)
+      if ((tid >> k) & 1) mine += s.load[s.member[k]][lane & 15];
+    const int4* row[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) row[k] = reinterpret_cast<const int4*>(s.load[s.member[k < np ? k : 0]]);
     W num = 0, peak = 0;
+#pragma unroll 1
     for (int q = 0; q < quads; ++q) {   // entries beyond D are zero
-      W w0 = 0, w1 = 0, w2 = 0, w3 = 0;
-      for (int k = 0; k < np; ++k) {
-        const int4 v = reinterpret_cast<const int4*>(s.load[s.member[k]])[q];
+      W w0 = __shfl_sync(0xffffffffu, mine, 4 * q), w1 = __shfl_sync(0xffffffffu, mine, 4 * q + 1),
+        w2 = __shfl_sync(0xffffffffu, mine, 4 * q + 2), w3 = __shfl_sync(0xffffffffu, mine, 4 * q + 3);
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        const int4 v = row[k][q];
         if ((tid >> k) & 1) {
           w0 += v.x;
           w1 += v.y;
@@ -255,7 +269,7 @@ __device__ __forceinline__ Cand maxutil_small(const SchedShared& s, int D, int n
       const W p = max4(w0, w1, w2, w3);
       peak = p > peak ? p : peak;
     }
-    best.offer(num, peak, D, n, tid);
+    if (tid < 1 << np && n >= m) best.offer(num, peak, D, n, tid);
   }
   return best.cand();
 }
@@ -325,8 +339,10 @@ __device__ __forceinline__ Cand maxutil_halves(const SchedShared& s, int D, int 
   return best.cand();
 }
 
-// Whether a schedule goes the way of maxutil_few_out.
-__host__ __device__ __forceinline__ bool few_out(int np, int m, int policy) { return policy == EB_POLICY_MAXUTIL && np > 10 && np > m && np - m <= kFewOut; }
+// Whether a schedule goes the way of maxutil_few_out: 3 or 4 out of 11 members, 2 to 4 out of 12, 1 to 4 out of more.
+__host__ __device__ __forceinline__ bool few_out(int np, int m, int policy) {
+  return policy == EB_POLICY_MAXUTIL && np > 10 && np - m > (np < 13 ? 13 - np : 0) && np - m <= kFewOut;
+}
 // Which micro-batches are in the pool, and the tables that the schedule takes; before the barrier behind the writes of s.load.
 __device__ __forceinline__ void schedule_prepare(SchedShared& s, uint32_t pool_mask, int m, int policy) {
   const int tid = threadIdx.x;

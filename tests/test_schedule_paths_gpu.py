@@ -8,8 +8,10 @@ from oracle import eb_oracle as O
 pytestmark = pytest.mark.gpu
 
 
-# members of the pool, members that may stay out: 10 | 11 members, 4 | 5 left out, the least and the most of either
-@pytest.mark.parametrize("members,out", [(2, 1), (5, 2), (9, 8), (10, 1), (10, 9), (11, 1), (11, 4), (11, 5), (13, 3), (14, 4), (14, 5), (16, 1), (16, 4), (16, 5)])
+# members of the pool, members that may stay out: 5 | 6 members, 10 | 11, few left out (from 3 for 11 members, 2 for 12, 1 for 13) up to 4 | 5,
+# the least and the most of each
+@pytest.mark.parametrize("members,out", [(2, 1), (4, 3), (5, 2), (5, 4), (6, 1), (6, 5), (8, 2), (9, 8), (10, 1), (10, 5), (10, 9), (11, 1), (11, 2),
+                                         (11, 3), (11, 4), (11, 5), (12, 1), (12, 2), (13, 1), (13, 3), (14, 4), (14, 5), (16, 1), (16, 4), (16, 5)])
 @pytest.mark.parametrize("D", [1, 3, 8, 16])
 def test_maxutil_takes_the_oracles_subset(members, out, D):
     from paper_2608_07964_b200 import binding as B
