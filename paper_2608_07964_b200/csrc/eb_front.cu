@@ -97,7 +97,6 @@ struct TablesArgs {
   int32_t *group_off, *group_w, *step_meta;
   TilePlan plan;
   SchedGrid sched;
-  ScheduleWatch watch;
 };
 
 // i / E for i < 2^16 (E <= 256): one multiplication by ceil(2^32 / E); larger i take the division
@@ -210,7 +209,7 @@ tables_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ Ba
     if (lane < EB_MAX_MB) s_rank[lane] = (run >> lane) & 1u ? __popc(active & ((1u << s_layer_of[lane]) - 1u)) : -1;
     if (lane == 0) s_nl = __popc(active);
   }
-  if (warp == 1) write_schedule(sc, D, a.pool_mask, run, a.res, a.watch);
+  if (warp == 1) write_schedule(sc, D, a.pool_mask, run, a.res);
   __syncthreads();
   const int nl = s_nl, G = nl * (E + D * S);
 
@@ -342,9 +341,11 @@ struct ScatterArgs {
   TileList list;
   int fill_blocks;
   int team;   // threads per token row
+  const int32_t* mb_load;
+  ScheduleWatch watch;
 };
 
-// Blocks below fill_blocks write the tile list.  Each of the others places TB tokens of a chunk: the chunk's assignments up to
+// A watched schedule is copied to host memory by a block ahead of the others.  Blocks below fill_blocks write the tile list.  Each of the others places TB tokens of a chunk: the chunk's assignments up to
 // them are ranked by warp matches while the token rows are on their way, then every row goes out to its K + S places, a team
 // of threads per row.  What bounds it is that chain of two trips to memory and three barriers per block, and the row traffic.
 // TB is small while there are few tokens (a block each keeps the chip busy) and 8 when there are many (ranking and tables are
@@ -357,9 +358,15 @@ template <int TB>
 __global__ void __launch_bounds__(kScatterThreads)
 scatter_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ BatchParams bp, const __grid_constant__ ScatterArgs a) {
   extern __shared__ int s_dyn[];
-  if ((int)blockIdx.x < a.fill_blocks) {
+  int block = blockIdx.x;
+  if (a.watch.rec && block-- == 0) {
     EB_GRID_DEP_SYNC();
-    fill_tiles(mp, a.group_off, a.group_w, a.list, s_dyn, blockIdx.x, a.fill_blocks);
+    if (threadIdx.x < 32) leave_record(a.watch, a.res, a.mb_load, bp.n_mb * mp.D);
+    return;
+  }
+  if (block < a.fill_blocks) {
+    EB_GRID_DEP_SYNC();
+    fill_tiles(mp, a.group_off, a.group_w, a.list, s_dyn, block, a.fill_blocks);
     return;
   }
   __shared__ StepShape ss;
@@ -373,7 +380,7 @@ scatter_kernel(const __grid_constant__ ModelParams mp, const __grid_constant__ B
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int E = mp.E, K = mp.K, S = mp.S, KS = K + S, vec = mp.H / 8;
   auto expert = [&](int e, int lane) { return (unsigned)e < (unsigned)E ? e : -1 - lane; };   // outside [0, E): equal to no other
-  const int part = (int)blockIdx.x - a.fill_blocks, c = part / (32 / TB);
+  const int part = block - a.fill_blocks, c = part / (32 / TB);
   const int j = mb_of_chunk(bp, c);
   const int c0 = bp.tok_off[j] + (c - bp.chunk_off[j]) * 32;      // first token of the chunk
   const int t0 = c0 + part % (32 / TB) * TB;                      // and of this part
@@ -567,26 +574,27 @@ eb_status ebi_front_run(eb_ctx* c, cudaStream_t st, const BatchParams& bp, uint3
                                       (const int32_t*)c->chunk_hist, c->chunk_base, c->chunk_seg));
     const TablesArgs a{pool_mask, route_mask, (int)m, (int)policy, c->chunk_hist, sums ? c->chunk_seg : nullptr, c->chunk_base, c->seg_base,
                        c->mb_base, b->mb_load, b->mb_cnt, seg, layers_of(bp), b->sched, b->group_off, b->group_w, b->step_meta, tile_plan_of(c),
-                       sched_grid_of(c), schedule_watch_of(c)};
+                       sched_grid_of(c)};
     int blocks = sched_blocks(pool_mask, m, policy);
     if ((int64_t)sched_subsets(pool_mask, m) * (blocks - 1) / blocks < kSchedSubsets) blocks = 1;
     EB_LAUNCH(c, "tables", ebi_launch(tables_kernel, dim3(blocks), dim3(kSchedThreads), tables_smem(bp.n_mb, g.E, bp.n_mb * (g.E + g.D * g.S)), st,
                                       c->mp, bp, a));
-    ebi_watch_launched(c, st);
   }
   {
     KernelTimer timer(c, EBK_PERMUTE_GATHER, st);
     const ScatterArgs a{b->sched, b->topk_idx, c->chunk_base, sums ? c->seg_base : nullptr, c->mb_base, b->group_off, b->group_w, seg, b->pos, b->row_src, b->step_meta,
-                        (const uint4*)b->x, (uint4*)b->xp, tile_list_of(c), c->num_sms / 2, row_team(g.H / 8)};
+                        (const uint4*)b->x, (uint4*)b->xp, tile_list_of(c), c->num_sms / 2, row_team(g.H / 8),
+                        b->mb_load, schedule_watch_of(c)};
     const size_t smem = sizeof(int) * (size_t)(ebi_groups_cap(c) + 1);
     auto launch = [&](auto kernel, int tb) {
-      return ebi_launch(kernel, dim3(a.fill_blocks + bp.n_chunks * (32 / tb)), dim3(kScatterThreads), smem, st, c->mp, bp, a);
+      return ebi_launch(kernel, dim3((a.watch.rec ? 1 : 0) + a.fill_blocks + bp.n_chunks * (32 / tb)), dim3(kScatterThreads), smem, st, c->mp, bp, a);
     };
     EB_LAUNCH(c, "scatter", bp.n_tok <= 2 * c->num_sms     ? launch(scatter_kernel<1>, 1)
                             : bp.n_tok <= 16 * c->num_sms  ? launch(scatter_kernel<4>, 4)
                             : g.H > kScatterNarrow || bp.n_tok <= 64 * c->num_sms ? launch(scatter_kernel<8>, 8)
                                                                                   : launch(scatter_kernel<32>, 32));
   }
+  ebi_watch_launched(c, st);
   EB_LAUNCH_CHECK(c, "step front end");
   return EB_OK;
 }

@@ -8,7 +8,7 @@ namespace {
 
 __global__ void __launch_bounds__(kSchedThreads)
 schedule_kernel(int D, int n_mb, uint32_t pool_mask, int m, int policy, const int32_t* __restrict__ mb_load,
-                eb_sched_result* __restrict__ res, SchedGrid grid, ScheduleWatch watch) {
+                eb_sched_result* res, SchedGrid grid, ScheduleWatch watch) {
   EB_GRID_DEP_SYNC();
   __shared__ SchedShared s;
   const int tid = threadIdx.x;
@@ -22,7 +22,13 @@ schedule_kernel(int D, int n_mb, uint32_t pool_mask, int m, int policy, const in
   const bool any_wide = __syncthreads_or(wide_load(load));
   uint32_t run;
   if (!schedule_grid(s, D, pool_mask, m, policy, any_wide, grid, &run)) return;
-  if (tid < 32) write_schedule(s, D, pool_mask, run, res, watch);
+  if (tid < 32) {
+    write_schedule(s, D, pool_mask, run, res);
+    if (watch.rec) {
+      __syncwarp();
+      leave_record(watch, res, mb_load, n_mb * D);
+    }
+  }
 }
 
 }  // namespace

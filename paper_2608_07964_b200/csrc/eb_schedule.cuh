@@ -547,9 +547,8 @@ inline SchedGrid sched_grid_of(const eb_ctx* c) {
   return SchedGrid{(Cand*)c->d_sched_scratch, (unsigned*)(c->d_sched_scratch + kMaxSchedBlocks * sizeof(Cand))};
 }
 
-// The result record, by one warp; and its copy in host memory, if that is watched.
-__device__ __forceinline__ void write_schedule(const SchedShared& s, int D, uint32_t pool_mask, uint32_t run, eb_sched_result* res,
-                                               const ScheduleWatch& watch) {
+// The result record, by one warp.
+__device__ __forceinline__ void write_schedule(const SchedShared& s, int D, uint32_t pool_mask, uint32_t run, eb_sched_result* res) {
   const int tid = threadIdx.x & 31;
   // lane d sums the chosen micro-batches' load on device d (zero beyond D); the warp adds and maximises
   long long v = 0;
@@ -557,7 +556,6 @@ __device__ __forceinline__ void write_schedule(const SchedShared& s, int D, uint
 #pragma unroll
     for (int j = 0; j < EB_MAX_MB; ++j) v += ((run >> j) & 1u) ? s.load[j][tid] : 0;
     res->joint_load[tid] = (int32_t)v;
-    if (watch.rec) watch.rec->res.joint_load[tid] = (int32_t)v;
   }
   long long num = v, peak = v;
 #pragma unroll
@@ -567,21 +565,28 @@ __device__ __forceinline__ void write_schedule(const SchedShared& s, int D, uint
     peak = p2 > peak ? p2 : peak;
   }
   if (tid == 0) {
-    for (eb_sched_result* r = res; r; r = watch.rec && r == res ? &watch.rec->res : nullptr) {
-      r->run_mask = run;
-      r->defer_mask = pool_mask & ~run;
-      r->n_run = __popc(run);
-      r->status = EB_OK;
-      r->util_num = num;
-      r->util_den = (long long)D * peak;
-    }
+    res->run_mask = run;
+    res->defer_mask = pool_mask & ~run;
+    res->n_run = __popc(run);
+    res->status = EB_OK;
+    res->util_num = num;
+    res->util_den = (long long)D * peak;
   }
-  if (watch.rec) {
-    for (int i = tid; i < EB_MAX_MB * D; i += 32) watch.rec->load[i] = s.load[i / D][i % D];
-    __threadfence_system();
-    __syncwarp();
-    if (tid == 0) asm volatile("st.release.sys.global.u32 [%0], %1;" ::"l"(&watch.rec->ticket), "r"(watch.ticket) : "memory");
-  }
+}
+
+// Copies a schedule and the loads it was made from, which are written, into the record, and marks it; by one warp.  The mark is a
+// release, which covers the words of the other lanes through the warp barrier, and waits until they are in host memory (1.5 us;
+// with a fence of every lane before it 3 us): no other warp of a step may have to wait for this one.  Ahead of a barrier of
+// tables_kernel it made a watched step of 4 x 64 tokens 32.8 us instead of 29.6; by a block of scatter_kernel of its own both are
+// 29.7, and 5 x 93 tokens 91.4 -> 87.9 (unwatched 87.9).  Out of line, as calls that are not watched pay for its place in the code:
+// eb_schedule of 4 members 2.98 us with it inlined, 2.83 without.
+static __device__ __noinline__ void leave_record(const ScheduleWatch& watch, const eb_sched_result* res, const int32_t* load, int n_load) {
+  const int lane = threadIdx.x & 31;
+  static_assert(sizeof(eb_sched_result) % 4 == 0 && sizeof(eb_sched_result) / 4 <= 32, "a word per lane");
+  if (lane < (int)sizeof(eb_sched_result) / 4) reinterpret_cast<int32_t*>(&watch.rec->res)[lane] = reinterpret_cast<const int32_t*>(res)[lane];
+  for (int i = lane; i < n_load; i += 32) watch.rec->load[i] = load[i];
+  __syncwarp();
+  if (lane == 0) asm volatile("st.release.sys.global.u32 [%0], %1;" ::"l"(&watch.rec->ticket), "r"(watch.ticket) : "memory");
 }
 
 }  // namespace

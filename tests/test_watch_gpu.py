@@ -1,4 +1,7 @@
 """Schedules left in host memory, and the copy of logits, against the calls they stand in for."""
+import ctypes as C
+import threading
+
 import pytest
 import torch
 
@@ -204,3 +207,59 @@ def test_a_copier_fills_the_rows_it_was_made_for():
     fill[3](torch.arange(step.E, device="cuda", dtype=torch.float64))
     want[33:] = torch.arange(step.E, device="cuda")
     assert torch.equal(step.logits, want)
+
+
+def _record(step, ticket, n_mb):
+    """What eb_schedule_wait gives when the device's buffers that it may fall back on hold something else: the record that the
+    kernels left in host memory, or -7 everywhere."""
+    from paper_2608_07964_b200 import binding as B
+    poison = torch.full((1024,), -7, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    h, ld, code = B.EbSchedResult(), (C.c_int32 * (16 * step.D))(), []
+    stream = B._stream()
+    t = threading.Thread(daemon=True, target=lambda: code.append(step.lib.eb_schedule_wait(
+        step.ctx, stream, ticket, n_mb, poison.data_ptr(), poison.data_ptr(), C.addressof(h), C.addressof(ld))))
+    t.start()
+    t.join(20)
+    assert code == [0], "the mark never came"
+    return B._sched_dict(h, step.D), [list(ld[j * step.D:(j + 1) * step.D]) for j in range(n_mb)]
+
+
+@pytest.mark.parametrize("how", ["step", "schedule", "graph"])
+@pytest.mark.parametrize("n_mb,tokens,m,policy", [(1, 1, 1, 0), (4, 37, 3, 0), (11, 8, 8, 0), (16, 5, 12, 0), (16, 5, 1, 0), (14, 9, 2, 0), (9, 33, 2, 1),
+                                                  (5, 70, 1, 3), (3, 0, 2, 0), (16, 400, 6, 0)])   # one block, several, no tokens, large grids
+def test_the_record_is_what_the_kernels_left_in_host_memory(how, n_mb, tokens, m, policy):
+    B, step = _step(n_mb, max(tokens, 1))
+    batch = B.Batch([tokens * j for j in range(n_mb + 1)], [j % 3 for j in range(n_mb)])
+    everything = (1 << n_mb) - 1
+    graph = torch.cuda.CUDAGraph()
+    step.eb_step(batch, m, policy)
+    torch.cuda.synchronize()
+    if how == "graph":
+        step.watch_schedule(40)
+        with torch.cuda.graph(graph):
+            step.eb_step(batch, m, policy)
+        step.watch_schedule(0)
+    for trial in range(3):
+        step.logits.normal_(generator=torch.Generator(device="cuda").manual_seed(trial))
+        ticket = 40 if how == "graph" else 41 + trial
+        step.watch_schedule(ticket)
+        route = everything if trial != 1 else everything >> 1   # the last micro-batch keeps its routing
+        if how == "graph":
+            step.watch_schedule(0)
+            graph.replay()
+        elif how == "step":
+            step.eb_step(batch, m, policy, route)
+        else:
+            if tokens:
+                step.eb_route(batch, route)
+            step.eb_schedule(batch, m, policy)
+        got, loads = _record(step, ticket, n_mb)
+        assert got == step.sched_result() and loads == step.mb_load[:n_mb].cpu().tolist(), trial
+        assert min(min(x) for x in loads) >= 0
+    # nothing is watched: the device's buffers answer, and these hold -7
+    step.watch_schedule(90)
+    step.watch_schedule(0)
+    step.eb_step(batch, m, policy)
+    got, loads = _record(step, 90, n_mb)
+    assert got["n_run"] == -7 and loads == [[-7] * step.D] * n_mb
