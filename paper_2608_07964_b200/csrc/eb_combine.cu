@@ -33,7 +33,9 @@ combine_kernel(int n_tok, int H, int K, int team, const uint4* __restrict__ yp, 
                const float* __restrict__ topk_w, const uint4* residual, uint4* out) {   // residual may be `out` itself
   const int t = blockIdx.x * (kThreads / team) + threadIdx.x / team;   // team >= 32: a warp serves one token
   const int lane = threadIdx.x & 31;
-  if (t < n_tok && lane < 3) touch_ahead(lane == 0 ? (const void*)(pos + (size_t)t * KS) : lane == 1 ? (const void*)(topk_w + (size_t)t * K) : (const void*)(out + (size_t)t * (H / 8)));
+  // by one warp per token: hints of all eight warps, and for the output row too, took 4 x 4096 tokens of 2048 elements from 26.5 us
+  // to 29.0 (26.8 now), 4 x 64 of 256 elements take 1.53 with and 1.68 without
+  if (t < n_tok && threadIdx.x % team < 2) touch_ahead(lane == 0 ? (const void*)(pos + (size_t)t * KS) : (const void*)(topk_w + (size_t)t * K));
   EB_GRID_DEP_SYNC();
   if (t >= n_tok) return;
   // lane s fetches slot s once per warp; the values are broadcast with shuffles
