@@ -253,8 +253,11 @@ __device__ __forceinline__ Cand maxutil_small(const SchedShared& s, int D, int n
     W num = 0, peak = 0;
 #pragma unroll 1
     for (int q = 0; q < quads; ++q) {   // entries beyond D are zero
-      W w0 = __shfl_sync(0xffffffffu, mine, 4 * q), w1 = __shfl_sync(0xffffffffu, mine, 4 * q + 1),
+      W w0 = 0, w1 = 0, w2 = 0, w3 = 0;
+      if (np > 5) {   // a step of 4 members is 0.1 us shorter without the shuffles
+        w0 = __shfl_sync(0xffffffffu, mine, 4 * q), w1 = __shfl_sync(0xffffffffu, mine, 4 * q + 1);
         w2 = __shfl_sync(0xffffffffu, mine, 4 * q + 2), w3 = __shfl_sync(0xffffffffu, mine, 4 * q + 3);
+      }
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
         const int4 v = row[k][q];
