@@ -22,6 +22,8 @@ std::map<const void*, size_t>& limits() {
 std::vector<std::string> launched;
 int refuse_at = -1, asked = 0;
 cudaError_t last = cudaSuccess;
+bool capturing = false;
+void* host_memory = nullptr;   // the last pinned allocation
 
 cudaError_t launch(const void* func, size_t smem) {
   const size_t limit = limits().count(func) ? limits()[func] : 48 * 1024;
@@ -41,6 +43,8 @@ void fake_reset(int refuse) {
 }
 int fake_launched() { return (int)launched.size(); }
 const char* fake_name(int i) { return launched[i].c_str(); }
+void fake_capturing(int on) { capturing = on != 0; }
+void* fake_host_memory() { return host_memory; }
 
 // ---- what the compiler's registration code calls
 void** __cudaRegisterFatBinary(void*) {
@@ -104,6 +108,16 @@ cudaError_t cudaMemcpyAsync(void*, const void*, size_t, cudaMemcpyKind, cudaStre
 cudaError_t cudaMemset(void*, int, size_t) { return cudaSuccess; }
 cudaError_t cudaMemsetAsync(void*, int, size_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
+cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { return host_memory = *p = calloc(1, n), cudaSuccess; }
+cudaError_t cudaFreeHost(void* p) {
+  if (p == host_memory) host_memory = nullptr;
+  return free(p), cudaSuccess;
+}
+cudaError_t cudaStreamQuery(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* s) {
+  *s = capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+  return cudaSuccess;
+}
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t*, unsigned) { return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }

@@ -24,6 +24,7 @@ def lib(tmp_path_factory):
     assert r.returncode == 0, r.stderr
     l = B.load_library(so)
     l.fake_name.restype = C.c_char_p
+    l.fake_host_memory.restype = C.c_void_p
     return l
 
 
@@ -84,6 +85,9 @@ def _calls(c, n_mb, tokens):
         permute_noalloc=lambda: l.eb_permute_noalloc(C.byref(cfg), None, ref, p, p, p, p, p, p, p, p, p, err, 256),
         expert_ffn=lambda: l.eb_expert_ffn_grouped(c.ctx, None, p, p, p, p, p),
         expert_ffn_device=lambda: l.eb_expert_ffn_device(c.ctx, None, p, p, p, p, p, 1),
+        copy_16=lambda: l.eb_copy(c.ctx, None, p, p + 4096, 48),
+        copy_4=lambda: l.eb_copy(c.ctx, None, p + 4, p + 4096, 48),
+        copy_1=lambda: l.eb_copy(c.ctx, None, p, p + 4096, 47),
         combine=lambda: l.eb_combine(c.ctx, None, ref, p, p, p, p, p),
         step=lambda: c.step(n_mb, tokens),
         step_host=lambda: l.eb_step_host(c.ctx, None, ref, b.pool_mask, 1, 0, C.byref(c.bufs), p, p, p, None),
@@ -111,3 +115,66 @@ def test_nothing_is_launched_behind_a_refused_kernel(lib, n_mb, tokens, timing):
             assert c.names() == chain[:i], (name, chain[i])
             lib.fake_reset(-1)
             assert call() == 0 and c.names() == chain, (name, chain[i], "afterwards")
+
+
+def test_the_library_finds_every_runtime_function_in_the_stand_in(lib):
+    """Nothing of the real runtime, which torch may have put in reach, is called in its place."""
+    r = subprocess.run(["nm", "-D", "--undefined-only", lib._name], capture_output=True, text=True)
+    assert r.returncode == 0
+    assert [n for n in r.stdout.split() if n.startswith(("cuda", "__cuda", "cu"))] == []
+
+
+def test_copies_look_at_their_arguments(lib):
+    lib.fake_reset(-1)
+    c = Context(lib, E=8, K=2, S=1, D=4, max_tokens=64)
+    assert lib.eb_copy(None, None, 16, 32, 4) == 1
+    assert lib.eb_copy(c.ctx, None, None, 32, 4) == 1 and lib.eb_copy(c.ctx, None, 16, None, 4) == 1
+    assert lib.eb_copy(c.ctx, None, None, None, 0) == 0 and c.names() == []
+
+
+def _wait(c, ticket, n_mb=4, res=1 << 30, load=1 << 30):
+    h, ld = B.EbSchedResult(), (C.c_int32 * (16 * c.D))()
+    code = c.lib.eb_schedule_wait(c.ctx, None, ticket, n_mb, res, load, C.addressof(h), C.addressof(ld))
+    return code, h, ld
+
+
+def test_watched_schedules_keep_their_contract(lib):
+    """Which tickets can be waited for, and when the device's buffers are fallen back on (the stand-in's copies leave the result
+    as it was: zeros), when the record is read."""
+    lib.fake_reset(-1)
+    c = Context(lib, E=8, K=2, S=1, D=4, max_tokens=4096)
+    INVALID, UNSUPPORTED = 1, 2
+    assert lib.eb_watch_schedule(None, 1) == INVALID
+    assert _wait(c, 5)[0] == INVALID                     # nothing was ever watched
+    assert lib.eb_watch_schedule(c.ctx, 0) == 0 and _wait(c, 5)[0] == INVALID
+    assert lib.eb_watch_schedule(c.ctx, 5) == 0
+    assert _wait(c, 0)[0] == INVALID and _wait(c, 6)[0] == INVALID
+    assert _wait(c, 5, res=None)[0] == INVALID and _wait(c, 5, load=None)[0] == INVALID
+    assert _wait(c, 5, n_mb=17)[0] == UNSUPPORTED and _wait(c, 5, n_mb=-1)[0] == UNSUPPORTED
+    assert _wait(c, 5)[0] == 0                           # nothing was launched: the stream is idle
+    assert lib.eb_watch_schedule(c.ctx, 6) == 0
+    assert _wait(c, 5)[0] == INVALID                     # its record may be written over
+    # captured, refused: no mark is on its way
+    lib.fake_capturing(1)
+    assert c.step(4, 3) == 0 and _wait(c, 6)[0] == 0
+    lib.fake_capturing(0)
+    lib.fake_reset(-1)
+    assert c.step(4, 3) == 0
+    chain = c.names()
+    scatter = [i for i, n in enumerate(chain) if "scatter" in n][0]
+    assert lib.eb_watch_schedule(c.ctx, 7) == 0
+    lib.fake_reset(scatter)
+    assert c.step(4, 3) == EB_ERR_CUDA and _wait(c, 7)[0] == 0
+    # launched: the mark is waited for, and the record is what comes back
+    lib.fake_reset(-1)
+    for call in (lambda: c.step(4, 3), _calls(c, 4, 3)["schedule"]):
+        assert lib.eb_watch_schedule(c.ctx, 8) == 0
+        assert call() == 0
+        words = (C.c_uint32 * (24 + 256 + 1)).from_address(lib.fake_host_memory())
+        assert words[280] == 0
+        words[0], words[24], words[39], words[280] = 0xb, 41, 43, 8
+        code, h, ld = _wait(c, 8)
+        assert code == 0 and h.run_mask == 0xb and ld[0] == 41 and ld[15] == 43 and ld[16] == 0
+    assert lib.eb_watch_schedule(c.ctx, 0) == 0 and _wait(c, 8)[0] == 0      # the mark stays
+    assert lib.eb_watch_schedule(c.ctx, 8) == 0 and words[280] == 0          # and is cleared with the next ticket
+    assert lib.eb_destroy(c.ctx) == 0 and lib.fake_host_memory() is None
