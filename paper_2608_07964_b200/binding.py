@@ -287,13 +287,15 @@ class MoEStep:
         """With a ticket other than 0 the schedules of this context are left in host memory too, see `schedule_wait`."""
         self._check(self.lib.eb_watch_schedule(self.ctx, ticket))
 
-    def schedule_wait(self, ticket: int, n_mb: int) -> Dict:
+    def schedule_wait(self, ticket: int, n_mb: int, mb_load: Optional[torch.Tensor] = None) -> Dict:
         """The schedule marked with `ticket` as soon as it is made, whatever the step has yet to do; with the load vectors it was
-        made from under "loads".  `ticket` is the last one that was set."""
+        made from under "loads".  `ticket` is the last one that was set; `mb_load` are the loads that eb_schedule was given, if they
+        were not the step's own: without a mark (a schedule that was not watched) they are read from there."""
         if not hasattr(self, "_wait_res"):
             self._wait_res, self._wait_load = EbSchedResult(), (C.c_int32 * (EB_MAX_MB * self.D))()
         h, ld = self._wait_res, self._wait_load
-        self._check(self.lib.eb_schedule_wait(self.ctx, _stream(), ticket, n_mb, self.sched.data_ptr(), self.mb_load.data_ptr(),
+        src = self.mb_load if mb_load is None else mb_load
+        self._check(self.lib.eb_schedule_wait(self.ctx, _stream(), ticket, n_mb, self.sched.data_ptr(), src.data_ptr(),
                                               C.addressof(h), C.addressof(ld)))
         self._waited = ticket
         res = _sched_dict(h, self.D)

@@ -263,3 +263,17 @@ def test_the_record_is_what_the_kernels_left_in_host_memory(how, n_mb, tokens, m
     step.eb_step(batch, m, policy)
     got, loads = _record(step, 90, n_mb)
     assert got["n_run"] == -7 and loads == [[-7] * step.D] * n_mb
+
+
+@pytest.mark.parametrize("watched", [True, False])
+def test_the_loads_are_those_the_schedule_was_made_from(watched):
+    B, step = _step(4, 16)
+    batch = B.Batch([0, 16, 32, 48, 64], [0, 1, 2, 0])
+    step.eb_step(batch, 3)
+    other = torch.arange(16 * step.D, dtype=torch.int32, device="cuda").view(16, step.D) % 11
+    step.watch_schedule(70)
+    if not watched:
+        step.watch_schedule(0)
+    step.eb_schedule(batch, 3, mb_load=other)
+    got = step.schedule_wait(70, 4, mb_load=other)
+    assert got.pop("loads") == other[:4].cpu().tolist() and got == step.sched_result()
