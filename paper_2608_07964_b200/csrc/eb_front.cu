@@ -506,9 +506,10 @@ constexpr int kSumsWords = 65536;
 constexpr int kSumsChunks = 64;
 
 // tables_kernel runs on several blocks when the others take at least this many subsets of a MaxUtil schedule off the first:
-// below, meeting in memory (1-3 us) costs more than it saves.  Steps on one / several blocks (us, 16 x 1 tokens, 64 experts):
-// pool of 16, m = 12 (2517 subsets) 41.5 / 41.6, m = 8 (39203) 57.0 / 43.6, m = 1 (65535) 67.5 / 44.4; pool of 14 (two blocks),
-// m = 8 (9908) 41.6 / 42.4, m = 6 (14913) 43.8 / 43.3.  256 experts, pool of 16, m = 1: 102.1 / 55.0.
+// below, meeting in memory (0.6 to 1.4 us) costs more than it saves.  Steps on one / several blocks (us, 16 x 1 tokens, 64 experts):
+// pool of 16 (eight blocks), m = 11 (6885 subsets) 33.5 / 32.2, m = 8 (39203) 46.2 / 32.5, m = 1 (65535) 56.6 / 33.0; pool of 15
+// (four), m = 10 (4944) 31.2 / 31.9, m = 9 (9949) 32.7 / 31.7; pool of 14 (two), m = 8 (6476) 30.6 / 31.2, m = 6 (12911) 32.5 /
+// 31.4.  256 experts: pool of 16, m = 1 62.8 / 39.0, m = 11 40.1 / 38.0; pool of 15, m = 10 37.8 / 37.9; pool of 14, m = 8 37.3 / 38.4.
 constexpr int kSchedSubsets = 5000;
 
 constexpr size_t tables_smem(int n_mb, int E, int groups) {

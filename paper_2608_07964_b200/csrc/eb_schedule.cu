@@ -58,7 +58,7 @@ extern "C" eb_status eb_schedule(eb_ctx* c, void* stream, const eb_batch* batch,
 }
 
 // Algorithm-1 loops wait for a schedule at every step.  Two blocking copies (result, loads) took 59 us of a scheduling step
-// together with the kernels, the record that the kernel writes to host memory 30.
+// together with the kernels (eb_route's two and eb_schedule's), the record that the kernel leaves in host memory 30.
 extern "C" eb_status eb_watch_schedule(eb_ctx* c, uint32_t ticket) {
   if (!c) return EB_ERR_INVALID_ARG;
   if (eb_status ds = ebi_check_device(c)) return ds;
