@@ -21,7 +21,7 @@ schedule_kernel(int D, int n_mb, uint32_t pool_mask, int m, int policy, const in
   schedule_prepare(s, pool_mask, m, policy);
   const bool any_wide = __syncthreads_or(wide_load(load));
   uint32_t run;
-  if (!schedule_grid(s, D, pool_mask, m, policy, any_wide, grid, &run)) return;
+  if (!schedule_grid<true>(s, D, pool_mask, m, policy, any_wide, grid, &run)) return;
   if (tid < 32) {
     write_schedule(s, D, pool_mask, run, res);
     if (watch.rec) {

@@ -346,6 +346,9 @@ __device__ __forceinline__ Cand maxutil_halves(const SchedShared& s, int D, int 
 __host__ __device__ __forceinline__ bool few_out(int np, int m, int policy) {
   return policy == EB_POLICY_MAXUTIL && np > 10 && np - m > (np < 13 ? 13 - np : 0) && np - m <= kFewOut;
 }
+// Whether a schedule goes through the subsets of more than 10 members.  What does not is spared their code (kLarge = false): the code
+// of a kernel that runs once per step comes from far away, and what lies between costs even what never runs.
+__host__ __device__ __forceinline__ bool large_pool(int np, int m, int policy) { return policy == EB_POLICY_MAXUTIL && np > 10 && np > m; }
 // Which micro-batches are in the pool, and the tables that the schedule takes; before the barrier behind the writes of s.load.
 __device__ __forceinline__ void schedule_prepare(SchedShared& s, uint32_t pool_mask, int m, int policy) {
   const int tid = threadIdx.x;
@@ -357,8 +360,10 @@ __device__ __forceinline__ void schedule_prepare(SchedShared& s, uint32_t pool_m
 __device__ __forceinline__ bool wide_load(int v) { return v < 0 || v > kNarrowLoad; }
 
 // Chooses the run set from s.load and returns it.  All kSchedThreads threads of the block call it after a barrier behind the writes
-// of s.load and schedule_prepare; `any_wide` (uniform) unless no load is a wide_load; `block` of n_blocks.  With n_blocks > 1, which
-// is for MaxUtil over a large pool, s.best[0] is this block's candidate.  Ends with a barrier.
+// of s.load and schedule_prepare; `any_wide` (uniform) unless no load is a wide_load; `block` of n_blocks; kLarge unless the schedule is
+// no large_pool.  With n_blocks > 1, which is for MaxUtil over a large pool, s.best[0] is this block's candidate.  Ends with a
+// barrier.
+template <bool kLarge>
 __device__ __forceinline__ uint32_t schedule_block(SchedShared& s, int D, uint32_t pool_mask, int m, int policy, bool any_wide, int block, int n_blocks) {
   const int tid = threadIdx.x;
   const int np = __popc(pool_mask);
@@ -368,7 +373,7 @@ __device__ __forceinline__ uint32_t schedule_block(SchedShared& s, int D, uint32
   }
   if (policy == EB_POLICY_MAXUTIL) {
     Cand best;
-    if (np <= 10) {
+    if (!kLarge || np <= 10) {
       best = any_wide ? maxutil_small<long long>(s, D, np, m) : maxutil_small<int>(s, D, np, m);
     } else if (few_out(np, m, policy)) {
       int* pairs = reinterpret_cast<int*>(s.lo);
@@ -498,10 +503,11 @@ struct SchedGrid {
   Cand* best;          // [gridDim.x]
   unsigned* arrived;
 };
+template <bool kLarge>
 __device__ __forceinline__ bool schedule_grid(SchedShared& s, int D, uint32_t pool_mask, int m, int policy, bool any_wide, const SchedGrid& g,
                                               uint32_t* run) {
-  *run = schedule_block(s, D, pool_mask, m, policy, any_wide, blockIdx.x, gridDim.x);
-  if (gridDim.x == 1) return true;
+  *run = schedule_block<kLarge>(s, D, pool_mask, m, policy, any_wide, blockIdx.x, gridDim.x);
+  if (!kLarge || gridDim.x == 1) return true;
   const int tid = threadIdx.x;
   if (tid == 0) {
     g.best[blockIdx.x] = s.best[0];

@@ -73,7 +73,7 @@ def test_halves_by_one_block_and_by_several(members, m):
             _same(got, ref, by, D, top, loads.tolist())
 
 
-@pytest.mark.parametrize("members,out", [(3, 1), (5, 4), (8, 2), (10, 3), (10, 9), (11, 2), (12, 4), (16, 4), (11, 5), (16, 6)])
+@pytest.mark.parametrize("members,out", [(3, 1), (5, 4), (8, 2), (10, 0), (10, 3), (10, 9), (11, 0), (11, 1), (11, 2), (12, 4), (16, 0), (16, 4), (11, 5), (16, 6)])
 @pytest.mark.parametrize("top", [1 << 11, 1 << 21, 1 << 22, (1 << 22) + 1, 1 << 25])
 def test_subsets_that_are_nearly_equal(members, out, top):
     """Members that are equal or differ by one on one device: quotients that floating point cannot tell apart, or rounds the wrong way
